@@ -3,6 +3,7 @@
 // idkm_kernels.cuh; nothing here computes on the data.
 #include <nvtx3/nvToolsExt.h>
 #include "idkm_kernels.cuh"
+#include "idkm_scalar.cuh"
 
 #include <math.h>
 #include <stdio.h>
@@ -33,37 +34,51 @@ extern const DualEntry k_table_dual_delta[3][2];
 extern const KernelEntry k_table_step_delta[3][N_FAMILY];
 extern const KernelEntry k_table_step_bulk[3][N_FAMILY];
 
-// Initialise the per-layer state and copy C0 into the working centroids.
-__global__ void idkm_init_forward(LayerState* st, int n_layers, const float* C0, float* C, int n_coord, int k, int d,
-                                  double inv_tau, unsigned int* gtickets, int n_groups, unsigned int* sync,
-                                  unsigned int* gtickets64, int n_groups64, int squared) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  for (int o = i; o < n_groups; o += gridDim.x * blockDim.x) gtickets[o] = 0u;
-  for (int o = i; o < n_groups64; o += gridDim.x * blockDim.x) gtickets64[o] = 0u;
+// Initialise the per-layer state and copy C0 into the working centroids: one block per layer (the bounding box of 1024
+// coordinates by one thread took 9 us).
+constexpr int INIT_T = 256;
+__global__ void __launch_bounds__(INIT_T) idkm_init_forward(LayerState* st, int n_layers, const float* C0, float* C, int k, int d,
+                                                            double inv_tau, unsigned int* gtickets, int n_groups, unsigned int* sync,
+                                                            unsigned int* gtickets64, int n_groups64, int squared) {
+  const int l = blockIdx.x, tid = threadIdx.x, all = gridDim.x * INIT_T, i = l * INIT_T + tid;
+  for (int o = i; o < n_groups; o += all) gtickets[o] = 0u;
+  for (int o = i; o < n_groups64; o += all) gtickets64[o] = 0u;
   if (i < 4) sync[i] = 0u;
-  if (i < n_layers) {
+  // bounding box of the starting centroids decides which step kernel takes the layer first; thread t keeps coordinate
+  // t % d (INIT_T is a multiple of d)
+  __shared__ float s_lo[INIT_T], s_hi[INIT_T];
+  float lo = 3.0e38f, hi = -3.0e38f;
+  for (int o = tid; o < k * d; o += INIT_T) {
+    const float v = C0[(size_t)l * k * d + o];
+    lo = fminf(lo, v);
+    hi = fmaxf(hi, v);
+    if (C0 != C) C[(size_t)l * k * d + o] = v;
+  }
+  s_lo[tid] = lo;
+  s_hi[tid] = hi;
+  __syncthreads();
+  for (int s = INIT_T / 2; s >= d; s >>= 1) {
+    if (tid < s) {
+      s_lo[tid] = fminf(s_lo[tid], s_lo[tid + s]);
+      s_hi[tid] = fmaxf(s_hi[tid], s_hi[tid + s]);
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    double box2 = 0.0;
+    for (int a = 0; a < d; ++a) {
+      const double e = (double)s_hi[a] - (double)s_lo[a];
+      box2 += e * e;
+    }
     LayerState s;
     s.fwd_done = 0; s.fwd_iters = 0; s.fwd_res = 0.f; s.dead = 0;
     s.adj_done = 0; s.adj_iters = 0; s.adj_res = 0.f; s.status = ST_OK;
     s.ticket = 0u; s.adj_up = 0; s.adj_prev = 3.0e38f;
     s.g_norm = 0.f;
     for (int q = 0; q < 2; ++q) s.pad[q] = 0;
-    // bounding box of the starting centroids decides which step kernel takes the layer first
-    double box2 = 0.0;
-    for (int a = 0; a < d; ++a) {
-      double lo = 1e300, hi = -1e300;
-      for (int j = 0; j < k; ++j) {
-        const double v = (double)C0[((size_t)i * k + j) * d + a];
-        lo = fmin(lo, v);
-        hi = fmax(hi, v);
-      }
-      box2 += (hi - lo) * (hi - lo);
-    }
     s.precise[0] = s.precise[1] = (!squared && sqrt(box2) * inv_tau <= PRECISE_SPAN) ? 1 : 0;
-    st[i] = s;
+    st[l] = s;
   }
-  if (C0 != C)
-    for (int o = i; o < n_coord; o += gridDim.x * blockDim.x) C[o] = C0[o];
 }
 
 static int d_index(int d) { return d == 1 ? 0 : (d == 2 ? 1 : (d == 4 ? 2 : -1)); }
@@ -165,7 +180,17 @@ struct WorkspaceLayout {
   size_t off_rowstat;   // two floats per weight-vector, or NO_ROWSTAT
   size_t off_partials64, off_gpartials64, off_gtickets64;   // second set for the fp64 half of the dual step kernel
   int max_slots, max_groups, max_groups64;
+  // scalar weights (idkm_scalar.cuh); sc_fine = 0: none
+  size_t off_sc_sync, off_sc_gcount, off_sc_fstart, off_sc_frec, off_sc_crec, off_sc_bstat, off_sc_tab, off_sc_perm, off_sc_ftab,
+      off_sc_gpart, off_sc_gtick;
+  int sc_fine, n_sc_groups, n_sc_grad_blocks;
 };
+
+// Fine bins the workspace holds for n_layers layers of scalar weights: the largest layers get more.
+static int scalar_fine_total(int n_layers) {
+  const int big = n_layers < SC_BIG_LAYERS ? n_layers : SC_BIG_LAYERS;
+  return big * SC_FINE_BIG + (n_layers - big) * SC_FINE_SMALL;
+}
 
 constexpr size_t NO_ROWSTAT = ~(size_t)0;
 
@@ -233,6 +258,25 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
       o = align_up(o + sizeof(float2) * (size_t)m_total, 256);
     }
   }
+  w.sc_fine = 0;
+  if (d == 1) {
+    const int L = n_layers, K1 = k + 1;
+    const size_t nf = (size_t)scalar_fine_total(L);
+    w.sc_fine = (int)nf;
+    w.n_sc_grad_blocks = 2 * sms + L;
+    w.n_sc_groups = w.n_sc_grad_blocks / RED_GROUP + 2 * L + 2;
+    w.off_sc_sync = o;   o = align_up(o + 4 * (size_t)L * SC_SYNC_WORDS, 256);
+    w.off_sc_gcount = o; o = align_up(o + 4 * nf, 256);
+    w.off_sc_fstart = o; o = align_up(o + 4 * (nf + L), 256);
+    w.off_sc_frec = o;   o = align_up(o + 32 * nf, 256);
+    w.off_sc_crec = o;   o = align_up(o + SC_REC_BYTES * nf + 16 * (size_t)L, 256);
+    w.off_sc_bstat = o;  o = align_up(o + 16 * (size_t)(sms + L), 256);
+    w.off_sc_tab = o;    o = align_up(o + 8 * (size_t)L * SC_NTAB * K1, 256);
+    w.off_sc_perm = o;   o = align_up(o + 4 * (size_t)L * k, 256);
+    w.off_sc_ftab = o;   o = align_up(o + 4 * (size_t)L * SC_NFTAB * K1, 256);
+    w.off_sc_gpart = o;  o = align_up(o + 8 * (size_t)(w.n_sc_grad_blocks + w.n_sc_groups) * 3 * K1, 256);
+    w.off_sc_gtick = o;  o = align_up(o + 4 * (size_t)w.n_sc_groups, 256);
+  }
   w.total = o;
   *out = w;
   return true;
@@ -248,6 +292,7 @@ struct idkm_ctx {
   int64_t launches;
   // last forward
   bool have_forward;
+  bool scalar_forward;   // the last forward ran in the interval form for scalar weights and left its tables in the workspace
   const float* W;
   float* C;
   void* workspace;
@@ -588,6 +633,135 @@ static int try_small_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPa
   return IDKM_OK;
 }
 
+// ---- scalar weights in the interval form (idkm_scalar.cuh) ----
+static void scalar_params(const idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, ScalarParams* sp) {
+  memset(sp, 0, sizeof(*sp));
+  char* ws = static_cast<char*>(ctx->workspace);
+  ScalarPtrs& q = sp->p;
+  q.W = ctx->W;
+  q.G = p.G;
+  q.C = ctx->C;
+  q.S = p.S;
+  q.F = p.F;
+  q.gvec = p.gvec;
+  q.u = p.u;
+  q.st = p.st;
+  q.hist_fwd = p.hist_fwd;
+  q.hist_adj = p.hist_adj;
+  q.sync = reinterpret_cast<unsigned int*>(ws + wl.off_sc_sync);
+  q.gcount = reinterpret_cast<unsigned int*>(ws + wl.off_sc_gcount);
+  q.fstart = reinterpret_cast<unsigned int*>(ws + wl.off_sc_fstart);
+  q.frec = reinterpret_cast<long long*>(ws + wl.off_sc_frec);
+  q.crec = reinterpret_cast<unsigned char*>(ws + wl.off_sc_crec);
+  q.bstat = reinterpret_cast<float4*>(ws + wl.off_sc_bstat);
+  q.tab = reinterpret_cast<double*>(ws + wl.off_sc_tab);
+  q.perm = reinterpret_cast<int*>(ws + wl.off_sc_perm);
+  q.ftab = reinterpret_cast<float*>(ws + wl.off_sc_ftab);
+  q.gpart = reinterpret_cast<double*>(ws + wl.off_sc_gpart);
+  q.gtick = reinterpret_cast<unsigned int*>(ws + wl.off_sc_gtick);
+  q.pair_ticks[0] = p.gtickets;
+  q.n_pair_ticks[0] = wl.max_groups;
+  q.pair_ticks[1] = reinterpret_cast<unsigned int*>(ws + wl.off_gtickets64);
+  q.n_pair_ticks[1] = wl.max_groups64;
+  sp->n_group_rows = wl.n_sc_groups;
+  sp->n_layers = ctx->n_layers;
+  sp->k = ctx->k;
+  sp->inv_tau_d = p.inv_tau_d;
+  sp->tol = p.tol;
+  sp->alpha = p.alpha;
+  sp->max_iter = p.max_iter;
+  sp->wq_dtype = ctx->wq_dtype;
+  const int L = ctx->n_layers;
+  for (int l = 0; l <= MAX_LAYERS; ++l) sp->row_off[l] = ctx->row_off[l < L ? l : L];
+  // fine bins: the SC_BIG_LAYERS largest layers get the larger share
+  for (int l = 0; l < L; ++l) {
+    const long long rows = ctx->row_off[l + 1] - ctx->row_off[l];
+    int larger = 0;
+    if (L > SC_BIG_LAYERS)
+      for (int o = 0; o < L; ++o) {
+        const long long r = ctx->row_off[o + 1] - ctx->row_off[o];
+        larger += (r > rows || (r == rows && o < l));
+      }
+    sp->fine_off[l + 1] = sp->fine_off[l] + (larger < SC_BIG_LAYERS ? SC_FINE_BIG : SC_FINE_SMALL);
+  }
+  for (int l = L + 1; l <= MAX_LAYERS; ++l) sp->fine_off[l] = sp->fine_off[L];
+}
+
+// Deals at most `grid` >= n_layers blocks to the layers: one each, the rest in proportion to the rows, none with fewer
+// than `min_rows`; returns the grid used.
+static int scalar_deal(ScalarParams* sp, int grid, long long min_rows) {
+  const int L = sp->n_layers;
+  const long long m = sp->row_off[L];
+  sp->blk_first[0] = 0;
+  const long long spare = grid - L;
+  for (int l = 0; l < L; ++l) {
+    const long long rows = sp->row_off[l + 1] - sp->row_off[l];
+    long long n = 1 + spare * rows / m;
+    const long long most = (rows + min_rows - 1) / min_rows;
+    if (n > most) n = most;
+    sp->blk_first[l + 1] = sp->blk_first[l] + (int)n;
+  }
+  for (int l = L + 1; l <= MAX_LAYERS; ++l) sp->blk_first[l] = sp->blk_first[L];
+  return sp->blk_first[L];
+}
+
+constexpr long long SCALAR_LOOP_ROWS = 8192;    // weights a block of the loop kernel summarises at least
+constexpr long long SCALAR_PASS_ROWS = 1024;    // ... of a streaming pass
+constexpr long long SCALAR_GRAD_ROWS = 256;     // weights a thread of the gradient pass takes before more blocks are used
+
+// Initialises the call and runs the forward loop in the interval form.  IDKM_OK after queueing it, 1 if this problem
+// takes another path.  scratch: room for two bytes per weight.
+static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, const float* C0, int max_iter, void* scratch) {
+  if (wl.sc_fine == 0 || ctx->squared || ctx->forward_loop != 0 || ctx->collapse_step != 0 || max_iter < 2 || scratch == nullptr ||
+      ctx->n_layers > ctx->sms)
+    return 1;
+  for (int l = 0; l < ctx->n_layers; ++l)
+    if (ctx->row_off[l + 1] - ctx->row_off[l] > 0x7fffffffLL) return 1;
+  ScalarParams sp;
+  scalar_params(ctx, wl, p, &sp);
+  sp.p.C0 = C0;
+  sp.p.grouped = static_cast<unsigned short*>(scratch);
+  const int grid = scalar_deal(&sp, ctx->sms, SCALAR_LOOP_ROWS);
+  sp.missing_arrivals = ctx->hook_missing_arrivals;
+  sp.spin_limit = SMALL_SPIN_LIMIT;
+  if (ctx->hook_spin_limit > 0 && ctx->hook_spin_limit < SMALL_SPIN_LIMIT) sp.spin_limit = ctx->hook_spin_limit;
+  if (launch_scalar_init(sp, grid, ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
+  mark(ctx, 1);
+  if (launch_scalar_loop(sp, grid, ctx->stream) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 1;   // the loop was not queued: the other paths start from their own initialisation
+  }
+  ctx->launches += 2;
+  ctx->scalar_forward = true;
+  return IDKM_OK;
+}
+
+enum ScalarPass { SP_FINAL, SP_GRAD, SP_ADJOINT, SP_DW };
+static int launch_scalar_pass(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, ScalarPass which, float* dC_out) {
+  ScalarParams sp;
+  scalar_params(ctx, wl, p, &sp);
+  sp.p.Wq = p.Wq;
+  sp.p.dW = p.dW;
+  sp.p.dC = dC_out;
+  cudaError_t rc = cudaSuccess;
+  switch (which) {
+    case SP_FINAL: rc = launch_scalar_final(sp, scalar_deal(&sp, ctx->sms * 8 + ctx->n_layers, SCALAR_PASS_ROWS), ctx->stream); break;
+    case SP_DW: rc = launch_scalar_dw(sp, scalar_deal(&sp, ctx->sms * 8 + ctx->n_layers, SCALAR_PASS_ROWS), ctx->stream); break;
+    case SP_GRAD: {
+      long long grid = ctx->m_total / (SCALAR_GRAD_ROWS * scalar_grad_threads(ctx->k));
+      if (grid < ctx->sms) grid = ctx->sms;
+      if (grid > 2 * ctx->sms) grid = 2 * ctx->sms;
+      if (grid < ctx->n_layers) grid = ctx->n_layers;
+      rc = launch_scalar_grad(sp, scalar_deal(&sp, (int)grid, SCALAR_PASS_ROWS), ctx->stream);
+      break;
+    }
+    case SP_ADJOINT: rc = launch_scalar_adjoint(sp, ctx->stream); break;
+  }
+  if (rc != cudaSuccess) return IDKM_ERR_CUDA;
+  ++ctx->launches;
+  return IDKM_OK;
+}
+
 static int launch_pass(idkm_ctx* ctx, int mode, PassParams* p, int repeat) {
   const int f = pick_family(mode, ctx->d, ctx->k);
   const KernelEntry* e = ctx_entry(ctx, mode, f);
@@ -605,11 +779,11 @@ static int launch_pass(idkm_ctx* ctx, int mode, PassParams* p, int repeat) {
 }
 
 // The last phase of a backward: the pass that writes dL/dW from the adjoint u in the workspace, and the copy of u.
-static int backward_outputs(idkm_ctx* ctx, PassParams* p, float* dW_out, float* dC_out) {
+static int backward_outputs(idkm_ctx* ctx, const WorkspaceLayout& wl, PassParams* p, bool scalar, float* dW_out, float* dC_out) {
   if (dW_out) {
     p->dW = dW_out;
     nvtxRangePushA("idkm dL/dW pass");
-    const int rc = launch_pass(ctx, SCATTER, p, 1);
+    const int rc = scalar ? launch_scalar_pass(ctx, wl, *p, SP_DW, nullptr) : launch_pass(ctx, SCATTER, p, 1);
     nvtxRangePop();
     if (rc != IDKM_OK) return rc;
   }
@@ -718,27 +892,32 @@ int idkm_forward_batched(idkm_ctx* ctx, const float* W_cat, const int64_t* layer
 
   ctx->ev_fwd_set = ctx->ev_bwd_set = false;
   mark(ctx, 0);
-  const int n_coord = n_layers * k * d;
-  const int init_threads = n_coord > n_layers ? n_coord : n_layers;
-  idkm_init_forward<<<(init_threads + 255) / 256, 256, 0, ctx->stream>>>(p.st, n_layers, C0, C_out, n_coord, k, d,
-                                                                                     p.inv_tau_d, p.gtickets, wl.max_groups,
-                                                                                     reinterpret_cast<unsigned int*>(static_cast<char*>(workspace) + wl.off_sync),
-                                                                                     reinterpret_cast<unsigned int*>(static_cast<char*>(workspace) + wl.off_gtickets64),
-                                                                                     wl.max_groups64, ctx->squared);
-  if (cudaGetLastError() != cudaSuccess) return IDKM_ERR_CUDA;
-  ++ctx->launches;
-  mark(ctx, 1);
-
   nvtxRangePushA("idkm forward loop");
-  int rc = try_small_loop(ctx, wl, p, max_iter);
-  if (rc == 1) rc = launch_step_loop(ctx, wl, &p, max_iter);
+  ctx->scalar_forward = false;
+  // scratch of the interval form: the buffer of Wq, which the final pass overwrites; without Wq the row cache of the
+  // backward, if there is one and no other one-launch loop takes the codebook
+  void* scratch = Wq_out ? static_cast<void*>(Wq_out) : (k > 16 ? static_cast<void*>(p.rowstat) : nullptr);
+  int rc = try_scalar_loop(ctx, wl, p, C0, max_iter, scratch);
+  if (rc == 1) {
+    char* wsb = static_cast<char*>(workspace);
+    idkm_init_forward<<<n_layers, INIT_T, 0, ctx->stream>>>(p.st, n_layers, C0, C_out, k, d, p.inv_tau_d, p.gtickets, wl.max_groups,
+                                                            reinterpret_cast<unsigned int*>(wsb + wl.off_sync),
+                                                            reinterpret_cast<unsigned int*>(wsb + wl.off_gtickets64), wl.max_groups64,
+                                                            ctx->squared);
+    if (cudaGetLastError() != cudaSuccess) return IDKM_ERR_CUDA;
+    ++ctx->launches;
+    mark(ctx, 1);
+    rc = try_small_loop(ctx, wl, p, max_iter);
+    if (rc == 1) rc = launch_step_loop(ctx, wl, &p, max_iter);
+  }
   nvtxRangePop();
   if (rc != IDKM_OK) return rc;
   mark(ctx, 2);
   p.Wq = Wq_out;
   p.A = A_out;
   nvtxRangePushA("idkm final pass");
-  rc = launch_pass(ctx, FINAL, &p, 1);
+  if (!ctx->scalar_forward || A_out) rc = launch_pass(ctx, FINAL, &p, 1);
+  else if (Wq_out) rc = launch_scalar_pass(ctx, wl, p, SP_FINAL, nullptr);   // (S and F came with the loop)
   nvtxRangePop();
   if (rc != IDKM_OK) return rc;
   mark(ctx, 3);
@@ -788,14 +967,19 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
   // the per-row softmax reference and normaliser are kept only if fused adjoint passes follow
   if (!solve || explicit_jac) p.rowstat = nullptr;
   mark(ctx, 4);
+  // scalar weights whose forward left its interval tables: gradient, adjoint and dL/dW in the interval form, unless the
+  // caller asked for the fused passes (1) or the exact solve (2)
+  const bool scalar = ctx->scalar_forward && (ctx->adjoint_method == 0 || !solve);
   nvtxRangePushA("idkm codebook gradient");
-  int rc = launch_pass(ctx, GRAD, &p, 1);
+  int rc = scalar ? launch_scalar_pass(ctx, wl, p, SP_GRAD, dC_out) : launch_pass(ctx, GRAD, &p, 1);
   nvtxRangePop();
   if (rc != IDKM_OK) return rc;
   mark(ctx, 5);
   if (solve) {
     nvtxRangePushA("idkm adjoint solve");
-    if (explicit_jac) {
+    if (scalar) {
+      rc = launch_scalar_pass(ctx, wl, p, SP_ADJOINT, dC_out);
+    } else if (explicit_jac) {
       if (exact) p.max_iter = -1;                  // the epilogue solves (I - J^T) u = g instead of iterating
       rc = launch_pass(ctx, JACOBIAN, &p, 1);      // one pass forms J_C; the whole iteration runs on it in the epilogue
       p.max_iter = adj_max_iter;
@@ -806,7 +990,7 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
     if (rc != IDKM_OK) return rc;
   }
   mark(ctx, 6);
-  return backward_outputs(ctx, &p, dW_out, dC_out);
+  return backward_outputs(ctx, wl, &p, scalar, dW_out, scalar ? nullptr : dC_out);   // (the scalar passes wrote dC)
 }
 
 int idkm_backward_restart(idkm_ctx* ctx, const float* dWq, float adj_tol, int adj_max_iter, float alpha0,
@@ -840,7 +1024,7 @@ int idkm_backward_restart(idkm_ctx* ctx, const float* dWq, float adj_tol, int ad
   fill_params(ctx, wl, &p);
   p.G = dWq;
   p.alpha = alpha;
-  return backward_outputs(ctx, &p, dW_out, dC_out);
+  return backward_outputs(ctx, wl, &p, ctx->scalar_forward && ctx->adjoint_method == 0, dW_out, dC_out);
 }
 
 int idkm_get_info(idkm_ctx* ctx, idkm_info* info_out) {

@@ -1,0 +1,1526 @@
+// Algorithm 1's whole loop for scalar weights, without a pass over the weights per iteration.
+//
+// The weights do not change during the loop, so they are summarised once: every layer's value range is cut into coarse
+// bins about tau / 6 wide, each with its count and the first four moments of its weights about the bin's centre, and
+// lambda(w) -- a logistic function of 2 w / tau inside an interval between centroids -- is summed over a bin by its
+// Taylor series (at that width the first dropped term is below 1e-6 of lambda at a bin's very edge, odd, and 1e-8 on
+// average; the exponential of the direct path is an approximation to 2e-7).  Far from an interval's even point, where
+// lambda or mu is below 2^-96, whole runs of bins are taken from running sums.  A bin that contains a centroid is split
+// at it: the moments of the weights below the centroid are the prefix over the fine bins of the coarse bin plus the
+// weights of the one fine bin the centroid lies in, which are looked at one by one.  For that the weights' places are
+// grouped by fine bin (two bytes per weight).  Everything that is accumulated in an order that can vary is a sum of
+// integers, so results are reproducible although the grouping uses atomic counters.
+//
+// Several blocks per layer build the summary (meetings at a bounded barrier), then one block per layer runs the
+// iterations: one warp (or a few) per interval between centroids, the M-step by the first warps in fp64.
+#include "idkm_scalar.cuh"
+
+namespace idkm {
+
+// Value range -> bins.  Index arithmetic is one fused multiply-add per weight, rounded once.
+struct ScGrid {
+  double hf, hc;     // widths of fine and coarse bins
+  double ctr0;       // centre of coarse bin 0
+  double inv_hc, iF; // 1 / hc, 1 / F
+  float inv_hf;
+  float lo, hi;      // value range, centroids are clamped to it for the choice of a bin
+  int fshift, F;     // fine bins per coarse bin: F = 1 << fshift
+  int base_f;        // index of the first fine bin
+  int nc, nf;
+  float eta;         // 2 hc / tau: range of the logistic's argument across a coarse bin
+};
+constexpr float SC_MAGIC = 12582912.f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
+__device__ __forceinline__ int sc_round_index(float w, float inv_hf) {
+  return __float_as_int(fmaf(w, inv_hf, SC_MAGIC)) - 0x4B400000;
+}
+__device__ __forceinline__ int sc_fine(const ScGrid& g, float w) { return sc_round_index(w, g.inv_hf) - g.base_f; }
+// index and place (in 1 / SC_PSCALE of a fine bin, from its centre)
+__device__ __forceinline__ int sc_fine_place(const ScGrid& g, float w, int& place) {
+  const float f = fmaf(w, g.inv_hf, SC_MAGIC);
+  place = __float2int_rn(fmaf(w, g.inv_hf, -(f - SC_MAGIC)) * (float)SC_PSCALE);
+  return __float_as_int(f) - 0x4B400000 - g.base_f;
+}
+__device__ __forceinline__ double sc_center(const ScGrid& g, int c) { return fma((double)c, g.hc, g.ctr0); }
+
+__device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int cap) {
+  ScGrid g;
+  if (!(lo <= hi)) lo = hi = 0.f;   // no weight besides zeros
+  const double amax = fmax(fmax(fabs((double)lo), fabs((double)hi)), 1e-30);
+  double range = (double)hi - (double)lo;
+  if (!(range > amax * 1e-6)) range = amax * 1e-6;
+  const double hmin = amax * (1.0 / 2097152.0);   // indices stay below 2^21 in magnitude
+  double hc = 0.17 * tau;
+  if (hc < range / (double)(cap - 8)) hc = range / (double)(cap - 8);
+  if (hc > range) hc = range;
+  if (hc < hmin) hc = hmin;
+  // fine bins: about 64 weights each, at least 16 to a coarse bin (see sc_bin_below), as many as the workspace holds
+  const long long nc0 = (long long)(range / hc) + 5;
+  long long want = m / 64 < 512 ? 512 : m / 64;
+  if (want < 16 * nc0) want = 16 * nc0;
+  if (want > cap) want = cap;
+  int f = 0;
+  while (f < 12 && hc / (double)(2 << f) >= hmin && (nc0 << (f + 1)) <= want) ++f;
+  g.inv_hf = (float)((double)(1 << f) / hc);
+  g.hf = 1.0 / (double)g.inv_hf;
+  g.fshift = f;
+  g.F = 1 << f;
+  g.hc = g.hf * (double)g.F;
+  g.inv_hc = 1.0 / g.hc;
+  g.iF = 1.0 / (double)g.F;
+  g.base_f = sc_round_index(lo, g.inv_hf) - 1;
+  const int nfn = sc_round_index(hi, g.inv_hf) - g.base_f + 2;
+  g.nc = (nfn + g.F - 1) >> f;
+  g.nf = g.nc << f;
+  g.ctr0 = ((double)g.base_f + 0.5 * (double)(g.F - 1)) * g.hf;
+  g.lo = lo;
+  g.hi = hi;
+  g.eta = (float)(2.0 * g.hc / tau);
+  return g;
+}
+
+// Barrier among the blocks of one layer: sync[0] arrivals (only grows), sync[1] error word.  Bounded wait.  `stay`: this
+// block goes on afterwards (otherwise it only arrives).
+__device__ __forceinline__ bool sc_team_barrier(unsigned int* sync, unsigned int target, long long spin_limit, int* s_ok, bool stay) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    volatile unsigned int* vs = sync;
+    int ok = 1;
+    __threadfence();
+    atomicAdd(&sync[0], 1u);
+    if (stay) {
+      const long long t0 = clock64();
+      while ((int)(vs[0] - target) < 0) {
+        if (vs[1] != 0u || clock64() - t0 > spin_limit) {
+          atomicExch(&sync[1], 1u);
+          ok = 0;
+          break;
+        }
+      }
+      if (vs[1] != 0u) ok = 0;
+      __threadfence();
+    }
+    *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// Integer powers of a place p (|p| <= 32767): p^2 / 2^14, p^3 / 2^29, p^4 / 2^44, each at most 2^16.
+__device__ __forceinline__ void sc_powers(int p, int& p2, int& p3, int& p4) {
+  p2 = (p * p + 8192) >> 14;
+  p3 = (p2 * p + 16384) >> 15;
+  p4 = (int)(((unsigned)p2 * (unsigned)p2 + 32768u) >> 16);
+}
+constexpr double SC_S1 = 1.0 / (double)SC_PSCALE;
+constexpr double SC_S2 = 16384.0 * SC_S1 * SC_S1;
+constexpr double SC_S3 = 536870912.0 * SC_S1 * SC_S1 * SC_S1;
+constexpr double SC_S4 = 17592186044416.0 * SC_S1 * SC_S1 * SC_S1 * SC_S1;
+constexpr int SC_CHUNK = 8192;   // elements whose 32-bit integer sums cannot overflow
+
+// Moments about the coarse bin's centre, in units of the coarse width, of n weights of fine bin kf (0 .. F - 1) whose
+// integer sums of powers of the place are s1 .. s4.
+__device__ __forceinline__ void sc_shift(const ScGrid& g, double x0, double n, double s1, double s2, double s3, double s4, double (&M)[4]) {
+  const double iF = g.iF, iF2 = iF * iF;
+  const double d1 = s1 * (SC_S1 * iF), d2 = s2 * (SC_S2 * iF2), d3 = s3 * (SC_S3 * iF2 * iF), d4 = s4 * (SC_S4 * iF2 * iF2);
+  M[0] = fma(n, x0, d1);
+  M[1] = fma(x0, fma(n, x0, 2.0 * d1), d2);
+  M[2] = fma(x0, fma(x0, fma(n, x0, 3.0 * d1), 3.0 * d2), d3);
+  M[3] = fma(x0, fma(x0, fma(x0, fma(n, x0, 4.0 * d1), 6.0 * d2), 4.0 * d3), d4);
+}
+// a fine bin's centre from its coarse bin's, in units of the coarse width
+__device__ __forceinline__ double sc_fine_x0(const ScGrid& g, int f) { return ((double)(f & (g.F - 1)) - 0.5 * (double)(g.F - 1)) * g.iF; }
+
+// Coarse records: running count and x sum up to every bin (doubles, nc + 1), then count and moments (floats).
+struct ScRec {
+  double *cn, *cx;
+  float* r;      // [5][stride]
+  int stride;
+};
+
+__device__ __forceinline__ ScRec sc_global_rec(const ScalarParams& sp, int layer, int cap) {
+  ScRec r;
+  r.cn = reinterpret_cast<double*>(sp.p.crec + (size_t)sp.fine_off[layer] * SC_REC_BYTES + (size_t)layer * 16);
+  r.cx = r.cn + cap + 1;
+  r.r = reinterpret_cast<float*>(r.cx + cap + 1);
+  r.stride = cap;
+  return r;
+}
+
+// What the iterations of one layer's block need besides the shared struct.
+struct ScLayer {
+  const unsigned short* grouped;   // all layers' (16-byte aligned); this layer's weights start at element row0
+  long long row0, total;   // ... of `total` in all layers
+  const unsigned int* fstart;
+  const double* frec;   // [nf][4]: moments of the weights of earlier fine bins of the coarse bin
+  ScRec rec;
+  int k, twl, wl;       // 2^twl warps share an interval, 2^wl the fine bin of a centroid
+  double tau, inv_tau;
+  double zone;          // half-width of the zone: SC_ZONE / slope
+  float slope;          // 2 log2(e) / tau
+};
+
+constexpr int SC_PARTS = 512;   // (centroid, slot) pairs: a slot per warp of an interval and one for its two ends
+constexpr int SC_BELOW = 272;   // (centroid, warp) pairs of the scan of the centroids' fine bins
+struct ScShared {
+  ScGrid g;
+  ScLayer ly;              // (copy for the functions that are not inlined)
+  int ok, bad, flag, done, iters, dead, status;
+  float res;
+  long long n0;            // weights that are exactly zero (kept out of the bins)
+  float v[257];            // sorted centroids
+  int id[256];             // their indices
+  float vn[256];
+  int idn[256];
+  int fb[256], pv[256];    // fine bin and place of every centroid
+  double even[257];        // e_s of interval s = 1 .. k - 1
+  double bs[SC_BELOW][5];  // twice the sums over a centroid's fine bin below it (sc_bin_below)
+  double Ls[SC_PARTS][2];  // sums of lambda (and lambda x) over the interval right of a centroid, per slot
+  double Ms[SC_PARTS][2];  // ... of mu over the interval left of it
+  double Xs[SC_PARTS][2];  // ... of lambda mu over the interval right of it (last evaluation only)
+  double cnew[256], cold[256];   // the last M-step, for the stop test
+  int dead_j[256];
+  double qs[256];
+  double tmp[32];
+  unsigned int scan[SC_WARPS + 1];
+  double scan_x[SC_WARPS + 1];
+};
+constexpr int SC_SH_BYTES = (int)((sizeof(ScShared) + 255) / 256 * 256);
+constexpr int SC_DYN = SC_SH_BYTES + ((SC_FINE_BIG * 4 > SC_REC_SMEM * SC_REC_BYTES + 16) ? SC_FINE_BIG * 4 : SC_REC_SMEM * SC_REC_BYTES + 16);
+constexpr int SC_SMALL_NC = 512;       // layers of up to this many coarse bins leave room for their weights' places
+constexpr int SC_SMALL_OFF = (SC_SMALL_NC * SC_REC_BYTES + 16 + 15) / 16 * 16;
+static_assert(SC_DYN <= 227 * 1024, "shared memory of the loop kernel");
+
+// exp(x) for x <= 0 in fp64: 2^n times the Taylor polynomial of degree 10 on |f ln 2| <= 0.3466 (remainder below 3e-13
+// relative), evaluated by Estrin's scheme: half the latency of the library function, which is on the iteration's chain.
+__device__ __forceinline__ double sc_exp(double x) {
+  const double y = fmax(x * 1.4426950408889634, -1020.0);
+  const double n = rint(y);
+  const double t = (y - n) * 0.6931471805599453, t2 = t * t, t4 = t2 * t2;
+  const double p01 = 1.0 + t, p23 = fma(t, 1.0 / 6.0, 0.5), p45 = fma(t, 1.0 / 120.0, 1.0 / 24.0);
+  const double p67 = fma(t, 1.0 / 5040.0, 1.0 / 720.0), p89 = fma(t, 1.0 / 362880.0, 1.0 / 40320.0);
+  const double q0 = fma(t2, p23, p01), q1 = fma(t2, p67, p45), q2 = fma(t2, 1.0 / 3628800.0, p89);
+  const double r = fma(t4, fma(t4, q2, q1), q0);
+  return r * __hiloint2double((1023 + (int)n) << 20, 0);
+}
+// 1 / x: fp32 seed and two Newton steps
+__device__ __forceinline__ double sc_rcp(double x) {
+  double r = (double)rcp_approx((float)x);
+  r = r * fma(-x, r, 2.0);
+  return r * fma(-x, r, 2.0);
+}
+
+// The recurrences over at most 32 centroids, both directions at once, by one warp.  cb[l], cf[l]: products of 2^l
+// coefficients a_j going right from, resp. left to, this lane (zero where they run over the end).
+template <int LOG>
+struct ScScan {
+  double cb[LOG > 0 ? LOG : 1], cf[LOG > 0 ? LOG : 1];
+};
+template <int NX, int LOG>
+__device__ __forceinline__ void sc_scan_both(const ScScan<LOG>& c, double (&x)[NX] /* from the right */, double (&y)[NX] /* from the left */) {
+#pragma unroll
+  for (int l = 0; l < LOG; ++l) {
+    double xs[NX], ys[NX];
+#pragma unroll
+    for (int i = 0; i < NX; ++i) {
+      xs[i] = __shfl_down_sync(0xffffffffu, x[i], 1 << l);
+      ys[i] = __shfl_up_sync(0xffffffffu, y[i], 1 << l);
+    }
+#pragma unroll
+    for (int i = 0; i < NX; ++i) {
+      x[i] = fma(c.cb[l], xs[i], x[i]);
+      y[i] = fma(c.cf[l], ys[i], y[i]);
+    }
+  }
+}
+
+// Where a centroid lies among the bins, and the even point of the interval to its right (own threads).
+__device__ __forceinline__ void sc_place(ScShared& sh, const ScLayer& ly, int j, float vf, double v, double vx, double ratio) {
+  if (j + 1 < ly.k) sh.even[j + 1] = 0.5 * (v + vx) - 0.5 * ly.tau * (double)logf((float)ratio);
+  const ScGrid& g = sh.g;
+  int place;
+  const int fi = sc_fine_place(g, fminf(fmaxf(vf, g.lo), g.hi), place);
+  // one beyond the ends of the scale where the centroid lies outside the weights' range
+  if (vf > g.hi) place = 40000;
+  if (vf < g.lo) place = -40000;
+  sh.fb[j] = fi;
+  sh.pv[j] = place;
+}
+
+// Interval tables of the sorted centroids: a_j, 1 / P_j, 1 / Q_j of this thread's centroid, e_s, bins.  One warp, k <= 32.
+template <int LOG>
+__device__ __forceinline__ void sc_tables_warp(ScShared& sh, const ScLayer& ly, float vf, ScScan<LOG>& sc, double& rP, double& rQ) {
+  const int j = threadIdx.x, k = ly.k;
+  const bool own = j < k;
+  const double v = (double)vf, vx = (double)__shfl_down_sync(0xffffffffu, vf, 1);
+  const double a = j + 1 < k ? sc_exp((v - vx) * ly.inv_tau) : 0.0;
+  sc.cb[0] = a;
+  const double al = __shfl_up_sync(0xffffffffu, a, 1);
+  sc.cf[0] = (j > 0 && own) ? al : 0.0;
+  double P = 1.0, Q = 1.0;
+#pragma unroll
+  for (int l = 0; l < LOG; ++l) {
+    const double qs = __shfl_down_sync(0xffffffffu, Q, 1 << l), ps = __shfl_up_sync(0xffffffffu, P, 1 << l);
+    Q = fma(sc.cb[l], qs, Q);
+    P = fma(sc.cf[l], ps, P);
+    if (l + 1 < LOG) {
+      sc.cb[l + 1] = sc.cb[l] * __shfl_down_sync(0xffffffffu, sc.cb[l], 1 << l);
+      sc.cf[l + 1] = sc.cf[l] * __shfl_up_sync(0xffffffffu, sc.cf[l], 1 << l);
+    }
+  }
+  const double Qn = __shfl_down_sync(0xffffffffu, Q, 1);
+  rP = own ? sc_rcp(P) : 0.0;
+  rQ = own ? sc_rcp(Q) : 0.0;
+  if (own) sc_place(sh, ly, j, vf, v, vx, Qn * rP);
+}
+// The same for up to 256 centroids, by the first kw warps.
+__device__ __forceinline__ void sc_tables_block(ScShared& sh, const ScLayer& ly, double& a, double& ap, double& rP, double& rQ) {
+  const int j = threadIdx.x, k = ly.k, kw = (k + 31) >> 5;
+  const bool own = j < k;
+  const double v = own ? (double)sh.v[j] : 0.0;
+  const double vx = (own && j + 1 < k) ? (double)sh.v[j + 1] : v;
+  a = (own && j + 1 < k) ? sc_exp((v - vx) * ly.inv_tau) : 0.0;
+  ap = __shfl_up_sync(0xffffffffu, a, 1);
+  if ((j & 31) == 0) ap = (own && j > 0) ? sc_exp(((double)sh.v[j - 1] - v) * ly.inv_tau) : 0.0;
+  if (!own) ap = 0.0;
+  double x[1] = {own ? 1.0 : 0.0}, y[1] = {own ? 1.0 : 0.0};
+  lin_scan<1, true>(ap, x, k, sh.tmp);
+  lin_scan<1, false>(a, y, k, sh.tmp);
+  sc_sync(kw);
+  if (own) sh.qs[j] = y[0];
+  sc_sync(kw);
+  rP = own ? sc_rcp(x[0]) : 0.0;
+  rQ = own ? sc_rcp(y[0]) : 0.0;
+  if (own) sc_place(sh, ly, j, sh.v[j], v, vx, j + 1 < k ? sh.qs[j + 1] * rP : 1.0);
+}
+
+// Sorts the k centroids in vn / idn into v / id (first kw warps; NaN sorts last).
+__device__ __forceinline__ void sc_sort(ScShared& sh, int k) {
+  const int j = threadIdx.x, kw = (k + 31) >> 5;
+  if (j < k) {
+    const float x = sh.vn[j];
+    const float key = (x == x) ? x : __int_as_float(0x7f800000);
+    int r = 0;
+    for (int i = 0; i < k; ++i) {
+      const float y = sh.vn[i];
+      const float ky = (y == y) ? y : __int_as_float(0x7f800000);
+      r += (ky < key || (ky == key && i < j)) ? 1 : 0;
+    }
+    sh.v[r] = x;
+    sh.id[r] = sh.idn[j];
+  }
+  sc_sync(kw);
+}
+
+// Eight places starting at element e (a multiple of 8); past the last of `total` elements zeros.
+__device__ __forceinline__ uint4 sc_load8(const unsigned short* grouped, long long e, long long total) {
+  if (e + 8 <= total) return *reinterpret_cast<const uint4*>(grouped + e);
+  unsigned int x[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (e + i < total) x[i >> 1] |= (unsigned int)grouped[e + i] << (16 * (i & 1));
+  return make_uint4(x[0], x[1], x[2], x[3]);
+}
+
+// A fine bin as a warp sees it: up to SC_HEAD of its weights in registers (kept from one iteration to the next while the
+// centroid stays in the bin), the rest read again every time.
+constexpr int SC_HEAD = 248;
+struct ScBin {
+  int f;                  // fine bin, -1: none
+  int groups;             // of 32 weights in pe
+  int pe[8];              // places (40001: no weight)
+  long long t0, t1;       // the rest, as elements of `grouped` (t0 is a multiple of 8)
+};
+// (n warps share a bin: this one takes share `sub`, boundaries at multiples of 8)
+__device__ __forceinline__ void sc_bin_load(const ScLayer& ly, int f, unsigned int e0, unsigned int e1, int sub, int n, ScBin& bn) {
+  const int lane = threadIdx.x & 31;
+  bn.f = f;
+  long long A0 = ly.row0 + e0, A1 = ly.row0 + e1;
+  if (n > 1) {
+    const long long len = A1 - A0, b = A0, e = A1;
+    A0 = sub == 0 ? b : ((b + len * sub / n) & ~7LL);
+    A1 = sub == n - 1 ? e : ((b + len * (sub + 1) / n) & ~7LL);
+    if (A0 < b) A0 = b;
+    if (A1 < A0) A1 = A0;
+  }
+  long long h = (A0 + SC_HEAD) & ~7LL;
+  if (h > A1) h = A1;
+  bn.t0 = h;
+  bn.t1 = A1;
+  bn.groups = (int)(h - A0 + 31) >> 5;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const long long e = A0 + 32 * i + lane;
+    bn.pe[i] = e < h ? (int)ly.grouped[e] - 32768 : 40001;
+  }
+}
+// Sums over the bin's weights that lie below place pv, weights at pv itself counting half: twice the count and twice the
+// sums of the powers of the place.  Result in every lane.  Which powers matter: a fine bin is 1 / F of a coarse bin, so
+// the fourth and third power of a place inside it change the interval's sums by less than 1e-8 from F = 64 on, and so
+// does the square in the one bin that is split.  This part: the weights that are not in registers, eight places per
+// load, two loads in flight beyond the one being counted, in stretches whose 32-bit sums cannot overflow.
+__device__ __noinline__ void sc_bin_below_rest(const ScLayer& ly, long long t0, long long t1, int pv, bool full, double* s) {
+  const int lane = threadIdx.x & 31;
+  for (long long tb = t0; tb < t1; tb += SC_CHUNK) {
+    const long long te = tb + SC_CHUNK < t1 ? tb + SC_CHUNK : t1;
+    int c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
+    long long e = tb + 8 * lane;
+    uint4 x = e < te ? sc_load8(ly.grouped, e, ly.total) : make_uint4(0u, 0u, 0u, 0u);
+    uint4 x1 = e + 256 < te ? sc_load8(ly.grouped, e + 256, ly.total) : make_uint4(0u, 0u, 0u, 0u);
+    for (; e < te; e += 256) {
+      const uint4 x2 = e + 512 < te ? sc_load8(ly.grouped, e + 512, ly.total) : make_uint4(0u, 0u, 0u, 0u);
+      const unsigned int xs[4] = {x.x, x.y, x.z, x.w};
+      const int left = (int)(te - e);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int p = i < left ? (int)((i & 1) ? xs[i >> 1] >> 16 : xs[i >> 1] & 0xffffu) - 32768 : 40001;
+        const int w = p < pv ? 2 : (p == pv ? 1 : 0);
+        c0 += w;
+        c1 += w ? w * p : 0;
+        if (full && w) {
+          int p2, p3, p4;
+          sc_powers(p, p2, p3, p4);
+          c2 += w * p2;
+          c3 += w * p3;
+          c4 += w * p4;
+        }
+      }
+      x = x1;
+      x1 = x2;
+    }
+    s[0] += (double)__reduce_add_sync(0xffffffffu, c0);
+    s[1] += (double)__reduce_add_sync(0xffffffffu, c1);
+    if (full) {
+      s[2] += (double)__reduce_add_sync(0xffffffffu, c2);
+      s[3] += (double)__reduce_add_sync(0xffffffffu, c3);
+      s[4] += (double)__reduce_add_sync(0xffffffffu, c4);
+    }
+  }
+}
+__device__ __forceinline__ void sc_bin_below(const ScLayer& ly, const ScBin& bn, int pv, bool full, double (&s)[5]) {
+  int lt = 0, eq = 0, s1 = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if (i >= bn.groups) break;
+    const int p = bn.pe[i];
+    if (p < pv) {
+      ++lt;
+      s1 += p;
+    }
+    eq += p == pv ? 1 : 0;
+  }
+  s[0] = (double)__reduce_add_sync(0xffffffffu, 2 * lt + eq);
+  s[1] = (double)__reduce_add_sync(0xffffffffu, 2 * s1 + eq * pv);
+  s[2] = s[3] = s[4] = 0.0;
+  if (full) {
+    int q2 = 0, q3 = 0, q4 = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (i >= bn.groups) break;
+      const int p = bn.pe[i], w = p < pv ? 2 : (p == pv ? 1 : 0);
+      int p2, p3, p4;
+      sc_powers(w ? p : 0, p2, p3, p4);
+      q2 += w * p2;
+      q3 += w * p3;
+      q4 += w * p4;
+    }
+    s[2] = (double)__reduce_add_sync(0xffffffffu, q2);
+    s[3] = (double)__reduce_add_sync(0xffffffffu, q3);
+    s[4] = (double)__reduce_add_sync(0xffffffffu, q4);
+  }
+  if (bn.t0 < bn.t1) {   // (through a copy: what is handed to a function by address would live in memory everywhere)
+    double t[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    sc_bin_below_rest(ly, bn.t0, bn.t1, pv, full, t);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) s[i] += t[i];
+  }
+}
+
+struct ScCoef {   // Taylor coefficients of a bin: lambda, mu and phi = lambda mu at its centre and derivatives
+  float lam, mu, phi, del, d3, d4;
+};
+__device__ __forceinline__ ScCoef sc_coef(float z) {
+  ScCoef c;
+  sc_lambda(z, c.lam, c.mu);
+  c.phi = c.lam * c.mu;
+  c.del = c.lam - c.mu;
+  c.d3 = fmaf(-6.f, c.phi, 1.f);
+  c.d4 = c.del * fmaf(-12.f, c.phi, 1.f);
+  return c;
+}
+// Sums over n weights with moments m1 .. m4 about the bin centre, which lies at x0 from the origin of the x sums.
+// (mu' = phi, mu'' = phi del, mu''' = phi d3, mu'''' = phi d4; lambda = 1 - mu)
+template <bool EXTRA, typename T>
+__device__ __forceinline__ void sc_bin_sums(const ScCoef& c, float eta, T n, T m1, T m2, T m3, T m4, double x0, double hc, double (&acc)[6]) {
+  const float e2 = 0.5f * eta * eta, e3 = e2 * eta * (1.f / 3.f), e4 = e3 * eta * 0.25f;
+  const T corr = (T)c.phi * ((T)eta * m1 + (T)(e2 * c.del) * m2 + (T)(e3 * c.d3) * m3 + (T)(e4 * c.d4) * m4);
+  const T cort = (T)c.phi * ((T)eta * m2 + (T)(e2 * c.del) * m3 + (T)(e3 * c.d3) * m4);
+  const double sl = (double)(n * (T)c.lam - corr), sm = (double)(n * (T)c.mu + corr);
+  acc[0] += sl;
+  acc[2] += sm;
+  acc[1] += fma(x0, sl, hc * (double)((T)c.lam * m1 - cort));
+  acc[3] += fma(x0, sm, hc * (double)((T)c.mu * m1 + cort));
+  if (EXTRA) {
+    const float d5 = fmaf(-12.f, c.phi, 1.f) * c.d3 - 12.f * c.phi * c.del * c.del;
+    const T sp = (T)c.phi * (n + (T)(eta * c.del) * m1 + (T)(e2 * c.d3) * m2 + (T)(e3 * c.d4) * m3 + (T)(e4 * d5) * m4);
+    const T tp = (T)c.phi * (m1 + (T)(eta * c.del) * m2 + (T)(e2 * c.d3) * m3 + (T)(e3 * c.d4) * m4);
+    acc[4] += (double)sp;
+    acc[5] += fma(x0, (double)sp, hc * (double)tp);
+  }
+}
+
+constexpr float SC_ETA_MAX = 0.6f;   // the series' limit; wider bins are evaluated weight by weight
+constexpr double SC_ZONE = 96.0;   // |z| beyond which lambda resp. mu (below 2^-96) is taken as zero for whole bins
+
+// Interval sums of the bins' weights one by one, for layers whose bins are too wide for the series (tau below about
+// range / 8000; fine bin = coarse bin there).  A lane takes whole bins; inside a bin the order of the weights can vary
+// from run to run, so the sums are integers relative to the largest value in the bin.
+template <bool EXTRA>
+__device__ __noinline__ void sc_wide_bin(const ScGrid& g, const ScLayer& ly, int f, int pl, int pr, double even, double v0, double* acc) {
+  const unsigned int e0 = ly.fstart[f], e1 = ly.fstart[f + 1];
+  if (e0 == e1) return;
+  const double ctr = (double)(g.base_f + f) * g.hf;
+  const float zc = (float)((ctr - even) * (double)ly.slope), dz = (float)(g.hf * (double)ly.slope);
+  // exponents of the largest lambda (left edge) and mu (right edge)
+  const float zl = zc - 0.5f * dz, zr = zc + 0.5f * dz;
+  const int el = (int)fmaxf(fminf(0.f, ceilf(-zl)), -126.f), em = (int)fmaxf(fminf(0.f, ceilf(zr)), -126.f);
+  const double sl = scalbn(1.0, 38 - el), sm = scalbn(1.0, 38 - em), sx = scalbn(1.0, 38 - el - em);
+  long long t[6] = {0, 0, 0, 0, 0, 0};
+  for (unsigned int e = e0; e < e1; ++e) {
+    const int p = (int)ly.grouped[ly.row0 + e] - 32768;
+    int wgt = (p > pl ? 2 : (p == pl ? 1 : 0)) - (p < pr ? 0 : (p == pr ? 1 : 2));   // twice the share in the interval
+    if (wgt <= 0) continue;
+    const float d = (float)p * (float)SC_S1;
+    float lam, mu;
+    sc_lambda(fmaf(d, dz, zc), lam, mu);
+    const double hw = 0.5 * (double)wgt;
+    const double xl = hw * (double)lam * sl, xm = hw * (double)mu * sm;
+    t[0] += __double2ll_rn(xl);
+    t[1] += __double2ll_rn(xl * (double)d);
+    t[2] += __double2ll_rn(xm);
+    t[3] += __double2ll_rn(xm * (double)d);
+    if (EXTRA) {
+      const double xx = hw * (double)lam * (double)mu * sx;
+      t[4] += __double2ll_rn(xx);
+      t[5] += __double2ll_rn(xx * (double)d);
+    }
+  }
+  const double x0 = ctr - v0;
+  const double S[3] = {1.0 / sl, 1.0 / sm, 1.0 / sx};
+#pragma unroll
+  for (int i = 0; i < (EXTRA ? 3 : 2); ++i) {
+    const double a0 = (double)t[2 * i] * S[i], a1 = (double)t[2 * i + 1] * S[i];
+    acc[2 * i] += a0;
+    acc[2 * i + 1] += fma(x0, a0, g.hf * a1);
+  }
+}
+
+// The weights that are exactly zero; on a centroid half of them belong to either side.
+__device__ __noinline__ void sc_zeros(const ScShared& sh, int s, double even, double v0, double* acc) {
+  const float vl = sh.v[s - 1], vr = sh.v[s];
+  const double share = (vl < 0.f && vr > 0.f) ? 1.0 : (((vl == 0.f && vr > 0.f) || (vl < 0.f && vr == 0.f)) ? 0.5 : 0.0);
+  float lam, mu;
+  sc_lambda((float)(-even * (double)sh.ly.slope), lam, mu);
+  const double n = share * (double)sh.n0, nl = n * (double)lam, nm = n * (double)mu, nx = n * (double)(lam * mu);
+  acc[0] += nl;
+  acc[1] -= nl * v0;
+  acc[2] += nm;
+  acc[3] -= nm * v0;
+  acc[4] += nx;
+  acc[5] -= nx * v0;
+}
+
+// Stop test of the M-step before (Algorithm 1's rule), by one warp while the others evaluate.
+__device__ __noinline__ void sc_stop_test(ScShared& sh, const ScalarParams& sp, int layer, int test) {
+  const int lane = threadIdx.x & 31, k = sp.k;
+  double num = 0.0, den = 0.0;
+  int dead = 0;
+  for (int j = lane; j < k; j += 32) {
+    const double c = sh.cnew[j], d = c - sh.cold[j];
+    num = fma(d, d, num);
+    den = fma(c, c, den);
+    dead += sh.dead_j[j];
+  }
+  const bool bad = __any_sync(0xffffffffu, dead < 0 || dead > 0x8000);
+  dead = __reduce_add_sync(0xffffffffu, dead & 0x7fff);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_xor_sync(0xffffffffu, num, o);
+    den += __shfl_xor_sync(0xffffffffu, den, o);
+  }
+  if (lane == 0) {
+    const float res = sqrtf((float)(num / fmax(den, 1e-300)));
+    sh.iters = test;
+    sh.res = res;
+    sh.dead = dead;
+    if (test <= HIST_CAP) sp.p.hist_fwd[(size_t)layer * HIST_CAP + test - 1] = res;
+    if (bad) {
+      sh.status = ST_NONFINITE;
+      sh.done = test;
+    } else if (sp.tol > 0.f && res < sp.tol) {
+      sh.done = test;
+      sh.status = ST_OK;
+    } else if (sp.tol > 0.f && test >= sp.max_iter) {
+      sh.status = ST_MAXITER;
+    }
+  }
+  }
+
+// First half of an evaluation: the weights of every centroid's fine bin below it, a warp (or 2^wl warps) per centroid.
+// `keep`: the bin this warp had in the evaluation before, in registers.
+__device__ __forceinline__ void sc_scan_bins(ScShared& sh, const ScLayer& ly, ScBin& keep, bool full) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int t = warp; t < ly.k << ly.wl; t += SC_WARPS) {
+    const int j = t >> ly.wl, sub = t & ((1 << ly.wl) - 1);
+    const int f = sh.fb[j];
+    if (keep.f != f || ly.k > SC_WARPS) sc_bin_load(ly, f, ly.fstart[f], ly.fstart[f + 1], sub, 1 << ly.wl, keep);
+    double s[5];
+    sc_bin_below(sh.ly, keep, sh.pv[j], full, s);
+    if (lane == 0) {
+      sh.bs[t][0] = s[0];
+      sh.bs[t][1] = s[1];
+      if (full) {
+        sh.bs[t][2] = s[2];
+        sh.bs[t][3] = s[3];
+        sh.bs[t][4] = s[4];
+      }
+    }
+  }
+}
+
+// Second half: every interval's sums.  Its two ends by two neighbouring threads (the block's last ones), the whole bins
+// between them by 2^twl warps; each leaves its share in a slot of Ls, Ms (and Xs).
+template <bool EXTRA>
+__device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly, bool full) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const ScGrid& g = sh.g;
+  const int k = ly.k, tw = 1 << ly.twl, slots = tw + 1;
+  const double v0 = (double)sh.v[0];
+  const bool wide = g.eta > SC_ETA_MAX;
+  if (k == 1) {
+    // one centroid: every weight counts on its left, with attention 1
+    if (threadIdx.x == 0) {
+      const double n = ly.rec.cn[g.nc] + (double)sh.n0;
+      sh.Ms[0][0] = n;
+      sh.Ms[0][1] = ly.rec.cx[g.nc] - v0 * n;
+    }
+    return;
+  }
+  // ---- the ends ----
+  {
+    const int e = SC_T - 1 - (int)threadIdx.x;   // 2 (s - 1) + (0: right end, 1: left end)
+    if (e - (e & 31) < 2 * (k - 1)) {            // whole warps: the two threads of an interval meet by a shuffle
+      const bool mine = e < 2 * (k - 1), left = e & 1;
+      const int s = mine ? (e >> 1) + 1 : 1, j = left ? s - 1 : s;
+      double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      const int fl = sh.fb[s - 1], fr = sh.fb[s], cl = fl >> g.fshift, cr = fr >> g.fshift;
+      const int f = left ? fl : fr, c = left ? cl : cr;
+      const double even = sh.even[s], ctr = sc_center(g, c);
+      if (mine) {
+        // weights of the coarse bin below the centroid: earlier fine bins, and those of its own
+        const double2 q0 = *reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4);
+        const double2 q1 = *reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4 + 2);
+        const double n0 = (double)ly.fstart[f];
+        double b[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int q = 0; q < (1 << ly.wl); ++q) {
+          const double* r = sh.bs[(j << ly.wl) + q];
+          b[0] += 0.5 * r[0];
+          b[1] += 0.5 * r[1];
+          if (full) {
+            b[2] += 0.5 * r[2];
+            b[3] += 0.5 * r[3];
+            b[4] += 0.5 * r[4];
+          }
+        }
+        double M[4];
+        sc_shift(g, sc_fine_x0(g, f), b[0], b[1], b[2], b[3], b[4], M);
+        const double nb = ly.rec.cn[c], xb = ly.rec.cx[c];
+        double n = b[0] + (n0 - nb);
+        M[0] += q0.x;
+        M[1] += q0.y;
+        M[2] += q1.x;
+        M[3] += q1.y;
+        if (left ? (s == 1) : (s == k - 1)) {
+          // the outer interval beyond this end: every weight there, and the zeros
+          double nn = n + nb, xx = fma(ctr, n, fma(g.hc, M[0], xb));
+          if (!left) {
+            nn = ly.rec.cn[g.nc] - nn;
+            xx = ly.rec.cx[g.nc] - xx;
+          }
+          if (sh.n0 > 0) {
+            const float v = left ? sh.v[0] : -sh.v[k - 1];
+            nn += (v > 0.f ? 1.0 : (v == 0.f ? 0.5 : 0.0)) * (double)sh.n0;
+          }
+          double* o = left ? sh.Ms[0] : sh.Ls[(k - 1) * slots];
+          o[0] = nn;
+          o[1] = xx - v0 * nn;
+        }
+        if (!wide) {
+          const ScCoef co = sc_coef((float)((ctr - even) * (double)ly.slope));
+          if (left) {   // the piece above the left end: the whole bin (unless the right end lies in it) minus what is below
+            const bool whole = cl != cr;
+            n = (whole ? (double)ly.rec.r[cl] : 0.0) - n;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) M[i] = (whole ? (double)ly.rec.r[(i + 1) * ly.rec.stride + cl] : 0.0) - M[i];
+          }
+          sc_bin_sums<EXTRA, double>(co, g.eta, n, M[0], M[1], M[2], M[3], ctr - v0, g.hc, acc);
+        } else if (left || fl != fr) {
+          // (fine bin = coarse bin)
+          double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+          sc_wide_bin<EXTRA>(sh.g, sh.ly, f, left ? sh.pv[s - 1] : -50000, (!left || fl == fr) ? sh.pv[s] : 50000, even, v0, t6);
+#pragma unroll
+          for (int i = 0; i < 6; ++i) acc[i] += t6[i];
+        }
+        if (cr - cl >= 2) {
+          // whole bins on this side of the zone: lambda = 1 left of it, mu = 1 right of it
+          int lo = cl + 1, hi = cr;
+          if (left) {
+            const int z = __double2int_rd((even - ly.zone - g.ctr0) * g.inv_hc);
+            hi = z < lo ? lo : (z < cr ? z : cr);
+          } else {
+            const int z = __double2int_ru((even + ly.zone - g.ctr0) * g.inv_hc) + 1;
+            lo = z < lo ? lo : (z < cr ? z : cr);
+          }
+          const double nn = ly.rec.cn[hi] - ly.rec.cn[lo], xx = ly.rec.cx[hi] - ly.rec.cx[lo] - v0 * nn;
+          acc[0] += left ? nn : 0.0;
+          acc[1] += left ? xx : 0.0;
+          acc[2] += left ? 0.0 : nn;
+          acc[3] += left ? 0.0 : xx;
+        }
+        if (left && sh.n0 > 0) {
+          double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+          sc_zeros(sh, s, even, v0, t6);
+#pragma unroll
+          for (int i = 0; i < 6; ++i) acc[i] += t6[i];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < (EXTRA ? 6 : 4); ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 1);
+      if (mine && left) {
+        double *lo = sh.Ls[(s - 1) * slots + tw], *mo = sh.Ms[s * slots + tw], *xo = sh.Xs[(s - 1) * slots + tw];
+        lo[0] = acc[0];
+        lo[1] = acc[1];
+        mo[0] = acc[2];
+        mo[1] = acc[3];
+        if (EXTRA) {
+          xo[0] = acc[4];
+          xo[1] = acc[5];
+        }
+      }
+    }
+  }
+  // ---- whole bins between the ends, inside the zone where neither lambda nor mu vanishes ----
+  for (int t = warp; t < (k - 1) << ly.twl; t += SC_WARPS) {
+    const int s = (t >> ly.twl) + 1, sub = t & (tw - 1);
+    const int cl = sh.fb[s - 1] >> g.fshift, cr = sh.fb[s] >> g.fshift;
+    const double even = sh.even[s];
+    int b0 = __double2int_rd((even - ly.zone - g.ctr0) * g.inv_hc), b1 = __double2int_ru((even + ly.zone - g.ctr0) * g.inv_hc);
+    if (b0 < cl + 1) b0 = cl + 1;
+    if (b1 > cr - 1) b1 = cr - 1;
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (!wide) {
+      for (int b = b0 + sub * 32 + lane; b <= b1; b += 32 * tw) {
+        const float n = ly.rec.r[b];
+        const double ctr = sc_center(g, b);
+        const ScCoef c = sc_coef((float)((ctr - even) * (double)ly.slope));
+        sc_bin_sums<EXTRA, float>(c, g.eta, n, ly.rec.r[ly.rec.stride + b], ly.rec.r[2 * ly.rec.stride + b], ly.rec.r[3 * ly.rec.stride + b],
+                                  ly.rec.r[4 * ly.rec.stride + b], ctr - v0, g.hc, acc);
+      }
+    } else {
+      double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      for (int b = b0 + sub * 32 + lane; b <= b1; b += 32 * tw) sc_wide_bin<EXTRA>(sh.g, sh.ly, b, -50000, 50000, even, v0, t6);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) acc[i] += t6[i];
+    }
+    // four sums over the warp: the first two levels also deal the sums out, so that lanes 0, 8, 16, 24 end with one each
+    {
+      const bool h4 = lane & 16, h3 = lane & 8;
+      double p = h4 ? acc[2] : acc[0], q = h4 ? acc[3] : acc[1];
+      p += __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[2], 16);
+      q += __shfl_xor_sync(0xffffffffu, h4 ? acc[1] : acc[3], 16);
+      double r = h3 ? q : p;
+      r += __shfl_xor_sync(0xffffffffu, h3 ? p : q, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+      if ((lane & 7) == 0) (h4 ? sh.Ms[s * slots + sub] : sh.Ls[(s - 1) * slots + sub])[h3 ? 1 : 0] = r;
+    }
+    if (EXTRA) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        acc[4] += __shfl_xor_sync(0xffffffffu, acc[4], o);
+        acc[5] += __shfl_xor_sync(0xffffffffu, acc[5], o);
+      }
+      if (lane == 0) {
+        sh.Xs[(s - 1) * slots + sub][0] = acc[4];
+        sh.Xs[(s - 1) * slots + sub][1] = acc[5];
+      }
+    }
+  }
+}
+
+// Both halves; the last warp first runs the stop test of the M-step before (`test` = its number, 0: none).
+template <bool EXTRA>
+__device__ __forceinline__ void sc_evaluate(ScShared& sh, const ScLayer& ly, ScBin& keep, const ScalarParams& sp, int layer, int test) {
+  const bool full = sh.g.F < 64;
+  if (test > 0 && threadIdx.x >= SC_T - 32) sc_stop_test(sh, sp, layer, test);
+  sc_scan_bins(sh, ly, keep, full);
+  __syncthreads();
+  sc_sum_intervals<EXTRA>(sh, ly, full);
+}
+
+// Sums a centroid sees on one of its sides (all slots; entries without a task stay zero).
+__device__ __forceinline__ void sc_gather(const double (*a)[2], int j, int twl, double& s0, double& s1) {
+  const int slots = (1 << twl) + 1;
+  s0 = s1 = 0.0;
+#pragma unroll
+  for (int q = 0; q < 5; ++q)
+    if (q < slots) {
+      s0 += a[j * slots + q][0];
+      s1 += a[j * slots + q][1];
+    }
+}
+
+constexpr int SI_T = 1024, SI_WARPS = SI_T / 32;
+// ---- first launch: layer states, working centroids, counters to zero, value range of the weights ----
+__global__ void __launch_bounds__(SI_T, 1) idkm_scalar_init(const __grid_constant__ ScalarParams sp) {
+  __shared__ float red_lo[SI_WARPS], red_hi[SI_WARPS];
+  __shared__ unsigned int red_z[SI_WARPS];
+  grid_dependency_sync();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = sp.k;
+  const int layer = sc_layer_of_block(sp, (int)blockIdx.x);
+  const int b = (int)blockIdx.x - sp.blk_first[layer], NB = sp.blk_first[layer + 1] - sp.blk_first[layer];
+  const long long m = sp.row_off[layer + 1] - sp.row_off[layer];
+  const float* Wl = sp.p.W + sp.row_off[layer];
+  if (b == 0) {
+    if (tid < SC_SYNC_WORDS) sp.p.sync[(size_t)layer * SC_SYNC_WORDS + tid] = 0u;
+    if (tid < k) sp.p.C[(size_t)layer * k + tid] = sp.p.C0[(size_t)layer * k + tid];
+    if (tid == 0) {
+      LayerState s;
+      memset(&s, 0, sizeof(s));
+      s.status = ST_OK;
+      s.adj_prev = 3.0e38f;
+      sp.p.st[layer] = s;
+    }
+  }
+  for (int i = (int)blockIdx.x * SI_T + tid; i < sp.n_group_rows; i += (int)gridDim.x * SI_T) sp.p.gtick[i] = 0u;
+  for (int h = 0; h < 2; ++h)
+    for (int i = (int)blockIdx.x * SI_T + tid; i < sp.p.n_pair_ticks[h]; i += (int)gridDim.x * SI_T) sp.p.pair_ticks[h][i] = 0u;
+  const int cap = sp.fine_off[layer + 1] - sp.fine_off[layer];
+  if (NB > 1)
+    for (int i = b * SI_T + tid; i < cap; i += NB * SI_T) sp.p.gcount[sp.fine_off[layer] + i] = 0u;
+  const long long r0 = m * b / NB, r1 = m * (b + 1) / NB;
+  float lo = __int_as_float(0x7f800000), hi = -lo;
+  int bad = 0;
+  unsigned int nz = 0;
+  auto take = [&](float w) {
+    bad |= !(fabsf(w) <= 3.4028235e38f);
+    const bool z = (w == 0.f);
+    nz += z ? 1u : 0u;
+    lo = z ? lo : fminf(lo, w);
+    hi = z ? hi : fmaxf(hi, w);
+  };
+  long long r = r0 + tid;
+  for (; r + 7 * SI_T < r1; r += 8 * SI_T) {
+    float w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = __ldg(Wl + r + i * SI_T);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) take(w[i]);
+  }
+  for (; r < r1; r += SI_T) take(__ldg(Wl + r));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  nz = __reduce_add_sync(0xffffffffu, nz);
+  if (lane == 0) {
+    red_lo[warp] = lo;
+    red_hi[warp] = hi;
+    red_z[warp] = nz;
+  }
+  bad = __syncthreads_or(bad);
+  if (warp == 0) {
+    lo = red_lo[lane];
+    hi = red_hi[lane];
+    nz = __reduce_add_sync(0xffffffffu, red_z[lane]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (lane == 0) sp.p.bstat[blockIdx.x] = make_float4(lo, hi, bad ? 1.f : 0.f, __uint_as_float(nz));
+  }
+}
+
+// LOG: codebooks of at most 2^LOG centroids, whose M-step one warp takes; 0: larger ones.
+template <int LOG>
+__global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constant__ ScalarParams sp) {
+  extern __shared__ __align__(16) unsigned char smem_all[];
+  ScShared& sh = *reinterpret_cast<ScShared*>(smem_all);
+  unsigned char* dyn = smem_all + SC_SH_BYTES;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int k = sp.k;
+  const int layer = sc_layer_of_block(sp, (int)blockIdx.x);
+  const int b = (int)blockIdx.x - sp.blk_first[layer], NB = sp.blk_first[layer + 1] - sp.blk_first[layer];
+  const long long m = sp.row_off[layer + 1] - sp.row_off[layer];
+  const float* Wl = sp.p.W + sp.row_off[layer];
+  unsigned short* grouped = sp.p.grouped + sp.row_off[layer];
+  const int fo = sp.fine_off[layer], cap = sp.fine_off[layer + 1] - fo;
+  unsigned int* fstart = sp.p.fstart + fo + layer;
+  unsigned int* gcount = sp.p.gcount + fo;
+  long long* frec = sp.p.frec + (size_t)fo * 4;
+  unsigned int* sync = sp.p.sync + (size_t)layer * SC_SYNC_WORDS;
+  LayerState* st = sp.p.st + layer;
+  float* Cl = sp.p.C + (size_t)layer * k;
+  const bool alone = (NB == 1) && (sp.missing_arrivals == 0);
+  unsigned int meet = 0;
+  auto barrier = [&](bool stay) {
+    if (alone) {
+      __syncthreads();
+      return true;
+    }
+    ++meet;
+    return sc_team_barrier(sync, meet * (unsigned int)(NB + sp.missing_arrivals), sp.spin_limit, &sh.ok, stay);
+  };
+  const long long r0 = m * b / NB, r1 = m * (b + 1) / NB;
+  unsigned int* cnt = reinterpret_cast<unsigned int*>(dyn);
+  grid_dependency_sync();
+  if (warp == 0) {
+    float lo = __int_as_float(0x7f800000), hi = -lo, bad = 0.f;
+    long long nz = 0;
+    for (int i = lane; i < NB; i += 32) {
+      const float4 s = __ldcg(sp.p.bstat + sp.blk_first[layer] + i);
+      lo = fminf(lo, s.x);
+      hi = fmaxf(hi, s.y);
+      bad = fmaxf(bad, s.z);
+      nz += (long long)__float_as_uint(s.w);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      bad = fmaxf(bad, __shfl_xor_sync(0xffffffffu, bad, o));
+      nz += __shfl_xor_sync(0xffffffffu, nz, o);
+    }
+    if (lane == 0) {
+      sh.bad = bad > 0.f;
+      sh.g = sc_make_grid(lo, hi, 1.0 / sp.inv_tau_d, m, cap);
+      sh.n0 = nz;
+    }
+  }
+  __syncthreads();
+  int status = ST_OK;
+  if (sh.bad) {
+    status = ST_NONFINITE;   // NaN or Inf among the weights (uniform over the layer's blocks)
+    if (b != 0) return;
+  } else {
+    const ScGrid g = sh.g;
+    const int nf = g.nf;
+    bool ok = true;
+    // ---- count the block's weights per fine bin ----
+    for (int i = tid; i < nf; i += SC_T) cnt[i] = 0u;
+    __syncthreads();
+    {
+      long long r = r0 + tid;
+      for (; r + 15 * SC_T < r1; r += 16 * SC_T) {
+        float w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = __ldg(Wl + r + i * SC_T);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (w[i] != 0.f) atomicAdd(&cnt[sc_fine(g, w[i])], 1u);
+      }
+      for (; r < r1; r += SC_T) {
+        const float w = __ldg(Wl + r);
+        if (w != 0.f) atomicAdd(&cnt[sc_fine(g, w)], 1u);
+      }
+    }
+    __syncthreads();
+    if (NB > 1) {
+      // where this block's share of every bin begins inside the bin (which block comes first does not matter)
+      for (int i = tid; i < nf; i += SC_T) {
+        const unsigned int c = cnt[i];
+        cnt[i] = c ? atomicAdd(&gcount[i], c) : 0u;
+      }
+    }
+    ok = barrier(true);
+    constexpr unsigned int BIG = 4 * SC_CHUNK;
+    if (ok) {
+      // ---- first element of every bin: exclusive prefix over the bins, four per thread and round ----
+      unsigned int carry = 0;
+      auto fetch = [&](int i) {
+        uint4 c = make_uint4(0u, 0u, 0u, 0u);
+        if (i < nf) {
+          // (capacities and shared memory are multiples of four bins; what lies past the last bin is masked)
+          c = NB > 1 ? __ldcg(reinterpret_cast<const uint4*>(gcount + i)) : *reinterpret_cast<const uint4*>(cnt + i);
+          if (i + 1 >= nf) c.y = 0u;
+          if (i + 2 >= nf) c.z = 0u;
+          if (i + 3 >= nf) c.w = 0u;
+        }
+        return c;
+      };
+      uint4 next = fetch(4 * tid);
+      for (int t = 0; t < nf; t += 4 * SC_T) {
+        const int i = t + 4 * tid;
+        const uint4 c = next;
+        if (NB > 1) next = fetch(i + 4 * SC_T);
+        const unsigned int sum = c.x + c.y + c.z + c.w;
+        unsigned int x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned int y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (lane == 31) sh.scan[warp] = x;
+        __syncthreads();
+        const unsigned int y = lane < SC_WARPS ? sh.scan[lane] : 0u;   // (every warp adds up the warp totals itself)
+        const unsigned int before = __reduce_add_sync(0xffffffffu, lane < warp ? y : 0u);
+        const unsigned int total = __reduce_add_sync(0xffffffffu, y);
+        if (i < nf) {
+          const unsigned int f0 = carry + before + x - sum;
+          const uint4 f = make_uint4(f0, f0 + c.x, f0 + c.x + c.y, f0 + c.x + c.y + c.z);
+          uint4* o = reinterpret_cast<uint4*>(cnt + i);
+          if (NB > 1) {
+            uint4 q = *o;
+            q.x += f.x;
+            q.y += f.y;
+            q.z += f.z;
+            q.w += f.w;
+            *o = q;
+          } else {
+            *o = f;
+          }
+          if (b == 0) {
+            const unsigned int fs[4] = {f.x, f.y, f.z, f.w}, cs[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (i + q < nf) {
+                fstart[i + q] = fs[q];
+                if (cs[q] > BIG) {   // (its moments are added up by all warps of the layer)
+                  long long* z = frec + (size_t)(i + q) * 4;
+                  z[0] = z[1] = z[2] = z[3] = 0;
+                }
+              }
+          }
+        }
+        carry += total;
+        __syncthreads();
+        if (NB == 1) next = fetch(i + 4 * SC_T);
+      }
+      if (b == 0 && tid == 0) fstart[nf] = carry;
+      // ---- group the weights' places by fine bin ----
+      auto put = [&](float w) {
+        if (w == 0.f) return;
+        int p;
+        const int i = sc_fine_place(g, w, p);
+        grouped[atomicAdd(&cnt[i], 1u)] = (unsigned short)(p + 32768);
+      };
+      long long r = r0 + tid;
+      for (; r + 7 * SC_T < r1; r += 8 * SC_T) {
+        float w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = __ldg(Wl + r + i * SC_T);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) put(w[i]);
+      }
+      for (; r < r1; r += SC_T) put(__ldg(Wl + r));
+      ok = barrier(true);
+    }
+    if (ok) {
+      // ---- integer sums of powers of the places, per fine bin; groups of 32 bins are dealt to the layer's warps ----
+      if (NB > 1) {
+        for (int i = tid; i < nf; i += SC_T) cnt[i] = __ldcg(fstart + i + 1);
+        __syncthreads();
+      }   // (otherwise the counters have moved on to the end of every bin)
+      int have_big = 0;
+      if (m <= 24LL * nf) {
+        // few weights per bin: one thread each
+        for (int i = b * SC_T + tid; i < nf; i += NB * SC_T) {
+          const unsigned int e0 = i > 0 ? cnt[i - 1] : 0u, e1 = cnt[i];
+          if (e1 - e0 > BIG) continue;
+          long long t1 = 0, t2 = 0, t3 = 0, t4 = 0;
+#pragma unroll 4
+          for (unsigned int e = e0; e < e1; ++e) {
+            const int p = (int)grouped[e] - 32768;
+            int p2, p3, p4;
+            sc_powers(p, p2, p3, p4);
+            t1 += p;
+            t2 += p2;
+            t3 += p3;
+            t4 += p4;
+          }
+          longlong2* o = reinterpret_cast<longlong2*>(frec + (size_t)i * 4);
+          o[0] = make_longlong2(t1, t2);
+          o[1] = make_longlong2(t3, t4);
+        }
+      } else {
+        // a quarter of a warp each, eight places per lane and load, the next bin's first two loads issued ahead
+        const unsigned short* all = sp.p.grouped;
+        const long long row0 = sp.row_off[layer], total = sp.row_off[sp.n_layers];
+        const int step = NB * SC_T / 8, ql = lane & 7;
+        const bool full = g.F < 64;   // (see sc_bin_below)
+        const unsigned int qmask = 0xffu << (lane & 24);
+        int i = (b * SC_T + tid) >> 3;
+        long long A0 = 0, A1 = 0;
+        uint4 x0 = make_uint4(0u, 0u, 0u, 0u), x1 = x0;
+        auto first = [&](int bi, long long& a0, long long& a1, uint4& y0, uint4& y1) {
+          a0 = a1 = 0;
+          y0 = y1 = make_uint4(0u, 0u, 0u, 0u);
+          if (bi < nf) {
+            a0 = row0 + (bi > 0 ? cnt[bi - 1] : 0u);
+            a1 = row0 + cnt[bi];
+            const long long e = (a0 & ~7LL) + 8 * ql;
+            if (e < a1) y0 = sc_load8(all, e, total);
+            if (e + 64 < a1) y1 = sc_load8(all, e + 64, total);
+          }
+        };
+        first(i, A0, A1, x0, x1);
+        for (; i < nf; i += step) {
+          long long B0, B1;
+          uint4 n0, n1;
+          first(i + step, B0, B1, n0, n1);
+          if (A1 - A0 <= (long long)BIG) {   // (32-bit sums per lane: at most BIG / 8 = 4096 places of at most 2^16)
+            int s1 = 0, s2 = 0, s3 = 0, s4 = 0;
+            long long e = (A0 & ~7LL) + 8 * ql;
+            while (e < A1) {
+              const unsigned int xs[4] = {x0.x, x0.y, x0.z, x0.w};
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const bool in = q >= (int)(A0 - e) && q < (int)(A1 - e);
+                const int p = in ? (int)((q & 1) ? xs[q >> 1] >> 16 : xs[q >> 1] & 0xffffu) - 32768 : 0;
+                s1 += p;
+                s2 += (p * p + 8192) >> 14;
+                if (full) {
+                  int p2, p3, p4;
+                  sc_powers(p, p2, p3, p4);
+                  s3 += p3;
+                  s4 += p4;
+                }
+              }
+              e += 64;
+              x0 = x1;
+              if (e + 64 < A1) x1 = sc_load8(all, e + 64, total);
+            }
+            long long t[4] = {s1, s2, s3, s4};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+              for (int o = 4; o > 0; o >>= 1) t[q] += __shfl_xor_sync(qmask, t[q], o);
+            if (ql < 4) frec[(size_t)i * 4 + ql] = ql == 0 ? t[0] : (ql == 1 ? t[1] : (ql == 2 ? t[2] : t[3]));
+          }
+          A0 = B0;
+          A1 = B1;
+          x0 = n0;
+          x1 = n1;
+        }
+      }
+      // bins with very many nearly equal weights: all warps of the layer share them
+      if (m > (long long)BIG)
+        for (int i = tid; i < nf; i += SC_T) have_big |= (cnt[i] - (i > 0 ? cnt[i - 1] : 0u) > BIG);
+      have_big = __syncthreads_or(have_big);
+      if (have_big) {   // (uniform over the layer's blocks: all read the same counts)
+        for (int i0 = 0; i0 < nf; i0 += SC_T) {
+          const int i = i0 + tid;
+          const unsigned int mask_w = __ballot_sync(0xffffffffu, i < nf && cnt[i] - (i > 0 ? cnt[i - 1] : 0u) > BIG);
+          if (lane == 0) sh.scan[warp] = mask_w;
+          __syncthreads();
+          for (int w = 0; w < SC_WARPS; ++w) {
+            unsigned int mask = sh.scan[w];
+            while (mask) {
+              const int bi = i0 + w * 32 + __ffs(mask) - 1;
+              mask &= mask - 1;
+              const unsigned int e0 = bi > 0 ? cnt[bi - 1] : 0u, e1 = cnt[bi];
+              for (unsigned long long eb = (unsigned long long)e0 + 1024ull * (b * SC_WARPS + warp); eb < e1; eb += 1024ull * NB * SC_WARPS) {
+                int t[4] = {0, 0, 0, 0};
+                for (int q = 0; q < 32; ++q) {
+                  const unsigned long long e = eb + 32ull * q + lane;
+                  if (e < e1) {
+                    const int p = (int)grouped[e] - 32768;
+                    int p2, p3, p4;
+                    sc_powers(p, p2, p3, p4);
+                    t[0] += p;
+                    t[1] += p2;
+                    t[2] += p3;
+                    t[3] += p4;
+                  }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  const int s = __reduce_add_sync(0xffffffffu, t[q]);
+                  if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(frec + (size_t)bi * 4 + q), (unsigned long long)(long long)s);
+                }
+              }
+            }
+          }
+          __syncthreads();
+        }
+      }
+      ok = barrier(true);
+    }
+    if (ok) {
+      // ---- moments about the coarse bins' centres, prefixed over the fine bins of every coarse bin; coarse records ----
+      const ScRec gr = sc_global_rec(sp, layer, cap);
+      const int wd = g.F < 32 ? g.F : 32;      // lanes per coarse bin
+      const int per = g.F < 32 ? 32 / g.F : 1; // coarse bins per step of a warp
+      for (int c0 = (b * SC_WARPS + warp) * per; c0 < g.nc; c0 += NB * SC_WARPS * per) {
+        const int c = c0 + lane / wd;
+        const bool in = c < g.nc;
+        double run[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int f0 = 0; f0 < g.F; f0 += wd) {
+          const int f = (c << g.fshift) + f0 + (lane % wd);
+          double x[4] = {0.0, 0.0, 0.0, 0.0}, y[4];
+          if (in) {
+            const longlong2 u0 = __ldcg(reinterpret_cast<const longlong2*>(frec + (size_t)f * 4));
+            const longlong2 u1 = __ldcg(reinterpret_cast<const longlong2*>(frec + (size_t)f * 4) + 1);
+            const double n = (double)(cnt[f] - (f > 0 ? cnt[f - 1] : 0u));
+            sc_shift(g, sc_fine_x0(g, f), n, (double)u0.x, (double)u0.y, (double)u1.x, (double)u1.y, x);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) y[q] = x[q];
+          for (int o = 1; o < wd; o <<= 1)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const double t = __shfl_up_sync(0xffffffffu, y[q], o, wd);
+              if ((lane % wd) >= o) y[q] += t;
+            }
+          if (in) {
+            double2* o = reinterpret_cast<double2*>(frec + (size_t)f * 4);
+            o[0] = make_double2(run[0] + (y[0] - x[0]), run[1] + (y[1] - x[1]));
+            o[1] = make_double2(run[2] + (y[2] - x[2]), run[3] + (y[3] - x[3]));
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) run[q] += __shfl_sync(0xffffffffu, y[q], wd - 1, wd);
+        }
+        if (in && lane % wd == 0) {
+          const unsigned int e0 = c > 0 ? cnt[(c << g.fshift) - 1] : 0u, e1 = cnt[((c + 1) << g.fshift) - 1];
+          gr.r[c] = (float)(e1 - e0);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) gr.r[(size_t)(q + 1) * cap + c] = (float)run[q];
+          gr.cx[c + 1] = fma(sc_center(g, c), (double)(e1 - e0), g.hc * run[0]);
+        }
+      }
+      ok = barrier(b == 0);
+    }
+    if (!ok) status = ST_TIMEOUT;
+  }
+  if (b != 0) return;
+
+  // ================= from here on one block per layer =================
+  const int kw = LOG > 0 ? 1 : (k + 31) >> 5;
+  if (tid < kw * 32) {
+    if (tid < k) {
+      sh.vn[tid] = Cl[tid];
+      sh.idn[tid] = tid;
+    }
+    sc_sync(kw);
+    sc_sort(sh, k);
+  }
+  const int K1 = k + 1;
+  double* tab = sp.p.tab + (size_t)layer * SC_NTAB * K1;
+  float* ft = sp.p.ftab + (size_t)layer * SC_NFTAB * K1;
+  if (status != ST_OK) {
+    // nothing was computed: report, and leave tables that later passes can read without harm
+    for (int i = tid; i < SC_NTAB * K1; i += SC_T) tab[i] = 0.0;
+    for (int i = tid; i < SC_NFTAB * K1; i += SC_T) ft[i] = 0.f;
+    const float nan = __int_as_float(0x7fc00000);
+    for (int i = tid; i < k; i += SC_T) {
+      sp.p.perm[(size_t)layer * k + i] = i;
+      sp.p.S[(size_t)layer * k + i] = 0.f;
+      sp.p.F[(size_t)layer * k + i] = status == ST_NONFINITE ? nan : sh.vn[i];
+      if (status == ST_NONFINITE) Cl[i] = nan;
+    }
+    if (tid == 0) {
+      st->status = status;
+      st->fwd_iters = st->fwd_done = status == ST_NONFINITE ? 1 : 0;
+      st->fwd_res = status == ST_NONFINITE ? nan : 0.f;
+    }
+    return;
+  }
+  const ScGrid& g = sh.g;
+  ScLayer ly;
+  ly.grouped = sp.p.grouped;
+  ly.row0 = sp.row_off[layer];
+  ly.total = sp.row_off[sp.n_layers];
+  ly.fstart = fstart;
+  ly.frec = reinterpret_cast<const double*>(frec);
+  ly.k = k;
+  ly.tau = 1.0 / sp.inv_tau_d;
+  ly.inv_tau = sp.inv_tau_d;
+  ly.slope = (float)(2.0 * 1.4426950408889634 * sp.inv_tau_d);
+  ly.zone = SC_ZONE / (double)ly.slope;
+  ly.twl = 0;
+  ly.wl = 0;
+  while (ly.wl < 3 && (k << (ly.wl + 1)) <= SC_WARPS) ++ly.wl;
+  while (ly.twl < 2 && k > 1 && ((k - 1) << (ly.twl + 1)) <= SC_WARPS) ++ly.twl;
+  {
+    // ---- coarse records: into shared memory where they fit; running counts and x sums ----
+    const ScRec gr = sc_global_rec(sp, layer, cap);
+    ly.rec = gr;
+    if (g.nc <= SC_REC_SMEM) {
+      const int stride = g.nc <= SC_SMALL_NC ? SC_SMALL_NC : SC_REC_SMEM;
+      ly.rec.cn = reinterpret_cast<double*>(dyn);
+      ly.rec.cx = ly.rec.cn + stride + 1;
+      ly.rec.r = reinterpret_cast<float*>(ly.rec.cx + stride + 1);
+      ly.rec.stride = stride;
+    }
+    __syncthreads();   // (the counters, which lie in the same place, are no longer read)
+    double carry = 0.0;
+    for (int t = 0; t < g.nc; t += SC_T) {
+      const int c = t + tid;
+      double x = c < g.nc ? __ldcg(gr.cx + c + 1) : 0.0;
+      if (c < g.nc && g.nc <= SC_REC_SMEM) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) ly.rec.r[q * ly.rec.stride + c] = __ldcg(gr.r + (size_t)q * cap + c);
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) sh.scan_x[warp] = x;
+      __syncthreads();
+      double before = 0.0, total = 0.0;
+      for (int w = 0; w < SC_WARPS; ++w) {
+        const double y = sh.scan_x[w];
+        before += w < warp ? y : 0.0;
+        total += y;
+      }
+      if (c < g.nc) {
+        ly.rec.cx[c + 1] = carry + before + x;
+        ly.rec.cn[c + 1] = (double)fstart[(c + 1) << g.fshift];
+      }
+      carry += total;
+      __syncthreads();
+    }
+    if (tid == 0) ly.rec.cx[0] = ly.rec.cn[0] = 0.0;
+    // a small layer's places, bin starts and moments too, behind the records (the records of few coarse bins are short:
+    // strides and arrays as above, so only what lies behind the last array's used part is free)
+    if (g.nc <= SC_SMALL_NC) {
+      unsigned char* q = dyn + SC_SMALL_OFF;
+      const int a0 = (int)(ly.row0 & 7);
+      const size_t need = 32 * (size_t)g.nf + 4 * (((size_t)g.nf + 4) & ~(size_t)3) + 2 * ((size_t)m + 16);
+      if (need <= (size_t)(SC_DYN - SC_SH_BYTES - SC_SMALL_OFF)) {
+        double* sf = reinterpret_cast<double*>(q);
+        unsigned int* ss = reinterpret_cast<unsigned int*>(q + 32 * (size_t)g.nf);
+        unsigned short* sg = reinterpret_cast<unsigned short*>(ss + ((g.nf + 4) & ~3));
+        for (int i = tid; i < 4 * g.nf; i += SC_T) sf[i] = ly.frec[i];
+        for (int i = tid; i <= g.nf; i += SC_T) ss[i] = fstart[i];
+        for (int i = tid; i < (int)m; i += SC_T) sg[a0 + i] = grouped[i];
+        ly.frec = sf;
+        ly.fstart = ss;
+        ly.grouped = sg;
+        ly.row0 = a0;
+        ly.total = a0 + m;
+      }
+    }
+  }
+  constexpr bool one_warp = LOG > 0;
+  double a = 0.0, ap = 0.0, rP = 0.0, rQ = 0.0;   // (more than 32 centroids)
+  ScScan<LOG> scn;
+#pragma unroll
+  for (int l = 0; l < (LOG > 0 ? LOG : 1); ++l) scn.cb[l] = scn.cf[l] = 0.0;
+  for (int i = tid; i < SC_PARTS * 2; i += SC_T) (&sh.Ls[0][0])[i] = (&sh.Ms[0][0])[i] = (&sh.Xs[0][0])[i] = 0.0;
+  if (tid == 0) {
+    sh.done = 0;
+    sh.iters = 0;
+    sh.dead = 0;
+    sh.status = ST_OK;
+    sh.res = 0.f;
+  }
+  if (tid == 0) sh.ly = ly;
+  auto tables = [&]() {
+    if constexpr (one_warp) {
+      if (warp == 0) sc_tables_warp(sh, ly, lane < k ? sh.v[lane] : sh.v[k - 1], scn, rP, rQ);
+    } else if (tid < kw * 32) {
+      sc_tables_block(sh, ly, a, ap, rP, rQ);
+    }
+  };
+  // sums of the two sides -> what every centroid receives from all intervals
+  auto spread2 = [&](double (&x)[2], double (&y)[2]) {
+    if constexpr (one_warp) {
+      sc_scan_both<2, LOG>(scn, x, y);
+    } else {
+      lin_scan<2, false>(a, x, k, sh.tmp);
+      lin_scan<2, true>(ap, y, k, sh.tmp);
+    }
+  };
+  tables();
+  ScBin keep;
+  keep.f = -1;
+  keep.groups = 0;
+  keep.t0 = keep.t1 = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) keep.pe[i] = 40001;
+  __syncthreads();
+
+  int it = 0;
+  while (it < sp.max_iter) {
+    sc_evaluate<false>(sh, ly, keep, sp, layer, it);
+    __syncthreads();
+    if (sh.done) break;
+    if (tid < kw * 32) {
+      // ---- M-step (Algorithm 1, step 5) ----
+      const int j = tid;
+      const bool own = j < k;
+      const int jc = own ? j : k - 1;
+      double L0, L1, M0, M1;
+      sc_gather(sh.Ls, jc, ly.twl, L0, L1);
+      sc_gather(sh.Ms, jc, ly.twl, M0, M1);
+      double x[2] = {L0 * rP, L1 * rP}, y[2] = {M0 * rQ, M1 * rQ};   // (rP = rQ = 0 in threads without a centroid)
+      spread2(x, y);
+      const double v0 = (double)sh.v[0], cold = (double)sh.v[jc];
+      const double s = x[0] + y[0];
+      const bool alive = (s >= S_MIN);
+      const double cnew = alive ? fma(x[1] + y[1], sc_rcp(s), v0) : cold;
+      float cn = (float)cnew;
+      if (own) {
+        sh.cnew[j] = cnew;
+        sh.cold[j] = cold;
+        sh.dead_j[j] = (alive ? 0 : 1) + ((!(s == s) || s > 1e300 || !(cnew == cnew) || fabs(cnew) > 1e300) ? 0x10000 : 0);
+      } else {
+        cn = __int_as_float(0x7f800000);
+      }
+      // (the map keeps the order of the centroids up to rounding)
+      float left = __shfl_up_sync(0xffffffffu, cn, 1);
+      bool out_of_order;
+      if constexpr (one_warp) {
+        out_of_order = __any_sync(0xffffffffu, own && j > 0 && !(left <= cn));
+      } else {
+        sc_bar(kw);   // (everybody has read the old centroids)
+        if (own) sh.vn[j] = cn;
+        if (j == 0) sh.flag = 0;
+        sc_bar(kw);
+        if ((j & 31) == 0 && j > 0) left = sh.vn[j - 1];
+        if (own && j > 0 && !(left <= cn)) sh.flag = 1;
+        sc_bar(kw);
+        out_of_order = sh.flag != 0;
+      }
+      if (out_of_order) {
+        if (own) {
+          sh.vn[j] = cn;
+          sh.idn[j] = sh.id[j];
+        }
+        sc_sync(kw);
+        sc_sort(sh, k);
+      } else {
+        if (one_warp) __syncwarp();
+        if (own) sh.v[j] = cn;
+        sc_sync(kw);
+      }
+    }
+    tables();
+    ++it;
+    __syncthreads();
+  }
+
+  // ---- sums at the returned centroids: S, F and the tables of the passes that follow ----
+  sc_evaluate<true>(sh, ly, keep, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
+  __syncthreads();
+  if (tid < kw * 32) {
+    const bool own = tid < k;
+    const int jc = own ? tid : k - 1;
+    double L0, L1, M0, M1, X0, X1;
+    sc_gather(sh.Ls, jc, ly.twl, L0, L1);
+    sc_gather(sh.Ms, jc, ly.twl, M0, M1);
+    sc_gather(sh.Xs, jc, ly.twl, X0, X1);
+    double x[2] = {L0 * rP, L1 * rP}, y[2] = {M0 * rQ, M1 * rQ};
+    spread2(x, y);
+    // averages of the centroids from every centroid on resp. up to it, relative to v_0
+    const double v0 = (double)sh.v[0], dv = own ? (double)sh.v[tid] - v0 : 0.0;
+    double qp[2] = {dv, 0.0}, pp[2] = {dv, 0.0};
+    spread2(qp, pp);
+    double bad[1] = {0.0};
+    sc_sync(kw);
+    if (own) {
+      const double s = x[0] + y[0];
+      const bool alive = (s >= S_MIN);
+      const double f = alive ? (x[1] + y[1]) / s : dv;
+      if (!(s == s) || s > 1e300 || !(f == f)) bad[0] = 1.0;
+      const int id = sh.id[tid];
+      const size_t lk = (size_t)layer * k;
+      sp.p.perm[lk + tid] = id;
+      Cl[id] = sh.v[tid];
+      sp.p.S[lk + id] = alive ? (float)s : 0.f;
+      sp.p.F[lk + id] = (float)(v0 + f);
+      double* t = tab + tid;
+      t[TB_V * K1] = dv;
+      t[TB_A * K1] = one_warp ? scn.cb[0] : a;
+      t[TB_RP * K1] = rP;
+      t[TB_RQ * K1] = rQ;
+      t[TB_L0 * K1] = L0;
+      t[TB_L1 * K1] = L1;
+      t[TB_M0 * K1] = M0;
+      t[TB_M1 * K1] = M1;
+      t[TB_X0 * K1] = X0;
+      t[TB_X1 * K1] = X1;
+      t[TB_S * K1] = alive ? s : 0.0;
+      t[TB_F * K1] = f;
+      if (tid == 0) tab[TB_V * K1 + k] = v0;
+      sh.qs[tid] = qp[0] * rQ;
+    }
+    sc_sync(kw);
+    if (own) {
+      // interval tid + 1 (and interval 0): the outer ones have their even point far outside
+      const double cl = pp[0] * rP, cr = tid + 1 < k ? sh.qs[tid + 1] : cl;
+      float* o = ft + tid + 1;
+      float e = 3.0e38f, off = 0.f;
+      if (tid + 1 < k) {
+        const double even = sh.even[tid + 1];
+        e = (float)even;
+        off = (float)(((double)e - even) * (double)ly.slope);
+      }
+      ft[FT_V * K1 + tid] = sh.v[tid];
+      o[FT_E * K1] = e;
+      o[FT_O * K1] = off;
+      o[FT_R * K1] = (float)(v0 + cr);
+      o[FT_D * K1] = (float)(cl - cr);
+      if (tid == 0) {
+        ft[FT_E * K1] = -3.0e38f;
+        ft[FT_O * K1] = 0.f;
+        ft[FT_R * K1] = (float)(v0 + sh.qs[0]);
+        ft[FT_D * K1] = 0.f;
+      }
+    }
+    sc_reduce<1>(bad, k, sh.tmp);
+    if (tid == 0) {
+      st->fwd_iters = sh.iters;
+      st->fwd_res = sh.res;
+      st->dead = sh.dead;
+      st->fwd_done = sh.done;
+      st->status = bad[0] > 0.0 ? ST_NONFINITE : sh.status;
+    }
+  }
+}
+
+cudaError_t launch_scalar_init(const ScalarParams& sp, int grid, cudaStream_t stream) {
+  idkm_scalar_init<<<grid, SI_T, 0, stream>>>(sp);
+  return cudaGetLastError();
+}
+
+template <int LOG>
+static cudaError_t launch_loop(const ScalarParams& sp, int grid, cudaStream_t stream) {
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t rc = cudaFuncSetAttribute(idkm_scalar_loop<LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_DYN);
+    if (rc != cudaSuccess) return rc;
+    configured = true;
+  }
+  // blocks of one layer wait for each other: a cooperative launch is refused if they cannot all be resident.  (A grid of
+  // one block per layer has no barriers and is launched plainly.)
+  void* args[1] = {const_cast<ScalarParams*>(&sp)};
+  if (grid == sp.n_layers && sp.missing_arrivals == 0) {
+    idkm_scalar_loop<LOG><<<grid, SC_T, SC_DYN, stream>>>(sp);
+    return cudaGetLastError();
+  }
+  return cudaLaunchCooperativeKernel((const void*)&idkm_scalar_loop<LOG>, dim3((unsigned)grid, 1, 1), dim3(SC_T, 1, 1), args, (size_t)SC_DYN, stream);
+}
+cudaError_t launch_scalar_loop(const ScalarParams& sp, int grid, cudaStream_t stream) {
+  if (sp.k <= 2) return launch_loop<1>(sp, grid, stream);
+  if (sp.k <= 4) return launch_loop<2>(sp, grid, stream);
+  if (sp.k <= 8) return launch_loop<3>(sp, grid, stream);
+  if (sp.k <= 16) return launch_loop<4>(sp, grid, stream);
+  if (sp.k <= 32) return launch_loop<5>(sp, grid, stream);
+  return launch_loop<0>(sp, grid, stream);
+}
+
+}  // namespace idkm

@@ -1,0 +1,130 @@
+"""Scalar weights in the interval form (bins with moments in the loop, one search per weight in the passes, the adjoint
+iteration on interval sums) against the float64 oracle (B200 only).  The backward is compared at the centroids the library
+itself returned, where no weight can lie between the two sides' centroids."""
+import numpy as np
+import pytest
+
+from paper_2312_07759_b200 import workloads as WL
+from parity_util import TOL_C, TOL_GRAD, assert_close
+
+pytestmark = pytest.mark.gpu
+
+
+def weights(kind, m, rng):
+    if kind == "normal":
+        return rng.standard_normal(m) * 0.03
+    if kind == "laplace":
+        return rng.laplace(0.0, 0.02, m)
+    if kind == "pruned":            # half the weights are exactly zero
+        return np.where(rng.random(m) < 0.5, 0.0, rng.standard_normal(m) * 0.03)
+    if kind == "levels":            # three quarters of the weights sit on two values: bins of very many equal weights
+        return np.where(rng.random(m) < 0.75, np.where(rng.random(m) < 0.5, 0.0125, -0.03125), rng.standard_normal(m) * 0.03)
+    if kind == "offset":            # a narrow range far from zero
+        return 1.0 + rng.standard_normal(m) * 1e-3
+    if kind == "outlier":           # one weight far outside the rest
+        w = rng.standard_normal(m) * 0.03
+        w[m // 2] = 4.0
+        return w
+    raise ValueError(kind)
+
+
+def check(W, C0, tau, iters, adj_iters, alpha=1.0, offs=None):
+    import torch
+    from oracle import idkm_ref as R
+    from paper_2312_07759_b200 import binding as B
+    m = W.shape[0]
+    offs = [0, m] if offs is None else offs
+    L = len(offs) - 1
+    k = C0.shape[0] // L
+    G = (np.random.default_rng(m).standard_normal(W.shape) * 0.3 + 0.1).astype(np.float32)
+    ctx = B.Context()
+    Wd, Cd, Gd = (torch.from_numpy(x).cuda() for x in (W, C0, G))
+    n0 = ctx.launches
+    fr = ctx.forward(Wd, Cd, tau, 0.0, iters, layer_offsets=offs)
+    torch.cuda.synchronize()
+    assert ctx.launches - n0 == 3
+    dWj, dCj = ctx.backward(Gd, B.JFB, 0.0, 0, 1.0)
+    dW, dC = ctx.backward(Gd, B.IMPLICIT, 0.0, adj_iters, alpha)
+    info = ctx.info()
+    for l in range(L):
+        a, b = offs[l], offs[l + 1]
+        W64, C64, G64 = W[a:b].astype(np.float64), C0[l * k:(l + 1) * k].astype(np.float64), G[a:b].astype(np.float64)
+        Ct, _, res, _ = R.forward(W64, C64, tau, 0.0, iters)
+        C = fr.C.cpu().numpy()[l * k:(l + 1) * k]
+        assert info[l].status in (0, B.ERR_DIVERGED) and info[l].fwd_iters == iters
+        assert_close(C, Ct, TOL_C, f"layer {l} C")
+        Cg = C.astype(np.float64)
+        Wq, _, S, F = R.final(W64, Cg, tau)
+        assert_close(fr.Wq.cpu().numpy()[a:b], Wq, TOL_C, f"layer {l} Wq")
+        rj, cj, _, _ = R.backward(W64, G64, Cg, tau, S, F, mode="jfb")
+        assert_close(dCj.cpu().numpy()[l * k:(l + 1) * k], cj, TOL_GRAD, f"layer {l} dC jfb")
+        assert_close(dWj.cpu().numpy()[a:b], rj, TOL_GRAD, f"layer {l} dW jfb")
+        if info[l].status == 0:
+            ri, ci, _, _ = R.backward(W64, G64, Cg, tau, S, F, mode="implicit", alpha=alpha, adj_max_iter=adj_iters)
+            assert info[l].adj_iters == adj_iters
+            assert_close(dC.cpu().numpy()[l * k:(l + 1) * k], ci, TOL_GRAD, f"layer {l} dC implicit")
+            assert_close(dW.cpu().numpy()[a:b], ri, TOL_GRAD, f"layer {l} dW implicit")
+    return ctx
+
+
+# one block and several, bins of one weight and of thousands, codebooks of one warp and of eight, tau from far below the
+# bin width the workspace allows (weights evaluated one by one) to far above the weights' range
+@pytest.mark.parametrize("kind,m,k,tau", [
+    ("normal", 5, 2, 0.01), ("normal", 257, 1, 0.01), ("normal", 4096, 4, 0.05), ("normal", 36864, 8, 0.01),
+    ("normal", 36865, 31, 0.004), ("laplace", 100003, 33, 0.003), ("normal", 200001, 64, 0.002), ("laplace", 300007, 256, 0.001),
+    ("normal", 50001, 256, 0.02), ("laplace", 65536, 16, 5e-4), ("normal", 8192, 8, 5e-5), ("laplace", 150000, 12, 2e-5),
+    ("pruned", 120001, 4, 0.01), ("pruned", 30000, 7, 0.002), ("levels", 150001, 5, 0.004), ("offset", 40000, 4, 5e-4),
+    ("outlier", 70000, 5, 0.003), ("outlier", 70000, 5, 2e-4), ("normal", 20000, 3, 10.0), ("normal", 1 << 20, 4, 0.002),
+])
+def test_interval_form_against_the_oracle(kind, m, k, tau):
+    rng = np.random.default_rng(m + k)
+    W = weights(kind, m, rng).astype(np.float32).reshape(m, 1)
+    # C0 in drawn order (unsorted), distinct values where the weights allow it
+    u = np.unique(W)
+    C0 = rng.choice(u, size=min(k, u.size), replace=False).reshape(-1, 1).astype(np.float32)
+    check(W, C0, float(np.float32(tau)), 6, 5, alpha=0.5)
+
+
+def test_interval_form_on_ragged_batches():
+    """Unaligned layer starts, layers of a few weights and of many blocks, one that collapses, in one call."""
+    rng = np.random.default_rng(5)
+    sizes = [1001, 37, 70003, 9, 200001, 4096]
+    stds = [0.05, 0.05, 0.0008, 0.03, 0.02, 0.1]
+    offs = [0] + [int(x) for x in np.cumsum(sizes)]
+    W = np.concatenate([rng.standard_normal((n, 1)) * s for n, s in zip(sizes, stds)]).astype(np.float32)
+    C0 = np.concatenate([WL.quantile_centroids(W[offs[l]:offs[l + 1]], 4) for l in range(len(sizes))])
+    ctx = check(W, C0, float(np.float32(0.01)), 12, 9, offs=offs)
+    assert ctx.busy_tickets() == 0
+
+
+def test_weights_on_centroids_take_the_zero_subgradient():
+    """Weights that equal a centroid exactly: n = 0 there (centroids handed over with the forward loop run once, from a
+    point that symmetry keeps in place: the outer centroids move, the weights at zero stay on the middle one)."""
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    W = np.concatenate([np.repeat(np.array([-0.03, -0.01, 0.01, 0.03], np.float32), 300), np.zeros(50, np.float32)]).reshape(-1, 1)
+    C0 = np.array([[-0.02], [0.0], [0.02]], np.float32)
+    ctx = B.Context()
+    C = ctx.forward(torch.from_numpy(W).cuda(), torch.from_numpy(C0).cuda(), 0.01, 0.0, 4).C.cpu().numpy()
+    if C[1, 0] != 0.0:
+        pytest.skip("rounding moved the middle centroid off the weights")
+    check(W, C0, float(np.float32(0.01)), 4, 4)
+
+
+def test_interval_form_agrees_with_the_pairwise_kernels_and_is_reproducible():
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    wl = WL.single_layer(500000, 1, 24, 0.004, std=0.03, seed=2, max_iter=20, adj_max_iter=30)
+    W, C0, G = (torch.from_numpy(x).cuda() for x in (wl.W, wl.C0, wl.G))
+    out = []
+    for method, adj in ((0, 0), (0, 0), (1, 1)):
+        ctx = B.Context()
+        ctx.set_forward_loop(method)
+        ctx.set_adjoint_method(adj)
+        fr = ctx.forward(W, C0, wl.tau, 0.0, wl.max_iter)
+        dW, dC = ctx.backward(G, B.IMPLICIT, 0.0, wl.adj_max_iter, 0.5)
+        out.append([t.cpu().numpy() for t in (fr.C, fr.Wq, dW, dC)])
+    for a, b in zip(out[0], out[1]):
+        assert np.array_equal(a, b)
+    assert_close(out[0][0], out[2][0], 2e-6, "C")
+    assert_close(out[0][1], out[2][1], 2e-6, "Wq")
