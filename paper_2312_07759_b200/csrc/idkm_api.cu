@@ -705,7 +705,7 @@ static int scalar_deal(ScalarParams* sp, int grid, long long min_rows) {
   return sp->blk_first[L];
 }
 
-constexpr long long SCALAR_LOOP_ROWS = 8192;    // weights a block of the loop kernel summarises at least
+constexpr long long SCALAR_LOOP_ROWS = 16384;   // weights a block of the loop kernel summarises at least
 constexpr long long SCALAR_PASS_ROWS = 1024;    // ... of a streaming pass
 constexpr long long SCALAR_GRAD_ROWS = 256;     // weights a thread of the gradient pass takes before more blocks are used
 

@@ -53,10 +53,11 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   if (hc < range / (double)(cap - 8)) hc = range / (double)(cap - 8);
   if (hc > range) hc = range;
   if (hc < hmin) hc = hmin;
-  // fine bins: about 64 weights each, at least 16 to a coarse bin (see sc_bin_below), as many as the workspace holds
+  // fine bins: about 64 weights each; 16 to a coarse bin (see sc_bin_below) while they hold 8 weights; as many as the
+  // workspace holds
   const long long nc0 = (long long)(range / hc) + 5;
   long long want = m / 64 < 512 ? 512 : m / 64;
-  if (want < 16 * nc0) want = 16 * nc0;
+  if (want < 16 * nc0) want = 16 * nc0 < m / 8 ? 16 * nc0 : (want < m / 8 ? m / 8 : want);
   if (want > cap) want = cap;
   int f = 0;
   while (f < 12 && hc / (double)(2 << f) >= hmin && (nc0 << (f + 1)) <= want) ++f;
@@ -884,6 +885,10 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
   };
   const long long r0 = m * b / NB, r1 = m * (b + 1) / NB;
   unsigned int* cnt = reinterpret_cast<unsigned int*>(dyn);
+  auto in_smem = [&](const ScGrid& g) {
+    return alone && g.nc <= SC_SMALL_NC &&
+           36 * (size_t)g.nf + 64 + 2 * ((size_t)m + 16) + 4 * (size_t)g.nf <= (size_t)(SC_DYN - SC_SH_BYTES - SC_SMALL_OFF);
+  };
   grid_dependency_sync();
   if (warp == 0) {
     float lo = __int_as_float(0x7f800000), hi = -lo, bad = 0.f;
@@ -917,6 +922,13 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
     const ScGrid g = sh.g;
     const int nf = g.nf;
     bool ok = true;
+    if (in_smem(g)) {
+      // a small layer of one block: everything stays in shared memory (the counters at its end)
+      frec = reinterpret_cast<long long*>(dyn + SC_SMALL_OFF);
+      fstart = reinterpret_cast<unsigned int*>(frec + 4 * (size_t)nf);
+      grouped = reinterpret_cast<unsigned short*>(fstart + ((nf + 4) & ~3));
+      cnt = reinterpret_cast<unsigned int*>(dyn + (SC_DYN - SC_SH_BYTES)) - ((nf + 3) & ~3);
+    }
     // ---- count the block's weights per fine bin ----
     for (int i = tid; i < nf; i += SC_T) cnt[i] = 0u;
     __syncthreads();
@@ -1055,8 +1067,9 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
         }
       } else {
         // a quarter of a warp each, eight places per lane and load, the next bin's first two loads issued ahead
-        const unsigned short* all = sp.p.grouped;
-        const long long row0 = sp.row_off[layer], total = sp.row_off[sp.n_layers];
+        const bool own = in_smem(g);
+        const unsigned short* all = own ? grouped : sp.p.grouped;
+        const long long row0 = own ? 0 : sp.row_off[layer], total = own ? m : sp.row_off[sp.n_layers];
         const int step = NB * SC_T / 8, ql = lane & 7;
         const bool full = g.F < 64;   // (see sc_bin_below)
         const unsigned int qmask = 0xffu << (lane & 24);
@@ -1170,8 +1183,9 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
           const int f = (c << g.fshift) + f0 + (lane % wd);
           double x[4] = {0.0, 0.0, 0.0, 0.0}, y[4];
           if (in) {
-            const longlong2 u0 = __ldcg(reinterpret_cast<const longlong2*>(frec + (size_t)f * 4));
-            const longlong2 u1 = __ldcg(reinterpret_cast<const longlong2*>(frec + (size_t)f * 4) + 1);
+            // (written by other blocks a barrier ago and not read before: plain loads see it; the place may be shared memory)
+            const longlong2 u0 = reinterpret_cast<const longlong2*>(frec + (size_t)f * 4)[0];
+            const longlong2 u1 = reinterpret_cast<const longlong2*>(frec + (size_t)f * 4)[1];
             const double n = (double)(cnt[f] - (f > 0 ? cnt[f - 1] : 0u));
             sc_shift(g, sc_fine_x0(g, f), n, (double)u0.x, (double)u0.y, (double)u1.x, (double)u1.y, x);
           }
@@ -1293,25 +1307,10 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
       __syncthreads();
     }
     if (tid == 0) ly.rec.cx[0] = ly.rec.cn[0] = 0.0;
-    // a small layer's places, bin starts and moments too, behind the records (the records of few coarse bins are short:
-    // strides and arrays as above, so only what lies behind the last array's used part is free)
-    if (g.nc <= SC_SMALL_NC) {
-      unsigned char* q = dyn + SC_SMALL_OFF;
-      const int a0 = (int)(ly.row0 & 7);
-      const size_t need = 32 * (size_t)g.nf + 4 * (((size_t)g.nf + 4) & ~(size_t)3) + 2 * ((size_t)m + 16);
-      if (need <= (size_t)(SC_DYN - SC_SH_BYTES - SC_SMALL_OFF)) {
-        double* sf = reinterpret_cast<double*>(q);
-        unsigned int* ss = reinterpret_cast<unsigned int*>(q + 32 * (size_t)g.nf);
-        unsigned short* sg = reinterpret_cast<unsigned short*>(ss + ((g.nf + 4) & ~3));
-        for (int i = tid; i < 4 * g.nf; i += SC_T) sf[i] = ly.frec[i];
-        for (int i = tid; i <= g.nf; i += SC_T) ss[i] = fstart[i];
-        for (int i = tid; i < (int)m; i += SC_T) sg[a0 + i] = grouped[i];
-        ly.frec = sf;
-        ly.fstart = ss;
-        ly.grouped = sg;
-        ly.row0 = a0;
-        ly.total = a0 + m;
-      }
+    if (in_smem(g)) {
+      ly.row0 = 0;
+      ly.grouped = grouped;
+      ly.total = m;
     }
   }
   constexpr bool one_warp = LOG > 0;
