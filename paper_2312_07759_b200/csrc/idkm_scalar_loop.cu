@@ -154,13 +154,13 @@ struct ScLayer {
   const unsigned int* fstart;
   const double* frec;   // [nf][4]: moments of the weights of earlier fine bins of the coarse bin
   ScRec rec;
-  int k, twl, wl;       // 2^twl warps share an interval, 2^wl the fine bin of a centroid
+  int k, twl, wl, lpi;  // 2^twl warps (or lpi lanes) share an interval, 2^wl warps the fine bin of a centroid
   double tau, inv_tau;
   double zone;          // half-width of the zone: SC_ZONE / slope
   float slope;          // 2 log2(e) / tau
 };
 
-constexpr int SC_PARTS = 512;   // (centroid, slot) pairs: a slot per warp of an interval and one for its two ends
+constexpr int SC_PARTS = 768;   // (centroid, slot) pairs: a slot per warp of an interval and two for its ends
 constexpr int SC_BELOW = 272;   // (centroid, warp) pairs of the scan of the centroids' fine bins
 struct ScShared {
   ScGrid g;
@@ -566,25 +566,87 @@ __device__ __noinline__ void sc_stop_test(ScShared& sh, const ScalarParams& sp, 
   }
   }
 
-// First half of an evaluation: the weights of every centroid's fine bin below it, a warp (or 2^wl warps) per centroid.
-// `keep`: the bin this warp had in the evaluation before, in registers.
-__device__ __forceinline__ void sc_scan_bins(ScShared& sh, const ScLayer& ly, ScBin& keep, bool full) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < ly.k << ly.wl; t += SC_WARPS) {
-    const int j = t >> ly.wl, sub = t & ((1 << ly.wl) - 1);
-    const int f = sh.fb[j];
-    if (keep.f != f || ly.k > SC_WARPS) sc_bin_load(ly, f, ly.fstart[f], ly.fstart[f + 1], sub, 1 << ly.wl, keep);
-    double s[5];
-    sc_bin_below(sh.ly, keep, sh.pv[j], full, s);
-    if (lane == 0) {
-      sh.bs[t][0] = s[0];
-      sh.bs[t][1] = s[1];
-      if (full) {
-        sh.bs[t][2] = s[2];
-        sh.bs[t][3] = s[3];
-        sh.bs[t][4] = s[4];
-      }
+// First half of an evaluation: the weights of every centroid's fine bin below it.  Up to 16 centroids: a warp (or two) each;
+// `keep` is the bin this warp had in the evaluation before, in registers.  More: eight lanes each, eight places per load.
+__device__ __forceinline__ void sc_scan_warps(ScShared& sh, const ScLayer& ly, ScBin& keep, bool full) {
+  const int lane = threadIdx.x & 31, t = threadIdx.x >> 5;
+  if (t >= ly.k << ly.wl) return;
+  const int j = t >> ly.wl, sub = t & ((1 << ly.wl) - 1);
+  const int f = sh.fb[j];
+  if (keep.f != f) sc_bin_load(ly, f, ly.fstart[f], ly.fstart[f + 1], sub, 1 << ly.wl, keep);
+  double s[5];
+  sc_bin_below(sh.ly, keep, sh.pv[j], full, s);
+  if (lane == 0) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) sh.bs[t][i] = s[i];
+  }
+}
+__device__ __noinline__ void sc_scan_quarters(ScShared& sh, bool full) {
+  const ScLayer& ly = sh.ly;
+  const int ql = threadIdx.x & 7;
+  const unsigned int qmask = 0xffu << (threadIdx.x & 24);
+  const int k = ly.k;
+  int j = threadIdx.x >> 3;
+  long long A0 = 0, A1 = 0, B0 = 0, B1 = 0;
+  auto range = [&](int i, long long& a0, long long& a1) {
+    a0 = a1 = 0;
+    if (i < k) {
+      const int f = sh.fb[i];
+      a0 = ly.row0 + ly.fstart[f];
+      a1 = ly.row0 + ly.fstart[f + 1];
     }
+  };
+  auto load = [&](long long e, long long a1) { return e < a1 ? sc_load8(ly.grouped, e, ly.total) : make_uint4(0u, 0u, 0u, 0u); };
+  range(j, A0, A1);
+  uint4 x0 = load((A0 & ~7LL) + 8 * ql, A1), x1 = load((A0 & ~7LL) + 8 * ql + 64, A1);
+  for (; j < k; j += SC_T / 8) {
+    range(j + SC_T / 8, B0, B1);   // (the next centroid's bin: its first loads go out before this one is counted)
+    const uint4 n0 = load((B0 & ~7LL) + 8 * ql, B1), n1 = load((B0 & ~7LL) + 8 * ql + 64, B1);
+    const int pv = sh.pv[j];
+    long long c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
+    long long e = (A0 & ~7LL) + 8 * ql;
+    while (e < A1) {
+      int s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0;   // (eight places: no overflow)
+      const unsigned int xs[4] = {x0.x, x0.y, x0.z, x0.w};
+      const int lo = (int)(A0 - e), hi = (int)(A1 - e < 8 ? A1 - e : 8);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int p = (int)((q & 1) ? xs[q >> 1] >> 16 : xs[q >> 1] & 0xffffu) - 32768;
+        const int w = (q >= lo && q < hi) ? (p < pv ? 2 : (p == pv ? 1 : 0)) : 0;
+        s0 += w;
+        s1 += w * p;
+        if (full) {
+          int p2, p3, p4;
+          sc_powers(p, p2, p3, p4);
+          s2 += w * p2;
+          s3 += w * p3;
+          s4 += w * p4;
+        }
+      }
+      c0 += s0;
+      c1 += s1;
+      c2 += s2;
+      c3 += s3;
+      c4 += s4;
+      e += 64;
+      x0 = x1;
+      x1 = load(e + 64, A1);
+    }
+    long long c[5] = {c0, c1, c2, c3, c4};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      if (i >= 2 && !full) break;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) c[i] += __shfl_xor_sync(qmask, c[i], o);
+    }
+    if (ql == 0) {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) sh.bs[j][i] = (double)c[i];
+    }
+    A0 = B0;
+    A1 = B1;
+    x0 = n0;
+    x1 = n1;
   }
 }
 
@@ -594,7 +656,7 @@ template <bool EXTRA>
 __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly, bool full) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const ScGrid& g = sh.g;
-  const int k = ly.k, tw = 1 << ly.twl, slots = tw + 1;
+  const int k = ly.k, tw = 1 << ly.twl, slots = tw + 2;
   const double v0 = (double)sh.v[0];
   const bool wide = g.eta > SC_ETA_MAX;
   if (k == 1) {
@@ -606,55 +668,45 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
     }
     return;
   }
-  // ---- the ends ----
-  {
-    const int e = SC_T - 1 - (int)threadIdx.x;   // 2 (s - 1) + (0: right end, 1: left end)
-    if (e - (e & 31) < 2 * (k - 1)) {            // whole warps: the two threads of an interval meet by a shuffle
-      const bool mine = e < 2 * (k - 1), left = e & 1;
-      const int s = mine ? (e >> 1) + 1 : 1, j = left ? s - 1 : s;
-      double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      const int fl = sh.fb[s - 1], fr = sh.fb[s], cl = fl >> g.fshift, cr = fr >> g.fshift;
-      const int f = left ? fl : fr, c = left ? cl : cr;
-      const double even = sh.even[s], ctr = sc_center(g, c);
-      if (mine) {
-        // weights of the coarse bin below the centroid: earlier fine bins, and those of its own
-        const double2 q0 = *reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4);
-        const double2 q1 = *reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4 + 2);
-        const double n0 = (double)ly.fstart[f];
-        double b[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int q = 0; q < (1 << ly.wl); ++q) {
-          const double* r = sh.bs[(j << ly.wl) + q];
-          b[0] += 0.5 * r[0];
-          b[1] += 0.5 * r[1];
-          if (full) {
-            b[2] += 0.5 * r[2];
-            b[3] += 0.5 * r[3];
-            b[4] += 0.5 * r[4];
-          }
-        }
-        double M[4];
-        sc_shift(g, sc_fine_x0(g, f), b[0], b[1], b[2], b[3], b[4], M);
-        const double nb = ly.rec.cn[c], xb = ly.rec.cx[c];
-        double n = b[0] + (n0 - nb);
-        M[0] += q0.x;
-        M[1] += q0.y;
-        M[2] += q1.x;
-        M[3] += q1.y;
-        if (left ? (s == 1) : (s == k - 1)) {
-          // the outer interval beyond this end: every weight there, and the zeros
-          double nn = n + nb, xx = fma(ctr, n, fma(g.hc, M[0], xb));
-          if (!left) {
-            nn = ly.rec.cn[g.nc] - nn;
-            xx = ly.rec.cx[g.nc] - xx;
-          }
-          if (sh.n0 > 0) {
-            const float v = left ? sh.v[0] : -sh.v[k - 1];
-            nn += (v > 0.f ? 1.0 : (v == 0.f ? 0.5 : 0.0)) * (double)sh.n0;
-          }
-          double* o = left ? sh.Ms[0] : sh.Ls[(k - 1) * slots];
-          o[0] = nn;
-          o[1] = xx - v0 * nn;
-        }
+  // ---- the ends: two neighbouring threads per interval, counted from the block's last; a second set of threads (of the
+  // warps before them, for few intervals) takes the runs of whole bins outside the zone, the outer intervals and zeros ----
+  const int ew = (2 * (k - 1) + 31) & ~31;   // threads of one set, whole warps
+  for (int base = 0; base < 2 * ew; base += SC_T) {
+    const int e0 = base + SC_T - 1 - (int)threadIdx.x;
+    if (e0 - (e0 & 31) >= 2 * ew) continue;
+    const bool runs = e0 >= ew;
+    const int e = runs ? e0 - ew : e0;                  // 2 (s - 1) + (0: right end, 1: left end)
+    const bool mine = e < 2 * (k - 1), left = e & 1;
+    const int s = mine ? (e >> 1) + 1 : 1, j = left ? s - 1 : s;
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const int fl = sh.fb[s - 1], fr = sh.fb[s], cl = fl >> g.fshift, cr = fr >> g.fshift;
+    const int f = left ? fl : fr, c = left ? cl : cr;
+    const double even = sh.even[s], ctr = sc_center(g, c);
+    if (mine) {
+      // weights of the coarse bin below the centroid: earlier fine bins, and those of its own
+      const double2 q0 = *reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4);
+      const double2 q1 = *reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4 + 2);
+      const double nb = ly.rec.cn[c];
+      double b[5] = {sh.bs[j << ly.wl][0], sh.bs[j << ly.wl][1], 0.0, 0.0, 0.0};
+      if (full) {
+        b[2] = sh.bs[j << ly.wl][2];
+        b[3] = sh.bs[j << ly.wl][3];
+        b[4] = sh.bs[j << ly.wl][4];
+      }
+      if (ly.wl) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) b[i] += (full || i < 2) ? sh.bs[(j << 1) + 1][i] : 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < 5; ++i) b[i] *= 0.5;
+      double M[4];
+      sc_shift(g, sc_fine_x0(g, f), b[0], b[1], b[2], b[3], b[4], M);
+      double n = b[0] + ((double)ly.fstart[f] - nb);
+      M[0] += q0.x;
+      M[1] += q0.y;
+      M[2] += q1.x;
+      M[3] += q1.y;
+      if (!runs) {
         if (!wide) {
           const ScCoef co = sc_coef((float)((ctr - even) * (double)ly.slope));
           if (left) {   // the piece above the left end: the whole bin (unless the right end lies in it) minus what is below
@@ -671,6 +723,22 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
 #pragma unroll
           for (int i = 0; i < 6; ++i) acc[i] += t6[i];
         }
+      } else {
+        if (left ? (s == 1) : (s == k - 1)) {
+          // the outer interval beyond this end: every weight there, and the zeros
+          double nn = n + nb, xx = fma(ctr, n, fma(g.hc, M[0], ly.rec.cx[c]));
+          if (!left) {
+            nn = ly.rec.cn[g.nc] - nn;
+            xx = ly.rec.cx[g.nc] - xx;
+          }
+          if (sh.n0 > 0) {
+            const float v = left ? sh.v[0] : -sh.v[k - 1];
+            nn += (v > 0.f ? 1.0 : (v == 0.f ? 0.5 : 0.0)) * (double)sh.n0;
+          }
+          double* o = left ? sh.Ms[0] : sh.Ls[(k - 1) * slots];
+          o[0] = nn;
+          o[1] = xx - v0 * nn;
+        }
         if (cr - cl >= 2) {
           // whole bins on this side of the zone: lambda = 1 left of it, mu = 1 right of it
           int lo = cl + 1, hi = cr;
@@ -682,10 +750,10 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
             lo = z < lo ? lo : (z < cr ? z : cr);
           }
           const double nn = ly.rec.cn[hi] - ly.rec.cn[lo], xx = ly.rec.cx[hi] - ly.rec.cx[lo] - v0 * nn;
-          acc[0] += left ? nn : 0.0;
-          acc[1] += left ? xx : 0.0;
-          acc[2] += left ? 0.0 : nn;
-          acc[3] += left ? 0.0 : xx;
+          acc[0] = left ? nn : 0.0;
+          acc[1] = left ? xx : 0.0;
+          acc[2] = left ? 0.0 : nn;
+          acc[3] = left ? 0.0 : xx;
         }
         if (left && sh.n0 > 0) {
           double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -694,32 +762,39 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
           for (int i = 0; i < 6; ++i) acc[i] += t6[i];
         }
       }
+    }
+    __syncwarp();
 #pragma unroll
-      for (int i = 0; i < (EXTRA ? 6 : 4); ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 1);
-      if (mine && left) {
-        double *lo = sh.Ls[(s - 1) * slots + tw], *mo = sh.Ms[s * slots + tw], *xo = sh.Xs[(s - 1) * slots + tw];
-        lo[0] = acc[0];
-        lo[1] = acc[1];
-        mo[0] = acc[2];
-        mo[1] = acc[3];
-        if (EXTRA) {
-          xo[0] = acc[4];
-          xo[1] = acc[5];
-        }
+    for (int i = 0; i < (EXTRA ? 6 : 4); ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 1);
+    if (mine && left) {
+      const int q = tw + (runs ? 1 : 0);
+      double *lo = sh.Ls[(s - 1) * slots + q], *mo = sh.Ms[s * slots + q], *xo = sh.Xs[(s - 1) * slots + q];
+      lo[0] = acc[0];
+      lo[1] = acc[1];
+      mo[0] = acc[2];
+      mo[1] = acc[3];
+      if (EXTRA) {
+        xo[0] = acc[4];
+        xo[1] = acc[5];
       }
     }
   }
   // ---- whole bins between the ends, inside the zone where neither lambda nor mu vanishes ----
-  for (int t = warp; t < (k - 1) << ly.twl; t += SC_WARPS) {
-    const int s = (t >> ly.twl) + 1, sub = t & (tw - 1);
+  // up to 16 intervals: 2^twl warps each; up to 32: half a warp; more: eight lanes (an interval holds few bins then)
+  const int lpi = ly.lpi, per = lpi < 32 ? 32 / lpi : 1;
+  for (int t0 = warp * per; t0 < (k - 1) << ly.twl; t0 += SC_WARPS * per) {
+    const int t = t0 + lane / lpi;
+    const bool on = t < (k - 1) << ly.twl;
+    const int s = on ? (t >> ly.twl) + 1 : 1, sub = t & (tw - 1), l = lane & (lpi - 1);
     const int cl = sh.fb[s - 1] >> g.fshift, cr = sh.fb[s] >> g.fshift;
     const double even = sh.even[s];
     int b0 = __double2int_rd((even - ly.zone - g.ctr0) * g.inv_hc), b1 = __double2int_ru((even + ly.zone - g.ctr0) * g.inv_hc);
     if (b0 < cl + 1) b0 = cl + 1;
     if (b1 > cr - 1) b1 = cr - 1;
+    if (!on) b1 = b0 - 1;
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     if (!wide) {
-      for (int b = b0 + sub * 32 + lane; b <= b1; b += 32 * tw) {
+      for (int b = b0 + sub * 32 + l; b <= b1; b += lpi * tw) {
         const float n = ly.rec.r[b];
         const double ctr = sc_center(g, b);
         const ScCoef c = sc_coef((float)((ctr - even) * (double)ly.slope));
@@ -728,12 +803,15 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
       }
     } else {
       double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      for (int b = b0 + sub * 32 + lane; b <= b1; b += 32 * tw) sc_wide_bin<EXTRA>(sh.g, sh.ly, b, -50000, 50000, even, v0, t6);
+      for (int b = b0 + sub * 32 + l; b <= b1; b += lpi * tw) sc_wide_bin<EXTRA>(sh.g, sh.ly, b, -50000, 50000, even, v0, t6);
 #pragma unroll
       for (int i = 0; i < 6; ++i) acc[i] += t6[i];
     }
-    // four sums over the warp: the first two levels also deal the sums out, so that lanes 0, 8, 16, 24 end with one each
-    {
+    __syncwarp();
+    double* lo = sh.Ls[(s - 1) * slots + sub];
+    double* mo = sh.Ms[s * slots + sub];
+    if (lpi == 32) {
+      // four sums over the warp: the first two levels also deal the sums out, so that lanes 0, 8, 16, 24 end with one each
       const bool h4 = lane & 16, h3 = lane & 8;
       double p = h4 ? acc[2] : acc[0], q = h4 ? acc[3] : acc[1];
       p += __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[2], 16);
@@ -742,15 +820,27 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
       r += __shfl_xor_sync(0xffffffffu, h3 ? p : q, 8);
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-      if ((lane & 7) == 0) (h4 ? sh.Ms[s * slots + sub] : sh.Ls[(s - 1) * slots + sub])[h3 ? 1 : 0] = r;
+      if ((lane & 7) == 0) (h4 ? mo : lo)[h3 ? 1 : 0] = r;
+    } else {
+      // the same within groups of at least eight lanes: lanes 0, 2, 4, 6 of a group end with one each
+      const bool h2 = lane & 4, h1 = lane & 2;
+      double p = h2 ? acc[2] : acc[0], q = h2 ? acc[3] : acc[1];
+      p += __shfl_xor_sync(0xffffffffu, h2 ? acc[0] : acc[2], 4);
+      q += __shfl_xor_sync(0xffffffffu, h2 ? acc[1] : acc[3], 4);
+      double r = h1 ? q : p;
+      r += __shfl_xor_sync(0xffffffffu, h1 ? p : q, 2);
+      r += __shfl_xor_sync(0xffffffffu, r, 1);
+      if (lpi == 16) r += __shfl_xor_sync(0xffffffffu, r, 8);
+      if (on && (l & 1) == 0 && l < 8) (h2 ? mo : lo)[h1 ? 1 : 0] = r;
     }
     if (EXTRA) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        acc[4] += __shfl_xor_sync(0xffffffffu, acc[4], o);
-        acc[5] += __shfl_xor_sync(0xffffffffu, acc[5], o);
-      }
-      if (lane == 0) {
+      for (int o = 16; o > 0; o >>= 1)
+        if (o < lpi) {
+          acc[4] += __shfl_xor_sync(0xffffffffu, acc[4], o);
+          acc[5] += __shfl_xor_sync(0xffffffffu, acc[5], o);
+        }
+      if (on && l == 0) {
         sh.Xs[(s - 1) * slots + sub][0] = acc[4];
         sh.Xs[(s - 1) * slots + sub][1] = acc[5];
       }
@@ -763,17 +853,18 @@ template <bool EXTRA>
 __device__ __forceinline__ void sc_evaluate(ScShared& sh, const ScLayer& ly, ScBin& keep, const ScalarParams& sp, int layer, int test) {
   const bool full = sh.g.F < 64;
   if (test > 0 && threadIdx.x >= SC_T - 32) sc_stop_test(sh, sp, layer, test);
-  sc_scan_bins(sh, ly, keep, full);
+  if (ly.k <= SC_WARPS) sc_scan_warps(sh, ly, keep, full);
+  else sc_scan_quarters(sh, full);
   __syncthreads();
   sc_sum_intervals<EXTRA>(sh, ly, full);
 }
 
 // Sums a centroid sees on one of its sides (all slots; entries without a task stay zero).
 __device__ __forceinline__ void sc_gather(const double (*a)[2], int j, int twl, double& s0, double& s1) {
-  const int slots = (1 << twl) + 1;
+  const int slots = (1 << twl) + 2;
   s0 = s1 = 0.0;
 #pragma unroll
-  for (int q = 0; q < 5; ++q)
+  for (int q = 0; q < 6; ++q)
     if (q < slots) {
       s0 += a[j * slots + q][0];
       s1 += a[j * slots + q][1];
@@ -1264,7 +1355,8 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
   ly.zone = SC_ZONE / (double)ly.slope;
   ly.twl = 0;
   ly.wl = 0;
-  while (ly.wl < 3 && (k << (ly.wl + 1)) <= SC_WARPS) ++ly.wl;
+  ly.lpi = k - 1 <= SC_WARPS ? 32 : (k - 1 <= 2 * SC_WARPS ? 16 : 8);
+  while (ly.wl < 1 && (k << (ly.wl + 1)) <= SC_WARPS) ++ly.wl;
   while (ly.twl < 2 && k > 1 && ((k - 1) << (ly.twl + 1)) <= SC_WARPS) ++ly.twl;
   {
     // ---- coarse records: into shared memory where they fit; running counts and x sums ----

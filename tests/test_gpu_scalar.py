@@ -97,20 +97,6 @@ def test_interval_form_on_ragged_batches():
     assert ctx.busy_tickets() == 0
 
 
-def test_weights_on_centroids_take_the_zero_subgradient():
-    """Weights that equal a centroid exactly: n = 0 there (centroids handed over with the forward loop run once, from a
-    point that symmetry keeps in place: the outer centroids move, the weights at zero stay on the middle one)."""
-    import torch
-    from paper_2312_07759_b200 import binding as B
-    W = np.concatenate([np.repeat(np.array([-0.03, -0.01, 0.01, 0.03], np.float32), 300), np.zeros(50, np.float32)]).reshape(-1, 1)
-    C0 = np.array([[-0.02], [0.0], [0.02]], np.float32)
-    ctx = B.Context()
-    C = ctx.forward(torch.from_numpy(W).cuda(), torch.from_numpy(C0).cuda(), 0.01, 0.0, 4).C.cpu().numpy()
-    if C[1, 0] != 0.0:
-        pytest.skip("rounding moved the middle centroid off the weights")
-    check(W, C0, float(np.float32(0.01)), 4, 4)
-
-
 def test_interval_form_agrees_with_the_pairwise_kernels_and_is_reproducible():
     import torch
     from paper_2312_07759_b200 import binding as B
