@@ -4,6 +4,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include "idkm_kernels.cuh"
 #include "idkm_scalar.cuh"
+#include "idkm_jac_mma.cuh"
 
 #include <math.h>
 #include <stdio.h>
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(INIT_T) idkm_init_forward(LayerState* st, int 
     s.adj_done = 0; s.adj_iters = 0; s.adj_res = 0.f; s.status = ST_OK;
     s.ticket = 0u; s.adj_up = 0; s.adj_prev = 3.0e38f;
     s.g_norm = 0.f;
-    for (int q = 0; q < 2; ++q) s.pad[q] = 0;
+    s.wmax = s.pad[0] = 0;
     s.precise[0] = s.precise[1] = (!squared && sqrt(box2) * inv_tau <= PRECISE_SPAN) ? 1 : 0;
     st[l] = s;
   }
@@ -184,7 +185,18 @@ struct WorkspaceLayout {
   size_t off_sc_sync, off_sc_gcount, off_sc_fstart, off_sc_frec, off_sc_crec, off_sc_bstat, off_sc_tab, off_sc_perm, off_sc_ftab,
       off_sc_gpart, off_sc_gtick;
   int sc_fine, n_sc_groups, n_sc_grad_blocks;
+  // explicit Jacobian on the tensor cores (idkm_jac_mma.cuh); jm.nt = 0: none
+  JacMmaPlan jm;
+  size_t off_jm_part, off_jm_ub, off_jm_pn, off_jm_sync;
 };
+constexpr int JM_SOLVE_ROWS = 8;   // rows of the matrix a block of the solve keeps
+static int jac_mma_solve_blocks(int d, int k) { return k * d <= 64 ? 0 : (k * d + JM_SOLVE_ROWS - 1) / JM_SOLVE_ROWS; }
+// Steps of the adjoint iteration from which the tensor-core Jacobian is used: it costs about k d^2 / 215 fused passes
+// (m = 2^22, d = 4, k = 256: see DESIGN's table of cases), and no fewer than the tiled kernels' 16.
+static int jac_mma_min_iters(int d, int k) {
+  const int n = k * d * d / 160;
+  return n < 16 ? 16 : n;
+}
 
 // Fine bins the workspace holds for n_layers layers of scalar weights: the largest layers get more.
 static int scalar_fine_total(int n_layers) {
@@ -256,6 +268,21 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
     if (rd || wr) {
       w.off_rowstat = o;
       o = align_up(o + sizeof(float2) * (size_t)m_total, 256);
+    }
+  }
+  w.jm.nt = 0;
+  {
+    JacMmaPlan jm;
+    if (w.off_rowstat != NO_ROWSTAT && jac_mma_plan(d, k, &jm)) {
+      const int nb = jac_mma_solve_blocks(d, k);
+      const size_t bytes = (size_t)jac_mma_units_max(jm, n_layers) * JM_M * jm.nt * sizeof(double);
+      if (bytes <= JM_PART_MAX && (long long)n_layers * nb <= 4LL * sms) {
+        w.jm = jm;
+        w.off_jm_part = o; o = align_up(o + bytes, 256);
+        w.off_jm_ub = o;   o = align_up(o + 16 * (size_t)n_layers * jm.kdp, 256);
+        w.off_jm_pn = o;   o = align_up(o + 32 * (size_t)n_layers * (nb + 1), 256);
+        w.off_jm_sync = o; o = align_up(o + 4 * (size_t)n_layers * JM_SYNC_WORDS, 256);
+      }
     }
   }
   w.sc_fine = 0;
@@ -778,6 +805,49 @@ static int launch_pass(idkm_ctx* ctx, int mode, PassParams* p, int repeat) {
   return IDKM_OK;
 }
 
+// The adjoint iteration on the explicit Jacobian formed by the tensor cores: one pass over the weights, then the whole
+// iteration on the matrix (in the same launch for k d <= 64).
+static int launch_jac_mma_adjoint(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p) {
+  JacMmaParams q;
+  memset(&q, 0, sizeof(q));
+  char* ws = static_cast<char*>(ctx->workspace);
+  q.W = ctx->W;
+  q.C = p.C;
+  q.S = p.S;
+  q.F = p.F;
+  q.gvec = p.gvec;
+  q.u = p.u;
+  q.rowstat = p.rowstat;
+  q.st = p.st;
+  q.hist_adj = p.hist_adj;
+  q.part = reinterpret_cast<double*>(ws + wl.off_jm_part);
+  q.ub = reinterpret_cast<double*>(ws + wl.off_jm_ub);
+  q.pn = reinterpret_cast<double*>(ws + wl.off_jm_pn);
+  q.sync = reinterpret_cast<unsigned int*>(ws + wl.off_jm_sync);
+  q.scale = p.scale;
+  q.inv_tau_d = p.inv_tau_d;
+  q.tol = p.tol;
+  q.alpha = p.alpha;
+  q.max_iter = p.max_iter;
+  q.k = ctx->k;
+  q.n_layers = ctx->n_layers;
+  q.tiles_m = wl.jm.tiles_m;
+  q.tiles_n = wl.jm.tiles_n;
+  q.solve_blocks = jac_mma_solve_blocks(ctx->d, ctx->k);
+  q.missing_arrivals = ctx->hook_missing_arrivals;
+  q.spin_limit = SMALL_SPIN_LIMIT;
+  if (ctx->hook_spin_limit > 0 && ctx->hook_spin_limit < SMALL_SPIN_LIMIT) q.spin_limit = ctx->hook_spin_limit;
+  for (int l = 0; l <= MAX_LAYERS; ++l) q.row_off[l] = ctx->row_off[l < ctx->n_layers ? l : ctx->n_layers];
+  const int units = jac_mma_split(wl.jm, &q);
+  if (launch_jac_mma(ctx->d, wl.jm, q, units, ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
+  ++ctx->launches;
+  if (q.solve_blocks > 0) {
+    if (launch_jac_solve(ctx->d, wl.jm, q, ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
+    ++ctx->launches;
+  }
+  return IDKM_OK;
+}
+
 // The last phase of a backward: the pass that writes dL/dW from the adjoint u in the workspace, and the copy of u.
 static int backward_outputs(idkm_ctx* ctx, const WorkspaceLayout& wl, PassParams* p, bool scalar, float* dW_out, float* dC_out) {
   if (dW_out) {
@@ -965,7 +1035,8 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
   const bool explicit_jac = exact || (ctx->adjoint_method == 0 && !ctx->squared && fj >= 0 &&
                                       (!jac_tile || adj_max_iter >= JAC_TILE_MIN_ITERS));
   // the per-row softmax reference and normaliser are kept only if fused adjoint passes follow
-  if (!solve || explicit_jac) p.rowstat = nullptr;
+  const bool jac_mma = solve && ctx->adjoint_method == 0 && !ctx->squared && wl.jm.nt > 0 && adj_max_iter >= jac_mma_min_iters(ctx->d, ctx->k);
+  if (!solve || (explicit_jac && !jac_mma)) p.rowstat = nullptr;
   mark(ctx, 4);
   // scalar weights whose forward left its interval tables: gradient, adjoint and dL/dW in the interval form, unless the
   // caller asked for the fused passes (1) or the exact solve (2)
@@ -979,6 +1050,8 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
     nvtxRangePushA("idkm adjoint solve");
     if (scalar) {
       rc = launch_scalar_pass(ctx, wl, p, SP_ADJOINT, dC_out);
+    } else if (jac_mma) {
+      rc = launch_jac_mma_adjoint(ctx, wl, p);
     } else if (explicit_jac) {
       if (exact) p.max_iter = -1;                  // the epilogue solves (I - J^T) u = g instead of iterating
       rc = launch_pass(ctx, JACOBIAN, &p, 1);      // one pass forms J_C; the whole iteration runs on it in the epilogue
@@ -1290,8 +1363,10 @@ int idkm_describe_path(int d, int k, int adj_max_iter, int adjoint_method, int* 
   out[2] = kernel_entry(ADJ, d, fa)->kpl;
   out[3] = kernel_entry(ADJ, d, fa)->lpw;
   const bool jac_tile = fj >= 0 && kernel_entry(JACOBIAN, d, fj)->plen > JAC_SMALL_PLEN_MAX;
-  const bool explicit_jac = adjoint_method == 0 && fj >= 0 && (!jac_tile || adj_max_iter >= JAC_TILE_MIN_ITERS);
-  out[4] = (adj_max_iter <= 0) ? 0 : ((adjoint_method == 2 && fj >= 0) ? 3 : (explicit_jac ? (jac_tile ? 2 : 1) : 0));
+  JacMmaPlan jm;
+  const bool explicit_jac = adjoint_method == 0 && ((fj >= 0 && (!jac_tile || adj_max_iter >= JAC_TILE_MIN_ITERS)) ||
+                                                    (jac_mma_plan(d, k, &jm) && adj_max_iter >= jac_mma_min_iters(d, k)));
+  out[4] = (adj_max_iter <= 0) ? 0 : ((adjoint_method == 2 && fj >= 0) ? 3 : (explicit_jac ? (fj >= 0 && !jac_tile ? 1 : 2) : 0));
   return IDKM_OK;
 }
 

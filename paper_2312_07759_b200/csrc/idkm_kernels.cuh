@@ -66,7 +66,9 @@ struct LayerState {   // 64 bytes, one per layer, in the workspace
                      // can never both take (or both skip) a layer.
   float g_norm;      // ||g||_2 of the last codebook-gradient pass: the adjoint iteration counts as diverged once
                      // ||u||_2 exceeds ADJ_GROWTH_LIMIT times it
-  int pad[2];
+  int wmax;          // largest |coordinate| of the layer's weights, as float bits (FINAL, d >= 2; read by the tensor-core
+                     // Jacobian, whose fp16 operands it scales)
+  int pad[1];
 };
 static_assert(sizeof(LayerState) == 64, "LayerState layout");
 
@@ -743,6 +745,9 @@ __device__ __forceinline__ void pass_body(const PassParams& p) {
     }
   };
   int since_spill = 0;
+  constexpr bool WMAX = (MODE == FINAL && D > 1);
+  float wmax = 0.f;   // largest |coordinate| of the layer's rows seen by this thread
+  (void)wmax;
   auto spill = [&]() {
     if constexpr (ACCUM) {
 #pragma unroll
@@ -868,6 +873,10 @@ __device__ __forceinline__ void pass_body(const PassParams& p) {
       }
     }
 
+    if constexpr (WMAX) {
+#pragma unroll
+      for (int a = 0; a < D; ++a) wmax = fmaxf(wmax, fabsf(w[a]));
+    }
     if constexpr (MODE == STEP || MODE == FINAL) {
       float rw[D];
 #pragma unroll
@@ -951,6 +960,11 @@ __device__ __forceinline__ void pass_body(const PassParams& p) {
       return;
     } else {
       float* red = reinterpret_cast<float*>(smem_raw);
+      if constexpr (WMAX) {
+        const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(wmax));
+        if (lane == 0) atomicMax(&p.st[l].wmax, wm);
+        wmax = 0.f;
+      }
       // across the groups of a warp (lanes with equal gl); the thread's own two levels are joined first
 #pragma unroll
       for (int t = 0; t < KPL; ++t)
