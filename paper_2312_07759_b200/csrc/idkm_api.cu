@@ -191,11 +191,14 @@ struct WorkspaceLayout {
 };
 constexpr int JM_SOLVE_ROWS = 8;   // rows of the matrix a block of the solve keeps
 static int jac_mma_solve_blocks(int d, int k) { return k * d <= 64 ? 0 : (k * d + JM_SOLVE_ROWS - 1) / JM_SOLVE_ROWS; }
-// Steps of the adjoint iteration from which the tensor-core Jacobian is used: it costs about k d^2 / 215 fused passes
-// (m = 2^22, d = 4, k = 256: see DESIGN's table of cases), and no fewer than the tiled kernels' 16.
+// Steps of the adjoint iteration from which the tensor-core Jacobian is used, measured against the fused passes' time a
+// step at 2 K, 20 K, 200 K and 2 M weights (alpha = 0.25, 48 steps on the matrix): k d <= 64 costs 8, 7, 6 and 5 passes
+// (d = 4, k = 16); larger codebooks 19, 19, 13 and 7 (d = 4, k = 32), 16, 12, 11 and 12 (d = 2, k = 256), and, where the
+// products count, 8, 11, 20 and 27 (d = 4, k = 256).
 static int jac_mma_min_iters(int d, int k) {
-  const int n = k * d * d / 160;
-  return n < 16 ? 16 : n;
+  const int n = k * d * d / 128;
+  const int least = k * d <= 64 ? 8 : 20;
+  return n < least ? least : n;
 }
 
 // Fine bins the workspace holds for n_layers layers of scalar weights: the largest layers get more.
@@ -275,8 +278,8 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
     JacMmaPlan jm;
     if (w.off_rowstat != NO_ROWSTAT && jac_mma_plan(d, k, &jm)) {
       const int nb = jac_mma_solve_blocks(d, k);
-      const size_t bytes = (size_t)jac_mma_units_max(jm, n_layers) * JM_M * jm.nt * sizeof(double);
-      if (bytes <= JM_PART_MAX && (long long)n_layers * nb <= 4LL * sms) {
+      const size_t bytes = jac_mma_part_bytes(jm, d, k, n_layers);
+      if (bytes <= JM_PART_MAX && (k * d > 64 || jac_mma_groups_max(n_layers) <= w.max_groups) && (long long)n_layers * nb <= 4LL * sms) {
         w.jm = jm;
         w.off_jm_part = o; o = align_up(o + bytes, 256);
         w.off_jm_ub = o;   o = align_up(o + 16 * (size_t)n_layers * jm.kdp, 256);
@@ -824,6 +827,7 @@ static int launch_jac_mma_adjoint(idkm_ctx* ctx, const WorkspaceLayout& wl, cons
   q.ub = reinterpret_cast<double*>(ws + wl.off_jm_ub);
   q.pn = reinterpret_cast<double*>(ws + wl.off_jm_pn);
   q.sync = reinterpret_cast<unsigned int*>(ws + wl.off_jm_sync);
+  q.gtickets = p.gtickets;
   q.scale = p.scale;
   q.inv_tau_d = p.inv_tau_d;
   q.tol = p.tol;
@@ -838,7 +842,7 @@ static int launch_jac_mma_adjoint(idkm_ctx* ctx, const WorkspaceLayout& wl, cons
   q.spin_limit = SMALL_SPIN_LIMIT;
   if (ctx->hook_spin_limit > 0 && ctx->hook_spin_limit < SMALL_SPIN_LIMIT) q.spin_limit = ctx->hook_spin_limit;
   for (int l = 0; l <= MAX_LAYERS; ++l) q.row_off[l] = ctx->row_off[l < ctx->n_layers ? l : ctx->n_layers];
-  const int units = jac_mma_split(wl.jm, &q);
+  const int units = jac_mma_split(wl.jm, ctx->d, &q);
   if (launch_jac_mma(ctx->d, wl.jm, q, units, ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
   ++ctx->launches;
   if (q.solve_blocks > 0) {

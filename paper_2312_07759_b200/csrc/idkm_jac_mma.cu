@@ -1,21 +1,27 @@
-// See idkm_jac_mma.cuh.  One block computes a 128 x NT tile of X^T Y over a range of weights.
+// See idkm_jac_mma.cuh.  One block computes 128 x NT tiles of X^T Y over ranges of weights.
 //
-// What bounds it: the products -- three fp16 products per multiply-add (below) -- and, almost as much, producing the
-// operands: nothing of X and Y exists in memory, every tile computes its 128 + NT columns of them from the weights, the
-// rows' softmax references and normalisers that the codebook-gradient pass left, and its centroids.  A tile of 128 x 256
-// makes 96 (weight, centroid) pairs of work per weight at d = 4 for 32 768 multiply-adds.
+// What bounds it: producing the operands.  Nothing of X and Y exists in memory; every tile computes its 128 + NT columns of
+// them from the weights, the rows' softmax references and normalisers that the codebook-gradient pass left, and its
+// centroids: at d = 4 and NT = 256, 96 (weight, centroid) pairs of ~300 instructions per eight weights and lane, two warps
+// to a scheduler (48 % of the issue slots, tensor pipe 34 % active), for 32 768 multiply-adds a weight, which three fp16
+// products take 1540 cycles a stage for.  Hence the tile as wide as the register file holds its sums, the packed fp32
+// instructions, and, where rows and columns of a tile are of the same centroids (k d <= 128), one pass for both operands.
+// Measured (adjoint of 50 steps against the fused passes): 4 M x 4, k = 256: 34 ms against 44; 1 M x 2, k = 256: 2.6
+// against 11.2; 3 M x 4, k = 16, 30 steps: 0.31 against 1.9 (1.3 with Jacobian tiles on the CUDA cores).
 //
 // Precision.  X and Y are split into two fp16 terms (22 bits, scaled by powers of two so that the second term stays
 // normal): hi hi + hi lo + lo hi; what is dropped is 2^-22 of a product, below the 2e-7 of the exponential and the
 // reciprocal square root they are made of.  The tensor core adds in fp32 without rounding to nearest, so an accumulator
-// takes one stage (64 weights) only -- small terms first -- and is then added to fp32 sums in registers, which move to an
-// fp64 partial every 16 K weights; the splits' partials are added in a fixed order.
+// takes one stage of 64 weights only -- its small terms first -- and is then added to fp32 sums in registers, which move to
+// an fp64 partial every JM_FOLD stages; the partials are added in a fixed order.  (Two stages to an accumulator were no
+// faster and 2 to 5 times less exact: 2.3e-6 to 5e-6 of the adjoint against 1e-6.)
 //
 // Roles: a producing warp makes eight weights' share of the stage (a lane holds a centroid, so nothing crosses lanes) and
 // writes it in the core-matrix order of the K-major operand, 16 bytes per lane and row of the operand: consecutive lanes
-// are consecutive rows, no bank conflicts.  One thread issues the products of a stage and commits them to the stage's
-// barrier, which frees its shared memory and hands its half of tensor memory to the accumulating warps.  Every wait is
-// bounded; if one runs out the layer's status says so.
+// are consecutive rows, no bank conflicts.  The diagonal sums Dg, d x d numbers a centroid, are added up on the way (as a
+// product of their own they took a third of the time for k d^2 useful of (k d)^2 entries).  The first accumulating warp
+// issues the products of a stage and commits them to the stage's barrier, which frees its shared memory and hands its half
+// of tensor memory over.  Every wait is bounded; if one runs out the layer's status says so.
 #include "idkm_jac_mma.cuh"
 
 #include <string.h>
@@ -23,16 +29,28 @@
 namespace idkm {
 
 constexpr int JM_POLLS = 1 << 22;
+constexpr int JM_DFOLD = 32;           // stages after which the diagonal's fp32 sums move to fp64 (one-tile codebooks)
+constexpr int JM_RED = 12;             // blocks whose partials one of them adds up (k d <= 64)
 
-template <int D, int NT>
+// PACK (k d <= 64): the lanes of a warp hold 16 centroids twice, for two sets of eight weights, so a stage takes twice the
+// weights; of the product the two diagonal blocks of lanes count, the others are between different weights.
+template <int D, int NT, bool PACK>
 struct JmCfg {
-  static constexpr int CPM = JM_M / D, CPN = NT / D;      // centroids of a tile's rows / columns
-  static constexpr int MU = CPM / 32, NU = CPN / 32;      // lane-per-centroid units of work per eight weights
+  static constexpr int LC = PACK ? 16 : 32;               // centroids of a unit of work per eight weights
+  static constexpr int MU = JM_M / D / 32, NU = NT / D / 32;
+  static constexpr int CPM = MU * LC, CPN = NU * LC;      // centroids of a tile's rows / columns
+  static constexpr int SETS = PACK ? 2 : 1;
+  static constexpr int ROWS = JM_ROWS * SETS;             // weights per stage
+  static constexpr bool BOTH = NT == JM_M;                // rows and columns are of the same centroids
   static constexpr int A_BYTES = JM_M * JM_ROWS * 2, B_BYTES = NT * JM_ROWS * 2;
   static constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
-  static constexpr int ROW_FLOATS = D + 2;
-  static constexpr int DYN = 2 * STAGE + 8 * 8 * 8 * 4;   // two stages, eight weights per producing warp
-};
+  static constexpr int SET_FLOATS = (D + 2) * 8 + 4;      // (the two sets' broadcasts fall into different banks)
+  static constexpr int OFF_DG = 2 * STAGE, OFF_ROW = OFF_DG + 8 * D * D * MU * 32 * 8;
+  static constexpr int DYN = OFF_ROW + 8 * SETS * SET_FLOATS * 4;
+  static constexpr int XY = PACK ? 64 * 64 : JM_M * NT;   // doubles of a partial: the product's, then the diagonal sums'
+  static constexpr int SLOT = XY + D * D * CPM;
+  };
+constexpr int JM_LAUNCH_REGS = 65536 / JM_THREADS;   // the two kinds of warps redistribute these: 112 + 144, 160 + 96
 
 __device__ __forceinline__ bool jm_wait(unsigned long long* bar, unsigned parity) {
   for (int i = 0; i < JM_POLLS; ++i)
@@ -55,7 +73,8 @@ __device__ __forceinline__ void jm_mma(unsigned tmem, unsigned long long a, unsi
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void jm_tmem_ld16(unsigned addr, float (&v)[16]) {
+// 16 columns of this warp's 32 lanes of tensor memory, added to v
+__device__ __forceinline__ void jm_tmem_add16(unsigned addr, float* v) {
   unsigned r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -65,7 +84,7 @@ __device__ __forceinline__ void jm_tmem_ld16(unsigned addr, float (&v)[16]) {
       : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) v[i] += __uint_as_float(r[i]);
 }
 
 // The largest |w - F_j| the operands are scaled by, a power of two.
@@ -81,26 +100,18 @@ __device__ __forceinline__ float jm_layer_range(const JacMmaParams& p, int layer
   return jm_range(__int_as_float(p.st[layer].wmax), fm);
 }
 
-// Where entry ((mt, mrow), column of centroid l, coordinate b) of the product, or of the diagonal tiles, lies in the
-// partial of unit 0 of its kind, and how far it is to the next split.
-template <int D, int NT>
-struct JmIndex {
-  using Cfg = JmCfg<D, NT>;
-  size_t xy, xy_step, dg, dg_step;
-  int ns_n, ns_d;
-  __device__ JmIndex(const JacMmaParams& p, int layer, int mt, int l, int b) {
-    constexpr size_t TILE = (size_t)JM_M * NT;
-    const int tn = p.tiles_m * p.tiles_n;
-    ns_n = p.ns_n[layer];
-    ns_d = p.ns_d[layer];
-    const size_t first = (size_t)p.unit_first[layer];
-    const int nt = l / Cfg::CPN, col = b * Cfg::CPN + l % Cfg::CPN;
-    xy = (first + (size_t)mt * p.tiles_n + nt) * TILE + (size_t)(col % (NT / 2)) * 256 + (size_t)(col / (NT / 2)) * 128;
-    xy_step = (size_t)tn * TILE;
-    const int dc = b * Cfg::CPM + l % Cfg::CPM;
-    dg = (first + (size_t)tn * ns_n + mt) * TILE + (size_t)(dc % 64) * 256 + (size_t)(dc / 64) * 128;
-    dg_step = (size_t)p.tiles_m * TILE;
+// A layer's work is dealt to its blocks as one line of (tile, stage) pairs; a block's share touches two tiles at most.  The
+// partial of block b and tile t has slot b + t of the layer: consecutive blocks of a tile lie SLOT doubles apart.
+struct JmDeal {
+  long long n_st, total, blocks;
+  __device__ JmDeal(const JacMmaParams& p, int layer, int rows_per_stage) {
+    n_st = (p.row_off[layer + 1] - p.row_off[layer] + rows_per_stage - 1) / rows_per_stage;
+    total = n_st * p.tiles_m * p.tiles_n;
+    blocks = p.unit_first[layer + 1] - p.unit_first[layer];
   }
+  __device__ long long first_of(long long b) const { return total * b / blocks; }
+  __device__ long long block_of(long long pos) const { return ((pos + 1) * blocks - 1) / total; }
+  __device__ size_t slot0(const JacMmaParams& p, int layer) const { return (size_t)p.unit_first[layer] + (size_t)layer * p.tiles_m * p.tiles_n; }
 };
 
 // Stop test of an adjoint step, as in the other forms of the iteration.
@@ -133,58 +144,203 @@ struct JmStop {
   }
 };
 
-// Eight weights of one centroid: the operand's entries for its D coordinates, split and stored.
-// KIND 0: X (rows), 1: Y (columns), 2: n (columns of the diagonal tiles).
-template <int D, int KIND>
-__device__ __forceinline__ void jm_unit(const float* rows, const float (&c)[D], const float (&f)[D], float scale, float mul, unsigned char* hi,
-                                        unsigned char* lo, int coord_bytes) {
-  unsigned ph[D][4], pl[D][4];
+// Two floats in one register pair: the packed fp32 instructions halve the issue slots of the producers, which compute the
+// same quantity for two neighbouring weights.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Splits eight values (four pairs of neighbouring weights) into two fp16 terms and stores them, 16 bytes each.  The first
+// term is the value cut to its 11 leading bits -- a mask, on the integer pipe, which the producers leave idle, instead of a
+// conversion and back -- so the second is exact before its rounding.
+__device__ __forceinline__ void jm_split_store(const f2 (&v)[4], unsigned char* hi, unsigned char* lo) {
+  unsigned ph[4], pl[4];
+  const f2 neg = f2_pack(-1.f, -1.f);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    float v[2][D];
+    float x, y, lx, ly;
+    f2_unpack(v[q], x, y);
+    const float hx = __uint_as_float(__float_as_uint(x) & 0xffffe000u), hy = __uint_as_float(__float_as_uint(y) & 0xffffe000u);
+    f2_unpack(f2_fma(f2_pack(hx, hy), neg, v[q]), lx, ly);
+    const __half2 h2 = __floats2half2_rn(hx, hy), l2 = __floats2half2_rn(lx, ly);
+    ph[q] = *reinterpret_cast<const unsigned*>(&h2);
+    pl[q] = *reinterpret_cast<const unsigned*>(&l2);
+  }
+  *reinterpret_cast<uint4*>(hi) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+  *reinterpret_cast<uint4*>(lo) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
+}
+
+// Eight weights of one centroid.  rows: [D + 2][8] -- the coordinates, the softmax references and the normalisers of the
+// eight weights; nc, nf: minus the centroid, minus its image F.  The eight weights go through every step together, so that
+// the special functions' latency is covered within the warp.
+// g: one over the distance; at: the attention
+// (The coordinates are loaded before anything is stored: the stores of the operands keep later loads behind them.)
+template <int D>
+__device__ __forceinline__ void jm_load(const float* rows, f2 (&w)[D][4]) {
+  const ulonglong2* r2 = reinterpret_cast<const ulonglong2*>(rows);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const float* r = rows + (2 * q + h) * 8;
-      float w[D];
-      if constexpr (D == 4) {
-        const float4 x = *reinterpret_cast<const float4*>(r);
-        w[0] = x.x; w[1] = x.y; w[2] = x.z; w[3] = x.w;
-      } else {
-        const float2 x = *reinterpret_cast<const float2*>(r);
-        w[0] = x.x; w[1] = x.y;
-      }
-      const float2 rs = *reinterpret_cast<const float2*>(r + 4);
-      float df[D], sq = 1e-30f;
+  for (int a = 0; a < D; ++a) {
+    const ulonglong2 x = r2[a * 2], y = r2[a * 2 + 1];
+    w[a][0] = x.x;
+    w[a][1] = x.y;
+    w[a][2] = y.x;
+    w[a][3] = y.y;
+  }
+}
+template <int D>
+__device__ __forceinline__ void jm_attention(const float* rows, const f2 (&w)[D][4], const float (&nc)[D], float scale, f2 (&g)[4], f2 (&at)[4]) {
+  const ulonglong2* r2 = reinterpret_cast<const ulonglong2*>(rows);
+  const ulonglong2 rf0 = r2[D * 2], rf1 = r2[D * 2 + 1], rn0 = r2[D * 2 + 2], rn1 = r2[D * 2 + 3];
+  const f2 rf[4] = {rf0.x, rf0.y, rf1.x, rf1.y}, rn[4] = {rn0.x, rn0.y, rn1.x, rn1.y};
+  f2 sq[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) sq[q] = f2_pack(1e-30f, 1e-30f);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const f2 c = f2_pack(nc[a], nc[a]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const f2 d = f2_add(w[a][q], c);
+      sq[q] = f2_fma(d, d, sq[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float x, y;
+    f2_unpack(sq[q], x, y);
+    g[q] = f2_pack(rsqrt_approx(x), rsqrt_approx(y));
+  }
+  const f2 ms = f2_pack(-scale, -scale);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float x, y;
+    f2_unpack(f2_fma(ms, f2_mul(sq[q], g[q]), rf[q]), x, y);
+    at[q] = f2_mul(f2_pack(ex2_approx(x), ex2_approx(y)), rn[q]);
+  }
+}
+// a coordinate of the eight weights, less what nx is minus of, times g
+__device__ __forceinline__ void jm_entries(const f2 (&w)[4], float nx, const f2 (&g)[4], f2 (&v)[4]) {
+  const f2 c = f2_pack(nx, nx);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = f2_mul(f2_add(w[q], c), g[q]);
+}
+__device__ __forceinline__ void jm_dot(const f2 (&p)[4], const f2 (&n)[4], float& acc) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float px, py, nx, ny;
+    f2_unpack(p[q], px, py);
+    f2_unpack(n[q], nx, ny);
+    acc = fmaf(py, ny, fmaf(px, nx, acc));
+  }
+}
+// X (rows of the tile); with DIAG also the diagonal sums, which are added to dsum in shared memory
+template <int D, bool DIAG>
+__device__ __forceinline__ void jm_unit_x(const float* rows, const float (&nc)[D], const float (&nf)[D], float scale, float xm, float ym,
+                                          double* dsum, int dstep, unsigned char* hi, unsigned char* lo, int coord_bytes) {
+  f2 w[D][4], g[4], at[4];
+  jm_load<D>(rows, w);
+  jm_attention<D>(rows, w, nc, scale, g, at);
+  const f2 m2 = f2_pack(xm, xm), y2 = f2_pack(ym, ym);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) at[q] = f2_mul(at[q], m2);
+  if constexpr (DIAG) {   // (only one tile of a row of tiles does it for a weight)
+    float dg[D * D];
+#pragma unroll
+    for (int e = 0; e < D * D; ++e) dg[e] = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const f2 gq = f2_mul(g[q], y2);
+      float nx[D], ny[D];
+#pragma unroll
+      for (int b = 0; b < D; ++b) f2_unpack(f2_mul(f2_add(w[b][q], f2_pack(nc[b], nc[b])), gq), nx[b], ny[b]);
 #pragma unroll
       for (int a = 0; a < D; ++a) {
-        df[a] = w[a] - c[a];
-        sq = fmaf(df[a], df[a], sq);
+        float px, py;
+        f2_unpack(f2_mul(f2_add(w[a][q], f2_pack(nf[a], nf[a])), at[q]), px, py);
+#pragma unroll
+        for (int b = 0; b < D; ++b) dg[a * D + b] = fmaf(py, ny[b], fmaf(px, nx[b], dg[a * D + b]));
       }
-      const float ri = rsqrt_approx(sq);
-      const float at = ex2_approx(fmaf(-scale, sq * ri, rs.x)) * rs.y;
-      const float g = KIND == 0 ? at * mul : (KIND == 1 ? at * ri * mul : ri * mul);
-#pragma unroll
-      for (int a = 0; a < D; ++a) v[h][a] = (KIND == 0 ? w[a] - f[a] : df[a]) * g;
     }
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-      const __half2 h2 = __floats2half2_rn(v[0][a], v[1][a]);
-      const float2 back = __half22float2(h2);
-      const __half2 l2 = __floats2half2_rn(v[0][a] - back.x, v[1][a] - back.y);
-      ph[a][q] = *reinterpret_cast<const unsigned*>(&h2);
-      pl[a][q] = *reinterpret_cast<const unsigned*>(&l2);
-    }
+    for (int e = 0; e < D * D; ++e) dsum[e * dstep] += (double)dg[e];
   }
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    *reinterpret_cast<uint4*>(hi + a * coord_bytes) = make_uint4(ph[a][0], ph[a][1], ph[a][2], ph[a][3]);
-    *reinterpret_cast<uint4*>(lo + a * coord_bytes) = make_uint4(pl[a][0], pl[a][1], pl[a][2], pl[a][3]);
+    f2 v[4];
+    jm_entries(w[a], nf[a], at, v);
+    jm_split_store(v, hi + a * coord_bytes, lo + a * coord_bytes);
+  }
+}
+// Y (columns of the tile)
+template <int D>
+__device__ __forceinline__ void jm_unit_y(const float* rows, const float (&nc)[D], float scale, float ym, unsigned char* hi, unsigned char* lo,
+                                          int coord_bytes) {
+  f2 w[D][4], g[4], at[4];
+  jm_load<D>(rows, w);
+  jm_attention<D>(rows, w, nc, scale, g, at);
+  const f2 m2 = f2_pack(ym, ym);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) at[q] = f2_mul(f2_mul(at[q], m2), g[q]);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    f2 v[4];
+    jm_entries(w[a], nc[a], at, v);
+    jm_split_store(v, hi + a * coord_bytes, lo + a * coord_bytes);
+  }
+}
+// both, and the diagonal sums, of a tile whose rows and columns are of the same centroids
+template <int D>
+__device__ __forceinline__ void jm_unit_both(const float* rows, const float (&nc)[D], const float (&nf)[D], float scale, float xm, float ym,
+                                             float* dg, unsigned char* xhi, unsigned char* xlo, unsigned char* yhi, unsigned char* ylo,
+                                             int coord_bytes) {
+  f2 w[D][4], g[4], at[4], n[D][4];
+  jm_load<D>(rows, w);
+  jm_attention<D>(rows, w, nc, scale, g, at);
+  const f2 m2 = f2_pack(xm, xm), y2 = f2_pack(ym, ym);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) g[q] = f2_mul(g[q], y2);
+#pragma unroll
+  for (int b = 0; b < D; ++b) {
+    f2 v[4];
+    jm_entries(w[b], nc[b], g, n[b]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = f2_mul(n[b][q], at[q]);
+    jm_split_store(v, yhi + b * coord_bytes, ylo + b * coord_bytes);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) at[q] = f2_mul(at[q], m2);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    f2 v[4];
+    jm_entries(w[a], nf[a], at, v);
+    jm_split_store(v, xhi + a * coord_bytes, xlo + a * coord_bytes);
+#pragma unroll
+    for (int b = 0; b < D; ++b) jm_dot(v, n[b], dg[a * D + b]);
   }
 }
 
-template <int D, int NT>
+template <int D, int NT, bool PACK>
 __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_constant__ JacMmaParams p) {
-  using Cfg = JmCfg<D, NT>;
+  using Cfg = JmCfg<D, NT, PACK>;
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ __align__(8) unsigned long long full[2], done[2], tfree[2];
   __shared__ unsigned s_tmem;
@@ -196,17 +352,14 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
   LayerState* st = p.st + layer;
   if (p.solve_blocks > 0 && (int)blockIdx.x == p.unit_first[layer] && tid < JM_SYNC_WORDS) p.sync[layer * JM_SYNC_WORDS + tid] = 0u;
   if (st->adj_done) return;
-  // ---- this unit's tile and rows ----
-  const int u0 = (int)blockIdx.x - p.unit_first[layer], tn = p.tiles_m * p.tiles_n;
-  const bool diag = u0 >= tn * p.ns_n[layer];
-  const int ud = diag ? u0 - tn * p.ns_n[layer] : u0, per = diag ? p.tiles_m : tn, ns = diag ? p.ns_d[layer] : p.ns_n[layer];
-  const int split = ud / per, tile = ud % per;
-  const int mt = diag ? tile : tile / p.tiles_n, nt = diag ? 0 : tile % p.tiles_n;
+  // ---- this block's share: stages lo .. lo + n - 1 of the layer's line, the first nb of them in tile t0 ----
+  const JmDeal dl(p, layer, Cfg::ROWS);
+  const int bl = (int)blockIdx.x - p.unit_first[layer];
+  const long long lo = dl.first_of(bl);
+  const int n = (int)(dl.first_of(bl + 1) - lo), t0 = (int)(lo / dl.n_st), st0 = (int)(lo - t0 * dl.n_st);
+  const int nb = (int)(dl.n_st - st0 < n ? dl.n_st - st0 : n);
+  double* part = p.part + (dl.slot0(p, layer) + bl + t0) * Cfg::SLOT;   // (the second tile's follows)
   const long long rows = p.row_off[layer + 1] - p.row_off[layer];
-  const long long n_st = (rows + JM_ROWS - 1) / JM_ROWS;
-  const long long st0 = n_st * split / ns, st1 = n_st * (split + 1) / ns;
-  const int n = (int)(st1 - st0);
-  const int ncols = diag ? JM_M : NT;
   const int k = p.k;
   const float range = jm_layer_range(p, layer, D);
 
@@ -232,116 +385,154 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
   const unsigned tmem = *reinterpret_cast<volatile unsigned*>(&s_tmem);
 
   if (warp < 8) {
-    // ================= accumulating warps; the first also issues the products =================
-    // (the registers of the two kinds of warps add up to the 128 x 512 of the launch)
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
+    // ================= accumulating warps: a quarter of the rows, half of the columns each =================
+    if constexpr (NT == 128)
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 112;");
+    else
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 160;");
     float acc[NT / 2];
 #pragma unroll
     for (int i = 0; i < NT / 2; ++i) acc[i] = 0.f;
-    const int half = warp >> 2, quad = warp & 3, cols = ncols / 2;
-    const unsigned base = tmem + ((unsigned)(quad * 32) << 16) + (unsigned)(half * cols);
-    double* mine = p.part + (size_t)blockIdx.x * (JM_M * NT) + half * 128 + quad * 32 + lane;
-    const unsigned idesc = (1u << 4) | ((unsigned)(ncols >> 3) << 17) | ((unsigned)(JM_M >> 4) << 24);   // fp16 in, fp32 out
-    const unsigned sbase = (unsigned)__cvta_generic_to_shared(dyn);
-    bool first = true, ok = true;
-    // products of stage i: all terms of the split, the small ones first; the commit frees the stage's shared memory and
-    // hands its half of tensor memory over
-    auto issue = [&](int i) {
+    const int half = warp >> 2, quad = warp & 3;
+    const unsigned base = tmem + ((unsigned)(quad * 32) << 16) + (unsigned)(half * (NT / 2));
+    // a quarter of what stage i left in tensor memory, added to the registers
+    auto take = [&](int i, int part4) {
       const int s = i & 1;
-      bool good = jm_wait(&full[s], (unsigned)((i >> 1) & 1));
-      if (good && i >= 2) good = jm_wait(&tfree[s], (unsigned)(((i >> 1) - 1) & 1));
-      if (!good) return false;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (lane == 0) {
-        const unsigned a0 = sbase + s * Cfg::STAGE, b0 = a0 + 2 * Cfg::A_BYTES, dst = tmem + (unsigned)(s * NT);
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {   // lo hi, hi lo, then hi hi
-#pragma unroll
-          for (int q = 0; q < JM_ROWS / 16; ++q) {
-            const unsigned long long da = jm_desc(a0 + (t == 0 ? Cfg::A_BYTES : 0) + q * 2 * (JM_M * 16), JM_M * 16);
-            const unsigned long long db = jm_desc(b0 + (t == 1 ? Cfg::B_BYTES : 0) + q * 2 * (NT * 16), NT * 16);
-            jm_mma(dst, da, db, idesc, (t == 0 && q == 0) ? 0u : 1u);
-          }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(&done[s])) : "memory");
+      if (part4 == 0) {
+        if (!jm_wait(&done[s], (unsigned)((i >> 1) & 1))) return false;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < NT / 8; q += 16)
+        jm_tmem_add16(base + (unsigned)(s * NT + part4 * (NT / 8) + q), acc + part4 * (NT / 8) + q);
+      if (part4 == 3) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) jm_arrive(&tfree[s]);
+      }
       return true;
     };
-    int issued = 0;
-    if (warp == 0 && n > 0) {
-      ok = issue(0);
-      issued = ok ? 1 : 0;
-    }
-    for (int i = 0; i < n && ok; ++i) {
-      const int s = i & 1;
-      if (warp == 0 && i + 1 < n) {   // the next stage's products before this one's sums are fetched
-        ok = issue(i + 1);
-        if (!ok) break;
-        issued = i + 2;
-      }
-      ok = jm_wait(&done[s], (unsigned)((i >> 1) & 1));
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (ok) {
+    // after stage i: the sums move on at the end of a run of stages
+    auto fold = [&](int i) {
+      const int at = i < nb ? i : i - nb, last = i < nb ? nb : n - nb;   // place within the tile's share, its length
+      if ((at + 1) % JM_FOLD == 0 || at + 1 == last) {
+        double* o = part + (i < nb ? 0 : Cfg::SLOT);
+        const bool first = at < JM_FOLD;
+        if constexpr (PACK) {   // the two sets' blocks of lanes: this lane's, and the one 16 lanes and 16 columns further
 #pragma unroll
-        for (int q = 0; q < NT / 32; ++q) {
-          if (q * 16 < cols) {
-            float v[16];
-            jm_tmem_ld16(base + (unsigned)(s * NT + q * 16), v);
+          for (int b = 0; b < 2; ++b)
 #pragma unroll
-            for (int e = 0; e < 16; ++e) acc[q * 16 + e] += v[e];
-          }
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) jm_arrive(&tfree[s]);
-      if ((i + 1) % JM_FOLD == 0 || i + 1 == n) {
+            for (int l = 0; l < 16; ++l) {
+              const double v = (double)acc[b * 32 + l] + (double)__shfl_xor_sync(0xffffffffu, acc[b * 32 + 16 + l], 16);
+              double* e = o + ((half * 2 + b) * 16 + l) * 64 + quad * 16 + lane;
+              if (lane < 16) *e = first ? v : *e + v;
+            }
 #pragma unroll
-        for (int q = 0; q < NT / 2; ++q)
-          if (q < cols) {
-            double* o = mine + (size_t)q * 256;
-            *o = first ? (double)acc[q] : *o + (double)acc[q];
+          for (int q = 0; q < NT / 2; ++q) acc[q] = 0.f;
+        } else {
+#pragma unroll
+          for (int q = 0; q < NT / 2; ++q) {
+            double* e = o + (size_t)q * 256 + half * 128 + quad * 32 + lane;
+            *e = first ? (double)acc[q] : *e + (double)acc[q];
             acc[q] = 0.f;
           }
-        first = false;
+        }
+      }};
+    bool ok = true;
+    if (warp != 0) {
+      for (int i = 0; i < n && ok; ++i) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ok = ok && take(i, c);
+        if (ok) fold(i);
       }
-    }
-    if (!ok) {
-      if (lane == 0) s_fail = 1;
+    } else {
+      // This warp also issues the products -- lo hi, hi lo, then hi hi --, three at a time: the tensor core's queue is
+      // short, and what the warp has to take of the stage before fits in between.
+      const unsigned idesc = (1u << 4) | ((unsigned)(NT >> 3) << 17) | ((unsigned)(JM_M >> 4) << 24);   // fp16 in, fp32 out
+      const unsigned sbase = (unsigned)__cvta_generic_to_shared(dyn);
+      int issued = 0;
+      for (int i = 0; i < n && ok; ++i) {
+        const int s = i & 1;
+        ok = jm_wait(&full[s], (unsigned)((i >> 1) & 1));
+        if (ok && i >= 2) ok = jm_wait(&tfree[s], (unsigned)(((i >> 1) - 1) & 1));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const unsigned a0 = sbase + s * Cfg::STAGE, b0 = a0 + 2 * Cfg::A_BYTES, dst = tmem + (unsigned)(s * NT);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          if (lane == 0) {
+#pragma unroll
+            for (int x = c * 3; x < c * 3 + 3; ++x) {
+              const int t = x / (JM_ROWS / 16), q = x % (JM_ROWS / 16);
+              const unsigned long long da = jm_desc(a0 + (t == 0 ? Cfg::A_BYTES : 0) + q * 2 * (JM_M * 16), JM_M * 16);
+              const unsigned long long db = jm_desc(b0 + (t == 1 ? Cfg::B_BYTES : 0) + q * 2 * (NT * 16), NT * 16);
+              jm_mma(dst, da, db, idesc, x == 0 ? 0u : 1u);
+            }
+            if (c == 3)
+              asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(&done[s])) : "memory");
+          }
+          __syncwarp();
+          issued = i + 1;
+          if (i > 0) ok = ok && take(i - 1, c);
+        }
+        if (ok && i > 0) fold(i - 1);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) ok = ok && take(n - 1, c);
+      if (ok) fold(n - 1);
       // (what is in flight ends before tensor memory is given back)
-      if (warp == 0 && issued > 0) (void)jm_wait(&done[(issued - 1) & 1], (unsigned)(((issued - 1) >> 1) & 1));
+      if (!ok && issued > 0) (void)jm_wait(&done[(issued - 1) & 1], (unsigned)(((issued - 1) >> 1) & 1));
     }
-    if (n == 0) {
-      for (int q = 0; q < cols; ++q) mine[(size_t)q * 256] = 0.0;
-    }
+    if (!ok && lane == 0) s_fail = 1;
   } else {
-    // ================= producing warps: weights 8 pw .. 8 pw + 7 of every stage =================
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
-    const int pw = warp - 8;
-    float cx[Cfg::MU][D], fx[Cfg::MU][D], cy[Cfg::NU][D];
+    // ================= producing warps: eight weights of every stage (twice eight: PACK) =================
+    if constexpr (NT == 128)
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
+    else
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
+    const int pw = warp - 8, cl = PACK ? lane & 15 : lane, set = PACK ? lane >> 4 : 0;
+    float cx[Cfg::MU][D], fx[Cfg::MU][D], cy[Cfg::BOTH ? 1 : Cfg::NU][D], dg[Cfg::BOTH ? Cfg::MU : 1][D * D];
+    double* dsum = reinterpret_cast<double*>(dyn + Cfg::OFF_DG);   // [8 warps][D * D][MU][32]
+    double* dmine = dsum + pw * (D * D * Cfg::MU * 32);
+    int mt = 0, nt = 0;
+    auto load_tile = [&](int t) {
+      mt = t / p.tiles_n;
+      nt = t % p.tiles_n;
 #pragma unroll
-    for (int h = 0; h < Cfg::MU; ++h) {
-      const int j = mt * Cfg::CPM + h * 32 + lane;
+      for (int h = 0; h < Cfg::MU; ++h) {
+        const int j = mt * Cfg::CPM + h * Cfg::LC + cl;
 #pragma unroll
-      for (int a = 0; a < D; ++a) {
-        cx[h][a] = j < k ? p.C[((size_t)layer * k + j) * D + a] : PAD_COORD;
-        fx[h][a] = j < k ? p.F[((size_t)layer * k + j) * D + a] : 0.f;
+        for (int a = 0; a < D; ++a) {
+          cx[h][a] = -(j < k ? p.C[((size_t)layer * k + j) * D + a] : PAD_COORD);
+          fx[h][a] = -(j < k ? p.F[((size_t)layer * k + j) * D + a] : 0.f);
+        }
+        if constexpr (Cfg::BOTH) {
+#pragma unroll
+          for (int e = 0; e < D * D; ++e) dg[h][e] = 0.f;
+        } else {
+#pragma unroll
+          for (int e = 0; e < D * D; ++e) dmine[(e * Cfg::MU + h) * 32 + lane] = 0.0;
+        }
       }
-    }
+      if constexpr (!Cfg::BOTH) {
 #pragma unroll
-    for (int h = 0; h < Cfg::NU; ++h) {
-      const int j = (diag ? mt * Cfg::CPM : nt * Cfg::CPN) + h * 32 + lane;
+        for (int h = 0; h < Cfg::NU; ++h) {
+          const int j = nt * Cfg::CPN + h * 32 + lane;
 #pragma unroll
-      for (int a = 0; a < D; ++a) cy[h][a] = j < k ? p.C[((size_t)layer * k + j) * D + a] : PAD_COORD;
-    }
-    float* rowsm = reinterpret_cast<float*>(dyn + 2 * Cfg::STAGE) + pw * 64;   // [8][8]: w, reference, normaliser
+          for (int a = 0; a < D; ++a) cy[h][a] = -(j < k ? p.C[((size_t)layer * k + j) * D + a] : PAD_COORD);
+        }
+      }
+    };
+    load_tile(t0);
+    float* rowsm = reinterpret_cast<float*>(dyn + Cfg::OFF_ROW) + pw * Cfg::SETS * Cfg::SET_FLOATS;   // [D + 2][8] per set
+    const float* myrows = rowsm + set * Cfg::SET_FLOATS;
     const long long row0 = p.row_off[layer];
     float4 wn = make_float4(0.f, 0.f, 0.f, 0.f);
     float2 rn = make_float2(0.f, 0.f);
     auto fetch = [&](int i) {
-      const long long loc = (st0 + i) * JM_ROWS + pw * 8 + lane;
-      if (lane < 8 && i < n) {
+      const int stage = i < nb ? st0 + i : i - nb;
+      const long long loc = (long long)stage * Cfg::ROWS + pw * (8 * Cfg::SETS) + lane;
+      if (lane < 8 * Cfg::SETS && i < n) {
         const bool ok = loc < rows;
         const long long g = row0 + (ok ? loc : 0);
         if constexpr (D == 4) {
@@ -357,35 +548,75 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
     fetch(0);
     const float xm = 16384.f / range, ym = 16384.f;
     bool ok = true;
-    for (int i = 0; i < n && ok; ++i) {
+    for (int i = 0; i < n; ++i) {
       const int s = i & 1;
+      if (i == nb) load_tile(t0 + 1);
       if (i >= 2) ok = jm_wait(&done[s], (unsigned)(((i >> 1) - 1) & 1));
+      if (!ok) break;
       __syncwarp();
-      if (lane < 8) {
-        *reinterpret_cast<float4*>(rowsm + lane * 8) = wn;
-        *reinterpret_cast<float2*>(rowsm + lane * 8 + 4) = rn;
+      if (lane < 8 * Cfg::SETS) {
+        float* o = rowsm + (lane >> 3) * Cfg::SET_FLOATS + (lane & 7);
+        o[0] = wn.x;
+        o[8] = wn.y;
+        if constexpr (D == 4) {
+          o[16] = wn.z;
+          o[24] = wn.w;
+        }
+        o[D * 8] = rn.x;
+        o[D * 8 + 8] = rn.y;
       }
       __syncwarp();
       fetch(i + 1);
       unsigned char* A = dyn + s * Cfg::STAGE + pw * (JM_M * 16) + lane * 16;
       unsigned char* B = dyn + s * Cfg::STAGE + 2 * Cfg::A_BYTES + pw * (NT * 16) + lane * 16;
-      if (ok) {
+      const int at = i < nb ? i : i - nb, last = i < nb ? nb : n - nb;
+      if constexpr (Cfg::BOTH) {
 #pragma unroll
         for (int h = 0; h < Cfg::MU; ++h)
-          jm_unit<D, 0>(rowsm, cx[h], fx[h], p.scale, xm, A + h * 512, A + Cfg::A_BYTES + h * 512, Cfg::CPM * 16);
-        if (!diag) {
+          jm_unit_both<D>(myrows, cx[h], fx[h], p.scale, xm, ym, dg[h], A + h * 512, A + Cfg::A_BYTES + h * 512, B + h * 512,
+                          B + Cfg::B_BYTES + h * 512, JM_M / D * 16);
+      } else {
+        // of the tiles that share these rows of X, one adds this stage to the diagonal sums
+        const bool diag = (i < nb ? st0 + i : i - nb) % p.tiles_n == nt;
 #pragma unroll
-          for (int h = 0; h < Cfg::NU; ++h)
-            jm_unit<D, 1>(rowsm, cy[h], cy[h], p.scale, ym, B + h * 512, B + Cfg::B_BYTES + h * 512, Cfg::CPN * 16);
-        } else {
-#pragma unroll
-          for (int h = 0; h < Cfg::MU; ++h)
-            jm_unit<D, 2>(rowsm, cy[h], cy[h], p.scale, ym, B + h * 512, B + Cfg::B_BYTES + h * 512, Cfg::CPM * 16);
+        for (int h = 0; h < Cfg::MU; ++h) {
+          unsigned char* o = A + h * 512;
+          if (diag)
+            jm_unit_x<D, true>(myrows, cx[h], fx[h], p.scale, xm, ym, dmine + h * 32 + lane, Cfg::MU * 32, o, o + Cfg::A_BYTES, JM_M / D * 16);
+          else
+            jm_unit_x<D, false>(myrows, cx[h], fx[h], p.scale, xm, ym, dmine + h * 32 + lane, Cfg::MU * 32, o, o + Cfg::A_BYTES, JM_M / D * 16);
         }
+#pragma unroll
+        for (int h = 0; h < Cfg::NU; ++h)
+          jm_unit_y<D>(myrows, cy[h], p.scale, ym, B + h * 512, B + Cfg::B_BYTES + h * 512, NT / D * 16);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) jm_arrive(&full[s]);
+      if (Cfg::BOTH && ((at + 1) % JM_DFOLD == 0 || at + 1 == last)) {
+#pragma unroll
+        for (int h = 0; h < (Cfg::BOTH ? Cfg::MU : 0); ++h)
+#pragma unroll
+          for (int e = 0; e < D * D; ++e) {
+            double* o = dmine + (e * Cfg::MU + h) * 32 + lane;
+            double v = (double)dg[h][e];
+            if constexpr (PACK) v += (double)__shfl_xor_sync(0xffffffffu, dg[h][e], 16);
+            *o = at < JM_DFOLD ? v : *o + v;
+            dg[h][e] = 0.f;
+          }
+      }
+      if (at + 1 == last) {   // (every producing warp comes here for the same stage)
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        double* o = part + (i < nb ? 0 : Cfg::SLOT) + Cfg::XY;
+        for (int x = tid - 256; x < D * D * Cfg::CPM; x += 256) {
+          const int e = x / Cfg::CPM, c = x % Cfg::CPM;
+          double v = 0.0;
+#pragma unroll
+          for (int w = 0; w < 8; ++w) v += dsum[w * (D * D * Cfg::MU * 32) + (e * Cfg::MU + c / Cfg::LC) * 32 + c % Cfg::LC];
+          o[x] = v;
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+      }
     }
     if (!ok && lane == 0) s_fail = 1;
   }
@@ -396,82 +627,108 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * NT));
   const bool failed = *reinterpret_cast<volatile int*>(&s_fail) != 0;
   if (failed && tid == 0) st->status = ST_TIMEOUT;
-  if (p.solve_blocks > 0) return;
-
-  // ================= k d <= 64: the layer's last unit adds the partials and runs the iteration =================
-  const int units = p.unit_first[layer + 1] - p.unit_first[layer];
-  if (tid == 0) s_flag = atomicAdd(&st->ticket, 1u) == (unsigned)(units - 1);
-  __syncthreads();
-  if (!s_flag) return;
-  __threadfence();
-  const int nd = k * D;
-  double* J = reinterpret_cast<double*>(dyn);   // [64][65]: J_C^T
-  double* ub = J + 64 * 65;                     // [2][64]
-  double* gs = ub + 128;                        // [64]
-  double* red = gs + 64;                        // [2][8][2]
-  for (int o = tid; o < 64 * 64; o += JM_THREADS) {
-    const int q = o & 63, r = o >> 6;           // output coordinate (l, b), input coordinate (j, a)
-    double s = 0.0;
-    if (q < nd && r < nd) {
-      const int l = q / D, b = q % D, j = r / D, a = r % D;
-      const JmIndex<D, NT> ix(p, layer, 0, l, b);
-      const int mrow = a * Cfg::CPM + j;
-#pragma unroll 16
-      for (int t = 0; t < ix.ns_n; ++t) s -= __ldcg(p.part + ix.xy + t * ix.xy_step + mrow);
+  if constexpr (PACK) {
+    // ================= k d <= 64: the blocks' partials are added in two stages, and the last block runs the iteration ======
+    const int units = p.unit_first[layer + 1] - p.unit_first[layer], ng = (units + JM_RED - 1) / JM_RED, grp = bl / JM_RED;
+    const int in_group = grp + 1 < ng ? JM_RED : units - grp * JM_RED;
+    if (tid == 0) s_flag = atomicAdd(&p.gtickets[p.group_first[layer] + grp], 1u) == (unsigned)(in_group - 1);
+    __syncthreads();
+    if (!s_flag) return;
+    __threadfence();
+    double* sum = p.part + (dl.slot0(p, layer) + (size_t)grp * JM_RED) * Cfg::SLOT;
+    for (int o = tid; o < Cfg::SLOT; o += JM_THREADS) {
+      double s = 0.0;
+#pragma unroll
+      for (int t = 0; t < JM_RED; ++t)
+        if (t < in_group) s += __ldcg(sum + (size_t)t * Cfg::SLOT + o);
+      __stcg(sum + o, s);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      p.gtickets[p.group_first[layer] + grp] = 0u;
+      s_flag = atomicAdd(&st->ticket, 1u) == (unsigned)(ng - 1);
+    }
+    __syncthreads();
+    if (!s_flag) return;
+    __threadfence();
+    const int nd = k * D;
+    double* J = reinterpret_cast<double*>(dyn);   // [64][65]: J_C^T
+    double* ub = J + 64 * 65;                     // [2][4][18]: a quarter per thread of an output, in banks of its own
+    double* red = ub + 2 * 72;                    // [2][8][2]
+    const double* all = p.part + dl.slot0(p, layer) * Cfg::SLOT;
+    for (int o = tid; o < 64 * 64; o += JM_THREADS) {
+      const int r = o & 63, q = o >> 6;           // places of the input coordinate (j, a) and the output coordinate (l, b)
+      const int j = r % Cfg::CPM, a = r / Cfg::CPM, l = q % Cfg::CPM, b = q / Cfg::CPM;
+      double s = 0.0;
+#pragma unroll
+      for (int t = 0; t < JM_RED + 1; ++t)
+        if (t < ng) s -= __ldcg(all + (size_t)t * JM_RED * Cfg::SLOT + o);
       if (j == l)
-#pragma unroll 16
-        for (int t = 0; t < ix.ns_d; ++t) s += __ldcg(p.part + ix.dg + t * ix.dg_step + mrow);
-      const float S = p.S[(size_t)layer * k + j];
+        for (int t = 0; t < ng; ++t) s += __ldcg(all + (size_t)t * JM_RED * Cfg::SLOT + Cfg::XY + (a * D + b) * Cfg::CPM + j);
+      const float S = j < k ? p.S[(size_t)layer * k + j] : 0.f;
       s *= (S >= S_MIN_F) ? p.inv_tau_d / (double)S * ((double)range / 268435456.0) : 0.0;
+      J[q * 65 + r] = l < k ? s : 0.0;
     }
-    J[q * 65 + r] = s;
-  }
-  if (tid < 64) {
-    gs[tid] = tid < nd ? (double)p.gvec[(size_t)layer * nd + tid] : 0.0;
-    ub[tid] = gs[tid];
-    ub[64 + tid] = 0.0;
-  }
-  __syncthreads();
-  if (warp >= 8) return;
-  const int q = tid >> 2, pr = tid & 3;         // four threads per output
-  const double al = (double)p.alpha, be = 1.0 - al;
-  JmStop stop;
-  stop.status = st->status;
-  double g2 = 0.0;
-  for (int r = 0; r < nd; ++r) g2 += gs[r] * gs[r];
-  const double u2_limit = ADJ_GROWTH_LIMIT * ADJ_GROWTH_LIMIT * g2;
-  if (failed || stop.status == ST_TIMEOUT) stop.done = 1;
-  while (stop.it < p.max_iter && !stop.done) {
-    const double* u = ub + (stop.it & 1) * 64;
-    double s = 0.0;
+    if (tid < 64) {
+      const int l = tid % Cfg::CPM, b = tid / Cfg::CPM;
+      ub[(tid >> 4) * 18 + (tid & 15)] = l < k ? (double)p.gvec[(size_t)layer * nd + l * D + b] : 0.0;
+    }
+    __syncthreads();
+    if (warp >= 8) return;
+    const int q = tid >> 2, pr = tid & 3;         // four threads per output, each with its part of the row in registers
+    const double al = (double)p.alpha, be = 1.0 - al;
+    JmStop stop;
+    stop.status = st->status;
+    const int place = (q >> 4) * 18 + (q & 15);
+    const double gq = ub[place];
+    double row[16], uo = gq, g2 = 0.0;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) s = fma(J[q * 65 + pr * 16 + r], u[pr * 16 + r], s);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    const double uo = u[q], un = q < nd ? al * (s + gs[q]) + be * uo : 0.0;
-    if (pr == 0) ub[((stop.it + 1) & 1) * 64 + q] = un;
-    double num = pr == 0 ? (un - uo) * (un - uo) : 0.0, den = pr == 0 ? un * un : 0.0;
+    for (int r = 0; r < 16; ++r) {
+      row[r] = J[q * 65 + pr * 16 + r];
+      const double x = ub[pr * 18 + r];
+      g2 = fma(x, x, g2);
+    }
+    g2 += __shfl_xor_sync(0xffffffffu, g2, 1);
+    g2 += __shfl_xor_sync(0xffffffffu, g2, 2);
+    const double u2_limit = ADJ_GROWTH_LIMIT * ADJ_GROWTH_LIMIT * g2;
+    if (failed || stop.status == ST_TIMEOUT) stop.done = 1;
+    while (stop.it < p.max_iter && !stop.done) {
+      const double* u = ub + (stop.it & 1) * 72 + pr * 18;
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
 #pragma unroll
-    for (int o = 16; o >= 4; o >>= 1) {
-      num += __shfl_xor_sync(0xffffffffu, num, o);
-      den += __shfl_xor_sync(0xffffffffu, den, o);
-    }
-    double* rd = red + (stop.it & 1) * 16;
-    if (lane == 0) {
-      rd[warp * 2] = num;
-      rd[warp * 2 + 1] = den;
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    num = den = 0.0;
+      for (int r = 0; r < 16; r += 4) {
+        s0 = fma(row[r], u[r], s0);
+        s1 = fma(row[r + 1], u[r + 1], s1);
+        s2 = fma(row[r + 2], u[r + 2], s2);
+        s3 = fma(row[r + 3], u[r + 3], s3);
+      }
+      double s = (s0 + s1) + (s2 + s3);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      const double un = al * (s + gq) + be * uo;
+      if (pr == 0) ub[((stop.it + 1) & 1) * 72 + place] = un;
+      double num = (un - uo) * (un - uo), den = un * un;
+      uo = un;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      num += rd[w * 2];
-      den += rd[w * 2 + 1];
+      for (int o = 16; o >= 4; o >>= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+      }
+      double* rd = red + (stop.it & 1) * 16;
+      if (lane == 0) {
+        rd[warp * 2] = num;
+        rd[warp * 2 + 1] = den;
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      num = ((rd[0] + rd[2]) + (rd[4] + rd[6])) + ((rd[8] + rd[10]) + (rd[12] + rd[14]));
+      den = ((rd[1] + rd[3]) + (rd[5] + rd[7])) + ((rd[9] + rd[11]) + (rd[13] + rd[15]));
+      stop.test(p, layer, num, den, u2_limit, tid == 0);
     }
-    stop.test(p, layer, num, den, u2_limit, tid == 0);
+    const int l = q % Cfg::CPM, b = q / Cfg::CPM;
+    if (pr == 0 && l < k) p.u[(size_t)layer * nd + l * D + b] = (float)uo;
+    if (tid == 0) stop.store(st);
   }
-  if (pr == 0 && q < nd) p.u[(size_t)layer * nd + q] = (float)ub[(stop.it & 1) * 64 + q];
-  if (tid == 0) stop.store(st);
 }
 
 // ---- larger codebooks: the iteration by many blocks, eight rows of J_C^T each, kept in shared memory ----
@@ -479,7 +736,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
 constexpr int JS_T = 256, JS_ROWS = 8;
 template <int D, int NT>
 __global__ void __launch_bounds__(JS_T) idkm_jac_solve(const __grid_constant__ JacMmaParams p) {
-  using Cfg = JmCfg<D, NT>;
+  using Cfg = JmCfg<D, NT, false>;
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ double red[JS_ROWS][2], tot[2];
   __shared__ int s_ok;
@@ -496,20 +753,37 @@ __global__ void __launch_bounds__(JS_T) idkm_jac_solve(const __grid_constant__ J
   const int q = b * JS_ROWS + warp, l = q / D, c = q % D;
   const bool own = q < nd;
   const int place = (l / Cfg::CPM) * JM_M + c * Cfg::CPM + l % Cfg::CPM;
+  const JmDeal dl(p, layer, Cfg::ROWS);
+  const size_t slot0 = dl.slot0(p, layer);
+  const int nt = l / Cfg::CPN, col = c * Cfg::CPN + l % Cfg::CPN;
+  const size_t entry = (size_t)(col % (NT / 2)) * 256 + (size_t)(col / (NT / 2)) * 128;
   for (int mt = 0; mt < p.tiles_m; ++mt) {
     double s[4] = {0.0, 0.0, 0.0, 0.0};
     if (own) {
-      const JmIndex<D, NT> ix(p, layer, mt, l, c);
-#pragma unroll 4
-      for (int t = 0; t < ix.ns_n; ++t)
+      const int t = mt * p.tiles_n + nt;
+      const int b0 = (int)dl.block_of(t * dl.n_st), nb = (int)dl.block_of((t + 1) * dl.n_st - 1) - b0 + 1;
+      const double* src = p.part + (slot0 + b0 + t) * Cfg::SLOT + entry + lane;
+#pragma unroll 8
+      for (int x = 0; x < nb; ++x)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) s[r] -= __ldcg(p.part + ix.xy + t * ix.xy_step + lane + 32 * r);
-      if (l / Cfg::CPM == mt)
-        for (int t = 0; t < ix.ns_d; ++t)
+        for (int r = 0; r < 4; ++r) s[r] -= __ldcg(src + (size_t)x * Cfg::SLOT + 32 * r);
+    }
+    if (own && l / Cfg::CPM == mt)
+      for (int t = mt * p.tiles_n; t < (mt + 1) * p.tiles_n; ++t) {
+        const int b0 = (int)dl.block_of(t * dl.n_st), nb = (int)dl.block_of((t + 1) * dl.n_st - 1) - b0 + 1;
+        const double* src = p.part + (slot0 + b0 + t) * Cfg::SLOT + Cfg::XY + c * Cfg::CPM + l % Cfg::CPM;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          double v = 0.0;
+          for (int x = lane; x < nb; x += 32) v += __ldcg(src + (size_t)x * Cfg::SLOT + a * D * Cfg::CPM);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          const int mrow = a * Cfg::CPM + l % Cfg::CPM;
 #pragma unroll
           for (int r = 0; r < 4; ++r)
-            if ((lane + 32 * r) % Cfg::CPM == l % Cfg::CPM) s[r] += __ldcg(p.part + ix.dg + t * ix.dg_step + lane + 32 * r);
-    }
+            if (lane + 32 * r == mrow) s[r] += v;
+        }
+      }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int mrow = lane + 32 * r, j = mt * Cfg::CPM + mrow % Cfg::CPM;
@@ -629,46 +903,55 @@ bool jac_mma_plan(int d, int k, JacMmaPlan* out) {
   return true;
 }
 
-int jac_mma_units_max(const JacMmaPlan& pl, int n_layers) { return JM_UNITS + n_layers * (pl.tiles_m * pl.tiles_n + pl.tiles_m); }
+static int plan_rows(int d, int k) { return k * d <= 64 ? 2 * JM_ROWS : JM_ROWS; }
+int jac_mma_units_max(const JacMmaPlan& pl, int n_layers) { return JM_UNITS + n_layers * pl.tiles_m * pl.tiles_n; }
+size_t jac_mma_part_bytes(const JacMmaPlan& pl, int d, int k, int n_layers) {
+  const size_t tiles = (size_t)pl.tiles_m * pl.tiles_n;
+  const size_t slot = k * d <= 64 ? 64 * 64 + (size_t)d * 64 : (size_t)JM_M * pl.nt + (size_t)d * JM_M;
+  return ((size_t)jac_mma_units_max(pl, n_layers) + n_layers * tiles) * slot * sizeof(double);
+}
 
-int jac_mma_split(const JacMmaPlan& pl, JacMmaParams* p) {
-  const int L = p->n_layers, tn = pl.tiles_m * pl.tiles_n, td = pl.tiles_m;
-  const double cd = pl.nt == 256 ? 0.6 : 1.0;   // a diagonal tile's cost against a product tile's
+// A layer gets its share of the blocks, at least one per tile (a block's share of the work then touches two tiles at most)
+// and no more than it has stages.
+int jac_mma_split(const JacMmaPlan& pl, int d, JacMmaParams* p) {
+  const int L = p->n_layers, tiles = pl.tiles_m * pl.tiles_n, per = plan_rows(d, p->k);
   const long long m = p->row_off[L];
-  int units = 0;
+  int units = 0, groups = 0;
   for (int l = 0; l < L; ++l) {
-    const long long rows = p->row_off[l + 1] - p->row_off[l], n_st = (rows + JM_ROWS - 1) / JM_ROWS;
-    const double budget = (double)JM_UNITS * (double)rows / (double)m;   // blocks this layer may use
-    long long nn = (long long)(budget / ((double)tn + cd * td));
-    if (nn < 1) nn = 1;
-    long long nd = ((long long)budget - nn * tn) / td;
-    if (nd < 1) nd = 1;
-    if (nn > n_st) nn = n_st;
-    if (nd > n_st) nd = n_st;
+    const long long rows = p->row_off[l + 1] - p->row_off[l], work = (rows + per - 1) / per * tiles;
+    long long n = (long long)JM_UNITS * rows / m;
+    if (n < tiles) n = tiles;
+    if (n > work) n = work;
     p->unit_first[l] = units;
-    p->ns_n[l] = (int)nn;
-    p->ns_d[l] = (int)nd;
-    units += (int)(nn * tn + nd * td);
+    p->group_first[l] = groups;
+    units += (int)n;
+    groups += (int)((n + JM_RED - 1) / JM_RED);
   }
   for (int l = L; l <= MAX_LAYERS; ++l) p->unit_first[l] = units;
   return units;
 }
+int jac_mma_groups_max(int n_layers) { return (JM_UNITS + n_layers) / JM_RED + n_layers; }   // k d <= 64
 
-template <int D, int NT>
+template <int D, int NT, bool PACK>
 static cudaError_t launch_mma(const JacMmaParams& p, int units, cudaStream_t stream) {
-  constexpr int DYN = JmCfg<D, NT>::DYN;
+  constexpr int DYN = JmCfg<D, NT, PACK>::DYN;
   static bool configured = false;
   if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_jac_mma<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN);
+    cudaFuncAttributes at;
+    cudaError_t rc = cudaFuncGetAttributes(&at, idkm_jac_mma<D, NT, PACK>);
+    if (rc != cudaSuccess) return rc;
+    if (at.numRegs != JM_LAUNCH_REGS) return cudaErrorInvalidConfiguration;   // (the warps' shares would not add up)
+    rc = cudaFuncSetAttribute(idkm_jac_mma<D, NT, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN);
     if (rc != cudaSuccess) return rc;
     configured = true;
   }
-  idkm_jac_mma<D, NT><<<units, JM_THREADS, DYN, stream>>>(p);
+  idkm_jac_mma<D, NT, PACK><<<units, JM_THREADS, DYN, stream>>>(p);
   return cudaGetLastError();
 }
 cudaError_t launch_jac_mma(int d, const JacMmaPlan& pl, const JacMmaParams& p, int units, cudaStream_t stream) {
-  if (d == 4) return pl.nt == 128 ? launch_mma<4, 128>(p, units, stream) : launch_mma<4, 256>(p, units, stream);
-  return pl.nt == 128 ? launch_mma<2, 128>(p, units, stream) : launch_mma<2, 256>(p, units, stream);
+  if (p.k * d <= 64) return d == 4 ? launch_mma<4, 128, true>(p, units, stream) : launch_mma<2, 128, true>(p, units, stream);
+  if (d == 4) return pl.nt == 128 ? launch_mma<4, 128, false>(p, units, stream) : launch_mma<4, 256, false>(p, units, stream);
+  return pl.nt == 128 ? launch_mma<2, 128, false>(p, units, stream) : launch_mma<2, 256, false>(p, units, stream);
 }
 template <int D, int NT>
 static cudaError_t launch_solve(const JacMmaPlan& pl, const JacMmaParams& p, cudaStream_t stream) {

@@ -16,7 +16,7 @@ constexpr int JM_M = 128;              // rows (j, a) of a tile
 constexpr int JM_FOLD = 256;           // stages after which the fp32 sums move into the fp64 partial
 constexpr int JM_UNITS = 148;          // blocks the splits of one call are dealt to
 constexpr int JM_SYNC_WORDS = 32;
-constexpr size_t JM_PART_MAX = 64u << 20;   // workspace for partial tiles
+constexpr size_t JM_PART_MAX = 96u << 20;   // workspace for partial tiles
 
 struct JacMmaParams {
   const float* W;
@@ -25,7 +25,8 @@ struct JacMmaParams {
   const float2* rowstat;
   LayerState* st;
   float* hist_adj;
-  double* part;            // [units][NT / 2][256]: one partial tile per unit
+  double* part;            // one partial tile per slot (idkm_jac_mma.cu)
+  unsigned int* gtickets;  // arrivals of the groups of blocks that add up their partials; zero at rest
   double* ub;              // [2][L][kdp] the adjoint, by permuted coordinate, alternating by step
   double* pn;              // [2][L][blocks per layer][2] squares of the step and of the adjoint
   unsigned int* sync;      // [L][JM_SYNC_WORDS] barrier words of the solve
@@ -39,7 +40,7 @@ struct JacMmaParams {
   long long spin_limit;
   long long row_off[MAX_LAYERS + 1];
   int unit_first[MAX_LAYERS + 1];
-  int ns_n[MAX_LAYERS], ns_d[MAX_LAYERS];   // row splits of the product's and of the diagonal tiles
+  int group_first[MAX_LAYERS];
 };
 
 struct JacMmaPlan {
@@ -49,7 +50,9 @@ struct JacMmaPlan {
 // false: this codebook has no such pass
 bool jac_mma_plan(int d, int k, JacMmaPlan* out);
 int jac_mma_units_max(const JacMmaPlan& pl, int n_layers);
-int jac_mma_split(const JacMmaPlan& pl, JacMmaParams* p);   // fills the unit table, returns the number of units
+int jac_mma_groups_max(int n_layers);
+size_t jac_mma_part_bytes(const JacMmaPlan& pl, int d, int k, int n_layers);
+int jac_mma_split(const JacMmaPlan& pl, int d, JacMmaParams* p);   // fills the unit table, returns the number of units
 cudaError_t launch_jac_mma(int d, const JacMmaPlan& pl, const JacMmaParams& p, int units, cudaStream_t stream);
 cudaError_t launch_jac_solve(int d, const JacMmaPlan& pl, const JacMmaParams& p, cudaStream_t stream);
 
