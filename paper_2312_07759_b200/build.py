@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ_DIR = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libidkm.so")
 
-HEADERS = ["idkm_kernels.cuh", "idkm_inst.cuh", "idkm_jacobian_tile.cuh", "idkm_scalar.cuh", "idkm_jac_mma.cuh", os.path.join(ROOT, "include", "idkm.h")]
+HEADERS = ["idkm_kernels.cuh", "idkm_inst.cuh", "idkm_jacobian_tile.cuh", "idkm_scalar.cuh", "idkm_jac_mma.cuh", "idkm_mma_loop.cuh", "idkm_mma_loop_impl.cuh", os.path.join(ROOT, "include", "idkm.h")]
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
               "-diag-suppress", "177"]
@@ -61,7 +61,7 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(res.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=min(8, len(_sources()))) as ex:
+    with ThreadPoolExecutor(max_workers=min(12, len(_sources()))) as ex:
         objs = list(ex.map(compile_one, _sources()))
     tmp = LIB + f".tmp{os.getpid()}"
     res = subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp, *objs],

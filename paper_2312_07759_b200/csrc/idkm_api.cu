@@ -5,6 +5,7 @@
 #include "idkm_kernels.cuh"
 #include "idkm_scalar.cuh"
 #include "idkm_jac_mma.cuh"
+#include "idkm_mma_loop.cuh"
 
 #include <math.h>
 #include <stdio.h>
@@ -180,7 +181,7 @@ struct WorkspaceLayout {
   size_t off_hist_fwd, off_hist_adj;
   size_t off_rowstat;   // two floats per weight-vector, or NO_ROWSTAT
   size_t off_partials64, off_gpartials64, off_gtickets64;   // second set for the fp64 half of the dual step kernel
-  int max_slots, max_groups, max_groups64;
+  int max_slots, max_groups, max_groups64, plen_max;
   // scalar weights (idkm_scalar.cuh); sc_fine = 0: none
   size_t off_sc_sync, off_sc_gcount, off_sc_fstart, off_sc_frec, off_sc_crec, off_sc_bstat, off_sc_tab, off_sc_perm, off_sc_ftab,
       off_sc_gpart, off_sc_gtick;
@@ -242,6 +243,7 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
   w.off_g = o;     o = align_up(o + sizeof(float) * (size_t)n_layers * k * d, 256);
   w.off_u = o;     o = align_up(o + sizeof(float) * (size_t)n_layers * k * d, 256);
   w.max_slots = sms * MAX_BLOCKS_PER_SM + n_layers;
+  w.plen_max = plen_max;
   size_t partial_doubles = (size_t)w.max_slots * plen_max;
   if (jac_tile_doubles > partial_doubles) partial_doubles = jac_tile_doubles;
   w.off_partials = o; o = align_up(o + sizeof(double) * partial_doubles, 256);
@@ -563,6 +565,46 @@ constexpr long long SMALL_SOLO_ROWS = 4096;   // a single layer up to this size 
 constexpr long long SMALL_SOLO_WORK = 32768;  // ... if rows x centroids x d stays below this (d = 4, k = 8: 1024 rows)
 constexpr long long SMALL_SPIN_LIMIT = 2000000000LL;   // about a second of SM clock ticks per barrier wait
 
+// Deals `grid` blocks to the layers: one each, the rest in proportion to the rows (largest remainders first).  Returns the
+// largest number of rows a block of any layer takes.
+static long long deal_blocks(const idkm_ctx* ctx, int grid, SmallLoopParams* sp) {
+  const int L = ctx->n_layers;
+  const long long m = ctx->m_total;
+  int cnt[MAX_LAYERS];
+  long long rem[MAX_LAYERS];
+  int given = 0;
+  const long long spare = grid - L;
+  for (int l = 0; l < L; ++l) {
+    const long long rows = ctx->row_off[l + 1] - ctx->row_off[l];
+    const long long share = (m > 0) ? spare * rows / m : 0;
+    cnt[l] = 1 + (int)share;
+    rem[l] = (m > 0) ? spare * rows % m : 0;
+    given += cnt[l];
+    sp->row_off[l] = ctx->row_off[l];
+  }
+  sp->row_off[L] = ctx->row_off[L];
+  while (given < grid) {
+    int best = 0;
+    for (int l = 1; l < L; ++l)
+      if (rem[l] > rem[best]) best = l;
+    ++cnt[best];
+    rem[best] = -1;
+    ++given;
+  }
+  long long most = 0;
+  sp->blk_first[0] = 0;
+  for (int l = 0; l < L; ++l) {
+    sp->blk_first[l + 1] = sp->blk_first[l] + cnt[l];
+    const long long per = (ctx->row_off[l + 1] - ctx->row_off[l] + cnt[l] - 1) / cnt[l];
+    if (per > most) most = per;
+  }
+  for (int l = L + 1; l <= MAX_LAYERS; ++l) {
+    sp->blk_first[l] = sp->blk_first[L];
+    sp->row_off[l] = sp->row_off[L];
+  }
+  return most;
+}
+
 // Returns IDKM_OK after queueing the loop, 1 if this problem should take the launch-per-iteration path.
 static int try_small_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, int max_iter) {
   static const bool env_off = (getenv("IDKM_NO_COOP") != nullptr);   // tuning knob: always a launch per iteration
@@ -605,40 +647,7 @@ static int try_small_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPa
   memset(&sp, 0, sizeof(sp));
   sp.W = ctx->W;
   sp.n_layers = L;
-  // blocks per layer: one each, the rest in proportion to the rows (largest remainders first)
-  int cnt[MAX_LAYERS];
-  long long rem[MAX_LAYERS];
-  int given = 0;
-  const long long spare = grid - L;
-  for (int l = 0; l < L; ++l) {
-    const long long rows = ctx->row_off[l + 1] - ctx->row_off[l];
-    const long long share = (m > 0) ? spare * rows / m : 0;
-    cnt[l] = 1 + (int)share;
-    rem[l] = (m > 0) ? spare * rows % m : 0;
-    given += cnt[l];
-    sp.row_off[l] = ctx->row_off[l];
-  }
-  sp.row_off[L] = ctx->row_off[L];
-  while (given < grid) {
-    int best = 0;
-    for (int l = 1; l < L; ++l)
-      if (rem[l] > rem[best]) best = l;
-    ++cnt[best];
-    rem[best] = -1;
-    ++given;
-  }
-  long long max_rows_per_thread = 0;
-  sp.blk_first[0] = 0;
-  for (int l = 0; l < L; ++l) {
-    sp.blk_first[l + 1] = sp.blk_first[l] + cnt[l];
-    const long long rows = ctx->row_off[l + 1] - ctx->row_off[l];
-    const long long per = (rows + (long long)cnt[l] * BLOCK - 1) / ((long long)cnt[l] * BLOCK);
-    if (per > max_rows_per_thread) max_rows_per_thread = per;
-  }
-  for (int l = L + 1; l <= MAX_LAYERS; ++l) {
-    sp.blk_first[l] = sp.blk_first[L];
-    sp.row_off[l] = sp.row_off[L];
-  }
+  const long long max_rows_per_thread = (deal_blocks(ctx, (int)grid, &sp) + BLOCK - 1) / BLOCK;
   sp.C = ctx->C;
   sp.st = p.st;
   sp.partials = p.partials;
@@ -656,6 +665,70 @@ static int try_small_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPa
   sp.missing_arrivals = ctx->hook_missing_arrivals;
   if (ctx->hook_spin_limit > 0 && ctx->hook_spin_limit < SMALL_SPIN_LIMIT) sp.spin_limit = ctx->hook_spin_limit;
   if (se->launch(sp, (int)grid, ctx->stream) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 1;   // nothing was queued: take the launch-per-iteration path
+  }
+  ++ctx->launches;
+  return IDKM_OK;
+}
+
+// The single-launch loop of idkm_mma_loop_impl.cuh: d = 2 and 4, codebooks the kernel above does not take.
+static const MmaLoopEntry* mma_loop_entry(int d, int k, bool squared) {
+  if (d != 2 && d != 4) return nullptr;
+  const MmaLoopEntry* t = d == 2 ? (squared ? k_mma_loop_d2_sq : k_mma_loop_d2) : (squared ? k_mma_loop_d4_sq : k_mma_loop_d4);
+  for (int i = 0; i < N_MMA_LOOP; ++i)
+    if (k <= t[i].kp) return t + i;
+  return nullptr;
+}
+constexpr int MMA_LOOP_ROWS = 128;   // weight-vectors a block takes at least
+// doubles that all blocks together may read for every block to add all partials (4 MB: about a microsecond; a second barrier
+// and a trip through memory cost two: m = 4096, d = 2, k = 64: 9.3 against 11.8 us an iteration, d = 4, k = 16: 8.7 against 10.2)
+constexpr long long MMA_LOOP_ONE_STAGE = 500000;
+// Batches with d = 4 and 9 to 16 centroids below this many weight-vectors keep a launch per iteration: callers of that path
+// count its launches.
+constexpr long long MMA_LOOP_BATCH_16 = 1 << 18;
+
+// Returns IDKM_OK after queueing the loop, 1 if this problem should take the launch-per-iteration path.
+static int try_mma_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, int max_iter) {
+  static const bool env_off = (getenv("IDKM_NO_COOP") != nullptr);
+  if (env_off || ctx->forward_loop != 0 || max_iter < 2 || (!ctx->squared && ctx->collapse_step != 0)) return 1;
+  const MmaLoopEntry* e = mma_loop_entry(ctx->d, ctx->k, ctx->squared != 0);
+  const int L = ctx->n_layers;
+  if (!e || !e->launch || ctx->k * ctx->d <= 32 || L > ctx->sms) return 1;
+  // (small batches of quadruples with at most 16 centroids: a launch per iteration, see MMA_LOOP_BATCH_16)
+  if (L > 1 && ctx->k <= 16 && ctx->m_total < MMA_LOOP_BATCH_16) return 1;
+  int grid = ctx->sms;
+  const long long most = (ctx->m_total + MMA_LOOP_ROWS - 1) / MMA_LOOP_ROWS;
+  if (grid > most) grid = (int)most;
+  if (grid < L) grid = L;
+  if ((size_t)grid * e->plen > (size_t)wl.max_slots * wl.plen_max || (size_t)L * e->plen > (size_t)wl.max_groups * wl.plen_max) return 1;
+  MmaLoopParams mp;
+  memset(&mp, 0, sizeof(mp));
+  SmallLoopParams& sp = mp.s;
+  sp.W = ctx->W;
+  sp.n_layers = L;
+  deal_blocks(ctx, grid, &sp);
+  long long reads = 0;   // doubles the blocks read if every one adds all partials of its layer
+  for (int l = 0; l < L; ++l) {
+    const long long n = sp.blk_first[l + 1] - sp.blk_first[l];
+    reads += n * n * e->plen;
+  }
+  mp.one_stage = reads <= MMA_LOOP_ONE_STAGE && 2 * (size_t)grid * e->plen <= (size_t)wl.max_slots * wl.plen_max;
+  sp.C = ctx->C;
+  sp.st = p.st;
+  sp.partials = p.partials;
+  mp.totals = p.gpartials;
+  sp.sync = reinterpret_cast<unsigned int*>(static_cast<char*>(ctx->workspace) + wl.off_sync);
+  sp.k = ctx->k;
+  sp.scale = p.scale;
+  sp.tol = p.tol;
+  sp.inv_tau_d = p.inv_tau_d;
+  sp.max_iter = max_iter;
+  sp.hist = p.hist_fwd;
+  sp.spin_limit = SMALL_SPIN_LIMIT;
+  sp.missing_arrivals = ctx->hook_missing_arrivals;
+  if (ctx->hook_spin_limit > 0 && ctx->hook_spin_limit < SMALL_SPIN_LIMIT) sp.spin_limit = ctx->hook_spin_limit;
+  if (e->launch(mp, grid, ctx->stream) != cudaSuccess) {
     (void)cudaGetLastError();
     return 1;   // nothing was queued: take the launch-per-iteration path
   }
@@ -982,6 +1055,7 @@ int idkm_forward_batched(idkm_ctx* ctx, const float* W_cat, const int64_t* layer
     ++ctx->launches;
     mark(ctx, 1);
     rc = try_small_loop(ctx, wl, p, max_iter);
+    if (rc == 1) rc = try_mma_loop(ctx, wl, p, max_iter);
     if (rc == 1) rc = launch_step_loop(ctx, wl, &p, max_iter);
   }
   nvtxRangePop();

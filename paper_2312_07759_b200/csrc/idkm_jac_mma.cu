@@ -144,31 +144,6 @@ struct JmStop {
   }
 };
 
-// Two floats in one register pair: the packed fp32 instructions halve the issue slots of the producers, which compute the
-// same quantity for two neighbouring weights.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 f2_pack(float a, float b) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void f2_unpack(f2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); }
-__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
-  f2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-  f2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-  f2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // Splits eight values (four pairs of neighbouring weights) into two fp16 terms and stores them, 16 bytes each.  The first
 // term is the value cut to its 11 leading bits -- a mask, on the integer pipe, which the producers leave idle, instead of a
 // conversion and back -- so the second is exact before its rounding.

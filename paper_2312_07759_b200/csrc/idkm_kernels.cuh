@@ -154,6 +154,30 @@ struct PassCfg {
 // full (there the two extra values per row in flight made the step spill and run 8 % slower).
 __host__ __device__ constexpr bool row_cache_layout(int d, int lpw) { return lpw > 1; }
 
+// Two floats in one register pair: the packed fp32 instructions take half the issue slots for the same arithmetic.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_pack(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // ---- special-function-unit wrappers ------------------------------------------------------------
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -2447,6 +2471,31 @@ struct SmallLoopParams {
                          // this many arrivals more than the grid has, so every wait runs out (see idkm.h)
   long long spin_limit;  // clock64() ticks a block waits at a barrier before it gives up
 };
+// Grid-wide barrier of a cooperative launch: one arrival counter that only grows (sync[0]) and an error word (sync[1]).
+// Bounded wait until the arrival counter has reached `target`.  Returns false if the wait ran out or another block
+// raised the error word.
+__device__ __forceinline__ bool small_barrier(unsigned int* sync, unsigned int target, long long spin_limit, int* s_ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    volatile unsigned int* vs = sync;
+    int ok = 1;
+    __threadfence();
+    atomicAdd(&sync[0], 1u);
+    const long long t0 = clock64();
+    while ((int)(vs[0] - target) < 0) {
+      if (vs[1] != 0u || clock64() - t0 > spin_limit) {
+        atomicExch(&sync[1], 1u);
+        ok = 0;
+        break;
+      }
+    }
+    if (vs[1] != 0u) ok = 0;
+    __threadfence();
+    *s_ok = ok;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
 typedef cudaError_t (*SmallLaunchFn)(const SmallLoopParams& sp, int grid, cudaStream_t stream);
 struct SmallLoopEntry {
   SmallLaunchFn launch;
