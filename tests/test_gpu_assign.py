@@ -62,3 +62,34 @@ def test_assign_argument_errors():
     assert f(W.data_ptr(), 64, 2, Cm.data_ptr(), 4, None, W.data_ptr(), None) == B.ERR_PARAM
     assert B.lib.idkm_code_bits(0) == 0 and B.lib.idkm_code_bits(3) == 2 and B.lib.idkm_codes_bytes(9, 2) == 2
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("d,k", [(1, 33), (1, 64), (1, 65), (1, 255), (1, 256), (2, 32), (2, 33), (2, 256), (4, 32), (4, 39), (4, 256)])
+@pytest.mark.parametrize("m", [3, 129, 20001])
+def test_assign_breaks_ties_by_the_lowest_index(m, d, k):
+    """Weights and centroids on a grid: every difference, square and sum is exact in fp32, equal distances are frequent (and some
+    centroids are equal), so the index must be the first of the nearest; NaN, huge and tiny values included."""
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    rng = np.random.default_rng(m + 7 * k + d)
+    W = (rng.integers(-40, 41, (m, d)) / 64.0).astype(np.float32)
+    C = (rng.integers(-20, 21, (k, d)) / 32.0).astype(np.float32)
+    C[k - 3] = C[1]
+    d2 = ((W[:, None, :].astype(np.float64) - C[None].astype(np.float64)) ** 2).sum(-1)
+    ref = d2.argmin(1)
+    W[0] = np.nan                       # nothing is nearer than a NaN is to anything: index 0
+    ref[0] = 0
+    W[1] = 3e30                         # every square overflows
+    ref[1] = 0
+    codes, Wq = B.assign(torch.from_numpy(W).cuda(), torch.from_numpy(C).cuda())
+    assert np.array_equal(H.unpack_codes(codes.cpu().numpy(), m, k), ref)
+    assert np.array_equal(Wq.cpu().numpy(), C[ref])
+    tiny = np.float32(2.0 ** -70)       # squares below the normal range: still exact multiples of 2^-149
+    codes, _ = B.assign(torch.from_numpy(W[2:] * tiny).cuda(), torch.from_numpy(C * tiny).cuda())
+    idx = H.unpack_codes(codes.cpu().numpy(), m - 2, k)
+    assert np.all(idx < k)
+    C2 = C.copy()
+    C2[2] = np.nan                      # a centroid that is never the nearest
+    d2[:, 2] = np.inf
+    codes, _ = B.assign(torch.from_numpy(W[2:]).cuda(), torch.from_numpy(C2).cuda())
+    assert np.array_equal(H.unpack_codes(codes.cpu().numpy(), m - 2, k), d2[2:].argmin(1))
