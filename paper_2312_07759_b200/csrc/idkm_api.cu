@@ -318,6 +318,8 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
 
 using namespace idkm;
 
+constexpr int HOST_GROUPS_MAX = 4;
+
 struct idkm_ctx {
   int device;
   int sms;
@@ -338,8 +340,8 @@ struct idkm_ctx {
   void* hbuf;
   size_t hbuf_bytes;
   bool host_streams_ok;
-  cudaStream_t hs_compute, hs_copy;
-  cudaEvent_t hev[4];
+  cudaStream_t hs_compute, hs_copy, hs_down;
+  cudaEvent_t hev[4 * HOST_GROUPS_MAX];   // per group of layers: W there, G there, forward done, backward done
   // optional phase timing (CUDA events on the call's stream)
   bool timing;
   bool ev_ok;
@@ -981,9 +983,10 @@ void idkm_destroy(idkm_ctx* ctx) {
   if (!ctx) return;
   if (ctx->hbuf) cudaFree(ctx->hbuf);
   if (ctx->host_streams_ok) {
-    for (int i = 0; i < 4; ++i) cudaEventDestroy(ctx->hev[i]);
+    for (int i = 0; i < 4 * HOST_GROUPS_MAX; ++i) cudaEventDestroy(ctx->hev[i]);
     cudaStreamDestroy(ctx->hs_compute);
     cudaStreamDestroy(ctx->hs_copy);
+    cudaStreamDestroy(ctx->hs_down);
   }
   if (ctx->chunk_ev_ok) {
     cudaEventDestroy(ctx->chunk_ev[0]);
@@ -1199,6 +1202,48 @@ int idkm_get_info(idkm_ctx* ctx, idkm_info* info_out) {
   return IDKM_OK;
 }
 
+// A call on host buffers in up to HOST_GROUPS_MAX groups of consecutive layers, each with buffers and a workspace of its own:
+// while one group is clustered the next one's weights come in, and what a group gives goes out at once.  The link carries
+// both directions at the same time, but one batch leaves the outgoing one idle until all weights are in and clustered
+// (47 MB of weights, d = 2, k = 4, 30 iterations: 0.87 ms in, 0.8 clustering, then twice 0.84 out).
+struct HostGroup {
+  int l0, l1;
+  int64_t m;
+  size_t wn, cn, w0, c0, ws_bytes, off;
+  float* w[5];   // W, G, Wq, dW, dW (Jacobian-free)
+  float* c[4];   // C0, C, dC, dC (Jacobian-free)
+  void* ws;
+  int64_t offs[IDKM_MAX_LAYERS + 1];
+  bool scalar_forward;
+  // the ctx as this group's forward left it
+  void make_current(idkm_ctx* ctx) const {
+    ctx->W = w[0];
+    ctx->C = c[1];
+    ctx->workspace = ws;
+    ctx->m_total = m;
+    ctx->n_layers = l1 - l0;
+    for (int l = 0; l <= l1 - l0; ++l) ctx->row_off[l] = offs[l];
+    ctx->scalar_forward = scalar_forward;
+  }
+};
+constexpr size_t HOST_GROUP_BYTES = 12u << 20;   // weights of a group at least: 0.2 ms of the link, more than its launches cost
+static int host_groups(const idkm_ctx* ctx, const int64_t* offs, int n_layers, size_t wn, HostGroup* grp) {
+  // (phase times are of one batch)
+  int want = ctx->timing ? 1 : (int)(wn / HOST_GROUP_BYTES);
+  if (want > HOST_GROUPS_MAX) want = HOST_GROUPS_MAX;
+  int n = 0, l = 0;
+  while (l < n_layers) {
+    grp[n].l0 = l;
+    ++l;
+    // up to the layer whose end is nearest to this group's share
+    const int64_t goal = want > 1 && n + 1 < want ? offs[n_layers] * (n + 1) / want : offs[n_layers];
+    while (l < n_layers && (goal == offs[n_layers] || offs[l + 1] - goal <= goal - offs[l])) ++l;
+    grp[n].l1 = l;
+    ++n;
+  }
+  return n;
+}
+
 int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* layer_offsets, int n_layers, int d,
                           const float* C0_host, int k, float tau, float tol, int max_iter, const float* dWq_host,
                           idkm_mode mode, float adj_tol, int adj_max_iter, float alpha, float* C_out_host,
@@ -1209,13 +1254,26 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
   if (n_layers < 1 || n_layers > IDKM_MAX_LAYERS || layer_offsets[0] != 0) return IDKM_ERR_SHAPE;
   const int64_t m = layer_offsets[n_layers];
   if (m < 1) return IDKM_ERR_SHAPE;
+  for (int l = 0; l < n_layers; ++l)
+    if (layer_offsets[l + 1] <= layer_offsets[l]) return IDKM_ERR_SHAPE;
   const size_t ws_bytes = idkm_workspace_bytes(m, d, k, n_layers);
   if (ws_bytes == 0) return IDKM_ERR_UNSUPPORTED;
   const bool also_jfb = (dW_jfb_out_host != nullptr || dC_jfb_out_host != nullptr) && mode == IDKM_IMPLICIT;
-  const size_t wbytes = align_up(sizeof(float) * (size_t)m * d, 256);
-  const size_t cbytes = align_up(sizeof(float) * (size_t)n_layers * k * d, 256);
-  // W, G, Wq, dW, dW (Jacobian-free) | C0, C, dC, dC (Jacobian-free) | workspace
-  const size_t need = 5 * wbytes + 4 * cbytes + align_up(ws_bytes, 256);
+  const size_t wn = sizeof(float) * (size_t)m * d, cn = sizeof(float) * (size_t)n_layers * k * d;
+  HostGroup grp[HOST_GROUPS_MAX];
+  const int ng = host_groups(ctx, layer_offsets, n_layers, wn, grp);
+  // each group's W, G, Wq, dW, dW (Jacobian-free), C0, C, dC, dC (Jacobian-free), workspace; the whole call's workspace
+  size_t need = ng > 1 ? align_up(ws_bytes, 256) : 0;
+  for (int g = 0; g < ng; ++g) {
+    HostGroup& q = grp[g];
+    q.m = layer_offsets[q.l1] - layer_offsets[q.l0];
+    q.wn = sizeof(float) * (size_t)q.m * d;
+    q.cn = sizeof(float) * (size_t)(q.l1 - q.l0) * k * d;
+    q.ws_bytes = idkm_workspace_bytes(q.m, d, k, q.l1 - q.l0);
+    if (q.ws_bytes == 0) return IDKM_ERR_UNSUPPORTED;
+    q.off = need;
+    need += 5 * align_up(q.wn, 256) + 4 * align_up(q.cn, 256) + align_up(q.ws_bytes, 256);
+  }
   if (need > ctx->hbuf_bytes) {
     if (ctx->hbuf) cudaFree(ctx->hbuf);
     ctx->hbuf = nullptr;
@@ -1226,70 +1284,119 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
     }
     ctx->hbuf_bytes = need;
   }
-  // two streams of the ctx's own: the kernels run on one, the copies that can overlap them on the other
+  // three streams of the ctx's own: the kernels run on one, uploads that can overlap them on another, downloads on a third (behind
+  // the upload of the gradient they would leave one direction of the link idle)
   if (!ctx->host_streams_ok) {
     if (cudaStreamCreateWithFlags(&ctx->hs_compute, cudaStreamNonBlocking) != cudaSuccess) return IDKM_ERR_CUDA;
     if (cudaStreamCreateWithFlags(&ctx->hs_copy, cudaStreamNonBlocking) != cudaSuccess) {
       cudaStreamDestroy(ctx->hs_compute);
       return IDKM_ERR_CUDA;
     }
-    for (int i = 0; i < 4; ++i)
+    if (cudaStreamCreateWithFlags(&ctx->hs_down, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaStreamDestroy(ctx->hs_compute);
+      cudaStreamDestroy(ctx->hs_copy);
+      return IDKM_ERR_CUDA;
+    }
+    for (int i = 0; i < 4 * HOST_GROUPS_MAX; ++i)
       if (cudaEventCreateWithFlags(&ctx->hev[i], cudaEventDisableTiming) != cudaSuccess) {
         for (int q = 0; q < i; ++q) cudaEventDestroy(ctx->hev[q]);
         cudaStreamDestroy(ctx->hs_compute);
         cudaStreamDestroy(ctx->hs_copy);
+        cudaStreamDestroy(ctx->hs_down);
         return IDKM_ERR_CUDA;
       }
     ctx->host_streams_ok = true;
   }
   char* base = static_cast<char*>(ctx->hbuf);
-  float* dW_ = reinterpret_cast<float*>(base);
-  float* dG = reinterpret_cast<float*>(base + wbytes);
-  float* dWq = reinterpret_cast<float*>(base + 2 * wbytes);
-  float* ddW = reinterpret_cast<float*>(base + 3 * wbytes);
-  float* ddWj = reinterpret_cast<float*>(base + 4 * wbytes);
-  float* dC0 = reinterpret_cast<float*>(base + 5 * wbytes);
-  float* dC = reinterpret_cast<float*>(base + 5 * wbytes + cbytes);
-  float* ddC = reinterpret_cast<float*>(base + 5 * wbytes + 2 * cbytes);
-  float* ddCj = reinterpret_cast<float*>(base + 5 * wbytes + 3 * cbytes);
-  void* ws = base + 5 * wbytes + 4 * cbytes;
-  cudaStream_t s = ctx->hs_compute, sc = ctx->hs_copy;
-  const size_t wn = sizeof(float) * (size_t)m * d, cn = sizeof(float) * (size_t)n_layers * k * d;
-#define IDKM_TRY(call) do { if ((call) != cudaSuccess) { (void)cudaGetLastError(); cudaStreamSynchronize(s); cudaStreamSynchronize(sc); return IDKM_ERR_CUDA; } } while (0)
-  // W and C0 go first on the compute stream; the upstream gradient is uploaded on the copy stream while the forward
-  // loop runs (it is first read by the backward)
-  IDKM_TRY(cudaMemcpyAsync(dW_, W_host, wn, cudaMemcpyHostToDevice, s));
-  IDKM_TRY(cudaMemcpyAsync(dC0, C0_host, cn, cudaMemcpyHostToDevice, s));
-  IDKM_TRY(cudaMemcpyAsync(dG, dWq_host, wn, cudaMemcpyHostToDevice, sc));
-  IDKM_TRY(cudaEventRecord(ctx->hev[0], sc));
-  const int wq_dtype_saved = ctx->wq_dtype;
-  ctx->wq_dtype = 0;   // the host buffers of this entry point are fp32
-  int rc = idkm_forward_batched(ctx, dW_, layer_offsets, n_layers, d, dC0, k, tau, tol, max_iter, dC, nullptr,
-                                Wq_out_host ? dWq : nullptr, ws, ws_bytes, s);
-  ctx->wq_dtype = wq_dtype_saved;
-  if (rc != IDKM_OK) { cudaStreamSynchronize(s); cudaStreamSynchronize(sc); return rc; }
-  // C and Wq go back on the copy stream while the backward runs
-  IDKM_TRY(cudaEventRecord(ctx->hev[1], s));
-  IDKM_TRY(cudaStreamWaitEvent(sc, ctx->hev[1], 0));
-  IDKM_TRY(cudaMemcpyAsync(C_out_host, dC, cn, cudaMemcpyDeviceToHost, sc));
-  if (Wq_out_host) IDKM_TRY(cudaMemcpyAsync(Wq_out_host, dWq, wn, cudaMemcpyDeviceToHost, sc));
-  IDKM_TRY(cudaStreamWaitEvent(s, ctx->hev[0], 0));
-  if (also_jfb) {
-    rc = idkm_backward(ctx, dG, IDKM_JFB, 0.f, 0, 1.f, dW_jfb_out_host ? ddWj : nullptr, dC_jfb_out_host ? ddCj : nullptr,
-                       ws, ws_bytes, s);
-    if (rc != IDKM_OK) { cudaStreamSynchronize(s); cudaStreamSynchronize(sc); return rc; }
-    IDKM_TRY(cudaEventRecord(ctx->hev[2], s));
-    IDKM_TRY(cudaStreamWaitEvent(sc, ctx->hev[2], 0));
-    if (dW_jfb_out_host) IDKM_TRY(cudaMemcpyAsync(dW_jfb_out_host, ddWj, wn, cudaMemcpyDeviceToHost, sc));
-    if (dC_jfb_out_host) IDKM_TRY(cudaMemcpyAsync(dC_jfb_out_host, ddCj, cn, cudaMemcpyDeviceToHost, sc));
+  cudaStream_t s = ctx->hs_compute, sc = ctx->hs_copy, sd = ctx->hs_down;
+  for (int g = 0; g < ng; ++g) {
+    HostGroup& q = grp[g];
+    char* at = base + q.off;
+    const size_t wb = align_up(q.wn, 256), cb = align_up(q.cn, 256);
+    for (int i = 0; i < 5; ++i, at += wb) q.w[i] = reinterpret_cast<float*>(at);
+    for (int i = 0; i < 4; ++i, at += cb) q.c[i] = reinterpret_cast<float*>(at);
+    q.ws = at;
+    for (int l = q.l0; l <= q.l1; ++l) q.offs[l - q.l0] = layer_offsets[l] - layer_offsets[q.l0];
+    q.w0 = (size_t)layer_offsets[q.l0] * d;
+    q.c0 = (size_t)q.l0 * k * d;
   }
-  rc = idkm_backward(ctx, dG, mode, adj_tol, adj_max_iter, alpha, dW_out_host ? ddW : nullptr,
-                     dC_out_host ? ddC : nullptr, ws, ws_bytes, s);
-  if (rc != IDKM_OK) { cudaStreamSynchronize(s); cudaStreamSynchronize(sc); return rc; }
-  if (dW_out_host) IDKM_TRY(cudaMemcpyAsync(dW_out_host, ddW, wn, cudaMemcpyDeviceToHost, s));
-  if (dC_out_host) IDKM_TRY(cudaMemcpyAsync(dC_out_host, ddC, cn, cudaMemcpyDeviceToHost, s));
+  const auto give_up = [&](int rc) {
+    cudaStreamSynchronize(s);
+    cudaStreamSynchronize(sc);
+    cudaStreamSynchronize(sd);
+    return rc;
+  };
+#define IDKM_TRY(call) do { if ((call) != cudaSuccess) { (void)cudaGetLastError(); return give_up(IDKM_ERR_CUDA); } } while (0)
+  // uploads: all weights, then all gradients (the link carries one upload at a time; the backward is what reads them)
+  for (int g = 0; g < ng; ++g) {
+    HostGroup& q = grp[g];
+    IDKM_TRY(cudaMemcpyAsync(q.c[0], C0_host + q.c0, q.cn, cudaMemcpyHostToDevice, sc));
+    IDKM_TRY(cudaMemcpyAsync(q.w[0], W_host + q.w0, q.wn, cudaMemcpyHostToDevice, sc));
+    IDKM_TRY(cudaEventRecord(ctx->hev[4 * g], sc));
+  }
+  for (int g = 0; g < ng; ++g) {
+    IDKM_TRY(cudaMemcpyAsync(grp[g].w[1], dWq_host + grp[g].w0, grp[g].wn, cudaMemcpyHostToDevice, sc));
+    IDKM_TRY(cudaEventRecord(ctx->hev[4 * g + 1], sc));
+  }
+  const int wq_dtype_saved = ctx->wq_dtype;
+  for (int g = 0; g < ng; ++g) {
+    HostGroup& q = grp[g];
+    IDKM_TRY(cudaStreamWaitEvent(s, ctx->hev[4 * g], 0));
+    ctx->wq_dtype = 0;   // the host buffers of this entry point are fp32
+    const int rc = idkm_forward_batched(ctx, q.w[0], q.offs, q.l1 - q.l0, d, q.c[0], k, tau, tol, max_iter, q.c[1], nullptr,
+                                        Wq_out_host ? q.w[2] : nullptr, q.ws, q.ws_bytes, s);
+    ctx->wq_dtype = wq_dtype_saved;
+    if (rc != IDKM_OK) return give_up(rc);
+    q.scalar_forward = ctx->scalar_forward;
+    // C and Wq go back while the rest comes in
+    IDKM_TRY(cudaEventRecord(ctx->hev[4 * g + 2], s));
+    IDKM_TRY(cudaStreamWaitEvent(sd, ctx->hev[4 * g + 2], 0));
+    IDKM_TRY(cudaMemcpyAsync(C_out_host + q.c0, q.c[1], q.cn, cudaMemcpyDeviceToHost, sd));
+    if (Wq_out_host) IDKM_TRY(cudaMemcpyAsync(Wq_out_host + q.w0, q.w[2], q.wn, cudaMemcpyDeviceToHost, sd));
+  }
+  for (int g = 0; g < ng; ++g) {
+    HostGroup& q = grp[g];
+    if (ng > 1) q.make_current(ctx);
+    IDKM_TRY(cudaStreamWaitEvent(s, ctx->hev[4 * g + 1], 0));
+    if (also_jfb) {
+      const int rc = idkm_backward(ctx, q.w[1], IDKM_JFB, 0.f, 0, 1.f, dW_jfb_out_host ? q.w[4] : nullptr,
+                                   dC_jfb_out_host ? q.c[3] : nullptr, q.ws, q.ws_bytes, s);
+      if (rc != IDKM_OK) return give_up(rc);
+      IDKM_TRY(cudaEventRecord(ctx->hev[4 * g + 3], s));
+      IDKM_TRY(cudaStreamWaitEvent(sd, ctx->hev[4 * g + 3], 0));
+      if (dW_jfb_out_host) IDKM_TRY(cudaMemcpyAsync(dW_jfb_out_host + q.w0, q.w[4], q.wn, cudaMemcpyDeviceToHost, sd));
+      if (dC_jfb_out_host) IDKM_TRY(cudaMemcpyAsync(dC_jfb_out_host + q.c0, q.c[3], q.cn, cudaMemcpyDeviceToHost, sd));
+    }
+    const int rc = idkm_backward(ctx, q.w[1], mode, adj_tol, adj_max_iter, alpha, dW_out_host ? q.w[3] : nullptr,
+                                 dC_out_host ? q.c[2] : nullptr, q.ws, q.ws_bytes, s);
+    if (rc != IDKM_OK) return give_up(rc);
+    IDKM_TRY(cudaEventRecord(ctx->hev[4 * g + 3], s));
+    IDKM_TRY(cudaStreamWaitEvent(sd, ctx->hev[4 * g + 3], 0));
+    if (dW_out_host) IDKM_TRY(cudaMemcpyAsync(dW_out_host + q.w0, q.w[3], q.wn, cudaMemcpyDeviceToHost, sd));
+    if (dC_out_host) IDKM_TRY(cudaMemcpyAsync(dC_out_host + q.c0, q.c[2], q.cn, cudaMemcpyDeviceToHost, sd));
+  }
+  if (ng > 1) {
+    // what can be asked about the call afterwards (layer states, residual histories) moves to one place
+    WorkspaceLayout all, part;
+    if (!make_layout(m, d, k, n_layers, ctx->sms, &all)) return give_up(IDKM_ERR_UNSUPPORTED);
+    IDKM_TRY(cudaMemsetAsync(base + all.off_gtickets, 0, sizeof(unsigned int) * (size_t)all.max_groups, s));
+    if (all.max_groups64 > 0) IDKM_TRY(cudaMemsetAsync(base + all.off_gtickets64, 0, sizeof(unsigned int) * (size_t)all.max_groups64, s));
+    for (int g = 0; g < ng; ++g) {
+      const HostGroup& q = grp[g];
+      const size_t n = (size_t)(q.l1 - q.l0), l0 = (size_t)q.l0, h = sizeof(float) * HIST_CAP;
+      if (!make_layout(q.m, d, k, q.l1 - q.l0, ctx->sms, &part)) return give_up(IDKM_ERR_UNSUPPORTED);
+      const char* ws = static_cast<const char*>(q.ws);
+      IDKM_TRY(cudaMemcpyAsync(base + all.off_state + l0 * sizeof(LayerState), ws + part.off_state, n * sizeof(LayerState), cudaMemcpyDeviceToDevice, s));
+      IDKM_TRY(cudaMemcpyAsync(base + all.off_hist_fwd + l0 * h, ws + part.off_hist_fwd, n * h, cudaMemcpyDeviceToDevice, s));
+      IDKM_TRY(cudaMemcpyAsync(base + all.off_hist_adj + l0 * h, ws + part.off_hist_adj, n * h, cudaMemcpyDeviceToDevice, s));
+    }
+    ctx->workspace = base;
+    ctx->m_total = m;
+    ctx->n_layers = n_layers;
+    for (int l = 0; l <= n_layers; ++l) ctx->row_off[l] = layer_offsets[l];
+  }
 #undef IDKM_TRY
-  if (cudaStreamSynchronize(sc) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return IDKM_ERR_CUDA;
+  if (cudaStreamSynchronize(sd) != cudaSuccess || cudaStreamSynchronize(sc) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return IDKM_ERR_CUDA;
   if (info_out) return idkm_get_info(ctx, info_out);
   return IDKM_OK;
 }

@@ -1,0 +1,37 @@
+"""Calls on host buffers large enough to be taken in groups of layers, against the same call as one batch (B200 only)."""
+import numpy as np
+import pytest
+
+from parity_util import assert_close
+
+pytestmark = pytest.mark.gpu
+
+
+# two to four groups; a layer larger than a group's share, tiny layers between large ones, unaligned layer starts
+@pytest.mark.parametrize("d,k,rows", [(1, 4, [3_000_001, 5, 3_500_003, 70_001]), (2, 4, [100_003, 2_900_001, 37, 1_700_000, 1_900_001, 12]),
+                                      (4, 16, [2_000_003, 33, 3001, 1_800_001])])
+def test_groups_equal_one_batch(d, k, rows):
+    from paper_2312_07759_b200 import binding as B
+    rng = np.random.default_rng(d)
+    offs = [0] + [int(x) for x in np.cumsum(rows)]
+    W = (rng.standard_normal((offs[-1], d), dtype=np.float32) * np.float32(0.03))
+    G = rng.standard_normal(W.shape, dtype=np.float32) * np.float32(0.1)
+    k = min([k] + rows)
+    C0 = np.concatenate([W[a:a + k] for a in offs[:-1]])
+    out = []
+    for one_batch in (False, True):
+        ctx = B.Context()
+        ctx.set_timing(one_batch)          # (phase times are of one batch)
+        n0 = ctx.launches
+        C, Wq, dW, dC, infos, dWj, dCj = ctx.quantize_host(W, C0, G, 0.02, 0.0, 5, B.IMPLICIT, 0.0, 6, 0.5, layer_offsets=offs, also_jfb=True)
+        n = ctx.launches - n0
+        assert ctx.busy_tickets() == 0 and len(infos) == len(rows)
+        assert [repr(i) for i in ctx.info()] == [repr(i) for i in infos]
+        out.append(([C, Wq, dW, dC, dWj, dCj], [(i.status, i.fwd_iters, i.adj_iters) for i in infos], n,
+                    [ctx.history(0, l) for l in range(len(rows))]))
+    assert out[0][2] > out[1][2]           # (the first call was split)
+    assert out[0][1] == out[1][1]
+    for name, a, b in zip(("C", "Wq", "dW", "dC", "dW jfb", "dC jfb"), out[0][0], out[1][0]):
+        assert_close(a, b, 2e-5 if d > 1 else 2e-4, name, l2_only=True)
+    for a, b in zip(out[0][3], out[1][3]):
+        assert len(a) == len(b) == 5 and np.allclose(a, b, rtol=1e-3, atol=1e-6)
