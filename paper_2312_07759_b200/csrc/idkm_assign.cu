@@ -142,6 +142,30 @@ __device__ __forceinline__ float assign_sq(const float (&w)[D], const float* c) 
   }
   return sq;
 }
+// The weights of the lanes in `left`, one by one, against all centroids, by the whole warp.
+template <int D>
+__device__ __forceinline__ void assign_unsure(unsigned left, const float (&w)[D], const float* cs, int k, int lane, int& bj) {
+  while (left) {
+    const int from = __ffs(left) - 1;
+    left &= left - 1;
+    float x[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) x[a] = __shfl_sync(0xffffffffu, w[a], from);
+    unsigned lo = 0xffffffffu;
+    int at = 0;
+    for (int j = lane; j < k; j += 32) {
+      const float sq = assign_sq<D>(x, cs + j * D);
+      const unsigned key = sq < 3.0e38f ? __float_as_uint(sq) : 0xffffffffu;   // (squares: ordered like their bits)
+      if (key < lo) {
+        lo = key;
+        at = j;
+      }
+    }
+    const unsigned all = __reduce_min_sync(0xffffffffu, lo);
+    const unsigned win = __reduce_min_sync(0xffffffffu, lo == all ? (unsigned)at : 0xffffffffu);
+    if (lane == from) bj = all == 0xffffffffu ? 0 : (int)win;
+  }
+}
 template <int D, int BITS>
 __global__ void __launch_bounds__(ASSIGN_BLOCK) idkm_assign_score(const float* __restrict__ W, long long m, const float* __restrict__ C,
                                                                   int k, unsigned char* __restrict__ codes, float* __restrict__ Wq) {
@@ -258,28 +282,7 @@ __global__ void __launch_bounds__(ASSIGN_BLOCK) idkm_assign_score(const float* _
           bj[v] = blk[v] * ASSIGN_BLK + e;
         }
       }
-      // the weights whose block is not certain, one by one, against all centroids
-      unsigned left = __ballot_sync(0xffffffffu, !sure);
-      while (left) {
-        const int from = __ffs(left) - 1;
-        left &= left - 1;
-        float x[D];
-#pragma unroll
-        for (int a = 0; a < D; ++a) x[a] = __shfl_sync(0xffffffffu, w[v][a], from);
-        unsigned lo = 0xffffffffu;
-        int at = 0;
-        for (int j = lane; j < k; j += 32) {
-          const float sq = assign_sq<D>(x, cs + j * D);
-          const unsigned key = sq < 3.0e38f ? __float_as_uint(sq) : 0xffffffffu;   // (squares: ordered like their bits)
-          if (key < lo) {
-            lo = key;
-            at = j;
-          }
-        }
-        const unsigned all = __reduce_min_sync(0xffffffffu, lo);
-        const unsigned win = __reduce_min_sync(0xffffffffu, lo == all ? (unsigned)at : 0xffffffffu);
-        if (lane == from) bj[v] = all == 0xffffffffu ? 0 : (int)win;
-      }
+      assign_unsure<D>(__ballot_sync(0xffffffffu, !sure), w[v], cs, k, lane, bj[v]);
     }
 #pragma unroll
     for (int q = 0; q < NG; ++q) {
@@ -293,6 +296,216 @@ __global__ void __launch_bounds__(ASSIGN_BLOCK) idkm_assign_score(const float* _
 // (m = 2.5 M, d = 4: k = 17 31 against 31 us for the kernel above, k = 32 47 against 42, k = 64 81 against 58, k = 256 284 against
 // 164; m = 5 M, d = 2: k = 32 55 against 51, k = 256 338 against 219)
 constexpr int ASSIGN_SCORE_MIN_K = 32;
+
+// Quadruples of weights, larger codebooks still: the scores on the tensor cores (tcgen05, kind::tf32), a row of the
+// accumulator per weight and a column per centroid, so that a thread finds all scores of its weight in its lane of tensor
+// memory and only keeps the smallest: one and a bit instructions a pair, and the load.  Each factor is split into two tf32
+// terms (hi + lo, rounded; |c|^2 / 2 into three) laid out along k: hi hi, hi lo, lo hi and ones for the constant, 15 of 16
+// columns.  What that drops is below 5 u of |w| |c|; the unit's sums are taken to be good to 20 u of
+// the terms' magnitudes: with the bounds above less than 66 u (|w|^2 + c_max^2) between two scores, ASSIGN_MMA_MARGIN is 128 u.
+// A block is 128 threads with 64 to 256 columns of tensor memory; several share an SM, so that while one waits for its
+// products another reads (two at k > 128: a weight and lane then takes 4 cycles a pair and 500 besides, of which the minima are
+// two thirds).  Every wait is bounded: if one ran out, the block would compare its weights with all centroids.
+constexpr float ASSIGN_MMA_MARGIN = 128.f * 5.9604645e-8f;
+constexpr int ASSIGN_MMA_T = 128;
+constexpr int ASSIGN_POLLS = 1 << 22;
+
+__device__ __forceinline__ unsigned assign_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes; ks: bytes between core matrices along k
+__device__ __forceinline__ unsigned long long assign_desc(unsigned addr, unsigned ks) {
+  return (unsigned long long)((addr >> 4) & 0x3fffu) | ((unsigned long long)(ks >> 4) << 16) | ((unsigned long long)(128u >> 4) << 32) |
+         (1ull << 46);
+}
+__device__ __forceinline__ float assign_tf32(float x) { return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u); }
+__device__ __forceinline__ void assign_tmem_ld32(unsigned addr, float (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,"
+      "%27,%28,%29,%30,%31}, [%32];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]),
+        "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17]), "=f"(v[18]), "=f"(v[19]),
+        "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]), "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]),
+        "=f"(v[30]), "=f"(v[31])
+      : "r"(addr)
+      : "memory");
+}
+// the loads issued so far have arrived; v depends on it
+__device__ __forceinline__ void assign_tmem_wait(float (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) asm volatile("" : "+f"(v[i]));
+}
+
+__global__ void __launch_bounds__(ASSIGN_MMA_T) idkm_assign_mma(const float* __restrict__ W, long long m, const float* __restrict__ C, int k,
+                                                                unsigned char* __restrict__ codes, float* __restrict__ Wq, int cols) {
+  constexpr int D = 4, K = 4 * D, CH = K / 4;   // columns of the operands, 16-byte chunks of them
+  constexpr int KB = ASSIGN_MAX_K / ASSIGN_BLK, BS = ASSIGN_BLK + 1, T = ASSIGN_MMA_T;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  unsigned char* opB = dyn;                         // [CH][ASSIGN_MAX_K][16]
+  unsigned char* opA = dyn + CH * ASSIGN_MAX_K * 16;   // [CH][T][16]
+  __shared__ __align__(16) float cs[ASSIGN_MAX_K * D];
+  __shared__ float ct[D][KB * BS];   // (see the kernel above)
+  __shared__ __align__(8) unsigned long long bar;
+  __shared__ unsigned s_tmem;
+  __shared__ float s_part[T / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nblk = (k + 31) / 32 * 4;
+  float h_max = 0.f;
+  for (int j = tid; j < nblk * ASSIGN_BLK; j += T) {
+    float c[D], hi[D], lo[D], q = 0.f, v[K];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      c[a] = j < k ? C[j * D + a] : 0.f;
+      cs[j * D + a] = c[a];
+      ct[a][(j / ASSIGN_BLK) * BS + j % ASSIGN_BLK] = j < k ? c[a] : 2.0e19f;
+      q = fmaf(c[a], c[a], q);
+      hi[a] = assign_tf32(c[a]);
+      lo[a] = assign_tf32(c[a] - hi[a]);
+    }
+    const float h = j < k ? 0.5f * q : 3.0e38f, h1 = assign_tf32(h), h2 = j < k ? assign_tf32(h - h1) : 0.f;
+    h_max = fmaxf(h_max, j < k ? (h < 1e37f ? h : 3.0e38f) : 0.f);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      v[a] = -hi[a];
+      v[D + a] = -lo[a];
+      v[2 * D + a] = -hi[a];
+    }
+    v[12] = h1;
+    v[13] = h2;
+    v[14] = j < k ? assign_tf32((h - h1) - h2) : 0.f;
+    v[15] = 0.f;
+#pragma unroll
+    for (int q4 = 0; q4 < CH; ++q4)
+      *reinterpret_cast<float4*>(opB + (q4 * ASSIGN_MAX_K + j) * 16) = make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) h_max = fmaxf(h_max, __shfl_xor_sync(0xffffffffu, h_max, o));
+  if (lane == 0) s_part[warp] = h_max;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(assign_smem(&s_tmem)), "r"(cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (lane == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(assign_smem(&bar)) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem = *reinterpret_cast<volatile unsigned*>(&s_tmem), mine = tmem + ((unsigned)(warp * 32) << 16);
+  h_max = fmaxf(fmaxf(s_part[0], s_part[1]), fmaxf(s_part[2], s_part[3]));
+  const float cmax2 = h_max < 1e37f ? 2.f * h_max : __int_as_float(0x7fc00000);   // (NaN: no weight passes the test)
+  const unsigned idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(nblk) << 17) | ((unsigned)(T >> 4) << 24);   // tf32 in, fp32 out
+  const long long n_tiles = (m + T - 1) / T;
+  bool dead = false;   // a wait ran out: nothing more is issued
+  unsigned phase = 0;
+  float wn[D];
+  auto fetch = [&](long long t) {
+    const long long row = t * T + tid;
+#pragma unroll
+    for (int a = 0; a < D; ++a) wn[a] = 0.f;
+    if (t < n_tiles && row < m) {
+      const float4 x = __ldg(reinterpret_cast<const float4*>(W) + row);
+      wn[0] = x.x; wn[1] = x.y; wn[2] = x.z; wn[3] = x.w;
+    }
+  };
+  fetch(blockIdx.x);
+  for (long long t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    float w[D], v[K], w2 = 0.f;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      w[a] = wn[a];
+      w2 = fmaf(w[a], w[a], w2);
+      const float x = w2 < 1e37f ? w[a] : 0.f;   // (what is not finite stays out of the products)
+      v[a] = v[D + a] = assign_tf32(x);
+      v[2 * D + a] = assign_tf32(x - v[a]);
+    }
+    v[12] = v[13] = v[14] = 1.f;
+    v[15] = 0.f;
+#pragma unroll
+    for (int q = 0; q < CH; ++q) *reinterpret_cast<float4*>(opA + (q * T + tid) * 16) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // (the last tile's scores have been read)
+    dead = __syncthreads_or(dead ? 1 : 0) != 0;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!dead && tid == 0) {
+#pragma unroll
+      for (int q = 0; q < K / 8; ++q) {
+        const unsigned long long da = assign_desc(assign_smem(opA) + q * 2 * (T * 16), T * 16);
+        const unsigned long long db = assign_desc(assign_smem(opB) + q * 2 * (ASSIGN_MAX_K * 16), ASSIGN_MAX_K * 16);
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+                     "l"(da), "l"(db), "r"(idesc), "r"(q > 0 ? 1u : 0u)
+                     : "memory");
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(assign_smem(&bar)) : "memory");
+    }
+    __syncwarp();
+    fetch(t + gridDim.x);
+    if (!dead) {
+      unsigned ok = 0;
+      for (int i = 0; i < ASSIGN_POLLS && !ok; ++i)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok)
+                     : "r"(assign_smem(&bar)), "r"(phase)
+                     : "memory");
+      phase ^= 1u;
+      dead = __any_sync(0xffffffffu, !ok);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    }
+    float best = 3.3e38f, second = 3.3e38f;
+    int blk = 0;
+    if (!dead) {
+      float s0[32], s1[32];
+      auto scan = [&](const float (&x)[32], int b0) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const float lo = min3(min3(x[8 * b], x[8 * b + 1], x[8 * b + 2]), min3(x[8 * b + 3], x[8 * b + 4], x[8 * b + 5]),
+                                fminf(x[8 * b + 6], x[8 * b + 7]));
+          second = fminf(second, fmaxf(best, lo));
+          blk = lo < best ? b0 + b : blk;
+          best = fminf(best, lo);
+        }
+      };
+      assign_tmem_ld32(mine, s0);
+#pragma unroll 1
+      for (int b0 = 0; b0 < nblk; b0 += 8) {   // (the next 32 scores are on their way while 32 are looked at)
+        assign_tmem_wait(s0);
+        const bool more = b0 + 4 < nblk;
+        if (more) assign_tmem_ld32(mine + (unsigned)((b0 + 4) * 8), s1);
+        scan(s0, b0);
+        if (!more) break;
+        assign_tmem_wait(s1);
+        if (b0 + 8 < nblk) assign_tmem_ld32(mine + (unsigned)((b0 + 8) * 8), s0);
+        scan(s1, b0 + 4);
+      }
+    }
+    const bool sure = !dead && second - best > fmaf(ASSIGN_MMA_MARGIN, w2 + cmax2, 1e-35f) && w2 < 1e37f;
+    float bd = 3.0e38f;
+    int bj = 0;
+#pragma unroll
+    for (int e = 0; e < ASSIGN_BLK; ++e) {
+      float sq = 0.f;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const float df = w[a] - ct[a][blk * BS + e];
+        sq = fmaf(df, df, sq);
+      }
+      if (sq < bd) {   // strict: ties keep the lower index
+        bd = sq;
+        bj = blk * ASSIGN_BLK + e;
+      }
+    }
+    const long long row = t * T + tid;
+    assign_unsure<D>(__ballot_sync(0xffffffffu, !sure && row < m), w, cs, k, lane, bj);
+    if (row < m) {
+      if (codes != nullptr) codes[row] = (unsigned char)bj;
+      if (Wq != nullptr) reinterpret_cast<float4*>(Wq)[row] = *reinterpret_cast<const float4*>(cs + bj * 4);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols));
+}
 
 // Scalar weights, larger codebooks: the codebook is sorted once per block (by counting), a weight finds its place in it by
 // bisection.  Rounding keeps the order of the differences and of their squares, so the smallest square is that of one of the
@@ -360,12 +573,15 @@ __global__ void __launch_bounds__(ASSIGN_BLOCK) idkm_assign_search(const float* 
 }
 // (m = 10 M: k = 32 74 against 78 us for the kernel that compares with every centroid, k = 64 131 against 78, k = 256 474 against 90)
 constexpr int ASSIGN_SEARCH_MIN_K = 33;
+// (m = 2.5 M, d = 4: k = 32 46 against 42 us for the scores on the CUDA cores, k = 64 51 against 58, k = 100 63 against 81, k = 256 106
+// against 164; 20 K: 17 against 17.  At d = 2, k = 256, 5 M: 203 against 219, k = 64 81 against 75: not taken)
+constexpr int ASSIGN_MMA_MIN_K = 48;
 
 
 int code_bits(int k) { return k <= 2 ? 1 : (k <= 4 ? 2 : (k <= 16 ? 4 : 8)); }
 
 template <int D, int BITS>
-void launch_bits(int grid, cudaStream_t st, const float* W, long long m, const float* C, int k, unsigned char* codes, float* Wq) {
+void launch_bits(int grid, int grid_max, cudaStream_t st, const float* W, long long m, const float* C, int k, unsigned char* codes, float* Wq) {
   if constexpr (D == 1 && BITS == 8) {
     if (k >= ASSIGN_SEARCH_MIN_K) {
       idkm_assign_search<BITS><<<grid, ASSIGN_BLOCK, 0, st>>>(W, m, C, k, codes, Wq);
@@ -373,6 +589,18 @@ void launch_bits(int grid, cudaStream_t st, const float* W, long long m, const f
     }
   }
   if constexpr (D > 1 && BITS == 8) {
+    if constexpr (D == 4) {
+      if (k >= ASSIGN_MMA_MIN_K) {
+        const int cols = k <= 64 ? 64 : (k <= 128 ? 128 : 256), per_sm = cols == 256 ? 2 : 4;
+        const int smem = 180 * 1024 / per_sm;   // (no more blocks on an SM than it has tensor memory for)
+        static bool configured = false;
+        if (!configured) configured = cudaFuncSetAttribute(idkm_assign_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, 90 * 1024) == cudaSuccess;
+        const long long tiles = (m + ASSIGN_MMA_T - 1) / ASSIGN_MMA_T;
+        const long long most = (long long)(grid_max / 8) * per_sm;
+        idkm_assign_mma<<<(int)(tiles < most ? tiles : most), ASSIGN_MMA_T, smem, st>>>(W, m, C, k, codes, Wq, cols);
+        return;
+      }
+    }
     if (k >= ASSIGN_SCORE_MIN_K) {
       idkm_assign_score<D, BITS><<<grid, ASSIGN_BLOCK, 0, st>>>(W, m, C, k, codes, Wq);
       return;
@@ -381,13 +609,13 @@ void launch_bits(int grid, cudaStream_t st, const float* W, long long m, const f
   idkm_assign_kernel<D, BITS><<<grid, ASSIGN_BLOCK, 0, st>>>(W, m, C, k, codes, Wq);
 }
 template <int D>
-cudaError_t launch_assign(int bits, int grid, cudaStream_t st, const float* W, long long m, const float* C, int k,
+cudaError_t launch_assign(int bits, int grid, int grid_max, cudaStream_t st, const float* W, long long m, const float* C, int k,
                           unsigned char* codes, float* Wq) {
   switch (bits) {
-    case 1: launch_bits<D, 1>(grid, st, W, m, C, k, codes, Wq); break;
-    case 2: launch_bits<D, 2>(grid, st, W, m, C, k, codes, Wq); break;
-    case 4: launch_bits<D, 4>(grid, st, W, m, C, k, codes, Wq); break;
-    default: launch_bits<D, 8>(grid, st, W, m, C, k, codes, Wq); break;
+    case 1: launch_bits<D, 1>(grid, grid_max, st, W, m, C, k, codes, Wq); break;
+    case 2: launch_bits<D, 2>(grid, grid_max, st, W, m, C, k, codes, Wq); break;
+    case 4: launch_bits<D, 4>(grid, grid_max, st, W, m, C, k, codes, Wq); break;
+    default: launch_bits<D, 8>(grid, grid_max, st, W, m, C, k, codes, Wq); break;
   }
   return cudaGetLastError();
 }
@@ -418,8 +646,8 @@ extern "C" int idkm_assign(const float* W, int64_t m, int d, const float* C, int
   if (grid > (long long)sms * 8) grid = (long long)sms * 8;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   cudaError_t rc;
-  if (d == 1) rc = launch_assign<1>(bits, (int)grid, st, W, m, C, k, codes_out, Wq_out);
-  else if (d == 2) rc = launch_assign<2>(bits, (int)grid, st, W, m, C, k, codes_out, Wq_out);
-  else rc = launch_assign<4>(bits, (int)grid, st, W, m, C, k, codes_out, Wq_out);
+  if (d == 1) rc = launch_assign<1>(bits, (int)grid, sms * 8, st, W, m, C, k, codes_out, Wq_out);
+  else if (d == 2) rc = launch_assign<2>(bits, (int)grid, sms * 8, st, W, m, C, k, codes_out, Wq_out);
+  else rc = launch_assign<4>(bits, (int)grid, sms * 8, st, W, m, C, k, codes_out, Wq_out);
   return rc == cudaSuccess ? IDKM_OK : IDKM_ERR_CUDA;
 }
