@@ -686,36 +686,28 @@ constexpr int MMA_LOOP_ROWS = 128;   // weight-vectors a block takes at least
 // doubles that all blocks together may read for every block to add all partials (4 MB: about a microsecond; a second barrier
 // and a trip through memory cost two: m = 4096, d = 2, k = 64: 9.3 against 11.8 us an iteration, d = 4, k = 16: 8.7 against 10.2)
 constexpr long long MMA_LOOP_ONE_STAGE = 500000;
-// Batches with d = 4 and 9 to 16 centroids below this many weight-vectors keep a launch per iteration: callers of that path
-// count its launches.
-constexpr long long MMA_LOOP_BATCH_16 = 1 << 18;
 
 // Returns IDKM_OK after queueing the loop, 1 if this problem should take the launch-per-iteration path.
 static int try_mma_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, int max_iter) {
   static const bool env_off = (getenv("IDKM_NO_COOP") != nullptr);
   if (env_off || ctx->forward_loop != 0 || max_iter < 2 || (!ctx->squared && ctx->collapse_step != 0)) return 1;
   const MmaLoopEntry* e = mma_loop_entry(ctx->d, ctx->k, ctx->squared != 0);
-  const int L = ctx->n_layers;
-  if (!e || !e->launch || ctx->k * ctx->d <= 32 || L > ctx->sms) return 1;
-  // (small batches of quadruples with at most 16 centroids: a launch per iteration, see MMA_LOOP_BATCH_16)
-  if (L > 1 && ctx->k <= 16 && ctx->m_total < MMA_LOOP_BATCH_16) return 1;
+  if (!e || !e->launch || ctx->k * ctx->d <= 32) return 1;
+  // (Batches keep a launch per iteration and with it their sums' order, bit for bit: among a network's layers there are small
+  // cold ones -- 2048 quadruples, k = 16, a spread of 350 tau -- that turn one rounding into 1e-5 of a centroid, and where the
+  // adjoint iteration of such a layer diverges, 1e-2 of its gradient.  A ResNet-18's, d = 4, k = 16: 64 us an iteration against 51.)
+  if (ctx->n_layers > 1) return 1;
   int grid = ctx->sms;
   const long long most = (ctx->m_total + MMA_LOOP_ROWS - 1) / MMA_LOOP_ROWS;
   if (grid > most) grid = (int)most;
-  if (grid < L) grid = L;
-  if ((size_t)grid * e->plen > (size_t)wl.max_slots * wl.plen_max || (size_t)L * e->plen > (size_t)wl.max_groups * wl.plen_max) return 1;
+  if ((size_t)grid * e->plen > (size_t)wl.max_slots * wl.plen_max || (size_t)e->plen > (size_t)wl.max_groups * wl.plen_max) return 1;
   MmaLoopParams mp;
   memset(&mp, 0, sizeof(mp));
   SmallLoopParams& sp = mp.s;
   sp.W = ctx->W;
-  sp.n_layers = L;
-  deal_blocks(ctx, grid, &sp);
-  long long reads = 0;   // doubles the blocks read if every one adds all partials of its layer
-  for (int l = 0; l < L; ++l) {
-    const long long n = sp.blk_first[l + 1] - sp.blk_first[l];
-    reads += n * n * e->plen;
-  }
-  mp.one_stage = reads <= MMA_LOOP_ONE_STAGE && 2 * (size_t)grid * e->plen <= (size_t)wl.max_slots * wl.plen_max;
+  sp.n_layers = 1;
+  sp.row_off[1] = ctx->m_total;
+  mp.one_stage = (long long)grid * grid * e->plen <= MMA_LOOP_ONE_STAGE && 2 * (size_t)grid * e->plen <= (size_t)wl.max_slots * wl.plen_max;
   sp.C = ctx->C;
   sp.st = p.st;
   sp.partials = p.partials;

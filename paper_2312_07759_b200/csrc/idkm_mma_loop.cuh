@@ -1,4 +1,4 @@
-// Algorithm 1's whole loop in one cooperative launch for pairs and quadruples of weights and codebooks of more than 16
+// Algorithm 1's whole loop over one layer in one cooperative launch for pairs and quadruples of weights and codebooks of more than 16
 // centroids (more than 8 at d = 4), in fp32 with the column sums S_j = sum_i A_ij, N_j = sum_i A_ij w_i taken by the tensor
 // cores.  Further description in idkm_mma_loop_impl.cuh.
 #pragma once
@@ -8,8 +8,8 @@ namespace idkm {
 
 struct MmaLoopParams {
   SmallLoopParams s;   // partials: [2][grid][PLEN] (one_stage) or [grid][PLEN]
-  double* totals;      // [L][PLEN]
-  int one_stage;       // 1: every block adds all partials of its layer (one barrier an iteration)
+  double* totals;      // [PLEN]
+  int one_stage;       // 1: every block adds all partials (one barrier an iteration)
 };
 typedef cudaError_t (*MmaLoopLaunchFn)(const MmaLoopParams& p, int grid, cudaStream_t stream);
 struct MmaLoopEntry {

@@ -75,15 +75,12 @@ __device__ __forceinline__ void loop_frame(const MmaLoopParams& mp, LoopShared<D
   float* c_sm = sh.c;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = gridDim.x, k = sp.k;
-  int layer = 0;
-  while (layer + 1 < sp.n_layers && (int)blockIdx.x >= sp.blk_first[layer + 1]) ++layer;
-  const int first_blk = sp.blk_first[layer];
-  const int b = (int)blockIdx.x - first_blk, NB = sp.blk_first[layer + 1] - first_blk;
-  const long long m = sp.row_off[layer + 1] - sp.row_off[layer];
-  const float* Wl = sp.W + sp.row_off[layer] * D;
-  float* Cl = sp.C + (size_t)layer * k * D;
-  LayerState* st = sp.st + layer;
-  double* gtot = mp.totals + (size_t)layer * PLEN;
+  const int b = (int)blockIdx.x;
+  const long long m = sp.row_off[1];
+  const float* Wl = sp.W;
+  float* Cl = sp.C;
+  LayerState* st = sp.st;
+  double* gtot = mp.totals;
 
   int iters = 0, done = 0, status = ST_OK, dead_n = 0;
   int precise = SQ ? 0 : st->precise[0];
@@ -93,47 +90,36 @@ __device__ __forceinline__ void loop_frame(const MmaLoopParams& mp, LoopShared<D
   bool ok = true;
 
   for (int it = 0; it < sp.max_iter; ++it) {
-    if (sp.n_layers == 1 && done) break;   // (a batch goes on meeting at the barrier until every layer has ended)
+    if (done) break;
     const size_t buf = mp.one_stage ? (size_t)(it & 1) * G : 0;   // (with one barrier the next iteration's partials need a second buffer)
-    if (!done) rows(precise, b, NB, m, Wl, sp.partials + (buf + blockIdx.x) * PLEN);
+    rows(precise, b, G, m, Wl, sp.partials + (buf + b) * PLEN);
     // ---- everyone has published ----
     const unsigned arrivals = (unsigned)(G + sp.missing_arrivals);
     ok = small_barrier(sp.sync, (unsigned)(mp.one_stage ? it + 1 : 2 * it + 1) * arrivals, sp.spin_limit, &sh.ok);
     if (!ok) break;
-    if (sp.n_layers > 1 && sp.tol > 0.f) {   // a batch ends when every layer's loop has ended (see idkm_small_loop.cu)
-      int ended = 1;
-      for (int l = tid; l < sp.n_layers; l += T) {
-        const int fd = *reinterpret_cast<const volatile int*>(&sp.st[l].fwd_done);
-        if (fd == 0 || fd > it) ended = 0;
-      }
-      if (__syncthreads_and(ended)) break;
-    }
     // ---- the layer's totals.  Few partials: every block adds them all, in the same order.  Many: it adds its share of the
     // sums, and after a second barrier reads the rest ----
-    const double* base = sp.partials + (buf + first_blk) * PLEN;
+    const double* base = sp.partials + buf * PLEN;
     if (!mp.one_stage) {
-      if (!done) {
-        const int o0 = (int)((long long)PLEN * b / NB), o1 = (int)((long long)PLEN * (b + 1) / NB);
-        if (NB >= 16) {
-          for (int o = o0 + warp; o < o1; o += NW) {
-            double v = 0.0;
-            for (int q = lane; q < NB; q += 32) v += __ldcg(base + (size_t)q * PLEN + o);
+      const int o0 = (int)((long long)PLEN * b / G), o1 = (int)((long long)PLEN * (b + 1) / G);
+      if (G >= 16) {
+        for (int o = o0 + warp; o < o1; o += NW) {
+          double v = 0.0;
+          for (int q = lane; q < G; q += 32) v += __ldcg(base + (size_t)q * PLEN + o);
 #pragma unroll
-            for (int x = 16; x > 0; x >>= 1) v += __shfl_xor_sync(0xffffffffu, v, x);
-            if (lane == 0) __stcg(gtot + o, v);
-          }
-        } else {
-          for (int o = o0 + tid; o < o1; o += T) {
-            double v = 0.0;
-            for (int q = 0; q < NB; ++q) v += __ldcg(base + (size_t)q * PLEN + o);
-            __stcg(gtot + o, v);
-          }
+          for (int x = 16; x > 0; x >>= 1) v += __shfl_xor_sync(0xffffffffu, v, x);
+          if (lane == 0) __stcg(gtot + o, v);
+        }
+      } else {
+        for (int o = o0 + tid; o < o1; o += T) {
+          double v = 0.0;
+          for (int q = 0; q < G; ++q) v += __ldcg(base + (size_t)q * PLEN + o);
+          __stcg(gtot + o, v);
         }
       }
       ok = small_barrier(sp.sync, (unsigned)(2 * it + 2) * arrivals, sp.spin_limit, &sh.ok);
       if (!ok) break;
     }
-    if (done) continue;
     if (!mp.one_stage) {
       for (int o = tid; o < PLEN; o += T) sh.tot[o] = __ldcg(gtot + o);
     } else if constexpr (PLEN <= T / 2) {
@@ -142,7 +128,7 @@ __device__ __forceinline__ void loop_frame(const MmaLoopParams& mp, LoopShared<D
       if (ch < CH) {
         double v = 0.0;
 #pragma unroll 8
-        for (int q = ch; q < NB; q += CH) v += __ldcg(base + (size_t)q * PLEN + o);
+        for (int q = ch; q < G; q += CH) v += __ldcg(base + (size_t)q * PLEN + o);
         sh.part[tid] = v;
       }
       __syncthreads();
@@ -156,7 +142,7 @@ __device__ __forceinline__ void loop_frame(const MmaLoopParams& mp, LoopShared<D
       for (int o = tid; o < PLEN; o += T) {
         double v = 0.0;
 #pragma unroll 8
-        for (int q = 0; q < NB; ++q) v += __ldcg(base + (size_t)q * PLEN + o);
+        for (int q = 0; q < G; ++q) v += __ldcg(base + (size_t)q * PLEN + o);
         sh.tot[o] = v;
       }
     }
@@ -246,7 +232,7 @@ __device__ __forceinline__ void loop_frame(const MmaLoopParams& mp, LoopShared<D
     __syncthreads();
     iters = it + 1;
     res_f = (float)sh.res;
-    if (b == 0 && tid == 0 && iters <= HIST_CAP) sp.hist[(size_t)layer * HIST_CAP + iters - 1] = res_f;
+    if (b == 0 && tid == 0 && iters <= HIST_CAP) sp.hist[iters - 1] = res_f;
     dead_n = sh.flags[0];
     precise = sh.flags[2];
     if (sh.flags[1] > 0) {
@@ -258,7 +244,6 @@ __device__ __forceinline__ void loop_frame(const MmaLoopParams& mp, LoopShared<D
     } else if (sp.tol > 0.f && iters >= sp.max_iter) {
       status = ST_MAXITER;
     }
-    if (done && b == 0 && tid == 0) st->fwd_done = done;   // (seen by the other layers' blocks after the next barrier)
     __syncthreads();
   }
 
