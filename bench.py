@@ -356,7 +356,7 @@ def main():
             r = {"bound": "alu", "achieved": pairs * sfu_ops / sec / 1e12, "peak": sfu_peak / 1e12,
                  "unit": "Tinst-lanes/s (sfu pipe)", "peak_source": "148 SMs x 16 sfu lanes/clk x 1965 MHz"}
         r["frac"] = r["achieved"] / r["peak"]
-        r["kernel"] = f"{label}, layout {layout[0]} centroids/lane x {layout[1]} lanes/weight"
+        r["kernel"] = f"{label}, layout {layout[0]} centroids/lane x {layout[1]} lanes/weight" if layout else label
         r["kernel_ms"] = kernel_ms
         r["share_of_step"] = share
         r["roofline_ms"] = max(t_hbm, t_fp32, t_sfu) * 1e3
@@ -365,12 +365,15 @@ def main():
         # dram__bytes_read.sum + dram__bytes_write.sum of one launch from the stored ncu capture of this kernel (ncu
         # flushes the caches before the launch, so this is the cold-L2 figure); null when none is stored for this
         # workload and layout, or when the kernel source has changed since the capture
-        r["traffic"] = traffic_table.get(f"{label.split(' ')[0]}:{layout[0]}x{layout[1]}")
+        r["traffic"] = traffic_table.get(f"{label.split(' ')[0]}:{layout[0]}x{layout[1]}") if layout else None
         r["frac_of_measured_pipes"] = max(t_hbm, pairs * fp32_ops / fp32_rate, pairs * sfu_ops / sfu_rate) / sec
         return r
 
     step_total = float(np.mean(step_ms))
-    roof_step = kernel_roofline("idkm_pass<STEP> (fused forward step)", path["step_layout"], step_kernel_ms, pair_ops(d),
+    # (single layers with larger codebooks run the whole loop in one launch: the time of one of its iterations)
+    one_launch = L == 1 and (d == 4 and k > 8 or d == 2 and k > 16)
+    roof_step = kernel_roofline("forward loop in one launch (one iteration)" if one_launch else "idkm_pass<STEP> (fused forward step)",
+                                None if one_launch else path["step_layout"], step_kernel_ms, pair_ops(d),
                                 ph["steps"] / step_total, 4.0 * d) if T_f > 0 and step_kernel_ms > 0 else None
     roof_adj = None
     if T_a > 0 and adj_kernel_ms > 0 and path["adjoint_route"] == "fused passes":

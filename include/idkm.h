@@ -156,9 +156,11 @@ int idkm_get_history(idkm_ctx* ctx, int which, int layer, float* host_out, int c
  * copies W, C0 and dWq to the device, runs idkm_forward_batched and idkm_backward, and copies
  * C, Wq, dW, dC back; returns after everything has completed.  Device buffers are allocated on
  * first use, kept in the ctx and grown on demand (with idkm_quantize_host_ex the only entry point that
- * allocates device memory); the work runs on two streams of the ctx's own, so that the upload of dWq
+ * allocates device memory); the work runs on three streams of the ctx's own, so that the upload of dWq
  * overlaps the forward loop and the download of C and Wq overlaps the backward (host buffers must be
- * page-locked for the overlap to happen; pageable buffers work, serially).
+ * page-locked for the overlap to happen; pageable buffers work, serially).  With 24 MB of weights or more
+ * the layers are taken in up to four groups of consecutive layers, each clustered while the next group's
+ * weights come in and the last group's results go out (not while phase times are recorded).
  * Any of Wq_out, dW_out, dC_out may be NULL; info_out (n_layers entries) too.
  * layer_offsets as in idkm_forward_batched (pass {0, m} and n_layers = 1 for one layer).
  */
@@ -231,11 +233,13 @@ int idkm_step_noalloc(const float* W, int64_t m, int d, const float* C_in, int k
 int idkm_step_noalloc_status(int* status_host_out, void* cuda_stream);
 
 /*
- * How IDKM_IMPLICIT runs the adjoint iteration.  0 (default): where k d <= 64 one pass over W forms the k d x k d
- * matrix dF/dC explicitly and the whole iteration u <- alpha (J^T u + g) + (1 - alpha) u then runs on that matrix on
- * the device -- the paper's own formulation (it iterates a k x k matrix, Section 4.2), same iterates, one pass
- * instead of adj_max_iter.  For k d <= 8 always; for 8 < k d <= 64 (the pass costs about ten fused passes) when
- * adj_max_iter >= 16.  Larger codebooks, and shorter iterations, use one fused vector-Jacobian pass per step.
+ * How IDKM_IMPLICIT runs the adjoint iteration.  0 (default): one pass over W forms the k d x k d matrix dF/dC
+ * explicitly and the whole iteration u <- alpha (J^T u + g) + (1 - alpha) u then runs on that matrix on the device --
+ * the paper's own formulation (it iterates a k x k matrix, Section 4.2), same iterates, one pass instead of
+ * adj_max_iter.  For k d <= 8 always; for 8 < k d <= 64 and k <= 8 (or where the interval form did not run) when
+ * adj_max_iter >= 16; for d = 2 or 4, Euclidean distance and k > 8 on the tensor cores when adj_max_iter is at least 8
+ * (k d <= 64), else 20 or k d^2 / 128; after an interval-form forward (d = 1) the matrix comes from interval sums, without
+ * a pass.  Other codebooks, and shorter iterations, use one fused vector-Jacobian pass per step.
  * 1: always the fused passes.
  * 2: no iteration where the matrix can be formed (k d <= 64): the same pass forms dF/dC and one warp then solves
  * (I - (dF/dC)^T) u = g exactly -- the system behind M* = (I - dF/dC)^-1 of Section 4.2 -- by Gaussian elimination
@@ -317,8 +321,11 @@ int idkm_measure_pipe_rates(double* fp32_lane_ops_per_s, double* sfu_lane_ops_pe
  * block then adds its layer's partials in the same order and takes the M-step itself, so only the partials cross L2
  * inside the loop.  A layer leaves the loop at the iteration whose stop test passes; a batch leaves at the first
  * barrier at which every layer has.  Layers that collapse on the way step in the fp32 increment form (see
- * idkm_set_collapse_step).  Everything else (larger layers, batches or codebooks, max_iter < 2, the squared
- * distance, the fp64 step for collapsing layers) takes one launch per iteration.  Every barrier wait is bounded
+ * idkm_set_collapse_step).  Scalar weights (d = 1, Euclidean distance, either Wq_out given or k > 16) of any size and
+ * number of layers up to the number of multiprocessors take the interval form instead: the weights are summarised once
+ * in bins with moments, and an iteration works on the bins.  Single layers with d = 2 and k > 16, or d = 4 and k > 8,
+ * of any size and either distance, have a one-launch loop of their own.  Everything else (larger layers of small
+ * codebooks, other batches, max_iter < 2, the fp64 step for collapsing layers) takes one launch per iteration.  Every barrier wait is bounded
  * (about a second): if one runs out the kernel returns and the status of the layer (of every layer of a batch) is
  * IDKM_ERR_TIMEOUT.  1: always one launch per iteration
  * (for the smallest codebooks -- k <= 4 at d = 1, k <= 2 at d = 2 -- that launch is a kernel that steps the fp32 and

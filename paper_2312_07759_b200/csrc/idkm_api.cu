@@ -812,6 +812,12 @@ static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassP
   if (wl.sc_fine == 0 || ctx->squared || ctx->forward_loop != 0 || ctx->collapse_step != 0 || max_iter < 2 || scratch == nullptr ||
       ctx->n_layers > ctx->sms)
     return 1;
+  // Few weights and a cold softmax: the bins are nearly as many as the weights, and summarising them costs more than the
+  // iterations save.  (The weights' spread is not known here; it is of the order of 0.05.  30 iterations and the Jacobian-free
+  // backward, spread 0.03, one-launch loop over the weights against this one: m = 4096, k = 4: tau = 0.05 128 against 115 us,
+  // 0.01 103 against 119, 5e-4 104 against 146; m = 8192, k = 16: 5e-4 185 against 222, 2e-3 faster here.)
+  const bool cold = (ctx->m_total <= 4096 && ctx->k <= 4 && ctx->tau < 0.03f) || (ctx->m_total <= 16384 && ctx->k <= 16 && ctx->tau < 1e-3f);
+  if (ctx->n_layers == 1 && cold) return 1;
   for (int l = 0; l < ctx->n_layers; ++l)
     if (ctx->row_off[l + 1] - ctx->row_off[l] > 0x7fffffffLL) return 1;
   ScalarParams sp;

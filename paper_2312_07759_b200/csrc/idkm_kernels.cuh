@@ -769,7 +769,7 @@ __device__ __forceinline__ void pass_body(const PassParams& p) {
     }
   };
   int since_spill = 0;
-  constexpr bool WMAX = (MODE == FINAL && D > 1);
+  constexpr bool WMAX = (MODE == FINAL && D > 1 && !SQ && Cfg::KP > 8);   // (what the tensor-core Jacobian can follow)
   float wmax = 0.f;   // largest |coordinate| of the layer's rows seen by this thread
   (void)wmax;
   auto spill = [&]() {
