@@ -11,6 +11,13 @@
 // grouped by fine bin (two bytes per weight).  Everything that is accumulated in an order that can vary is a sum of
 // integers, so results are reproducible although the grouping uses atomic counters.
 //
+// What bounds it.  Building: the grouping pass stores two bytes per weight to scattered places, 67 cycles a warp store
+// (110 us per 11.7 M weights on all SMs).  Iterating: the chain of one block a layer -- evaluate, sum, M-step, four meetings of
+// the block -- 2.6 us at k <= 4 to 6 us, whatever the number of weights.  Measured, loop with the summary against one that
+// visits the pairs: 21 layers of a ResNet-18, k = 4, 50 iterations 382 against 1473 us; k = 8, tau = 5e-4, 30 iterations 366
+// against 1268; 16 M weights, k = 16, 100 iterations 1.42 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 101
+// against 112.
+//
 // Several blocks per layer build the summary (meetings at a bounded barrier), then one block per layer runs the
 // iterations: one warp (or a few) per interval between centroids, the M-step by the first warps in fp64.
 #include "idkm_scalar.cuh"

@@ -1,6 +1,10 @@
 // The passes around the loop for scalar weights: soft-quantised weights, codebook gradient, adjoint iteration and dL/dW,
 // all in the interval form of idkm_scalar.cuh.  A weight costs a search for its interval, one exponential and one
 // reciprocal whatever the number of centroids; the adjoint iteration (Section 4.2) does not visit the weights at all.
+// Bound by memory and the search's shared-memory lookups.  Measured (soft weights / gradient / dL/dW against the passes over
+// pairs): 11.7 M weights, k = 4 38 / 56 / 46 us against 48 / 54 / 56; k = 8 43 / 61 / 49 against 75 / 95 / 101; 16 M, k = 16
+// 63 / 80 / 72 against 152 / 234 / 244.  Adjoint iteration of 50 steps, 21 layers, k = 4: 26 us against 104 on a matrix that a
+// pass over the weights forms.
 #include "idkm_scalar.cuh"
 
 namespace idkm {
