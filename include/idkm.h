@@ -100,7 +100,9 @@ size_t idkm_workspace_bytes(int64_t m_total, int d, int k, int n_layers);
  * writes Wq = A C (Wq_out, may be NULL), optionally A itself (A_out, may be NULL: m*k floats, the
  * paper's O(m 2^b) term), and stashes S_j = sum_i A_ij and F(C, W)_j in the workspace.
  *
- * C_out receives the last C+ ("return C+", Algorithm 1).  C0 and C_out may alias.
+ * C_out receives the last C+ ("return C+", Algorithm 1).  C0 and C_out may alias.  Wq_out is written from the start of
+ * the call (for d = 1 the loop keeps intermediate results there), not only by the final pass.  Wq_out = W overwrites the
+ * weights when the loop has ended; nothing but another forward can follow such a call, since the backward reads W.
  */
 int idkm_forward(idkm_ctx* ctx, const float* W, int64_t m, int d, const float* C0, int k, float tau, float tol,
                  int max_iter, float* C_out, float* A_out, float* Wq_out, void* workspace, size_t workspace_bytes,

@@ -368,6 +368,10 @@ static void mark(idkm_ctx* ctx, int i) {
   if (ctx->timing && ctx->ev_ok) cudaEventRecord(ctx->ev[i], ctx->stream);
 }
 
+static bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + b_bytes && y < x + a_bytes;
+}
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // The kernel that runs a pass for this ctx: the squared-distance variant of the fused passes when the ctx asks for it.
@@ -1042,9 +1046,11 @@ int idkm_forward_batched(idkm_ctx* ctx, const float* W_cat, const int64_t* layer
   mark(ctx, 0);
   nvtxRangePushA("idkm forward loop");
   ctx->scalar_forward = false;
-  // scratch of the interval form: the buffer of Wq, which the final pass overwrites; without Wq the row cache of the
-  // backward, if there is one and no other one-launch loop takes the codebook
-  void* scratch = Wq_out ? static_cast<void*>(Wq_out) : (k > 16 ? static_cast<void*>(p.rowstat) : nullptr);
+  // scratch of the interval form: the buffer of Wq, which the final pass overwrites, unless it overlaps the weights, which
+  // the loop still reads; otherwise the row cache of the backward, if there is one and no other one-launch loop takes the codebook
+  const size_t w_bytes = sizeof(float) * (size_t)m_total * d, wq_bytes = ctx->wq_dtype == 0 ? w_bytes : w_bytes / 2;
+  const bool own_wq = Wq_out && !overlap(W_cat, w_bytes, Wq_out, wq_bytes);
+  void* scratch = own_wq ? static_cast<void*>(Wq_out) : (k > 16 ? static_cast<void*>(p.rowstat) : nullptr);
   int rc = try_scalar_loop(ctx, wl, p, C0, max_iter, scratch);
   if (rc == 1) {
     char* wsb = static_cast<char*>(workspace);
