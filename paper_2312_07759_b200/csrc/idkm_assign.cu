@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include "idkm_per_device.h"
 #include "../../include/idkm.h"
 
 namespace {
@@ -593,12 +594,14 @@ void launch_bits(int grid, int grid_max, cudaStream_t st, const float* W, long l
       if (k >= ASSIGN_MMA_MIN_K) {
         const int cols = k <= 64 ? 64 : (k <= 128 ? 128 : 256), per_sm = cols == 256 ? 2 : 4;
         const int smem = 180 * 1024 / per_sm;   // (no more blocks on an SM than it has tensor memory for)
-        static bool configured = false;
-        if (!configured) configured = cudaFuncSetAttribute(idkm_assign_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, 90 * 1024) == cudaSuccess;
+        static idkm::PerDevice limit;
         const long long tiles = (m + ASSIGN_MMA_T - 1) / ASSIGN_MMA_T;
         const long long most = (long long)(grid_max / 8) * per_sm;
-        idkm_assign_mma<<<(int)(tiles < most ? tiles : most), ASSIGN_MMA_T, smem, st>>>(W, m, C, k, codes, Wq, cols);
-        return;
+        if (idkm::allow_smem(limit, idkm_assign_mma, 90 * 1024) == cudaSuccess) {   // (otherwise the scores on the CUDA cores)
+          idkm_assign_mma<<<(int)(tiles < most ? tiles : most), ASSIGN_MMA_T, smem, st>>>(W, m, C, k, codes, Wq, cols);
+          return;
+        }
+        (void)cudaGetLastError();
       }
     }
     if (k >= ASSIGN_SCORE_MIN_K) {

@@ -31,13 +31,9 @@ static cudaError_t launch_pdl(Kernel kernel, const PassParams& p, int grid, int 
 template <int MODE, int D, int KPL, int LPW, bool SQ>
 static cudaError_t launch_one(const PassParams& p, int grid, cudaStream_t stream) {
   constexpr int DYN = PassCfg<MODE, D, KPL, LPW>::DYN_SMEM;
-  static bool configured = false;   // static + dynamic shared memory may exceed the 48 KB default
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_pass<MODE, D, KPL, LPW, SQ>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, DYN > 0 ? DYN : 1);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;   // static + dynamic shared memory may exceed the 48 KB default
+  const cudaError_t allowed = allow_smem(limit, idkm_pass<MODE, D, KPL, LPW, SQ>, DYN > 0 ? DYN : 1);
+  if (allowed != cudaSuccess) return allowed;
   return launch_pdl(idkm_pass<MODE, D, KPL, LPW, SQ>, p, grid, DYN, stream);
 }
 
@@ -68,13 +64,9 @@ template <int D, int KPL>
 static cudaError_t launch_step_bulk(const PassParams& p, int grid, cudaStream_t stream) {
   using Cfg = PassCfg<STEP, D, KPL, 1>;
   constexpr int DYN = Cfg::DYN_SMEM + BULK_STAGES * Cfg::UNROLL * BLOCK * 16;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_pass<STEP, D, KPL, 1, false, true>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_pass<STEP, D, KPL, 1, false, true>, DYN);
+  if (allowed != cudaSuccess) return allowed;
   return launch_pdl(idkm_pass<STEP, D, KPL, 1, false, true>, p, grid, DYN, stream);
 }
 #define IDKM_BULK_ENTRY(D, KPL)                                                                              \

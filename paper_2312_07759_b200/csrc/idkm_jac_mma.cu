@@ -910,16 +910,15 @@ int jac_mma_groups_max(int n_layers) { return (JM_UNITS + n_layers) / JM_RED + n
 template <int D, int NT, bool PACK>
 static cudaError_t launch_mma(const JacMmaParams& p, int units, cudaStream_t stream) {
   constexpr int DYN = JmCfg<D, NT, PACK>::DYN;
-  static bool configured = false;
-  if (!configured) {
+  static PerDevice shares, limit;
+  // (the warps' shares of the registers have to add up)
+  cudaError_t rc = shares.once(0, [] {
     cudaFuncAttributes at;
-    cudaError_t rc = cudaFuncGetAttributes(&at, idkm_jac_mma<D, NT, PACK>);
-    if (rc != cudaSuccess) return rc;
-    if (at.numRegs != JM_LAUNCH_REGS) return cudaErrorInvalidConfiguration;   // (the warps' shares would not add up)
-    rc = cudaFuncSetAttribute(idkm_jac_mma<D, NT, PACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+    const cudaError_t got = cudaFuncGetAttributes(&at, idkm_jac_mma<D, NT, PACK>);
+    return got != cudaSuccess ? got : (at.numRegs == JM_LAUNCH_REGS ? cudaSuccess : cudaErrorInvalidConfiguration);
+  });
+  if (rc == cudaSuccess) rc = allow_smem(limit, idkm_jac_mma<D, NT, PACK>, DYN);
+  if (rc != cudaSuccess) return rc;
   idkm_jac_mma<D, NT, PACK><<<units, JM_THREADS, DYN, stream>>>(p);
   return cudaGetLastError();
 }
@@ -931,12 +930,9 @@ cudaError_t launch_jac_mma(int d, const JacMmaPlan& pl, const JacMmaParams& p, i
 template <int D, int NT>
 static cudaError_t launch_solve(const JacMmaPlan& pl, const JacMmaParams& p, cudaStream_t stream) {
   const int smem = (JS_ROWS + 1) * pl.kdp * 8;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_jac_solve<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (JS_ROWS + 1) * 1024 * 8);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_jac_solve<D, NT>, (JS_ROWS + 1) * 1024 * 8);
+  if (allowed != cudaSuccess) return allowed;
   void* args[1] = {const_cast<JacMmaParams*>(&p)};
   return cudaLaunchCooperativeKernel((const void*)&idkm_jac_solve<D, NT>, dim3((unsigned)(p.n_layers * p.solve_blocks), 1, 1), dim3(JS_T, 1, 1),
                                      args, (size_t)smem, stream);

@@ -18,6 +18,8 @@
 #include <stdint.h>
 #include <type_traits>
 
+#include "idkm_per_device.h"
+
 namespace idkm {
 
 constexpr int BLOCK = 256;

@@ -717,12 +717,9 @@ __global__ void __launch_bounds__(GrpCfg<D, KPL, LPW>::T, 1) idkm_group_loop(con
 template <int D, int KPL, int LPW, bool SQ>
 static cudaError_t launch_group_loop(const MmaLoopParams& p, int grid, cudaStream_t stream) {
   using Cfg = GrpCfg<D, KPL, LPW>;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_group_loop<D, KPL, LPW, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_group_loop<D, KPL, LPW, SQ>, Cfg::DYN);
+  if (allowed != cudaSuccess) return allowed;
   void* args[1] = {const_cast<MmaLoopParams*>(&p)};
   return cudaLaunchCooperativeKernel((const void*)&idkm_group_loop<D, KPL, LPW, SQ>, dim3((unsigned)grid, 1, 1), dim3(Cfg::T, 1, 1), args,
                                      (size_t)Cfg::DYN, stream);
@@ -732,12 +729,9 @@ static cudaError_t launch_group_loop(const MmaLoopParams& p, int grid, cudaStrea
 template <int MT, bool SQ>
 static cudaError_t launch_mma_loop(const MmaLoopParams& p, int grid, cudaStream_t stream) {
   using Cfg = MmlCfg<MT>;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_mma_loop<MT, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_mma_loop<MT, SQ>, Cfg::DYN);
+  if (allowed != cudaSuccess) return allowed;
   void* args[1] = {const_cast<MmaLoopParams*>(&p)};
   // cooperative launch: refused (instead of hanging at the first barrier) if the grid cannot be co-resident
   return cudaLaunchCooperativeKernel((const void*)&idkm_mma_loop<MT, SQ>, dim3((unsigned)grid, 1, 1), dim3(Cfg::T, 1, 1), args,

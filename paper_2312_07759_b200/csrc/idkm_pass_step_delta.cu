@@ -5,12 +5,9 @@ namespace idkm {
 template <int D, int KPL, int LPW>
 static cudaError_t launch_delta(const PassParams& p, int grid, cudaStream_t stream) {
   constexpr int DYN = DeltaCfg<D, KPL, LPW>::DYN_SMEM;
-  static bool configured = false;   // static + dynamic shared memory may exceed the 48 KB default
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_step_delta<D, KPL, LPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;   // static + dynamic shared memory may exceed the 48 KB default
+  const cudaError_t allowed = allow_smem(limit, idkm_step_delta<D, KPL, LPW>, DYN);
+  if (allowed != cudaSuccess) return allowed;
   return launch_pdl(idkm_step_delta<D, KPL, LPW>, p, grid, DYN, stream);
 }
 #define IDKM_DELTA_ENTRY(D, KPL, LPW)                                                             \

@@ -7,13 +7,9 @@ template <int D, int KPL, bool DELTA>
 static cudaError_t launch_dual(const DualParams& dp, int grid, cudaStream_t stream) {
   constexpr int DYN_A = PassCfg<STEP, D, KPL, 1>::DYN_SMEM, DYN_B = DELTA ? DeltaCfg<D, KPL, 1>::DYN_SMEM : 0;
   constexpr int DYN = DYN_A > DYN_B ? DYN_A : DYN_B;   // the two halves use the dynamic region one after the other
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_step_dual<D, KPL, DELTA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                DYN > 0 ? DYN : 1);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_step_dual<D, KPL, DELTA>, DYN > 0 ? DYN : 1);
+  if (allowed != cudaSuccess) return allowed;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = dim3((unsigned)grid, 1, 1);

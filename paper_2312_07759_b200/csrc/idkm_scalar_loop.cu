@@ -1597,12 +1597,9 @@ cudaError_t launch_scalar_init(const ScalarParams& sp, int grid, cudaStream_t st
 
 template <int LOG>
 static cudaError_t launch_loop(const ScalarParams& sp, int grid, cudaStream_t stream) {
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_scalar_loop<LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_scalar_loop<LOG>, SC_DYN);
+  if (allowed != cudaSuccess) return allowed;
   // blocks of one layer wait for each other: a cooperative launch is refused if they cannot all be resident.  (A grid of
   // one block per layer has no barriers and is launched plainly.)
   void* args[1] = {const_cast<ScalarParams*>(&sp)};

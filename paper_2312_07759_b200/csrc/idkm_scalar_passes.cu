@@ -593,12 +593,9 @@ int scalar_grad_threads(int k) {
   return T > 1024 ? 1024 : T;
 }
 cudaError_t launch_scalar_grad(const ScalarParams& sp, int grid, cudaStream_t stream) {
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_scalar_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_GRAD_BYTES);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  const cudaError_t allowed = allow_smem(limit, idkm_scalar_grad, SP_GRAD_BYTES);
+  if (allowed != cudaSuccess) return allowed;
   const int T = scalar_grad_threads(sp.k);
   return launch_after(idkm_scalar_grad, grid, T < 256 ? 256 : T, 12 * (sp.k + 1) * T, stream, sp, T);
 }

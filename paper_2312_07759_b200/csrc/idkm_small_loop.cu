@@ -436,12 +436,9 @@ __global__ void __launch_bounds__(BLOCK, 2) idkm_small_loop(const __grid_constan
 template <int D, int KPL>
 static cudaError_t launch_small(const SmallLoopParams& sp, int grid, cudaStream_t stream) {
   constexpr int DYN = SmallCfg<D, KPL>::DYN_SMEM;
-  static bool configured = false;   // the slots of the widest layouts reach the 48 KB default limit
-  if (!configured) {
-    const cudaError_t rc = cudaFuncSetAttribute(idkm_small_loop<D, KPL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DYN);
-    if (rc != cudaSuccess) return rc;
-    configured = true;
-  }
+  static PerDevice limit;   // the slots of the widest layouts reach the 48 KB default limit
+  const cudaError_t allowed = allow_smem(limit, idkm_small_loop<D, KPL, true>, DYN);
+  if (allowed != cudaSuccess) return allowed;
   void* args[1] = {const_cast<SmallLoopParams*>(&sp)};
   // cooperative launch: refused (instead of hanging at the first barrier) if the grid cannot be co-resident
   if (sp.chunked)
