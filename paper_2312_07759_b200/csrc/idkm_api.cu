@@ -1342,6 +1342,21 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
     IDKM_TRY(cudaMemcpyAsync(grp[g].w[1], dWq_host + grp[g].w0, grp[g].wn, cudaMemcpyHostToDevice, sc));
     IDKM_TRY(cudaEventRecord(ctx->hev[4 * g + 1], sc));
   }
+  // Downloads start while uploads are on their way.  A result that goes to the memory of an input waits until all inputs are in,
+  // unless the two are the same array and a group's result follows that group's input anyway (all but Wq over dL/dWq).
+  {
+    const void* in[3] = {W_host, dWq_host, C0_host};
+    const size_t in_bytes[3] = {wn, wn, cn};
+    const void* out[6] = {Wq_out_host, dW_out_host, dW_jfb_out_host, C_out_host, dC_out_host, dC_jfb_out_host};
+    bool wait = false;
+    for (int o = 0; o < 6; ++o)
+      for (int i = 0; i < 3; ++i) {
+        const size_t bytes = o < 3 ? wn : cn;
+        const bool follows = out[o] == in[i] && bytes == in_bytes[i] && !(o == 0 && i == 1);
+        wait = wait || (out[o] && !follows && overlap(out[o], bytes, in[i], in_bytes[i]));
+      }
+    if (wait) IDKM_TRY(cudaStreamWaitEvent(sd, ctx->hev[4 * (ng - 1) + 1], 0));
+  }
   const int wq_dtype_saved = ctx->wq_dtype;
   for (int g = 0; g < ng; ++g) {
     HostGroup& q = grp[g];

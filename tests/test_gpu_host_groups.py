@@ -35,3 +35,28 @@ def test_groups_equal_one_batch(d, k, rows):
         assert_close(a, b, 2e-5 if d > 1 else 2e-4, name, l2_only=True)
     for a, b in zip(out[0][3], out[1][3]):
         assert len(a) == len(b) == 5 and np.allclose(a, b, rtol=1e-3, atol=1e-6)
+
+
+# one array for two purposes: (input, output) pairs that share their memory, one batch and several groups
+@pytest.mark.parametrize("rows", [[900_001], [2_000_003, 1_900_001, 1_900_005]])
+@pytest.mark.parametrize("pairs", [[("G", "Wq")], [("G", "dW"), ("W", "Wq"), ("C0", "C")], [("G", "Wq"), ("W", "dW"), ("C0", "dC")]])
+def test_results_may_go_where_inputs_came_from(rows, pairs):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    rng = np.random.default_rng(len(rows))
+    offs, d, k = [0] + [int(x) for x in np.cumsum(rows)], 2, 4
+    W = rng.standard_normal((offs[-1], d), dtype=np.float32) * np.float32(0.03)
+    G = rng.standard_normal(W.shape, dtype=np.float32) * np.float32(0.1)
+    C0 = np.concatenate([W[a:a + k] for a in offs[:-1]])
+    names = ("C", "Wq", "dW", "dC")
+    got = []
+    for shared in (False, True):
+        pin = lambda x: torch.from_numpy(x.copy()).pin_memory().numpy()
+        ins = {"W": pin(W), "G": pin(G), "C0": pin(C0)}
+        out = {n: pin(np.zeros_like(W if n in ("Wq", "dW") else C0)) for n in names}
+        if shared:
+            out.update({o: ins[i] for i, o in pairs})
+        res = B.Context().quantize_host(ins["W"], ins["C0"], ins["G"], 0.02, 0.0, 2, B.JFB, 0.0, 0, 1.0, layer_offsets=offs, out=out)
+        got.append([x.copy() for x in res[:4]])
+    for n, a, b in zip(names, *got):
+        assert np.array_equal(a, b), n
