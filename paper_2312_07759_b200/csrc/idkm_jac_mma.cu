@@ -28,7 +28,6 @@
 
 namespace idkm {
 
-constexpr int JM_POLLS = 1 << 22;
 constexpr int JM_DFOLD = 32;           // stages after which the diagonal's fp32 sums move to fp64 (one-tile codebooks)
 constexpr int JM_RED = 12;             // blocks whose partials one of them adds up (k d <= 64)
 
@@ -52,10 +51,14 @@ struct JmCfg {
   };
 constexpr int JM_LAUNCH_REGS = 65536 / JM_THREADS;   // the two kinds of warps redistribute these: 112 + 144, 160 + 96
 
-__device__ __forceinline__ bool jm_wait(unsigned long long* bar, unsigned parity) {
-  for (int i = 0; i < JM_POLLS; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  return false;
+__device__ __forceinline__ bool jm_wait(unsigned long long* bar, unsigned parity, long long limit /* SM clock ticks */) {
+  bool ok = mbar_try_wait(bar, parity);
+  if (!ok) {
+    const long long t0 = clock64();
+    do ok = mbar_try_wait(bar, parity);
+    while (!ok && clock64() - t0 < limit);
+  }
+  return __all_sync(0xffffffffu, ok);   // (by whole warps, which stay together whatever comes of it)
 }
 __device__ __forceinline__ void jm_arrive(unsigned long long* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
@@ -346,7 +349,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
     if (lane == 0) {
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        mbar_init(&full[i], 8);
+        mbar_init(&full[i], 8u + (PACK ? (unsigned)p.missing_arrivals : 0u));
         mbar_init(&done[i], 1);
         mbar_init(&tfree[i], 8);
       }
@@ -374,7 +377,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
     auto take = [&](int i, int part4) {
       const int s = i & 1;
       if (part4 == 0) {
-        if (!jm_wait(&done[s], (unsigned)((i >> 1) & 1))) return false;
+        if (!jm_wait(&done[s], (unsigned)((i >> 1) & 1), p.spin_limit)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
 #pragma unroll
@@ -428,8 +431,8 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
       int issued = 0;
       for (int i = 0; i < n && ok; ++i) {
         const int s = i & 1;
-        ok = jm_wait(&full[s], (unsigned)((i >> 1) & 1));
-        if (ok && i >= 2) ok = jm_wait(&tfree[s], (unsigned)(((i >> 1) - 1) & 1));
+        ok = jm_wait(&full[s], (unsigned)((i >> 1) & 1), p.spin_limit);
+        if (ok && i >= 2) ok = jm_wait(&tfree[s], (unsigned)(((i >> 1) - 1) & 1), p.spin_limit);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const unsigned a0 = sbase + s * Cfg::STAGE, b0 = a0 + 2 * Cfg::A_BYTES, dst = tmem + (unsigned)(s * NT);
@@ -456,7 +459,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
       for (int c = 0; c < 4; ++c) ok = ok && take(n - 1, c);
       if (ok) fold(n - 1);
       // (what is in flight ends before tensor memory is given back)
-      if (!ok && issued > 0) (void)jm_wait(&done[(issued - 1) & 1], (unsigned)(((issued - 1) >> 1) & 1));
+      if (!ok && issued > 0) (void)jm_wait(&done[(issued - 1) & 1], (unsigned)(((issued - 1) >> 1) & 1), p.spin_limit);
     }
     if (!ok && lane == 0) s_fail = 1;
   } else {
@@ -526,48 +529,50 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
     for (int i = 0; i < n; ++i) {
       const int s = i & 1;
       if (i == nb) load_tile(t0 + 1);
-      if (i >= 2) ok = jm_wait(&done[s], (unsigned)(((i >> 1) - 1) & 1));
-      if (!ok) break;
-      __syncwarp();
-      if (lane < 8 * Cfg::SETS) {
-        float* o = rowsm + (lane >> 3) * Cfg::SET_FLOATS + (lane & 7);
-        o[0] = wn.x;
-        o[8] = wn.y;
-        if constexpr (D == 4) {
-          o[16] = wn.z;
-          o[24] = wn.w;
-        }
-        o[D * 8] = rn.x;
-        o[D * 8 + 8] = rn.y;
-      }
-      __syncwarp();
-      fetch(i + 1);
-      unsigned char* A = dyn + s * Cfg::STAGE + pw * (JM_M * 16) + lane * 16;
-      unsigned char* B = dyn + s * Cfg::STAGE + 2 * Cfg::A_BYTES + pw * (NT * 16) + lane * 16;
+      // (a warp whose wait ran out makes nothing more, but meets the others at the ends of the tiles)
+      if (i >= 2 && ok) ok = jm_wait(&done[s], (unsigned)(((i >> 1) - 1) & 1), p.spin_limit);
       const int at = i < nb ? i : i - nb, last = i < nb ? nb : n - nb;
-      if constexpr (Cfg::BOTH) {
-#pragma unroll
-        for (int h = 0; h < Cfg::MU; ++h)
-          jm_unit_both<D>(myrows, cx[h], fx[h], p.scale, xm, ym, dg[h], A + h * 512, A + Cfg::A_BYTES + h * 512, B + h * 512,
-                          B + Cfg::B_BYTES + h * 512, JM_M / D * 16);
-      } else {
-        // of the tiles that share these rows of X, one adds this stage to the diagonal sums
-        const bool diag = (i < nb ? st0 + i : i - nb) % p.tiles_n == nt;
-#pragma unroll
-        for (int h = 0; h < Cfg::MU; ++h) {
-          unsigned char* o = A + h * 512;
-          if (diag)
-            jm_unit_x<D, true>(myrows, cx[h], fx[h], p.scale, xm, ym, dmine + h * 32 + lane, Cfg::MU * 32, o, o + Cfg::A_BYTES, JM_M / D * 16);
-          else
-            jm_unit_x<D, false>(myrows, cx[h], fx[h], p.scale, xm, ym, dmine + h * 32 + lane, Cfg::MU * 32, o, o + Cfg::A_BYTES, JM_M / D * 16);
+      if (ok) {
+        __syncwarp();
+        if (lane < 8 * Cfg::SETS) {
+          float* o = rowsm + (lane >> 3) * Cfg::SET_FLOATS + (lane & 7);
+          o[0] = wn.x;
+          o[8] = wn.y;
+          if constexpr (D == 4) {
+            o[16] = wn.z;
+            o[24] = wn.w;
+          }
+          o[D * 8] = rn.x;
+          o[D * 8 + 8] = rn.y;
         }
+        __syncwarp();
+        fetch(i + 1);
+        unsigned char* A = dyn + s * Cfg::STAGE + pw * (JM_M * 16) + lane * 16;
+        unsigned char* B = dyn + s * Cfg::STAGE + 2 * Cfg::A_BYTES + pw * (NT * 16) + lane * 16;
+        if constexpr (Cfg::BOTH) {
 #pragma unroll
-        for (int h = 0; h < Cfg::NU; ++h)
-          jm_unit_y<D>(myrows, cy[h], p.scale, ym, B + h * 512, B + Cfg::B_BYTES + h * 512, NT / D * 16);
+          for (int h = 0; h < Cfg::MU; ++h)
+            jm_unit_both<D>(myrows, cx[h], fx[h], p.scale, xm, ym, dg[h], A + h * 512, A + Cfg::A_BYTES + h * 512, B + h * 512,
+                            B + Cfg::B_BYTES + h * 512, JM_M / D * 16);
+        } else {
+          // of the tiles that share these rows of X, one adds this stage to the diagonal sums
+          const bool diag = (i < nb ? st0 + i : i - nb) % p.tiles_n == nt;
+#pragma unroll
+          for (int h = 0; h < Cfg::MU; ++h) {
+            unsigned char* o = A + h * 512;
+            if (diag)
+              jm_unit_x<D, true>(myrows, cx[h], fx[h], p.scale, xm, ym, dmine + h * 32 + lane, Cfg::MU * 32, o, o + Cfg::A_BYTES, JM_M / D * 16);
+            else
+              jm_unit_x<D, false>(myrows, cx[h], fx[h], p.scale, xm, ym, dmine + h * 32 + lane, Cfg::MU * 32, o, o + Cfg::A_BYTES, JM_M / D * 16);
+          }
+#pragma unroll
+          for (int h = 0; h < Cfg::NU; ++h)
+            jm_unit_y<D>(myrows, cy[h], p.scale, ym, B + h * 512, B + Cfg::B_BYTES + h * 512, NT / D * 16);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) jm_arrive(&full[s]);
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) jm_arrive(&full[s]);
       if (Cfg::BOTH && ((at + 1) % JM_DFOLD == 0 || at + 1 == last)) {
 #pragma unroll
         for (int h = 0; h < (Cfg::BOTH ? Cfg::MU : 0); ++h)
@@ -601,7 +606,10 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * NT));
   const bool failed = *reinterpret_cast<volatile int*>(&s_fail) != 0;
-  if (failed && tid == 0) st->status = ST_TIMEOUT;
+  if (failed && tid == 0) {
+    st->status = ST_TIMEOUT;
+    __threadfence();   // (before this block announces itself: the last block of the layer reads the status)
+  }
   if constexpr (PACK) {
     // ================= k d <= 64: the blocks' partials are added in two stages, and the last block runs the iteration ======
     const int units = p.unit_first[layer + 1] - p.unit_first[layer], ng = (units + JM_RED - 1) / JM_RED, grp = bl / JM_RED;
@@ -654,7 +662,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
     const int q = tid >> 2, pr = tid & 3;         // four threads per output, each with its part of the row in registers
     const double al = (double)p.alpha, be = 1.0 - al;
     JmStop stop;
-    stop.status = st->status;
+    stop.status = *reinterpret_cast<volatile int*>(&st->status);
     const int place = (q >> 4) * 18 + (q & 15);
     const double gq = ub[place];
     double row[16], uo = gq, g2 = 0.0;

@@ -36,8 +36,8 @@ struct JacMmaParams {
   int max_iter, k, n_layers;
   int tiles_m, tiles_n;
   int solve_blocks;        // blocks per layer of the solve kernel; 0: the last unit of a layer solves
-  int missing_arrivals;    // host-side fault injection of the solve's barrier, 0 in production
-  long long spin_limit;
+  int missing_arrivals;    // host-side fault injection, 0 in production: of the solve's barrier, for k d <= 64 of a full stage's
+  long long spin_limit;    // SM clock ticks of every wait
   long long row_off[MAX_LAYERS + 1];
   int unit_first[MAX_LAYERS + 1];
   int group_first[MAX_LAYERS];

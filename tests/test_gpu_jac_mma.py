@@ -91,3 +91,27 @@ def test_a_lost_arrival_ends_the_iteration_with_a_status():
     ctx.forward(W, C0, 0.01, 0.0, 5)
     again = ctx.backward(G, B.IMPLICIT, 0.0, 30, 0.25)[1].cpu().numpy()
     assert ctx.info()[0].status == 0 and np.array_equal(again, good)
+
+
+@pytest.mark.parametrize("d,k", [(2, 9), (4, 16)])
+def test_a_stage_that_never_fills_ends_the_pass_with_a_status(d, k):
+    """k d <= 64: the pass and the iteration are one launch.  A block whose wait for its operands ran out says so before it
+    joins the others, and the block that iterates on their sums keeps the status."""
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    W, C0, G, _ = data([60000], d, k, 0.03, 5)
+    W, C0, G = (torch.from_numpy(x).cuda() for x in (W, C0, G))
+    ctx = B.Context()
+    ctx.forward(W, C0, 0.01, 0.0, 5)
+    good = ctx.backward(G, B.IMPLICIT, 0.0, 30, 0.25)[1].cpu().numpy()
+    ctx.set_test_hooks(missing_arrivals=1, spin_limit_ticks=2000000)      # about a millisecond per wait
+    try:
+        ctx.backward(G, B.IMPLICIT, 0.0, 30, 0.25)
+        torch.cuda.synchronize()
+        assert ctx.info()[0].status == B.ERR_TIMEOUT
+    finally:
+        ctx.set_test_hooks(0, 0)
+    assert ctx.busy_tickets() == 0
+    ctx.forward(W, C0, 0.01, 0.0, 5)
+    again = ctx.backward(G, B.IMPLICIT, 0.0, 30, 0.25)[1].cpu().numpy()
+    assert ctx.info()[0].status == 0 and np.array_equal(again, good)
