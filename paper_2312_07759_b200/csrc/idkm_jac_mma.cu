@@ -6,15 +6,17 @@
 // to a scheduler (48 % of the issue slots, tensor pipe 34 % active), for 32 768 multiply-adds a weight, which three fp16
 // products take 1540 cycles a stage for.  Hence the tile as wide as the register file holds its sums, the packed fp32
 // instructions, and, where rows and columns of a tile are of the same centroids (k d <= 128), one pass for both operands.
-// Measured (adjoint of 50 steps against the fused passes): 4 M x 4, k = 256: 34 ms against 44; 1 M x 2, k = 256: 2.6
+// Measured (adjoint of 50 steps against the fused passes): 4 M x 4, k = 256: 35 ms against 44; 1 M x 2, k = 256: 2.6
 // against 11.2; 3 M x 4, k = 16, 30 steps: 0.31 against 1.9 (1.3 with Jacobian tiles on the CUDA cores).
 //
 // Precision.  X and Y are split into two fp16 terms (22 bits, scaled by powers of two so that the second term stays
-// normal): hi hi + hi lo + lo hi; what is dropped is 2^-22 of a product, below the 2e-7 of the exponential and the
-// reciprocal square root they are made of.  The tensor core adds in fp32 without rounding to nearest, so an accumulator
-// takes one stage of 64 weights only -- its small terms first -- and is then added to fp32 sums in registers, which move to
-// an fp64 partial every JM_FOLD stages; the partials are added in a fixed order.  (Two stages to an accumulator were no
-// faster and 2 to 5 times less exact: 2.3e-6 to 5e-6 of the adjoint against 1e-6.)
+// normal): hi hi + hi lo + lo hi; what is dropped is at most 2^-24 of a product and of either sign.  The tensor core adds in
+// fp32 and cuts instead of rounding, so an accumulator takes one stage of 64 weights only -- its small terms first --, what
+// the cuts take on average is given back (JM_CUT), and the result is added to fp32 sums in registers, which move to an fp64
+// partial every JM_FOLD stages; the partials are added in a fixed order.  Error of the adjoint against float64, with the fused
+// passes' in brackets, 40 000 weights, 40 steps: d = 4, k = 16 3.2e-7 (2.9e-7), at tau = 0.002 4e-7 (5e-7); k = 64 3.5e-7 (3.4e-7);
+// d = 2, k = 64 3.7e-7 (3.3e-7).  With the first term cut to its leading bits and nothing given back it was 5e-7, and 3e-6 at
+// tau = 0.002; two stages to an accumulator were no faster and 2 to 5 times less exact.
 //
 // Roles: a producing warp makes eight weights' share of the stage (a lane holds a centroid, so nothing crosses lanes) and
 // writes it in the core-matrix order of the K-major operand, 16 bytes per lane and row of the operand: consecutive lanes
@@ -28,6 +30,9 @@
 
 namespace idkm {
 
+// What an accumulator loses by being cut: four steps of the large products leave a quarter, a half, three quarters and all of an
+// entry, each cut by half a unit in the last place on average, 0.36 x 2^-23 of itself: 2.5 x 0.36 x 2^-23 of the entry.
+constexpr double JM_CUT = 1.0 + 0.9017 / 8388608.0;
 constexpr int JM_DFOLD = 32;           // stages after which the diagonal's fp32 sums move to fp64 (one-tile codebooks)
 constexpr int JM_RED = 12;             // blocks whose partials one of them adds up (k d <= 64)
 
@@ -148,8 +153,9 @@ struct JmStop {
 };
 
 // Splits eight values (four pairs of neighbouring weights) into two fp16 terms and stores them, 16 bytes each.  The first
-// term is the value cut to its 11 leading bits -- a mask, on the integer pipe, which the producers leave idle, instead of a
-// conversion and back -- so the second is exact before its rounding.
+// term is the value rounded to its 11 leading bits -- an addition and a mask, on the integer pipe, which the producers leave
+// idle, instead of a conversion and back -- so the second is exact before its rounding and of either sign: what the products
+// leave out, lo lo, averages out.  (Cut instead of rounded, it is up to 2^-20 of a product and always of its sign.)
 __device__ __forceinline__ void jm_split_store(const f2 (&v)[4], unsigned char* hi, unsigned char* lo) {
   unsigned ph[4], pl[4];
   const f2 neg = f2_pack(-1.f, -1.f);
@@ -157,7 +163,7 @@ __device__ __forceinline__ void jm_split_store(const f2 (&v)[4], unsigned char* 
   for (int q = 0; q < 4; ++q) {
     float x, y, lx, ly;
     f2_unpack(v[q], x, y);
-    const float hx = __uint_as_float(__float_as_uint(x) & 0xffffe000u), hy = __uint_as_float(__float_as_uint(y) & 0xffffe000u);
+    const float hx = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u), hy = __uint_as_float((__float_as_uint(y) + 0x1000u) & 0xffffe000u);
     f2_unpack(f2_fma(f2_pack(hx, hy), neg, v[q]), lx, ly);
     const __half2 h2 = __floats2half2_rn(hx, hy), l2 = __floats2half2_rn(lx, ly);
     ph[q] = *reinterpret_cast<const unsigned*>(&h2);
@@ -401,7 +407,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
           for (int b = 0; b < 2; ++b)
 #pragma unroll
             for (int l = 0; l < 16; ++l) {
-              const double v = (double)acc[b * 32 + l] + (double)__shfl_xor_sync(0xffffffffu, acc[b * 32 + 16 + l], 16);
+              const double v = JM_CUT * ((double)acc[b * 32 + l] + (double)__shfl_xor_sync(0xffffffffu, acc[b * 32 + 16 + l], 16));
               double* e = o + ((half * 2 + b) * 16 + l) * 64 + quad * 16 + lane;
               if (lane < 16) *e = first ? v : *e + v;
             }
@@ -411,7 +417,7 @@ __global__ void __launch_bounds__(JM_THREADS, 1) idkm_jac_mma(const __grid_const
 #pragma unroll
           for (int q = 0; q < NT / 2; ++q) {
             double* e = o + (size_t)q * 256 + half * 128 + quad * 32 + lane;
-            *e = first ? (double)acc[q] : *e + (double)acc[q];
+            *e = first ? JM_CUT * (double)acc[q] : fma(JM_CUT, (double)acc[q], *e);
             acc[q] = 0.f;
           }
         }
