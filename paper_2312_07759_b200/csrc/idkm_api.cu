@@ -886,7 +886,8 @@ static int launch_pass(idkm_ctx* ctx, int mode, PassParams* p, int repeat) {
 }
 
 // The adjoint iteration on the explicit Jacobian formed by the tensor cores: one pass over the weights, then the whole
-// iteration on the matrix (in the same launch for k d <= 64).
+// iteration on the matrix (in the same launch for k d <= 64).  1: a launch was refused (the blocks that iterate on the matrix
+// have to be resident together), and the adjoint still is where the codebook-gradient pass left it: the fused passes take over.
 static int launch_jac_mma_adjoint(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p) {
   JacMmaParams q;
   memset(&q, 0, sizeof(q));
@@ -920,10 +921,16 @@ static int launch_jac_mma_adjoint(idkm_ctx* ctx, const WorkspaceLayout& wl, cons
   if (ctx->hook_spin_limit > 0 && ctx->hook_spin_limit < SMALL_SPIN_LIMIT) q.spin_limit = ctx->hook_spin_limit;
   for (int l = 0; l <= MAX_LAYERS; ++l) q.row_off[l] = ctx->row_off[l < ctx->n_layers ? l : ctx->n_layers];
   const int units = jac_mma_split(wl.jm, ctx->d, &q);
-  if (launch_jac_mma(ctx->d, wl.jm, q, units, ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
+  if (launch_jac_mma(ctx->d, wl.jm, q, units, ctx->stream) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 1;
+  }
   ++ctx->launches;
   if (q.solve_blocks > 0) {
-    if (launch_jac_solve(ctx->d, wl.jm, q, ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
+    if (launch_jac_solve(ctx->d, wl.jm, q, ctx->stream) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return 1;
+    }
     ++ctx->launches;
   }
   return IDKM_OK;
@@ -1137,6 +1144,7 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
       rc = launch_scalar_pass(ctx, wl, p, SP_ADJOINT, dC_out);
     } else if (jac_mma) {
       rc = launch_jac_mma_adjoint(ctx, wl, p);
+      if (rc == 1) rc = launch_pass(ctx, ADJ, &p, adj_max_iter);
     } else if (explicit_jac) {
       if (exact) p.max_iter = -1;                  // the epilogue solves (I - J^T) u = g instead of iterating
       rc = launch_pass(ctx, JACOBIAN, &p, 1);      // one pass forms J_C; the whole iteration runs on it in the epilogue

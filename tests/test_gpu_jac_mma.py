@@ -140,3 +140,24 @@ def test_no_less_exact_than_the_passes(d, k, tau):
             _, u, _, _ = R.backward(W64, G.astype(np.float64), C, tau, S, F, alpha=0.25, adj_max_iter=40, want_dW=False)
             err[method] += float(np.linalg.norm(dC - u) / np.linalg.norm(u)) / 4
     assert err[0] <= 1.5 * err[1] + 1e-7, err
+
+
+# as many blocks as the workspace rule lets iterate on matrices at a time (576, 384, 576), which have to be resident together
+@pytest.mark.parametrize("d,k,layers", [(2, 256, 9), (4, 256, 3), (4, 192, 6)])
+def test_the_largest_batches_keep_the_route(d, k, layers):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    W, C0, G, offs = data([300 + 64 * l for l in range(layers)], d, k, 0.03, layers)
+    W, C0, G = (torch.from_numpy(x).cuda() for x in (W, C0, G))
+    out = []
+    for method in (0, 1):
+        ctx = B.Context()
+        ctx.set_adjoint_method(method)
+        ctx.forward(W, C0, 0.02, 0.0, 8, layer_offsets=offs)
+        n0 = ctx.launches
+        dW, dC = ctx.backward(G, B.IMPLICIT, 0.0, 100, 0.25)
+        out.append((ctx.launches - n0, dW.cpu().numpy(), dC.cpu().numpy(), [i.status for i in ctx.info()]))
+    assert out[0][0] == 4 and out[1][0] == 102 and out[0][3] == out[1][3]
+    if all(s == 0 for s in out[0][3]):
+        assert_close(out[0][2], out[1][2], TOL_GRAD, "dC")
+        assert_close(out[0][1], out[1][1], TOL_GRAD, "dW")
