@@ -306,7 +306,9 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
     w.off_sc_tab = o;    o = align_up(o + 8 * (size_t)L * SC_NTAB * K1, 256);
     w.off_sc_perm = o;   o = align_up(o + 4 * (size_t)L * k, 256);
     w.off_sc_ftab = o;   o = align_up(o + 4 * (size_t)L * SC_NFTAB * K1, 256);
-    w.off_sc_gpart = o;  o = align_up(o + 8 * (size_t)(w.n_sc_grad_blocks + w.n_sc_groups) * 3 * K1, 256);
+    const size_t grad_rows = (size_t)(w.n_sc_grad_blocks + w.n_sc_groups) * 3 * K1;
+    const size_t loop_rows = (size_t)(k <= SD_TWO_ROWS_K ? 2 * sms : sms + L) * SD_SUMS(k);
+    w.off_sc_gpart = o;  o = align_up(o + 8 * (grad_rows > loop_rows ? grad_rows : loop_rows), 256);
     w.off_sc_gtick = o;  o = align_up(o + 4 * (size_t)w.n_sc_groups, 256);
   }
   w.total = o;

@@ -24,6 +24,8 @@ constexpr int SC_BIG_LAYERS = 8;
 constexpr int SC_REC_SMEM = 3584;      // coarse bins whose records fit in shared memory (36 bytes each)
 constexpr int SC_REC_BYTES = 36;
 constexpr int SC_SYNC_WORDS = 32;      // barrier words of one layer (one 128-byte line)
+constexpr int SD_TWO_ROWS_K = 32;      // loop without bins: up to this many centroids two rows of sums for every block
+__host__ __device__ constexpr int SD_SUMS(int k) { return 6 * (k + 1); }
 constexpr int SC_PSCALE = 65534;       // a weight's place in its fine bin is kept in 1 / 65534 of the bin's width
 
 // Per-layer tables the loop leaves for the passes that follow: doubles, [SC_NTAB][k + 1], sorted order.  V: relative to
@@ -56,7 +58,8 @@ struct ScalarPtrs {            // per-call pointers into the workspace (and the 
   double* tab;                 // [L][SC_NTAB][k + 1]
   int* perm;                   // [L][k] sorted position -> centroid index
   float* ftab;                 // [L][SC_NFTAB][k + 1]
-  double* gpart;               // partial sums of the codebook gradient, [blocks + groups][3 (k + 1)]
+  double* gpart;               // partial sums of the codebook gradient, [blocks + groups][3 (k + 1)], and of the loop without
+                               // bins, rows of SD_SUMS(k), [blocks] twice (k <= SD_TWO_ROWS_K) or [blocks + L]
   unsigned int* gtick;         // [groups] arrival counters, zero at rest
   unsigned int* pair_ticks[2]; // arrival counters of the pairwise passes, which may follow: zeroed with the rest
   int n_pair_ticks[2];

@@ -18,6 +18,12 @@
 // against 1268; 16 M weights, k = 16, 100 iterations 1.42 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 101
 // against 112.
 //
+// Layers that bins do not suit -- tau below 1 / 5700 of the weights' range (1 / 2800 in layers beyond the eighth), which an outlier
+// is enough for, or thousands of weights in one fine bin -- are evaluated weight by weight by all their blocks (sd_pass): without
+// bins an iteration's time does not depend on where the weights lie.  m = 1 M, one weight at 1e5 standard deviations, an iteration
+// at k = 4 / 16 / 64 / 256: 17 / 24 / 63 / 63 us; two values for 3/4 of the weights: 19 / 22 / 63.  (Loops over the pairs on such
+// weights: 8 / 14 / 37 / 125 us, 16 M weights 27 / 73 / 395 / 1000 against 58 / 78 / 332 / 325.)
+//
 // Several blocks per layer build the summary (meetings at a bounded barrier), then one block per layer runs the
 // iterations: one warp (or a few) per interval between centroids, the M-step by the first warps in fp64.
 #include "idkm_scalar.cuh"
@@ -173,6 +179,10 @@ struct ScShared {
   ScGrid g;
   ScLayer ly;              // (copy for the functions that are not inlined)
   int ok, bad, flag, done, iters, dead, status;
+  // what the evaluations without bins need (here, so that it does not live in registers in the others)
+  unsigned int meet;       // barriers of the layer's blocks so far
+  const float* W;          // the layer's weights, and this block's share
+  long long r0, r1;
   float res;
   long long n0;            // weights that are exactly zero (kept out of the bins)
   float v[257];            // sorted centroids
@@ -193,7 +203,10 @@ struct ScShared {
   double scan_x[SC_WARPS + 1];
 };
 constexpr int SC_SH_BYTES = (int)((sizeof(ScShared) + 255) / 256 * 256);
-constexpr int SC_DYN = SC_SH_BYTES + ((SC_FINE_BIG * 4 > SC_REC_SMEM * SC_REC_BYTES + 16) ? SC_FINE_BIG * 4 : SC_REC_SMEM * SC_REC_BYTES + 16);
+constexpr int SC_BIN_BYTES = (SC_FINE_BIG * 4 > SC_REC_SMEM * SC_REC_BYTES + 16) ? SC_FINE_BIG * 4 : SC_REC_SMEM * SC_REC_BYTES + 16;
+// without bins (sd_pass): sums of every thread, of every warp, tables of the search
+constexpr int SD_COLS = SC_WARPS * 257 * 4 * 8, SD_WSUM = 8448, SD_BYTES = SD_COLS + SD_WSUM + (512 + 2 * 257) * 4;
+constexpr int SC_DYN = SC_SH_BYTES + (SC_BIN_BYTES > SD_BYTES ? SC_BIN_BYTES : SD_BYTES);
 constexpr int SC_SMALL_NC = 512;       // layers of up to this many coarse bins leave room for their weights' places
 constexpr int SC_SMALL_OFF = (SC_SMALL_NC * SC_REC_BYTES + 16 + 15) / 16 * 16;
 static_assert(SC_DYN <= 227 * 1024, "shared memory of the loop kernel");
@@ -476,51 +489,7 @@ __device__ __forceinline__ void sc_bin_sums(const ScCoef& c, float eta, T n, T m
   }
 }
 
-constexpr float SC_ETA_MAX = 0.6f;   // the series' limit; wider bins are evaluated weight by weight
 constexpr double SC_ZONE = 96.0;   // |z| beyond which lambda resp. mu (below 2^-96) is taken as zero for whole bins
-
-// Interval sums of the bins' weights one by one, for layers whose bins are too wide for the series (tau below about
-// range / 8000; fine bin = coarse bin there).  A lane takes whole bins; inside a bin the order of the weights can vary
-// from run to run, so the sums are integers relative to the largest value in the bin.
-template <bool EXTRA>
-__device__ __noinline__ void sc_wide_bin(const ScGrid& g, const ScLayer& ly, int f, int pl, int pr, double even, double v0, double* acc) {
-  const unsigned int e0 = ly.fstart[f], e1 = ly.fstart[f + 1];
-  if (e0 == e1) return;
-  const double ctr = (double)(g.base_f + f) * g.hf;
-  const float zc = (float)((ctr - even) * (double)ly.slope), dz = (float)(g.hf * (double)ly.slope);
-  // exponents of the largest lambda (left edge) and mu (right edge)
-  const float zl = zc - 0.5f * dz, zr = zc + 0.5f * dz;
-  const int el = (int)fmaxf(fminf(0.f, ceilf(-zl)), -126.f), em = (int)fmaxf(fminf(0.f, ceilf(zr)), -126.f);
-  const double sl = scalbn(1.0, 38 - el), sm = scalbn(1.0, 38 - em), sx = scalbn(1.0, 38 - el - em);
-  long long t[6] = {0, 0, 0, 0, 0, 0};
-  for (unsigned int e = e0; e < e1; ++e) {
-    const int p = (int)ly.grouped[ly.row0 + e] - 32768;
-    int wgt = (p > pl ? 2 : (p == pl ? 1 : 0)) - (p < pr ? 0 : (p == pr ? 1 : 2));   // twice the share in the interval
-    if (wgt <= 0) continue;
-    const float d = (float)p * (float)SC_S1;
-    float lam, mu;
-    sc_lambda(fmaf(d, dz, zc), lam, mu);
-    const double hw = 0.5 * (double)wgt;
-    const double xl = hw * (double)lam * sl, xm = hw * (double)mu * sm;
-    t[0] += __double2ll_rn(xl);
-    t[1] += __double2ll_rn(xl * (double)d);
-    t[2] += __double2ll_rn(xm);
-    t[3] += __double2ll_rn(xm * (double)d);
-    if (EXTRA) {
-      const double xx = hw * (double)lam * (double)mu * sx;
-      t[4] += __double2ll_rn(xx);
-      t[5] += __double2ll_rn(xx * (double)d);
-    }
-  }
-  const double x0 = ctr - v0;
-  const double S[3] = {1.0 / sl, 1.0 / sm, 1.0 / sx};
-#pragma unroll
-  for (int i = 0; i < (EXTRA ? 3 : 2); ++i) {
-    const double a0 = (double)t[2 * i] * S[i], a1 = (double)t[2 * i + 1] * S[i];
-    acc[2 * i] += a0;
-    acc[2 * i + 1] += fma(x0, a0, g.hf * a1);
-  }
-}
 
 // The weights that are exactly zero; on a centroid half of them belong to either side.
 __device__ __noinline__ void sc_zeros(const ScShared& sh, int s, double even, double v0, double* acc) {
@@ -560,7 +529,7 @@ __device__ __noinline__ void sc_stop_test(ScShared& sh, const ScalarParams& sp, 
     sh.iters = test;
     sh.res = res;
     sh.dead = dead;
-    if (test <= HIST_CAP) sp.p.hist_fwd[(size_t)layer * HIST_CAP + test - 1] = res;
+    if (test <= HIST_CAP && (int)blockIdx.x == sp.blk_first[layer]) sp.p.hist_fwd[(size_t)layer * HIST_CAP + test - 1] = res;
     if (bad) {
       sh.status = ST_NONFINITE;
       sh.done = test;
@@ -665,7 +634,6 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
   const ScGrid& g = sh.g;
   const int k = ly.k, tw = 1 << ly.twl, slots = tw + 2;
   const double v0 = (double)sh.v[0];
-  const bool wide = g.eta > SC_ETA_MAX;
   if (k == 1) {
     // one centroid: every weight counts on its left, with attention 1
     if (threadIdx.x == 0) {
@@ -714,22 +682,14 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
       M[2] += q1.x;
       M[3] += q1.y;
       if (!runs) {
-        if (!wide) {
-          const ScCoef co = sc_coef((float)((ctr - even) * (double)ly.slope));
-          if (left) {   // the piece above the left end: the whole bin (unless the right end lies in it) minus what is below
-            const bool whole = cl != cr;
-            n = (whole ? (double)ly.rec.r[cl] : 0.0) - n;
+        const ScCoef co = sc_coef((float)((ctr - even) * (double)ly.slope));
+        if (left) {   // the piece above the left end: the whole bin (unless the right end lies in it) minus what is below
+          const bool whole = cl != cr;
+          n = (whole ? (double)ly.rec.r[cl] : 0.0) - n;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) M[i] = (whole ? (double)ly.rec.r[(i + 1) * ly.rec.stride + cl] : 0.0) - M[i];
-          }
-          sc_bin_sums<EXTRA, double>(co, g.eta, n, M[0], M[1], M[2], M[3], ctr - v0, g.hc, acc);
-        } else if (left || fl != fr) {
-          // (fine bin = coarse bin)
-          double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-          sc_wide_bin<EXTRA>(sh.g, sh.ly, f, left ? sh.pv[s - 1] : -50000, (!left || fl == fr) ? sh.pv[s] : 50000, even, v0, t6);
-#pragma unroll
-          for (int i = 0; i < 6; ++i) acc[i] += t6[i];
+          for (int i = 0; i < 4; ++i) M[i] = (whole ? (double)ly.rec.r[(i + 1) * ly.rec.stride + cl] : 0.0) - M[i];
         }
+        sc_bin_sums<EXTRA, double>(co, g.eta, n, M[0], M[1], M[2], M[3], ctr - v0, g.hc, acc);
       } else {
         if (left ? (s == 1) : (s == k - 1)) {
           // the outer interval beyond this end: every weight there, and the zeros
@@ -800,19 +760,12 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
     if (b1 > cr - 1) b1 = cr - 1;
     if (!on) b1 = b0 - 1;
     double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (!wide) {
-      for (int b = b0 + sub * 32 + l; b <= b1; b += lpi * tw) {
-        const float n = ly.rec.r[b];
-        const double ctr = sc_center(g, b);
-        const ScCoef c = sc_coef((float)((ctr - even) * (double)ly.slope));
-        sc_bin_sums<EXTRA, float>(c, g.eta, n, ly.rec.r[ly.rec.stride + b], ly.rec.r[2 * ly.rec.stride + b], ly.rec.r[3 * ly.rec.stride + b],
-                                  ly.rec.r[4 * ly.rec.stride + b], ctr - v0, g.hc, acc);
-      }
-    } else {
-      double t6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      for (int b = b0 + sub * 32 + l; b <= b1; b += lpi * tw) sc_wide_bin<EXTRA>(sh.g, sh.ly, b, -50000, 50000, even, v0, t6);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) acc[i] += t6[i];
+    for (int b = b0 + sub * 32 + l; b <= b1; b += lpi * tw) {
+      const float n = ly.rec.r[b];
+      const double ctr = sc_center(g, b);
+      const ScCoef c = sc_coef((float)((ctr - even) * (double)ly.slope));
+      sc_bin_sums<EXTRA, float>(c, g.eta, n, ly.rec.r[ly.rec.stride + b], ly.rec.r[2 * ly.rec.stride + b], ly.rec.r[3 * ly.rec.stride + b],
+                                ly.rec.r[4 * ly.rec.stride + b], ctr - v0, g.hc, acc);
     }
     __syncwarp();
     double* lo = sh.Ls[(s - 1) * slots + sub];
@@ -876,6 +829,319 @@ __device__ __forceinline__ void sc_gather(const double (*a)[2], int j, int twl, 
       s0 += a[j * slots + q][0];
       s1 += a[j * slots + q][1];
     }
+}
+
+// ---- layers whose bins would not pay: the sums of an evaluation from the weights themselves ----
+// Where tau is far below the weights' range (bins as wide as the workspace allows are then too wide for the series, and
+// places of 16 bits in them too coarse), or very many weights share a few values (the bin of a centroid is looked at weight by
+// weight by one or two warps), every evaluation is a pass over the weights by all blocks of the layer.  A weight costs a search
+// for its interval, an exponential and a reciprocal whatever the number of centroids, and four additions in shared memory, so
+// the time does not depend on where the weights lie.
+constexpr float SC_ETA_MAX = 0.35f;          // coarse bins of 0.17 tau and their rounding
+constexpr unsigned int SC_CROWD = 4096;      // weights of a fine bin, besides 1 / 256 of the layer's
+// Up to SD_OWN_K centroids every thread has fp32 sums of its own for every interval (as many threads take weights as there is
+// room for); more have fp64 sums for every warp, to which the lanes that have weights of the same interval add one after the
+// other, or, where few intervals have many, after a sum over the warp.  (m = 1 M, an iteration, own sums against the warp's:
+// k = 64 58 against 85 us, k = 256 248 against 63.)
+constexpr int SD_OWN_K = 100;
+__device__ __forceinline__ int sd_threads(int k) {
+  if (k > SD_OWN_K) return SC_T;
+  const int t = (SD_COLS / (16 * (k + 1))) & ~31;
+  return t > SC_T ? SC_T : t;
+}
+struct SdView {
+  float4* own;        // [k + 1][threads]: by interval, sums of lambda, lambda x, mu, mu x
+  double* wsum;       // [warps][4 (k + 1)] the same of a warp
+  float *v, *te, *to; // sorted centroids, even points and what their rounding adds to the exponent
+};
+__device__ __forceinline__ SdView sd_view(int k) {
+  extern __shared__ __align__(16) unsigned char smem_all[];
+  SdView d;
+  d.own = reinterpret_cast<float4*>(smem_all + SC_SH_BYTES);
+  d.wsum = reinterpret_cast<double*>(smem_all + SC_SH_BYTES + (k <= SD_OWN_K ? SD_COLS : 0));
+  d.v = reinterpret_cast<float*>(smem_all + SC_SH_BYTES + SD_COLS + SD_WSUM);
+  d.te = d.v + 512;
+  d.to = d.te + 257;
+  return d;
+}
+// A warp's fp32 sums move to its fp64 sums and start at zero again.  A thread adds at most SD_FOLD terms to one between two such
+// calls (a longer fp32 sum loses the many terms below half its last place, see PassCfg).  A lane takes an interval, or several
+// lanes share one: few conversions a lane.  Each starts from a thread of its own: the lanes read different banks.
+constexpr int SD_FOLD = 64;
+__device__ __forceinline__ void sd_fold(const SdView& d, int T, int k, double* wsum, bool first) {
+  const int tid = threadIdx.x, lane = tid & 31, n = k + 1, P = n < 32 ? 32 / n : 1, c = n < 32 ? lane / n : 0;
+  __syncwarp();
+  for (int s0 = 0; s0 < n; s0 += 32) {   // (one round where lanes share)
+    const int s = n < 32 ? lane % n : s0 + lane, N = (31 - c) / P + 1;
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    if (c < P && s < n) {
+      const float4* col = d.own + (size_t)s * T + (tid - lane) + c;
+      int j = s % N;
+#pragma unroll 4
+      for (int i = 0; i < N; ++i) {
+        const float4 y = col[P * j];
+        x[0] += (double)y.x;
+        x[1] += (double)y.y;
+        x[2] += (double)y.z;
+        x[3] += (double)y.w;
+        j = j + 1 == N ? 0 : j + 1;
+      }
+    }
+    double t[4] = {x[0], x[1], x[2], x[3]};
+    for (int q = 1; q < P; ++q)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) t[i] += __shfl_sync(0xffffffffu, x[i], s + q * n);
+    if (c == 0 && s < n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) wsum[s * 4 + i] = first ? t[i] : wsum[s * 4 + i] + t[i];
+  }
+  __syncwarp();
+  for (int i = 0; i < n; ++i) d.own[(size_t)i * T + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+// MODE 0: sums of lambda and mu; 1: the same, a weight on a centroid counting half on either side (sub-gradient 0 of its
+// distance); 2: of lambda mu in place of lambda.  x: from the interval's left centroid.
+template <int MODE, bool OWN>
+__device__ __noinline__ void sd_pass(const float* __restrict__ Wl, long long r0, long long r1, int k, float slope) {
+  const SdView d = sd_view(k);
+  const int tid = threadIdx.x, lane = tid & 31, T = OWN ? sd_threads(k) : SC_T;
+  if (OWN && tid >= T) {   // (whole warps)
+    __syncthreads();
+    return;
+  }
+  double* wsum = d.wsum + (size_t)(tid >> 5) * 4 * (k + 1);
+  if (OWN) {
+    for (int s = 0; s <= k; ++s) d.own[(size_t)s * T + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+  } else {
+    for (int e = lane; e < 4 * (k + 1); e += 32) wsum[e] = 0.0;
+    __syncwarp();
+  }
+  int top = 1;
+  while (2 * top <= k) top *= 2;
+  // what a weight adds to its interval (outside the centroids lambda resp. mu is 1)
+  auto terms = [&](int s, float w, float g) {
+    const float x = w - d.v[s > 0 ? s - 1 : 0];
+    float lam, mu;
+    sc_lambda(fmaf(w - d.te[s], slope, d.to[s]), lam, mu);
+    const bool in = s > 0 && s < k;
+    if (MODE == 2) {
+      lam = in ? g * lam * mu : 0.f;
+      mu = 0.f;
+    } else {
+      lam = in ? g * lam : (s > 0 ? g : 0.f);
+      mu = in ? g * mu : (s < k ? g : 0.f);
+    }
+    return make_float4(lam, lam * x, mu, mu * x);
+  };
+  auto add = [&](int s, const float4& y, bool real) {   // (by whole warps)
+    if (OWN) {
+      if (!real) return;
+      float4* c = d.own + (size_t)s * T + tid;
+      float4 x = *c;
+      x.x += y.x;
+      x.y += y.y;
+      x.z += y.z;
+      x.w += y.w;
+      *c = x;
+    } else {
+      const unsigned int same = __match_any_sync(0xffffffffu, real ? s : -1);
+      const int turn = real ? __popc(same & ((1u << lane) - 1u)) : -1;
+      const int turns = __reduce_max_sync(0xffffffffu, turn);
+      const unsigned int firsts = __ballot_sync(0xffffffffu, turn == 0);
+      if (2 * __popc(firsts) <= turns) {
+        for (unsigned int left = firsts; left; left &= left - 1) {
+          const int lead = __ffs(left) - 1, sl = __shfl_sync(0xffffffffu, s, lead);
+          const bool mine = real && s == sl;
+          float x[4] = {mine ? y.x : 0.f, mine ? y.y : 0.f, mine ? y.z : 0.f, mine ? y.w : 0.f};
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] += __shfl_xor_sync(0xffffffffu, x[i], o);
+          if (lane < 4) wsum[4 * sl + lane] += (double)(lane == 0 ? x[0] : (lane == 1 ? x[1] : (lane == 2 ? x[2] : x[3])));
+        }
+        __syncwarp();
+        return;
+      }
+      double2* c = reinterpret_cast<double2*>(wsum + 4 * s);
+      for (int t = 0; t <= turns; ++t) {
+        if (t == turn) {
+          double2 a = c[0], b = c[1];
+          a.x += (double)y.x;
+          a.y += (double)y.y;
+          b.x += (double)y.z;
+          b.y += (double)y.w;
+          c[0] = a;
+          c[1] = b;
+        }
+        __syncwarp();
+      }
+    }
+  };
+  constexpr int U = OWN ? 8 : 4;
+  static_assert(SD_FOLD % U == 0, "");
+  const long long step = (long long)T * U;
+  long long r = r0 + tid;
+  float wn[U];
+  auto fetch = [&](long long q) {
+#pragma unroll
+    for (int i = 0; i < U; ++i) wn[i] = q + i * T < r1 ? __ldg(Wl + q + i * T) : 0.f;
+  };
+  fetch(r);
+  bool first = true;
+  int since = 0;
+  for (long long q = r0; q < r1; q += step, r += step) {   // (the same trips for all threads)
+    float w[U];
+    float4 y[U];
+    int s[U];
+    bool real[U], on[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      w[i] = wn[i];
+      s[i] = 0;
+      real[i] = r + i * T < r1;
+    }
+    fetch(r + step);
+    for (int h = top; h > 0; h >>= 1)
+#pragma unroll
+      for (int i = 0; i < U; ++i) s[i] += d.v[s[i] + h - 1] < w[i] ? h : 0;
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      on[i] = MODE > 0 && real[i] && s[i] < k && d.v[s[i] < k ? s[i] : 0] == w[i];
+      y[i] = terms(s[i], w[i], on[i] ? 0.5f : 1.f);
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      add(s[i], y[i], real[i]);
+      if (MODE > 0 && __any_sync(0xffffffffu, on[i])) {
+        int s2 = s[i];
+        while (on[i] && s2 < k && d.v[s2] == w[i]) ++s2;
+        add(s2, terms(s2, w[i], 0.5f), on[i]);
+      }
+    }
+    if (OWN && (since += U) == SD_FOLD) {
+      sd_fold(d, T, k, wsum, first);
+      first = false;
+      since = 0;
+    }
+  }
+  if (OWN && (first || since > 0)) sd_fold(d, T, k, wsum, first);
+  __syncthreads();
+}
+// One evaluation, by all threads of a block of the layer.  A block that is the layer's only one leaves the sums where the M-step
+// looks for them; several leave a row of SD_SUMS each: 4 (k + 1) by interval and kind, then 2 (k + 1) of lambda mu.
+__device__ __forceinline__ void sd_place(ScShared& sh, int k, int o, double x) {
+  const int n = 4 * (k + 1);
+  if (o < n) {
+    const int s = o >> 2, c = o & 3;   // interval s: lambda for the centroid on its left, mu for the one on its right
+    if (c < 2) {
+      if (s > 0) sh.Ls[(s - 1) * 3][c] = x;
+    } else if (s < k) {
+      sh.Ms[s * 3][c - 2] = x;
+    }
+  } else {
+    const int s = (o - n) >> 1;
+    if (s > 0) sh.Xs[(s - 1) * 3][o & 1] = x;
+  }
+}
+template <int MODE>
+__device__ __forceinline__ void sd_one(ScShared& sh, int k, float slope, double* row) {
+  if (k <= SD_OWN_K) sd_pass<MODE, true>(sh.W, sh.r0, sh.r1, k, slope);
+  else sd_pass<MODE, false>(sh.W, sh.r0, sh.r1, k, slope);
+  const SdView d = sd_view(k);
+  const int n4 = 4 * (k + 1), warps = sd_threads(k) / 32;
+  for (int i = threadIdx.x; i < (MODE == 2 ? n4 / 2 : n4); i += SC_T) {
+    const int e = MODE == 2 ? (i >> 1) * 4 + (i & 1) : i, o = MODE == 2 ? n4 + i : i;
+    double s[2] = {0.0, 0.0};
+#pragma unroll
+    for (int w = 0; w < SC_WARPS; ++w) s[w & 1] += w < warps ? d.wsum[(size_t)w * n4 + e] : 0.0;
+    if (row) __stcg(row + o, s[0] + s[1]);
+    else sd_place(sh, k, o, s[0] + s[1]);
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void sd_evaluate(ScShared& sh, int k, float slope, bool last, double* row) {
+  if (!last) {
+    sd_one<0>(sh, k, slope, row);
+  } else {
+    sd_one<1>(sh, k, slope, row);
+    sd_one<2>(sh, k, slope, row);
+  }
+}
+// Sums of all blocks of the layer, which all call (the last warp runs the stop test of the M-step before first, as in
+// sc_evaluate), in the same order in every one of them: slot 0 of Ls, Ms (and, in the last evaluation, Xs); x sums from v_0.  Few
+// rows: every block adds them all up, and the next evaluation's go to a second buffer.  Many: it adds up its share of the sums, and
+// reads the others' after a second barrier.
+constexpr long long SD_ONE_STAGE = 1 << 20;   // doubles that all blocks together may read (8 MB)
+__device__ __noinline__ bool sd_sums(ScShared& sh, const ScalarParams& sp, int layer, bool last, int test) {
+  const SdView d = sd_view(sp.k);
+  if (test > 0 && threadIdx.x >= SC_T - 32) sc_stop_test(sh, sp, layer, test);
+  const int tid = threadIdx.x, k = sp.k, NB = sp.blk_first[layer + 1] - sp.blk_first[layer], b = (int)blockIdx.x - sp.blk_first[layer];
+  const bool alone = NB == 1 && sp.missing_arrivals == 0;
+  const float slope = sh.ly.slope;
+  const unsigned int meet = sh.meet;
+  for (int i = tid; i < 512; i += SC_T) d.v[i] = i < k ? sh.v[i] : __int_as_float(0x7f800000);
+  for (int i = tid; i <= k; i += SC_T) {
+    const double even = i > 0 && i < k ? sh.even[i] : 0.0;
+    const float e = (float)even;
+    d.te[i] = e;
+    d.to[i] = (float)(((double)e - even) * (double)slope);
+  }
+  __syncthreads();
+  if (alone) {
+    sd_evaluate(sh, k, slope, last, nullptr);
+  } else {
+    const int R = SD_SUMS(k), n = last ? R : 4 * (k + 1);
+    const bool one_stage = k <= SD_TWO_ROWS_K && (long long)NB * NB * 4 * k <= SD_ONE_STAGE;
+    const unsigned int arrivals = (unsigned int)(NB + sp.missing_arrivals);
+    unsigned int* sync = sp.p.sync + (size_t)layer * SC_SYNC_WORDS;
+    // rows: [blocks][R], then (one stage) as many again, or the layers' totals, [layers][R]
+    const size_t all = (size_t)gridDim.x * R;
+    double* rows = sp.p.gpart + (size_t)sp.blk_first[layer] * R + ((one_stage && (meet & 1u)) ? all : 0);
+    sd_evaluate(sh, k, slope, last, rows + (size_t)b * R);
+    if (!sc_team_barrier(sync, (meet + 1) * arrivals, sp.spin_limit, &sh.ok, true)) return false;
+    const double* from = rows;
+    int n_rows = NB;
+    if (!one_stage) {
+      double* tot = sp.p.gpart + all + (size_t)layer * R;
+      const int o0 = (int)((long long)n * b / NB), o1 = (int)((long long)n * (b + 1) / NB);
+      for (int o = o0 + (tid >> 5); o < o1; o += SC_WARPS) {
+        double s = 0.0;
+        for (int q = tid & 31; q < NB; q += 32) s += __ldcg(rows + (size_t)q * R + o);
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) s += __shfl_xor_sync(0xffffffffu, s, x);
+        if ((tid & 31) == 0) __stcg(tot + o, s);
+      }
+      if (!sc_team_barrier(sync, (meet + 2) * arrivals, sp.spin_limit, &sh.ok, true)) return false;
+      from = tot;
+      n_rows = 1;
+    }
+    if (tid == 0) sh.meet = meet + (one_stage ? 1u : 2u);   // (read again after the next barriers of the block)
+    // few sums: several threads each
+    const int per = (n >= SC_T || n_rows == 1) ? 1 : SC_T / n;
+    double* part = reinterpret_cast<double*>(d.own);   // (what it holds has been read)
+    for (int o = tid; o < n * per; o += SC_T) {
+      const int e = o % n, c = o / n;
+      double s = 0.0;
+#pragma unroll 8
+      for (int q = c; q < n_rows; q += per) s += __ldcg(from + (size_t)q * R + e);
+      if (per == 1) sd_place(sh, k, e, s);
+      else part[o] = s;
+    }
+    __syncthreads();
+    if (per > 1 && tid < n) {
+      double s = 0.0;
+      for (int c = 0; c < per; ++c) s += part[c * n + tid];
+      sd_place(sh, k, tid, s);
+    }
+    __syncthreads();
+  }
+  for (int j = tid; j < k; j += SC_T) {
+    const double right = (double)sh.v[j] - (double)sh.v[0], left = j > 0 ? (double)sh.v[j - 1] - (double)sh.v[0] : 0.0;
+    sh.Ls[j * 3][1] = fma(right, sh.Ls[j * 3][0], sh.Ls[j * 3][1]);
+    sh.Ms[j * 3][1] = fma(left, sh.Ms[j * 3][0], sh.Ms[j * 3][1]);
+    if (last) sh.Xs[j * 3][1] = fma(right, sh.Xs[j * 3][0], sh.Xs[j * 3][1]);
+  }
+  __syncthreads();
+  return true;
 }
 
 constexpr int SI_T = 1024, SI_WARPS = SI_T / 32;
@@ -951,7 +1217,307 @@ __global__ void __launch_bounds__(SI_T, 1) idkm_scalar_init(const __grid_constan
   }
 }
 
-// LOG: codebooks of at most 2^LOG centroids, whose M-step one warp takes; 0: larger ones.
+// Nothing was computed: report, and leave tables that later passes can read without harm.
+__device__ __noinline__ void sc_give_up(const ScalarParams& sp, int layer, int status) {
+  const int tid = threadIdx.x, k = sp.k, K1 = k + 1;
+  double* tab = sp.p.tab + (size_t)layer * SC_NTAB * K1;
+  float* ft = sp.p.ftab + (size_t)layer * SC_NFTAB * K1;
+  float* Cl = sp.p.C + (size_t)layer * k;
+  LayerState* st = sp.p.st + layer;
+  for (int i = tid; i < SC_NTAB * K1; i += SC_T) tab[i] = 0.0;
+  for (int i = tid; i < SC_NFTAB * K1; i += SC_T) ft[i] = 0.f;
+  const float nan = __int_as_float(0x7fc00000);
+  for (int i = tid; i < k; i += SC_T) {
+    sp.p.perm[(size_t)layer * k + i] = i;
+    sp.p.S[(size_t)layer * k + i] = 0.f;
+    sp.p.F[(size_t)layer * k + i] = status == ST_NONFINITE ? nan : Cl[i];
+    if (status == ST_NONFINITE) Cl[i] = nan;
+  }
+  if (tid == 0) {
+    st->status = status;
+    st->fwd_iters = st->fwd_done = status == ST_NONFINITE ? 1 : 0;
+    st->fwd_res = status == ST_NONFINITE ? nan : 0.f;
+  }
+}
+
+// The iterations of a layer, by its first block, once the bins are there (DIRECT: without bins, by all its blocks alike).  LOG:
+// codebooks of at most 2^LOG centroids, whose M-step one warp takes; 0: larger ones.
+template <int LOG, bool DIRECT>
+__device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, int layer, bool in_smem, const unsigned int* fstart,
+                                        const long long* frec, const unsigned short* grouped) {
+  extern __shared__ __align__(16) unsigned char smem_all[];
+  unsigned char* dyn = smem_all + SC_SH_BYTES;
+  (void)dyn;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = sp.k, K1 = k + 1;
+  const int kw = LOG > 0 ? 1 : (k + 31) >> 5;
+  const int cap = sp.fine_off[layer + 1] - sp.fine_off[layer];
+  double* tab = sp.p.tab + (size_t)layer * SC_NTAB * K1;
+  float* ft = sp.p.ftab + (size_t)layer * SC_NFTAB * K1;
+  LayerState* st = sp.p.st + layer;
+  float* Cl = sp.p.C + (size_t)layer * k;
+  const bool leader = !DIRECT || (int)blockIdx.x == sp.blk_first[layer];   // (all blocks of the layer come to the same results)
+  const ScGrid& g = sh.g;
+  ScLayer ly;
+  ly.grouped = sp.p.grouped;
+  ly.row0 = sp.row_off[layer];
+  ly.total = sp.row_off[sp.n_layers];
+  ly.fstart = fstart;
+  ly.frec = reinterpret_cast<const double*>(frec);
+  ly.k = k;
+  ly.tau = 1.0 / sp.inv_tau_d;
+  ly.inv_tau = sp.inv_tau_d;
+  ly.slope = (float)(2.0 * 1.4426950408889634 * sp.inv_tau_d);
+  ly.zone = SC_ZONE / (double)ly.slope;
+  ly.twl = 0;
+  ly.wl = 0;
+  ly.lpi = k - 1 <= SC_WARPS ? 32 : (k - 1 <= 2 * SC_WARPS ? 16 : 8);
+  while (ly.wl < 1 && (k << (ly.wl + 1)) <= SC_WARPS) ++ly.wl;
+  while (!DIRECT && ly.twl < 2 && k > 1 && ((k - 1) << (ly.twl + 1)) <= SC_WARPS) ++ly.twl;
+  if constexpr (!DIRECT) {
+    // ---- coarse records: into shared memory where they fit; running counts and x sums ----
+    const ScRec gr = sc_global_rec(sp, layer, cap);
+    ly.rec = gr;
+    if (g.nc <= SC_REC_SMEM) {
+      const int stride = g.nc <= SC_SMALL_NC ? SC_SMALL_NC : SC_REC_SMEM;
+      ly.rec.cn = reinterpret_cast<double*>(dyn);
+      ly.rec.cx = ly.rec.cn + stride + 1;
+      ly.rec.r = reinterpret_cast<float*>(ly.rec.cx + stride + 1);
+      ly.rec.stride = stride;
+    }
+    __syncthreads();   // (the counters, which lie in the same place, are no longer read)
+    double carry = 0.0;
+    for (int t = 0; t < g.nc; t += SC_T) {
+      const int c = t + tid;
+      double x = c < g.nc ? __ldcg(gr.cx + c + 1) : 0.0;
+      if (c < g.nc && g.nc <= SC_REC_SMEM) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) ly.rec.r[q * ly.rec.stride + c] = __ldcg(gr.r + (size_t)q * cap + c);
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) sh.scan_x[warp] = x;
+      __syncthreads();
+      double before = 0.0, total = 0.0;
+      for (int w = 0; w < SC_WARPS; ++w) {
+        const double y = sh.scan_x[w];
+        before += w < warp ? y : 0.0;
+        total += y;
+      }
+      if (c < g.nc) {
+        ly.rec.cx[c + 1] = carry + before + x;
+        ly.rec.cn[c + 1] = (double)fstart[(c + 1) << g.fshift];
+      }
+      carry += total;
+      __syncthreads();
+    }
+    if (tid == 0) ly.rec.cx[0] = ly.rec.cn[0] = 0.0;
+    if (in_smem) {
+      ly.row0 = 0;
+      ly.grouped = grouped;
+      ly.total = sp.row_off[layer + 1] - sp.row_off[layer];
+    }
+  }
+  constexpr bool one_warp = LOG > 0;
+  double a = 0.0, ap = 0.0, rP = 0.0, rQ = 0.0;   // (more than 32 centroids)
+  ScScan<LOG> scn;
+#pragma unroll
+  for (int l = 0; l < (LOG > 0 ? LOG : 1); ++l) scn.cb[l] = scn.cf[l] = 0.0;
+  for (int i = tid; i < SC_PARTS * 2; i += SC_T) (&sh.Ls[0][0])[i] = (&sh.Ms[0][0])[i] = (&sh.Xs[0][0])[i] = 0.0;
+  if (tid == 0) {
+    sh.done = 0;
+    sh.iters = 0;
+    sh.dead = 0;
+    sh.status = ST_OK;
+    sh.res = 0.f;
+  }
+  if (tid == 0) sh.ly = ly;
+  auto tables = [&]() {
+    if constexpr (one_warp) {
+      if (warp == 0) sc_tables_warp(sh, ly, lane < k ? sh.v[lane] : sh.v[k - 1], scn, rP, rQ);
+    } else if (tid < kw * 32) {
+      sc_tables_block(sh, ly, a, ap, rP, rQ);
+    }
+  };
+  // sums of the two sides -> what every centroid receives from all intervals
+  auto spread2 = [&](double (&x)[2], double (&y)[2]) {
+    if constexpr (one_warp) {
+      sc_scan_both<2, LOG>(scn, x, y);
+    } else {
+      lin_scan<2, false>(a, x, k, sh.tmp);
+      lin_scan<2, true>(ap, y, k, sh.tmp);
+    }
+  };
+  tables();
+  ScBin keep;
+  keep.f = -1;
+  keep.groups = 0;
+  keep.t0 = keep.t1 = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) keep.pe[i] = 40001;
+  __syncthreads();
+
+  int it = 0;
+  while (it < sp.max_iter) {
+    if constexpr (DIRECT) {
+      if (!sd_sums(sh, sp, layer, false, it)) {
+        if (leader) sc_give_up(sp, layer, ST_TIMEOUT);
+        return;
+      }
+    } else {
+      sc_evaluate<false>(sh, ly, keep, sp, layer, it);
+      __syncthreads();
+    }
+    if (sh.done) break;
+    if (tid < kw * 32) {
+      // ---- M-step (Algorithm 1, step 5) ----
+      const int j = tid;
+      const bool own = j < k;
+      const int jc = own ? j : k - 1;
+      double L0, L1, M0, M1;
+      sc_gather(sh.Ls, jc, ly.twl, L0, L1);
+      sc_gather(sh.Ms, jc, ly.twl, M0, M1);
+      double x[2] = {L0 * rP, L1 * rP}, y[2] = {M0 * rQ, M1 * rQ};   // (rP = rQ = 0 in threads without a centroid)
+      spread2(x, y);
+      const double v0 = (double)sh.v[0], cold = (double)sh.v[jc];
+      const double s = x[0] + y[0];
+      const bool alive = (s >= S_MIN);
+      const double cnew = alive ? fma(x[1] + y[1], sc_rcp(s), v0) : cold;
+      float cn = (float)cnew;
+      if (own) {
+        sh.cnew[j] = cnew;
+        sh.cold[j] = cold;
+        sh.dead_j[j] = (alive ? 0 : 1) + ((!(s == s) || s > 1e300 || !(cnew == cnew) || fabs(cnew) > 1e300) ? 0x10000 : 0);
+      } else {
+        cn = __int_as_float(0x7f800000);
+      }
+      // (the map keeps the order of the centroids up to rounding)
+      float left = __shfl_up_sync(0xffffffffu, cn, 1);
+      bool out_of_order;
+      if constexpr (one_warp) {
+        out_of_order = __any_sync(0xffffffffu, own && j > 0 && !(left <= cn));
+      } else {
+        sc_bar(kw);   // (everybody has read the old centroids)
+        if (own) sh.vn[j] = cn;
+        if (j == 0) sh.flag = 0;
+        sc_bar(kw);
+        if ((j & 31) == 0 && j > 0) left = sh.vn[j - 1];
+        if (own && j > 0 && !(left <= cn)) sh.flag = 1;
+        sc_bar(kw);
+        out_of_order = sh.flag != 0;
+      }
+      if (out_of_order) {
+        if (own) {
+          sh.vn[j] = cn;
+          sh.idn[j] = sh.id[j];
+        }
+        sc_sync(kw);
+        sc_sort(sh, k);
+      } else {
+        if (one_warp) __syncwarp();
+        if (own) sh.v[j] = cn;
+        sc_sync(kw);
+      }
+    }
+    tables();
+    ++it;
+    __syncthreads();
+  }
+
+  // ---- sums at the returned centroids: S, F and the tables of the passes that follow ----
+  if constexpr (DIRECT) {
+    if (!sd_sums(sh, sp, layer, true, (it == sp.max_iter && !sh.done) ? it : 0)) {
+      if (leader) sc_give_up(sp, layer, ST_TIMEOUT);
+      return;
+    }
+    if (!leader) return;
+  } else {
+    sc_evaluate<true>(sh, ly, keep, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
+  }
+  __syncthreads();
+  if (tid < kw * 32) {
+    const bool own = tid < k;
+    const int jc = own ? tid : k - 1;
+    double L0, L1, M0, M1, X0, X1;
+    sc_gather(sh.Ls, jc, ly.twl, L0, L1);
+    sc_gather(sh.Ms, jc, ly.twl, M0, M1);
+    sc_gather(sh.Xs, jc, ly.twl, X0, X1);
+    double x[2] = {L0 * rP, L1 * rP}, y[2] = {M0 * rQ, M1 * rQ};
+    spread2(x, y);
+    // averages of the centroids from every centroid on resp. up to it, relative to v_0
+    const double v0 = (double)sh.v[0], dv = own ? (double)sh.v[tid] - v0 : 0.0;
+    double qp[2] = {dv, 0.0}, pp[2] = {dv, 0.0};
+    spread2(qp, pp);
+    double bad[1] = {0.0};
+    sc_sync(kw);
+    if (own) {
+      const double s = x[0] + y[0];
+      const bool alive = (s >= S_MIN);
+      const double f = alive ? (x[1] + y[1]) / s : dv;
+      if (!(s == s) || s > 1e300 || !(f == f)) bad[0] = 1.0;
+      const int id = sh.id[tid];
+      const size_t lk = (size_t)layer * k;
+      sp.p.perm[lk + tid] = id;
+      Cl[id] = sh.v[tid];
+      sp.p.S[lk + id] = alive ? (float)s : 0.f;
+      sp.p.F[lk + id] = (float)(v0 + f);
+      double* t = tab + tid;
+      t[TB_V * K1] = dv;
+      t[TB_A * K1] = one_warp ? scn.cb[0] : a;
+      t[TB_RP * K1] = rP;
+      t[TB_RQ * K1] = rQ;
+      t[TB_L0 * K1] = L0;
+      t[TB_L1 * K1] = L1;
+      t[TB_M0 * K1] = M0;
+      t[TB_M1 * K1] = M1;
+      t[TB_X0 * K1] = X0;
+      t[TB_X1 * K1] = X1;
+      t[TB_S * K1] = alive ? s : 0.0;
+      t[TB_F * K1] = f;
+      if (tid == 0) tab[TB_V * K1 + k] = v0;
+      sh.qs[tid] = qp[0] * rQ;
+    }
+    sc_sync(kw);
+    if (own) {
+      // interval tid + 1 (and interval 0): the outer ones have their even point far outside
+      const double cl = pp[0] * rP, cr = tid + 1 < k ? sh.qs[tid + 1] : cl;
+      float* o = ft + tid + 1;
+      float e = 3.0e38f, off = 0.f;
+      if (tid + 1 < k) {
+        const double even = sh.even[tid + 1];
+        e = (float)even;
+        off = (float)(((double)e - even) * (double)ly.slope);
+      }
+      ft[FT_V * K1 + tid] = sh.v[tid];
+      o[FT_E * K1] = e;
+      o[FT_O * K1] = off;
+      o[FT_R * K1] = (float)(v0 + cr);
+      o[FT_D * K1] = (float)(cl - cr);
+      if (tid == 0) {
+        ft[FT_E * K1] = -3.0e38f;
+        ft[FT_O * K1] = 0.f;
+        ft[FT_R * K1] = (float)(v0 + sh.qs[0]);
+        ft[FT_D * K1] = 0.f;
+      }
+    }
+    sc_reduce<1>(bad, k, sh.tmp);
+    if (tid == 0) {
+      st->fwd_iters = sh.iters;
+      st->fwd_res = sh.res;
+      st->dead = sh.dead;
+      st->fwd_done = sh.done;
+      st->status = bad[0] > 0.0 ? ST_NONFINITE : sh.status;
+    }
+  }
+}
+template <int LOG>
+__device__ __noinline__ void sd_rest(ScShared& sh, const ScalarParams& sp, int layer) {
+  sc_rest<LOG, true>(sh, sp, layer, false, nullptr, nullptr, nullptr);
+}
+
+// LOG: as above.
 template <int LOG>
 __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constant__ ScalarParams sp) {
   extern __shared__ __align__(16) unsigned char smem_all[];
@@ -985,7 +1551,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
   unsigned int* cnt = reinterpret_cast<unsigned int*>(dyn);
   auto in_smem = [&](const ScGrid& g) {
     return alone && g.nc <= SC_SMALL_NC &&
-           36 * (size_t)g.nf + 64 + 2 * ((size_t)m + 16) + 4 * (size_t)g.nf <= (size_t)(SC_DYN - SC_SH_BYTES - SC_SMALL_OFF);
+           36 * (size_t)g.nf + 64 + 2 * ((size_t)m + 16) + 4 * (size_t)g.nf <= (size_t)(SC_BIN_BYTES - SC_SMALL_OFF);
   };
   grid_dependency_sync();
   if (warp == 0) {
@@ -1013,10 +1579,11 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
   }
   __syncthreads();
   int status = ST_OK;
+  bool direct = sh.g.eta > SC_ETA_MAX;   // (uniform over the layer's blocks, as all that is read here and below)
   if (sh.bad) {
-    status = ST_NONFINITE;   // NaN or Inf among the weights (uniform over the layer's blocks)
+    status = ST_NONFINITE;   // NaN or Inf among the weights
     if (b != 0) return;
-  } else {
+  } else if (!direct) {
     const ScGrid g = sh.g;
     const int nf = g.nf;
     bool ok = true;
@@ -1025,7 +1592,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
       frec = reinterpret_cast<long long*>(dyn + SC_SMALL_OFF);
       fstart = reinterpret_cast<unsigned int*>(frec + 4 * (size_t)nf);
       grouped = reinterpret_cast<unsigned short*>(fstart + ((nf + 4) & ~3));
-      cnt = reinterpret_cast<unsigned int*>(dyn + (SC_DYN - SC_SH_BYTES)) - ((nf + 3) & ~3);
+      cnt = reinterpret_cast<unsigned int*>(dyn + SC_BIN_BYTES) - ((nf + 3) & ~3);
     }
     // ---- count the block's weights per fine bin ----
     for (int i = tid; i < nf; i += SC_T) cnt[i] = 0u;
@@ -1057,7 +1624,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
     constexpr unsigned int BIG = 4 * SC_CHUNK;
     if (ok) {
       // ---- first element of every bin: exclusive prefix over the bins, four per thread and round ----
-      unsigned int carry = 0;
+      unsigned int carry = 0, most = 0;
       auto fetch = [&](int i) {
         uint4 c = make_uint4(0u, 0u, 0u, 0u);
         if (i < nf) {
@@ -1075,6 +1642,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
         const uint4 c = next;
         if (NB > 1) next = fetch(i + 4 * SC_T);
         const unsigned int sum = c.x + c.y + c.z + c.w;
+        most = max(max(most, max(c.x, c.y)), max(c.z, c.w));
         unsigned int x = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1118,6 +1686,9 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
         if (NB == 1) next = fetch(i + 4 * SC_T);
       }
       if (b == 0 && tid == 0) fstart[nf] = carry;
+      direct = __syncthreads_or((long long)most > SC_CROWD + m / 256) != 0;
+    }
+    if (ok && !direct) {
       // ---- group the weights' places by fine bin ----
       auto put = [&](float w) {
         if (w == 0.f) return;
@@ -1136,7 +1707,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
       for (; r < r1; r += SC_T) put(__ldg(Wl + r));
       ok = barrier(true);
     }
-    if (ok) {
+    if (ok && !direct) {
       // ---- integer sums of powers of the places, per fine bin; groups of 32 bins are dealt to the layer's warps ----
       if (NB > 1) {
         for (int i = tid; i < nf; i += SC_T) cnt[i] = __ldcg(fstart + i + 1);
@@ -1268,7 +1839,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
       }
       ok = barrier(true);
     }
-    if (ok) {
+    if (ok && !direct) {
       // ---- moments about the coarse bins' centres, prefixed over the fine bins of every coarse bin; coarse records ----
       const ScRec gr = sc_global_rec(sp, layer, cap);
       const int wd = g.F < 32 ? g.F : 32;      // lanes per coarse bin
@@ -1315,9 +1886,15 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
     }
     if (!ok) status = ST_TIMEOUT;
   }
-  if (b != 0) return;
+  if (tid == 0) {
+    sh.meet = meet;
+    sh.W = Wl;
+    sh.r0 = r0;
+    sh.r1 = r1;
+  }
+  if (b != 0 && !(direct && status == ST_OK)) return;
 
-  // ================= from here on one block per layer =================
+  // ================= from here on one block per layer (or all, without bins) =================
   const int kw = LOG > 0 ? 1 : (k + 31) >> 5;
   if (tid < kw * 32) {
     if (tid < k) {
@@ -1327,267 +1904,15 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
     sc_sync(kw);
     sc_sort(sh, k);
   }
-  const int K1 = k + 1;
-  double* tab = sp.p.tab + (size_t)layer * SC_NTAB * K1;
-  float* ft = sp.p.ftab + (size_t)layer * SC_NFTAB * K1;
   if (status != ST_OK) {
-    // nothing was computed: report, and leave tables that later passes can read without harm
-    for (int i = tid; i < SC_NTAB * K1; i += SC_T) tab[i] = 0.0;
-    for (int i = tid; i < SC_NFTAB * K1; i += SC_T) ft[i] = 0.f;
-    const float nan = __int_as_float(0x7fc00000);
-    for (int i = tid; i < k; i += SC_T) {
-      sp.p.perm[(size_t)layer * k + i] = i;
-      sp.p.S[(size_t)layer * k + i] = 0.f;
-      sp.p.F[(size_t)layer * k + i] = status == ST_NONFINITE ? nan : sh.vn[i];
-      if (status == ST_NONFINITE) Cl[i] = nan;
-    }
-    if (tid == 0) {
-      st->status = status;
-      st->fwd_iters = st->fwd_done = status == ST_NONFINITE ? 1 : 0;
-      st->fwd_res = status == ST_NONFINITE ? nan : 0.f;
-    }
+    sc_give_up(sp, layer, status);
     return;
   }
-  const ScGrid& g = sh.g;
-  ScLayer ly;
-  ly.grouped = sp.p.grouped;
-  ly.row0 = sp.row_off[layer];
-  ly.total = sp.row_off[sp.n_layers];
-  ly.fstart = fstart;
-  ly.frec = reinterpret_cast<const double*>(frec);
-  ly.k = k;
-  ly.tau = 1.0 / sp.inv_tau_d;
-  ly.inv_tau = sp.inv_tau_d;
-  ly.slope = (float)(2.0 * 1.4426950408889634 * sp.inv_tau_d);
-  ly.zone = SC_ZONE / (double)ly.slope;
-  ly.twl = 0;
-  ly.wl = 0;
-  ly.lpi = k - 1 <= SC_WARPS ? 32 : (k - 1 <= 2 * SC_WARPS ? 16 : 8);
-  while (ly.wl < 1 && (k << (ly.wl + 1)) <= SC_WARPS) ++ly.wl;
-  while (ly.twl < 2 && k > 1 && ((k - 1) << (ly.twl + 1)) <= SC_WARPS) ++ly.twl;
-  {
-    // ---- coarse records: into shared memory where they fit; running counts and x sums ----
-    const ScRec gr = sc_global_rec(sp, layer, cap);
-    ly.rec = gr;
-    if (g.nc <= SC_REC_SMEM) {
-      const int stride = g.nc <= SC_SMALL_NC ? SC_SMALL_NC : SC_REC_SMEM;
-      ly.rec.cn = reinterpret_cast<double*>(dyn);
-      ly.rec.cx = ly.rec.cn + stride + 1;
-      ly.rec.r = reinterpret_cast<float*>(ly.rec.cx + stride + 1);
-      ly.rec.stride = stride;
-    }
-    __syncthreads();   // (the counters, which lie in the same place, are no longer read)
-    double carry = 0.0;
-    for (int t = 0; t < g.nc; t += SC_T) {
-      const int c = t + tid;
-      double x = c < g.nc ? __ldcg(gr.cx + c + 1) : 0.0;
-      if (c < g.nc && g.nc <= SC_REC_SMEM) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) ly.rec.r[q * ly.rec.stride + c] = __ldcg(gr.r + (size_t)q * cap + c);
-      }
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-      }
-      if (lane == 31) sh.scan_x[warp] = x;
-      __syncthreads();
-      double before = 0.0, total = 0.0;
-      for (int w = 0; w < SC_WARPS; ++w) {
-        const double y = sh.scan_x[w];
-        before += w < warp ? y : 0.0;
-        total += y;
-      }
-      if (c < g.nc) {
-        ly.rec.cx[c + 1] = carry + before + x;
-        ly.rec.cn[c + 1] = (double)fstart[(c + 1) << g.fshift];
-      }
-      carry += total;
-      __syncthreads();
-    }
-    if (tid == 0) ly.rec.cx[0] = ly.rec.cn[0] = 0.0;
-    if (in_smem(g)) {
-      ly.row0 = 0;
-      ly.grouped = grouped;
-      ly.total = m;
-    }
+  if (direct) {
+    sd_rest<LOG>(sh, sp, layer);
+    return;
   }
-  constexpr bool one_warp = LOG > 0;
-  double a = 0.0, ap = 0.0, rP = 0.0, rQ = 0.0;   // (more than 32 centroids)
-  ScScan<LOG> scn;
-#pragma unroll
-  for (int l = 0; l < (LOG > 0 ? LOG : 1); ++l) scn.cb[l] = scn.cf[l] = 0.0;
-  for (int i = tid; i < SC_PARTS * 2; i += SC_T) (&sh.Ls[0][0])[i] = (&sh.Ms[0][0])[i] = (&sh.Xs[0][0])[i] = 0.0;
-  if (tid == 0) {
-    sh.done = 0;
-    sh.iters = 0;
-    sh.dead = 0;
-    sh.status = ST_OK;
-    sh.res = 0.f;
-  }
-  if (tid == 0) sh.ly = ly;
-  auto tables = [&]() {
-    if constexpr (one_warp) {
-      if (warp == 0) sc_tables_warp(sh, ly, lane < k ? sh.v[lane] : sh.v[k - 1], scn, rP, rQ);
-    } else if (tid < kw * 32) {
-      sc_tables_block(sh, ly, a, ap, rP, rQ);
-    }
-  };
-  // sums of the two sides -> what every centroid receives from all intervals
-  auto spread2 = [&](double (&x)[2], double (&y)[2]) {
-    if constexpr (one_warp) {
-      sc_scan_both<2, LOG>(scn, x, y);
-    } else {
-      lin_scan<2, false>(a, x, k, sh.tmp);
-      lin_scan<2, true>(ap, y, k, sh.tmp);
-    }
-  };
-  tables();
-  ScBin keep;
-  keep.f = -1;
-  keep.groups = 0;
-  keep.t0 = keep.t1 = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) keep.pe[i] = 40001;
-  __syncthreads();
-
-  int it = 0;
-  while (it < sp.max_iter) {
-    sc_evaluate<false>(sh, ly, keep, sp, layer, it);
-    __syncthreads();
-    if (sh.done) break;
-    if (tid < kw * 32) {
-      // ---- M-step (Algorithm 1, step 5) ----
-      const int j = tid;
-      const bool own = j < k;
-      const int jc = own ? j : k - 1;
-      double L0, L1, M0, M1;
-      sc_gather(sh.Ls, jc, ly.twl, L0, L1);
-      sc_gather(sh.Ms, jc, ly.twl, M0, M1);
-      double x[2] = {L0 * rP, L1 * rP}, y[2] = {M0 * rQ, M1 * rQ};   // (rP = rQ = 0 in threads without a centroid)
-      spread2(x, y);
-      const double v0 = (double)sh.v[0], cold = (double)sh.v[jc];
-      const double s = x[0] + y[0];
-      const bool alive = (s >= S_MIN);
-      const double cnew = alive ? fma(x[1] + y[1], sc_rcp(s), v0) : cold;
-      float cn = (float)cnew;
-      if (own) {
-        sh.cnew[j] = cnew;
-        sh.cold[j] = cold;
-        sh.dead_j[j] = (alive ? 0 : 1) + ((!(s == s) || s > 1e300 || !(cnew == cnew) || fabs(cnew) > 1e300) ? 0x10000 : 0);
-      } else {
-        cn = __int_as_float(0x7f800000);
-      }
-      // (the map keeps the order of the centroids up to rounding)
-      float left = __shfl_up_sync(0xffffffffu, cn, 1);
-      bool out_of_order;
-      if constexpr (one_warp) {
-        out_of_order = __any_sync(0xffffffffu, own && j > 0 && !(left <= cn));
-      } else {
-        sc_bar(kw);   // (everybody has read the old centroids)
-        if (own) sh.vn[j] = cn;
-        if (j == 0) sh.flag = 0;
-        sc_bar(kw);
-        if ((j & 31) == 0 && j > 0) left = sh.vn[j - 1];
-        if (own && j > 0 && !(left <= cn)) sh.flag = 1;
-        sc_bar(kw);
-        out_of_order = sh.flag != 0;
-      }
-      if (out_of_order) {
-        if (own) {
-          sh.vn[j] = cn;
-          sh.idn[j] = sh.id[j];
-        }
-        sc_sync(kw);
-        sc_sort(sh, k);
-      } else {
-        if (one_warp) __syncwarp();
-        if (own) sh.v[j] = cn;
-        sc_sync(kw);
-      }
-    }
-    tables();
-    ++it;
-    __syncthreads();
-  }
-
-  // ---- sums at the returned centroids: S, F and the tables of the passes that follow ----
-  sc_evaluate<true>(sh, ly, keep, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
-  __syncthreads();
-  if (tid < kw * 32) {
-    const bool own = tid < k;
-    const int jc = own ? tid : k - 1;
-    double L0, L1, M0, M1, X0, X1;
-    sc_gather(sh.Ls, jc, ly.twl, L0, L1);
-    sc_gather(sh.Ms, jc, ly.twl, M0, M1);
-    sc_gather(sh.Xs, jc, ly.twl, X0, X1);
-    double x[2] = {L0 * rP, L1 * rP}, y[2] = {M0 * rQ, M1 * rQ};
-    spread2(x, y);
-    // averages of the centroids from every centroid on resp. up to it, relative to v_0
-    const double v0 = (double)sh.v[0], dv = own ? (double)sh.v[tid] - v0 : 0.0;
-    double qp[2] = {dv, 0.0}, pp[2] = {dv, 0.0};
-    spread2(qp, pp);
-    double bad[1] = {0.0};
-    sc_sync(kw);
-    if (own) {
-      const double s = x[0] + y[0];
-      const bool alive = (s >= S_MIN);
-      const double f = alive ? (x[1] + y[1]) / s : dv;
-      if (!(s == s) || s > 1e300 || !(f == f)) bad[0] = 1.0;
-      const int id = sh.id[tid];
-      const size_t lk = (size_t)layer * k;
-      sp.p.perm[lk + tid] = id;
-      Cl[id] = sh.v[tid];
-      sp.p.S[lk + id] = alive ? (float)s : 0.f;
-      sp.p.F[lk + id] = (float)(v0 + f);
-      double* t = tab + tid;
-      t[TB_V * K1] = dv;
-      t[TB_A * K1] = one_warp ? scn.cb[0] : a;
-      t[TB_RP * K1] = rP;
-      t[TB_RQ * K1] = rQ;
-      t[TB_L0 * K1] = L0;
-      t[TB_L1 * K1] = L1;
-      t[TB_M0 * K1] = M0;
-      t[TB_M1 * K1] = M1;
-      t[TB_X0 * K1] = X0;
-      t[TB_X1 * K1] = X1;
-      t[TB_S * K1] = alive ? s : 0.0;
-      t[TB_F * K1] = f;
-      if (tid == 0) tab[TB_V * K1 + k] = v0;
-      sh.qs[tid] = qp[0] * rQ;
-    }
-    sc_sync(kw);
-    if (own) {
-      // interval tid + 1 (and interval 0): the outer ones have their even point far outside
-      const double cl = pp[0] * rP, cr = tid + 1 < k ? sh.qs[tid + 1] : cl;
-      float* o = ft + tid + 1;
-      float e = 3.0e38f, off = 0.f;
-      if (tid + 1 < k) {
-        const double even = sh.even[tid + 1];
-        e = (float)even;
-        off = (float)(((double)e - even) * (double)ly.slope);
-      }
-      ft[FT_V * K1 + tid] = sh.v[tid];
-      o[FT_E * K1] = e;
-      o[FT_O * K1] = off;
-      o[FT_R * K1] = (float)(v0 + cr);
-      o[FT_D * K1] = (float)(cl - cr);
-      if (tid == 0) {
-        ft[FT_E * K1] = -3.0e38f;
-        ft[FT_O * K1] = 0.f;
-        ft[FT_R * K1] = (float)(v0 + sh.qs[0]);
-        ft[FT_D * K1] = 0.f;
-      }
-    }
-    sc_reduce<1>(bad, k, sh.tmp);
-    if (tid == 0) {
-      st->fwd_iters = sh.iters;
-      st->fwd_res = sh.res;
-      st->dead = sh.dead;
-      st->fwd_done = sh.done;
-      st->status = bad[0] > 0.0 ? ST_NONFINITE : sh.status;
-    }
-  }
+  sc_rest<LOG, false>(sh, sp, layer, in_smem(sh.g), fstart, frec, grouped);
 }
 
 cudaError_t launch_scalar_init(const ScalarParams& sp, int grid, cudaStream_t stream) {
