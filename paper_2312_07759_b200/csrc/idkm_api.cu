@@ -613,11 +613,16 @@ static long long deal_blocks(const idkm_ctx* ctx, int grid, SmallLoopParams* sp)
   return most;
 }
 
+// Tuning knob: always a launch per iteration (and scalar weights in pairs with the centroids).
+static bool no_coop() {
+  static const bool off = (getenv("IDKM_NO_COOP") != nullptr);
+  return off;
+}
+
 // Returns IDKM_OK after queueing the loop, 1 if this problem should take the launch-per-iteration path.
 static int try_small_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, int max_iter) {
-  static const bool env_off = (getenv("IDKM_NO_COOP") != nullptr);   // tuning knob: always a launch per iteration
   // (the loop kernel steps a collapsing layer in the fp32 increment form; the fp64 step exists as launches only)
-  if (env_off || ctx->forward_loop != 0 || max_iter < 2 || ctx->squared || ctx->collapse_step != 0)
+  if (no_coop() || ctx->forward_loop != 0 || max_iter < 2 || ctx->squared || ctx->collapse_step != 0)
     return 1;
   const int di = d_index(ctx->d);
   int f = -1;
@@ -695,8 +700,7 @@ constexpr long long MMA_LOOP_ONE_STAGE = 500000;
 
 // Returns IDKM_OK after queueing the loop, 1 if this problem should take the launch-per-iteration path.
 static int try_mma_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, int max_iter) {
-  static const bool env_off = (getenv("IDKM_NO_COOP") != nullptr);
-  if (env_off || ctx->forward_loop != 0 || max_iter < 2 || (!ctx->squared && ctx->collapse_step != 0)) return 1;
+  if (no_coop() || ctx->forward_loop != 0 || max_iter < 2 || (!ctx->squared && ctx->collapse_step != 0)) return 1;
   const MmaLoopEntry* e = mma_loop_entry(ctx->d, ctx->k, ctx->squared != 0);
   if (!e || !e->launch || ctx->k * ctx->d <= 32) return 1;
   // (Batches keep a launch per iteration and with it their sums' order, bit for bit: among a network's layers there are small
@@ -815,7 +819,7 @@ constexpr long long SCALAR_GRAD_ROWS = 256;     // weights a thread of the gradi
 // Initialises the call and runs the forward loop in the interval form.  IDKM_OK after queueing it, 1 if this problem
 // takes another path.  scratch: room for two bytes per weight.
 static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassParams& p, const float* C0, int max_iter, void* scratch) {
-  if (wl.sc_fine == 0 || ctx->squared || ctx->forward_loop != 0 || ctx->collapse_step != 0 || max_iter < 2 || scratch == nullptr ||
+  if (no_coop() || wl.sc_fine == 0 || ctx->squared || ctx->forward_loop != 0 || ctx->collapse_step != 0 || max_iter < 2 || scratch == nullptr ||
       ctx->n_layers > ctx->sms)
     return 1;
   // Few weights and a cold softmax: the bins are nearly as many as the weights, and summarising them costs more than the
