@@ -752,7 +752,7 @@ static cudaError_t launch_mma_loop(const MmaLoopParams& p, int grid, cudaStream_
 //          k = 256: 16 x 16 16.5 / 24.2 / 181 / 680, 8 x 32 13.4 / 22 / 195 / 749, matrix 15.7 / 24 / 199 / 764 (18 / 31 / 192 / 704)
 // (a matrix instruction holds the fp32 pipe for 8 cycles -- mma and three packed multiply-adds: 13.7 cycles, alone 8.2 and
 // 5.7 -- so at d = 2, where a pair has three sums instead of five, it does not pay)
-#define IDKM_LOOP_ROW_2(SQ, LAST) { IDKM_GRP(2, 8, 2, SQ), IDKM_GRP(2, 16, 2, SQ), IDKM_GRP(2, 16, 4, SQ), IDKM_GRP(2, 16, 8, SQ), LAST }
+#define IDKM_LOOP_ROW_2(SQ, LAST) { { nullptr, 0, 0 }, IDKM_GRP(2, 16, 2, SQ), IDKM_GRP(2, 16, 4, SQ), IDKM_GRP(2, 16, 8, SQ), LAST }
 #define IDKM_LOOP_ROW_4(SQ) { IDKM_GRP(4, 8, 2, SQ), IDKM_GRP(4, 8, 4, SQ), IDKM_MML(4, SQ), IDKM_MML(8, SQ), IDKM_MML(16, SQ) }
 
 }  // namespace idkm
