@@ -336,14 +336,20 @@ struct idkm_ctx {
   int d, k, n_layers;
   float tau;
   long long row_off[MAX_LAYERS + 1];
+  bool in_groups;        // the layers of this call are part of a larger batch, whose routes they take:
+  int64_t batch_m;       // its rows,
+  bool batch_jac;        // and whether its adjoint may run on the tensor-core Jacobian
+  // a call on host buffers may have run in groups of layers, each with a workspace of its own
+  struct Part { void* ws; int64_t m; int l0, n; } parts[HOST_GROUPS_MAX];
+  int n_parts;           // 0: the last forward's workspace has all layers
   cudaStream_t stream;
   int occupancy[2][N_MODES][3][N_FAMILY];   // cached blocks/SM per kernel ([1]: squared-distance variants), 0 = not queried
   // device buffers, streams and events of the host-pointer entry point
   void* hbuf;
   size_t hbuf_bytes;
-  bool host_streams_ok;
-  cudaStream_t hs_compute, hs_copy, hs_down;
+  cudaStream_t hs_compute, hs_copy, hs_down;   // null until the first such call
   cudaEvent_t hev[4 * HOST_GROUPS_MAX];   // per group of layers: W there, G there, forward done, backward done
+  int n_hev;                              // of which exist
   // optional phase timing (CUDA events on the call's stream)
   bool timing;
   bool ev_ok;
@@ -644,16 +650,17 @@ static int try_small_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPa
   const int L = ctx->n_layers;
   const long long m = ctx->m_total;
   if (L > nb || L > MAX_LAYERS) return 1;
-  const int per_thread = L > 1 ? SMALL_BATCH_ROWS_PER_THREAD : (ctx->d == 4 ? SMALL_ROWS_PER_THREAD_D4 : SMALL_ROWS_PER_THREAD);
-  if (m > (long long)per_thread * nb * BLOCK) return 1;
+  const int per_thread = (L > 1 || ctx->in_groups) ? SMALL_BATCH_ROWS_PER_THREAD : (ctx->d == 4 ? SMALL_ROWS_PER_THREAD_D4 : SMALL_ROWS_PER_THREAD);
+  const long long batch = ctx->in_groups ? ctx->batch_m : m;
+  if (batch > (long long)per_thread * nb * BLOCK) return 1;
   // (weights that do not stay in L2 are faster by a launch per iteration, whose kernels keep more loads in flight:
   // 16 x 1 M rows at d = 2, k = 2: 68 against 38 us per iteration; 8 x 1 M at d = 4, k = 2: 65 against 41 us)
-  if (m * ctx->d > SMALL_MAX_FLOATS) return 1;
+  if (batch * ctx->d > SMALL_MAX_FLOATS) return 1;
   long long grid = (m + (long long)SMALL_MIN_ROWS_PER_THREAD * BLOCK - 1) / ((long long)SMALL_MIN_ROWS_PER_THREAD * BLOCK);
   if (grid > nb) grid = nb;
   // a single layer of a few thousand weights: one block, which then skips the partial buffers and the barrier
   // (m = 4096, d = 1, k = 4: 2.6 against 4.7 us per iteration on four blocks; d = 4, k = 8 at that size is faster spread out)
-  if (L == 1 && m <= SMALL_SOLO_ROWS && m * ctx->k * ctx->d <= SMALL_SOLO_WORK) grid = 1;
+  if (L == 1 && !ctx->in_groups && m <= SMALL_SOLO_ROWS && m * ctx->k * ctx->d <= SMALL_SOLO_WORK) grid = 1;
   if (grid < L) grid = L;
   if (2 * grid > wl.max_slots) return 1;   // the two partial buffers live in the partial-slot region
   SmallLoopParams sp;
@@ -706,7 +713,7 @@ static int try_mma_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPara
   // (Batches keep a launch per iteration and with it their sums' order, bit for bit: among a network's layers there are small
   // cold ones -- 2048 quadruples, k = 16, a spread of 350 tau -- that turn one rounding into 1e-5 of a centroid, and where the
   // adjoint iteration of such a layer diverges, 1e-2 of its gradient.  A ResNet-18's, d = 4, k = 16: 64 us an iteration against 51.)
-  if (ctx->n_layers > 1) return 1;
+  if (ctx->n_layers > 1 || ctx->in_groups) return 1;
   int grid = ctx->sms;
   const long long most = (ctx->m_total + MMA_LOOP_ROWS - 1) / MMA_LOOP_ROWS;
   if (grid > most) grid = (int)most;
@@ -827,7 +834,7 @@ static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassP
   // backward, spread 0.03, one-launch loop over the weights against this one: m = 4096, k = 4: tau = 0.05 128 against 115 us,
   // 0.01 103 against 119, 5e-4 104 against 146; m = 8192, k = 16: 5e-4 185 against 222, 2e-3 faster here.)
   const bool cold = (ctx->m_total <= 4096 && ctx->k <= 4 && ctx->tau < 0.03f) || (ctx->m_total <= 16384 && ctx->k <= 16 && ctx->tau < 1e-3f);
-  if (ctx->n_layers == 1 && cold) return 1;
+  if (ctx->n_layers == 1 && !ctx->in_groups && cold) return 1;
   for (int l = 0; l < ctx->n_layers; ++l)
     if (ctx->row_off[l + 1] - ctx->row_off[l] > 0x7fffffffLL) return 1;
   ScalarParams sp;
@@ -997,12 +1004,10 @@ int idkm_create(idkm_ctx** out) {
 void idkm_destroy(idkm_ctx* ctx) {
   if (!ctx) return;
   if (ctx->hbuf) cudaFree(ctx->hbuf);
-  if (ctx->host_streams_ok) {
-    for (int i = 0; i < 4 * HOST_GROUPS_MAX; ++i) cudaEventDestroy(ctx->hev[i]);
-    cudaStreamDestroy(ctx->hs_compute);
-    cudaStreamDestroy(ctx->hs_copy);
-    cudaStreamDestroy(ctx->hs_down);
-  }
+  for (int i = 0; i < ctx->n_hev; ++i) cudaEventDestroy(ctx->hev[i]);
+  if (ctx->hs_compute) cudaStreamDestroy(ctx->hs_compute);
+  if (ctx->hs_copy) cudaStreamDestroy(ctx->hs_copy);
+  if (ctx->hs_down) cudaStreamDestroy(ctx->hs_down);
   if (ctx->chunk_ev_ok) {
     cudaEventDestroy(ctx->chunk_ev[0]);
     cudaEventDestroy(ctx->chunk_ev[1]);
@@ -1039,6 +1044,7 @@ int idkm_forward_batched(idkm_ctx* ctx, const float* W_cat, const int64_t* layer
   if (workspace_bytes < wl.total) return IDKM_ERR_WORKSPACE;
 
   ctx->have_forward = false;
+  ctx->n_parts = 0;
   ctx->W = W_cat;
   ctx->C = C_out;
   ctx->workspace = workspace;
@@ -1133,7 +1139,8 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
   const bool explicit_jac = exact || (ctx->adjoint_method == 0 && !ctx->squared && fj >= 0 &&
                                       (!jac_tile || adj_max_iter >= JAC_TILE_MIN_ITERS));
   // the per-row softmax reference and normaliser are kept only if fused adjoint passes follow
-  const bool jac_mma = solve && ctx->adjoint_method == 0 && !ctx->squared && wl.jm.nt > 0 && adj_max_iter >= jac_mma_min_iters(ctx->d, ctx->k);
+  const bool jac_mma = solve && ctx->adjoint_method == 0 && !ctx->squared && wl.jm.nt > 0 && (!ctx->in_groups || ctx->batch_jac) &&
+                       adj_max_iter >= jac_mma_min_iters(ctx->d, ctx->k);
   if (!solve || (explicit_jac && !jac_mma)) p.rowstat = nullptr;
   mark(ctx, 4);
   // scalar weights whose forward left its interval tables: gradient, adjoint and dL/dW in the interval form, unless the
@@ -1199,16 +1206,44 @@ int idkm_backward_restart(idkm_ctx* ctx, const float* dWq, float adj_tol, int ad
   return backward_outputs(ctx, wl, &p, ctx->scalar_forward && ctx->adjoint_method == 0, dW_out, dC_out);
 }
 
+// The workspace that holds a layer of the last call: its layout, its base, and the layer's place in it.
+static bool layer_place(const idkm_ctx* ctx, int layer, WorkspaceLayout* wl, const char** ws, int* at) {
+  if (ctx->n_parts == 0) {
+    *ws = static_cast<const char*>(ctx->workspace);
+    *at = layer;
+    return make_layout(ctx->m_total, ctx->d, ctx->k, ctx->n_layers, ctx->sms, wl);
+  }
+  for (int i = 0; i < ctx->n_parts; ++i) {
+    const idkm_ctx::Part& q = ctx->parts[i];
+    if (layer >= q.l0 && layer < q.l0 + q.n) {
+      *ws = static_cast<const char*>(q.ws);
+      *at = layer - q.l0;
+      return make_layout(q.m, ctx->d, ctx->k, q.n, ctx->sms, wl);
+    }
+  }
+  return false;
+}
+static int read_states(const idkm_ctx* ctx, LayerState* host) {
+  for (int l = 0; l < ctx->n_layers;) {
+    WorkspaceLayout wl;
+    const char* ws;
+    int at, n = ctx->n_layers;
+    if (!layer_place(ctx, l, &wl, &ws, &at)) return IDKM_ERR_UNSUPPORTED;
+    for (int i = 0; i < ctx->n_parts; ++i)
+      if (ctx->parts[i].ws == ws) n = ctx->parts[i].n;
+    if (cudaMemcpy(host + l, ws + wl.off_state, sizeof(LayerState) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess) return IDKM_ERR_CUDA;
+    l += n;
+  }
+  return IDKM_OK;
+}
+
 int idkm_get_info(idkm_ctx* ctx, idkm_info* info_out) {
   if (!ctx || !info_out) return IDKM_ERR_NULL;
   if (!ctx->have_forward) return IDKM_ERR_ORDER;
-  WorkspaceLayout wl;
-  if (!make_layout(ctx->m_total, ctx->d, ctx->k, ctx->n_layers, ctx->sms, &wl)) return IDKM_ERR_UNSUPPORTED;
   LayerState host[MAX_LAYERS];
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
-  if (cudaMemcpy(host, static_cast<char*>(ctx->workspace) + wl.off_state, sizeof(LayerState) * (size_t)ctx->n_layers,
-                 cudaMemcpyDeviceToHost) != cudaSuccess)
-    return IDKM_ERR_CUDA;
+  const int rc = read_states(ctx, host);
+  if (rc != IDKM_OK) return rc;
   for (int l = 0; l < ctx->n_layers; ++l) {
     info_out[l].status = host[l].status;
     info_out[l].fwd_iters = host[l].fwd_iters;
@@ -1245,10 +1280,7 @@ struct HostGroup {
   }
 };
 constexpr size_t HOST_GROUP_BYTES = 12u << 20;   // weights of a group at least: 0.2 ms of the link, more than its launches cost
-static int host_groups(const idkm_ctx* ctx, const int64_t* offs, int n_layers, size_t wn, HostGroup* grp) {
-  // (phase times are of one batch)
-  int want = ctx->timing ? 1 : (int)(wn / HOST_GROUP_BYTES);
-  if (want > HOST_GROUPS_MAX) want = HOST_GROUPS_MAX;
+static int host_groups(const int64_t* offs, int n_layers, int want, HostGroup* grp) {
   int n = 0, l = 0;
   while (l < n_layers) {
     grp[n].l0 = l;
@@ -1274,57 +1306,51 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
   if (m < 1) return IDKM_ERR_SHAPE;
   for (int l = 0; l < n_layers; ++l)
     if (layer_offsets[l + 1] <= layer_offsets[l]) return IDKM_ERR_SHAPE;
-  const size_t ws_bytes = idkm_workspace_bytes(m, d, k, n_layers);
-  if (ws_bytes == 0) return IDKM_ERR_UNSUPPORTED;
+  if (idkm_workspace_bytes(m, d, k, n_layers) == 0) return IDKM_ERR_UNSUPPORTED;
   const bool also_jfb = (dW_jfb_out_host != nullptr || dC_jfb_out_host != nullptr) && mode == IDKM_IMPLICIT;
   const size_t wn = sizeof(float) * (size_t)m * d, cn = sizeof(float) * (size_t)n_layers * k * d;
   HostGroup grp[HOST_GROUPS_MAX];
-  const int ng = host_groups(ctx, layer_offsets, n_layers, wn, grp);
-  // each group's W, G, Wq, dW, dW (Jacobian-free), C0, C, dC, dC (Jacobian-free), workspace; the whole call's workspace
-  size_t need = ng > 1 ? align_up(ws_bytes, 256) : 0;
-  for (int g = 0; g < ng; ++g) {
-    HostGroup& q = grp[g];
-    q.m = layer_offsets[q.l1] - layer_offsets[q.l0];
-    q.wn = sizeof(float) * (size_t)q.m * d;
-    q.cn = sizeof(float) * (size_t)(q.l1 - q.l0) * k * d;
-    q.ws_bytes = idkm_workspace_bytes(q.m, d, k, q.l1 - q.l0);
-    if (q.ws_bytes == 0) return IDKM_ERR_UNSUPPORTED;
-    q.off = need;
-    need += 5 * align_up(q.wn, 256) + 4 * align_up(q.cn, 256) + align_up(q.ws_bytes, 256);
-  }
-  if (need > ctx->hbuf_bytes) {
+  int ng = 0, want = ctx->timing ? 1 : (int)(wn / HOST_GROUP_BYTES);   // (phase times are of one batch)
+  if (want > HOST_GROUPS_MAX) want = HOST_GROUPS_MAX;
+  // What several groups need besides one batch is their workspaces; where the device has not that much left, the call is one batch.
+  for (;; want = 1) {
+    ng = host_groups(layer_offsets, n_layers, want, grp);
+    size_t need = 0;   // each group's W, G, Wq, dW, dW (Jacobian-free), C0, C, dC, dC (Jacobian-free), workspace
+    for (int g = 0; g < ng; ++g) {
+      HostGroup& q = grp[g];
+      q.m = layer_offsets[q.l1] - layer_offsets[q.l0];
+      q.wn = sizeof(float) * (size_t)q.m * d;
+      q.cn = sizeof(float) * (size_t)(q.l1 - q.l0) * k * d;
+      q.ws_bytes = idkm_workspace_bytes(q.m, d, k, q.l1 - q.l0);
+      if (q.ws_bytes == 0) return IDKM_ERR_UNSUPPORTED;
+      q.off = need;
+      need += 5 * align_up(q.wn, 256) + 4 * align_up(q.cn, 256) + align_up(q.ws_bytes, 256);
+    }
+    if (need <= ctx->hbuf_bytes) break;
     if (ctx->hbuf) cudaFree(ctx->hbuf);
     ctx->hbuf = nullptr;
     ctx->hbuf_bytes = 0;
-    if (cudaMalloc(&ctx->hbuf, need) != cudaSuccess) {
+    if (cudaMalloc(&ctx->hbuf, need) == cudaSuccess) {
+      ctx->hbuf_bytes = need;
+      break;
+    }
+    (void)cudaGetLastError();
+    if (ng == 1) return IDKM_ERR_CUDA;
+  }
+  // three streams of the ctx's own: the kernels run on one, uploads that can overlap them on another, downloads on a third (behind
+  // the upload of the gradient they would leave one direction of the link idle); four events per group, as many as were needed yet
+  cudaStream_t* streams[3] = {&ctx->hs_compute, &ctx->hs_copy, &ctx->hs_down};
+  for (int i = 0; i < 3; ++i)
+    if (!*streams[i] && cudaStreamCreateWithFlags(streams[i], cudaStreamNonBlocking) != cudaSuccess) {
+      *streams[i] = nullptr;
       (void)cudaGetLastError();
       return IDKM_ERR_CUDA;
     }
-    ctx->hbuf_bytes = need;
-  }
-  // three streams of the ctx's own: the kernels run on one, uploads that can overlap them on another, downloads on a third (behind
-  // the upload of the gradient they would leave one direction of the link idle)
-  if (!ctx->host_streams_ok) {
-    if (cudaStreamCreateWithFlags(&ctx->hs_compute, cudaStreamNonBlocking) != cudaSuccess) return IDKM_ERR_CUDA;
-    if (cudaStreamCreateWithFlags(&ctx->hs_copy, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaStreamDestroy(ctx->hs_compute);
+  for (; ctx->n_hev < 4 * ng; ++ctx->n_hev)
+    if (cudaEventCreateWithFlags(&ctx->hev[ctx->n_hev], cudaEventDisableTiming) != cudaSuccess) {
+      (void)cudaGetLastError();
       return IDKM_ERR_CUDA;
     }
-    if (cudaStreamCreateWithFlags(&ctx->hs_down, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaStreamDestroy(ctx->hs_compute);
-      cudaStreamDestroy(ctx->hs_copy);
-      return IDKM_ERR_CUDA;
-    }
-    for (int i = 0; i < 4 * HOST_GROUPS_MAX; ++i)
-      if (cudaEventCreateWithFlags(&ctx->hev[i], cudaEventDisableTiming) != cudaSuccess) {
-        for (int q = 0; q < i; ++q) cudaEventDestroy(ctx->hev[q]);
-        cudaStreamDestroy(ctx->hs_compute);
-        cudaStreamDestroy(ctx->hs_copy);
-        cudaStreamDestroy(ctx->hs_down);
-        return IDKM_ERR_CUDA;
-      }
-    ctx->host_streams_ok = true;
-  }
   char* base = static_cast<char*>(ctx->hbuf);
   cudaStream_t s = ctx->hs_compute, sc = ctx->hs_copy, sd = ctx->hs_down;
   for (int g = 0; g < ng; ++g) {
@@ -1339,6 +1365,7 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
     q.c0 = (size_t)q.l0 * k * d;
   }
   const auto give_up = [&](int rc) {
+    ctx->in_groups = false;
     cudaStreamSynchronize(s);
     cudaStreamSynchronize(sc);
     cudaStreamSynchronize(sd);
@@ -1370,6 +1397,13 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
         wait = wait || (out[o] && !follows && overlap(out[o], bytes, in[i], in_bytes[i]));
       }
     if (wait) IDKM_TRY(cudaStreamWaitEvent(sd, ctx->hev[4 * (ng - 1) + 1], 0));
+  }
+  {
+    WorkspaceLayout all;
+    if (!make_layout(m, d, k, n_layers, ctx->sms, &all)) return give_up(IDKM_ERR_UNSUPPORTED);
+    ctx->in_groups = ng > 1;
+    ctx->batch_m = m;
+    ctx->batch_jac = all.jm.nt > 0;
   }
   const int wq_dtype_saved = ctx->wq_dtype;
   for (int g = 0; g < ng; ++g) {
@@ -1409,26 +1443,15 @@ int idkm_quantize_host_ex(idkm_ctx* ctx, const float* W_host, const int64_t* lay
     if (dC_out_host) IDKM_TRY(cudaMemcpyAsync(dC_out_host + q.c0, q.c[2], q.cn, cudaMemcpyDeviceToHost, sd));
   }
   if (ng > 1) {
-    // what can be asked about the call afterwards (layer states, residual histories) moves to one place
-    WorkspaceLayout all, part;
-    if (!make_layout(m, d, k, n_layers, ctx->sms, &all)) return give_up(IDKM_ERR_UNSUPPORTED);
-    IDKM_TRY(cudaMemsetAsync(base + all.off_gtickets, 0, sizeof(unsigned int) * (size_t)all.max_groups, s));
-    if (all.max_groups64 > 0) IDKM_TRY(cudaMemsetAsync(base + all.off_gtickets64, 0, sizeof(unsigned int) * (size_t)all.max_groups64, s));
-    for (int g = 0; g < ng; ++g) {
-      const HostGroup& q = grp[g];
-      const size_t n = (size_t)(q.l1 - q.l0), l0 = (size_t)q.l0, h = sizeof(float) * HIST_CAP;
-      if (!make_layout(q.m, d, k, q.l1 - q.l0, ctx->sms, &part)) return give_up(IDKM_ERR_UNSUPPORTED);
-      const char* ws = static_cast<const char*>(q.ws);
-      IDKM_TRY(cudaMemcpyAsync(base + all.off_state + l0 * sizeof(LayerState), ws + part.off_state, n * sizeof(LayerState), cudaMemcpyDeviceToDevice, s));
-      IDKM_TRY(cudaMemcpyAsync(base + all.off_hist_fwd + l0 * h, ws + part.off_hist_fwd, n * h, cudaMemcpyDeviceToDevice, s));
-      IDKM_TRY(cudaMemcpyAsync(base + all.off_hist_adj + l0 * h, ws + part.off_hist_adj, n * h, cudaMemcpyDeviceToDevice, s));
-    }
-    ctx->workspace = base;
+    // where the layers are that can be asked about afterwards
+    for (int g = 0; g < ng; ++g) ctx->parts[g] = {grp[g].ws, grp[g].m, grp[g].l0, grp[g].l1 - grp[g].l0};
+    ctx->n_parts = ng;
     ctx->m_total = m;
     ctx->n_layers = n_layers;
     for (int l = 0; l <= n_layers; ++l) ctx->row_off[l] = layer_offsets[l];
   }
 #undef IDKM_TRY
+  ctx->in_groups = false;
   if (cudaStreamSynchronize(sd) != cudaSuccess || cudaStreamSynchronize(sc) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return IDKM_ERR_CUDA;
   if (info_out) return idkm_get_info(ctx, info_out);
   return IDKM_OK;
@@ -1487,17 +1510,18 @@ int idkm_get_history(idkm_ctx* ctx, int which, int layer, float* host_out, int c
   if (!ctx->have_forward) return IDKM_ERR_ORDER;
   if ((which != 0 && which != 1) || layer < 0 || layer >= ctx->n_layers || capacity < 0) return IDKM_ERR_PARAM;
   WorkspaceLayout wl;
-  if (!make_layout(ctx->m_total, ctx->d, ctx->k, ctx->n_layers, ctx->sms, &wl)) return IDKM_ERR_UNSUPPORTED;
+  const char* ws;
+  int at;
+  if (!layer_place(ctx, layer, &wl, &ws, &at)) return IDKM_ERR_UNSUPPORTED;
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
   LayerState st;
-  const char* ws = static_cast<const char*>(ctx->workspace);
-  if (cudaMemcpy(&st, ws + wl.off_state + sizeof(LayerState) * (size_t)layer, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (cudaMemcpy(&st, ws + wl.off_state + sizeof(LayerState) * (size_t)at, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess)
     return IDKM_ERR_CUDA;
   int n = which == 0 ? st.fwd_iters : st.adj_iters;
   if (n > HIST_CAP) n = HIST_CAP;
   if (n > capacity) n = capacity;
   if (n < 0) n = 0;
-  const size_t off = (which == 0 ? wl.off_hist_fwd : wl.off_hist_adj) + sizeof(float) * (size_t)layer * HIST_CAP;
+  const size_t off = (which == 0 ? wl.off_hist_fwd : wl.off_hist_adj) + sizeof(float) * (size_t)at * HIST_CAP;
   if (n > 0 && cudaMemcpy(host_out, ws + off, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess)
     return IDKM_ERR_CUDA;
   *n_out = n;
@@ -1544,26 +1568,29 @@ int idkm_set_test_hooks(idkm_ctx* ctx, int missing_arrivals, int64_t spin_limit_
 int idkm_count_busy_tickets(idkm_ctx* ctx, int* count_out) {
   if (!ctx || !count_out) return IDKM_ERR_NULL;
   if (!ctx->have_forward) return IDKM_ERR_ORDER;
-  WorkspaceLayout wl;
-  if (!make_layout(ctx->m_total, ctx->d, ctx->k, ctx->n_layers, ctx->sms, &wl)) return IDKM_ERR_UNSUPPORTED;
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return IDKM_ERR_CUDA;
-  const char* ws = static_cast<const char*>(ctx->workspace);
   int busy = 0;
   LayerState host[MAX_LAYERS];
-  if (cudaMemcpy(host, ws + wl.off_state, sizeof(LayerState) * (size_t)ctx->n_layers, cudaMemcpyDeviceToHost) != cudaSuccess)
-    return IDKM_ERR_CUDA;
+  const int rs = read_states(ctx, host);
+  if (rs != IDKM_OK) return rs;
   for (int l = 0; l < ctx->n_layers; ++l) busy += (host[l].ticket != 0u);
-  const size_t offs[2] = {wl.off_gtickets, wl.off_gtickets64};
-  const int counts[2] = {wl.max_groups, wl.max_groups64};
-  for (int s = 0; s < 2; ++s) {
-    if (counts[s] <= 0) continue;
-    unsigned int* t = new (std::nothrow) unsigned int[counts[s]];
-    if (!t) return IDKM_ERR_CUDA;
-    const cudaError_t rc = cudaMemcpy(t, ws + offs[s], sizeof(unsigned int) * (size_t)counts[s], cudaMemcpyDeviceToHost);
-    if (rc == cudaSuccess)
-      for (int i = 0; i < counts[s]; ++i) busy += (t[i] != 0u);
-    delete[] t;
-    if (rc != cudaSuccess) return IDKM_ERR_CUDA;
+  for (int part = 0; part < (ctx->n_parts > 0 ? ctx->n_parts : 1); ++part) {
+    WorkspaceLayout wl;
+    const char* ws;
+    int at;
+    if (!layer_place(ctx, ctx->n_parts > 0 ? ctx->parts[part].l0 : 0, &wl, &ws, &at)) return IDKM_ERR_UNSUPPORTED;
+    const size_t offs[2] = {wl.off_gtickets, wl.off_gtickets64};
+    const int counts[2] = {wl.max_groups, wl.max_groups64};
+    for (int s = 0; s < 2; ++s) {
+      if (counts[s] <= 0) continue;
+      unsigned int* t = new (std::nothrow) unsigned int[counts[s]];
+      if (!t) return IDKM_ERR_CUDA;
+      const cudaError_t rc = cudaMemcpy(t, ws + offs[s], sizeof(unsigned int) * (size_t)counts[s], cudaMemcpyDeviceToHost);
+      if (rc == cudaSuccess)
+        for (int i = 0; i < counts[s]; ++i) busy += (t[i] != 0u);
+      delete[] t;
+      if (rc != cudaSuccess) return IDKM_ERR_CUDA;
+    }
   }
   *count_out = busy;
   return IDKM_OK;

@@ -60,3 +60,27 @@ def test_results_may_go_where_inputs_came_from(rows, pairs):
         got.append([x.copy() for x in res[:4]])
     for n, a, b in zip(names, *got):
         assert np.array_equal(a, b), n
+
+
+# a large layer and a small cold one, which lands in a group of its own: quadruples with a codebook whose single layers have a
+# loop of their own, and scalar weights that would be few and cold
+@pytest.mark.parametrize("d,k,rows,tau", [(4, 16, [1_600_000, 2048], 5e-4), (1, 4, [6_500_001, 3000], 1e-3), (4, 64, [2_000_000, 3000, 2_000_000, 1000], 2e-3)])
+def test_a_group_takes_the_routes_of_the_whole_call(d, k, rows, tau):
+    """The routes are counted in launches: groups of one layer must not take what only single layers take."""
+    from paper_2312_07759_b200 import binding as B
+    rng = np.random.default_rng(k)
+    offs = [0] + [int(x) for x in np.cumsum(rows)]
+    W = rng.standard_normal((offs[-1], d), dtype=np.float32) * np.float32(0.17)
+    G = rng.standard_normal(W.shape, dtype=np.float32) * np.float32(0.1)
+    C0 = np.concatenate([W[a:a + k] for a in offs[:-1]])
+    iters, n, out = 12, [], []
+    for one_batch in (False, True):
+        ctx = B.Context()
+        ctx.set_timing(one_batch)
+        n0 = ctx.launches
+        res = ctx.quantize_host(W, C0, G, tau, 0.0, iters, B.JFB, 0.0, 0, 1.0, layer_offsets=offs)
+        n.append(ctx.launches - n0)
+        out.append(res)
+    groups = n[0] / n[1]
+    assert groups == int(groups) and 2 <= groups <= 4
+    assert [i.status for i in out[0][4]] == [i.status for i in out[1][4]]
