@@ -336,7 +336,7 @@ def main():
     pairs = float(m) * k
     peaks, which = measured_peaks()
     fp32_rate, sfu_rate = B.measure_pipe_rates()      # register-only micro-benchmarks of the two pipes, measured now
-    path = B.describe_path(d, k, T_a, 0)
+    path, route = B.describe_path(d, k, T_a, 0), ctx.last_route()
     traffic_table = stored_traffic(wl.name if args.iters == 0 else None)
 
     def kernel_roofline(label, layout, kernel_ms, ops, share, bytes_per_row):
@@ -370,13 +370,16 @@ def main():
         return r
 
     step_total = float(np.mean(step_ms))
-    # (single layers with larger codebooks run the whole loop in one launch: the time of one of its iterations)
-    one_launch = L == 1 and (d == 4 and k > 8 or d == 2 and k > 16)
-    roof_step = kernel_roofline("forward loop in one launch (one iteration)" if one_launch else "idkm_pass<STEP> (fused forward step)",
-                                None if one_launch else path["step_layout"], step_kernel_ms, pair_ops(d),
-                                ph["steps"] / step_total, 4.0 * d) if T_f > 0 and step_kernel_ms > 0 else None
+    # (the interval form visits no pairs of a weight and a centroid: their count says nothing about its time; a loop of one launch
+    # is given by the time of one of its iterations)
+    per_launch = route["forward"] == "a launch per iteration"
+    roof_step = None
+    if T_f > 0 and step_kernel_ms > 0 and route["forward"] != "interval form":
+        roof_step = kernel_roofline("idkm_pass<STEP> (fused forward step)" if per_launch else f"{route['forward']} (one iteration)",
+                                    path["step_layout"] if per_launch else None, step_kernel_ms, pair_ops(d), ph["steps"] / step_total,
+                                    4.0 * d)
     roof_adj = None
-    if T_a > 0 and adj_kernel_ms > 0 and path["adjoint_route"] == "fused passes":
+    if T_a > 0 and adj_kernel_ms > 0 and route["adjoint"] == "fused passes":
         # the group-per-weight adjoint layouts also read each row's cached softmax reference and normaliser (8 bytes)
         roof_adj = kernel_roofline("idkm_pass<ADJ> (fused adjoint step)", path["adjoint_layout"], adj_kernel_ms,
                                    adjoint_pair_ops(d), ph["adjoint"] / step_total,
@@ -388,7 +391,7 @@ def main():
         roof["pipes_measured"] = {"fp32_lane_ops_per_s": fp32_rate, "sfu_lane_ops_per_s": sfu_rate,
                                   "fp32_lanes_per_clk_per_sm_at_max_clock": fp32_rate / (SM_COUNT * SM_MAX_MHZ * 1e6),
                                   "sfu_lanes_per_clk_per_sm_at_max_clock": sfu_rate / (SM_COUNT * SM_MAX_MHZ * 1e6)}
-        roof["adjoint_route"] = path["adjoint_route"]
+        roof["adjoint_route"] = route["adjoint"]
 
     # ---- end to end through the host-buffer entry point: the same work as the timed step ----------------------------
     e2e = None
@@ -444,7 +447,7 @@ def main():
             "adjoint_wit_per_s": world * m * T_a / (ph["adjoint"] * 1e-3) if T_a else None,
             "step_ms": [round(x, 3) for x in step_ms],
             "step_phase_sum_ms": [round(sum(p.values()), 3) for p in phases], "phase_ms": ph, "step_kernel_ms": step_kernel_ms, "adjoint_kernel_ms": adj_kernel_ms,
-            "roofline": roof, "roofline_second": roof_second, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": int(n_launch), "clocks": clocks,
+            "route": route, "roofline": roof, "roofline_second": roof_second, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": int(n_launch), "clocks": clocks,
             "info": {"status": [i.status for i in info][:4], "fwd_residual": info[0].fwd_residual,
                      "adj_residual": info[0].adj_residual},
         }

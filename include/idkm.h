@@ -82,7 +82,9 @@ void idkm_destroy(idkm_ctx* ctx);
  * per-layer state and the per-block partial sums it holds, for most codebooks of more than 8
  * centroids, 8 bytes per row: each row's softmax reference and normaliser, which the codebook-
  * gradient pass leaves for the adjoint steps (the iteration of Section 4.2 re-evaluates the same attention
- * rows at every step). */
+ * rows at every step), for scalar weights the bins of the interval form (1 to 3 MB a layer), and for d >= 2 and more than
+ * 8 centroids the partial tiles of the Jacobian formed by the tensor cores (16 MB at d = 4, k = 16, 51 and 69 MB at d = 2 and
+ * 4, k = 256, hardly depending on m_total; batches for which they would pass 96 MB have none and use fused passes). */
 size_t idkm_workspace_bytes(int64_t m_total, int d, int k, int n_layers);
 
 /*
@@ -276,8 +278,9 @@ int idkm_backward_restart(idkm_ctx* ctx, const float* dWq, float adj_tol, int ad
  * operation (the exponential) instead of two.  Everything else -- F, Wq, the implicit and Jacobian-free gradients,
  * statuses -- is defined as above with that D.  Applies to the following idkm_forward* / idkm_backward /
  * idkm_quantize_host* calls of the ctx; a backward must follow a forward made with the same setting (else
- * IDKM_ERR_ORDER).  In this setting every forward iteration is one launch per iteration of the fused fp32 step
- * (no one-launch loop, no fp64 step for collapsing layers) and the implicit backward always iterates fused passes.
+ * IDKM_ERR_ORDER).  In this setting single layers with d = 2 and k > 16, or d = 4 and k > 8, run the forward loop in one
+ * launch, all others one launch per iteration of the fused fp32 step (no fp64 step for collapsing layers), and the implicit
+ * backward always iterates fused passes.
  * A temperature schedule (start warm, end cold, as the paper's closing section suggests) is a sequence of forward
  * calls in which each call's C0 is the previous call's C_out.
  * Returns IDKM_OK, IDKM_ERR_NULL or IDKM_ERR_PARAM.
@@ -325,7 +328,8 @@ int idkm_measure_pipe_rates(double* fp32_lane_ops_per_s, double* sfu_lane_ops_pe
  * barrier at which every layer has.  Layers that collapse on the way step in the fp32 increment form (see
  * idkm_set_collapse_step).  Scalar weights (d = 1, Euclidean distance, either Wq_out given or k > 16) of any size and
  * number of layers up to the number of multiprocessors take the interval form instead: the weights are summarised once
- * in bins with moments, and an iteration works on the bins.  Single layers with d = 2 and k > 16, or d = 4 and k > 8,
+ * in bins with moments, and an iteration works on the bins (or, for layers that bins do not suit -- tau far below the
+ * weights' range, thousands of weights on one value -- weight by weight, in the same launch).  Single layers with d = 2 and k > 16, or d = 4 and k > 8,
  * of any size and either distance, have a one-launch loop of their own.  Everything else (larger layers of small
  * codebooks, other batches, max_iter < 2, the fp64 step for collapsing layers) takes one launch per iteration.  Every barrier wait is bounded
  * (about a second): if one runs out the kernel returns and the status of the layer (of every layer of a batch) is
@@ -388,11 +392,21 @@ int idkm_count_busy_tickets(idkm_ctx* ctx, int* count_out);
  * ints to the HOST array out: [0], [1] centroids per lane and lanes per weight-vector of the fused forward step
  * (Algorithm 1, steps 3-5); [2], [3] the same of the fused adjoint step (Section 4.2); [4] how an implicit backward
  * of adj_max_iter steps with idkm_set_adjoint_method = adjoint_method runs the iteration: 0 one fused pass per step,
- * 1 explicit k d x k d matrix held in registers (k d <= 8), 2 explicit matrix in tiles (k d <= 64, from 16 steps),
- * 3 exact solve on the explicit matrix (adjoint_method 2, k d <= 64).
+ * 1 explicit k d x k d matrix held in registers (k d <= 8), 2 explicit matrix in tiles (k d <= 64, from 16 steps) or from the
+ * tensor cores, 3 exact solve on the explicit matrix (adjoint_method 2, k d <= 64).  What (d, k) alone decides: whether a call
+ * takes these kernels depends on its size, its layers and the ctx's settings too (idkm_last_route).
  * Returns IDKM_OK, IDKM_ERR_NULL or IDKM_ERR_UNSUPPORTED.  Needs no device.
  */
 int idkm_describe_path(int d, int k, int adj_max_iter, int adjoint_method, int* out);
+
+/*
+ * Which kernels the last forward and the last backward of the ctx took (for benchmarks that attribute time to kernels).
+ * *forward_out: 0 a launch per iteration, 1 the one-launch loop of small codebooks, 2 that of larger ones, 3 the interval
+ * form.  *adjoint_out: -1 no adjoint iteration since the last forward, 0 fused passes, 1 explicit matrix held in registers, 2 in
+ * tiles, 3 exact solve, 4 matrix formed by the tensor cores, 5 interval sums.  HOST locations; of a call on host buffers that ran
+ * in groups, the last group's.  Returns IDKM_OK, IDKM_ERR_NULL or IDKM_ERR_ORDER (no forward yet).
+ */
+int idkm_last_route(const idkm_ctx* ctx, int* forward_out, int* adjoint_out);
 
 /* Number of kernels this ctx has launched since idkm_create (for accounting in benchmarks). */
 int64_t idkm_launch_count(const idkm_ctx* ctx);

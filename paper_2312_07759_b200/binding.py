@@ -88,6 +88,8 @@ lib.idkm_set_forward_loop.argtypes = [_vp, C.c_int]
 lib.idkm_set_forward_loop.restype = C.c_int
 lib.idkm_describe_path.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
 lib.idkm_describe_path.restype = C.c_int
+lib.idkm_last_route.argtypes = [_vp, C.POINTER(C.c_int), C.POINTER(C.c_int)]
+lib.idkm_last_route.restype = C.c_int
 lib.idkm_launch_count.argtypes = [_vp]
 lib.idkm_launch_count.restype = C.c_int64
 lib.idkm_measure_pipe_rates.argtypes = [C.POINTER(C.c_double), C.POINTER(C.c_double), _vp]
@@ -378,6 +380,14 @@ class Context:
         arr = (C.c_float * 6)()
         _check(lib.idkm_get_phase_ms(self._h, arr))
         return dict(zip(("init", "steps", "final", "grad", "adjoint", "scatter"), [float(x) for x in arr]))
+
+    def last_route(self) -> dict:
+        """``idkm_last_route``: which kernels the last forward and the last backward took."""
+        f, a = C.c_int(0), C.c_int(0)
+        _check(lib.idkm_last_route(self._h, C.byref(f), C.byref(a)))
+        return {"forward": ("a launch per iteration", "one-launch loop", "one-launch loop of larger codebooks", "interval form")[f.value],
+                "adjoint": ("none", "fused passes", "explicit Jacobian in registers", "explicit Jacobian in tiles",
+                            "exact solve on the explicit Jacobian", "explicit Jacobian from the tensor cores", "interval sums")[a.value + 1]}
 
     @property
     def launches(self) -> int:

@@ -328,6 +328,7 @@ struct idkm_ctx {
   int64_t launches;
   // last forward
   bool have_forward;
+  int route_forward, route_adjoint;   // what the last forward and the last backward took (idkm_last_route)
   bool scalar_forward;   // the last forward ran in the interval form for scalar weights and left its tables in the workspace
   const float* W;
   float* C;
@@ -710,9 +711,10 @@ static int try_mma_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPara
   if (no_coop() || ctx->forward_loop != 0 || max_iter < 2 || (!ctx->squared && ctx->collapse_step != 0)) return 1;
   const MmaLoopEntry* e = mma_loop_entry(ctx->d, ctx->k, ctx->squared != 0);
   if (!e || !e->launch || ctx->k * ctx->d <= 32) return 1;
-  // (Batches keep a launch per iteration and with it their sums' order, bit for bit: among a network's layers there are small
-  // cold ones -- 2048 quadruples, k = 16, a spread of 350 tau -- that turn one rounding into 1e-5 of a centroid, and where the
-  // adjoint iteration of such a layer diverges, 1e-2 of its gradient.  A ResNet-18's, d = 4, k = 16: 64 us an iteration against 51.)
+  // (Single layers only: a batch keeps a launch per iteration.  A ResNet-18's, d = 4, k = 16: 64 us an iteration against 51 in a
+  // version of this kernel for batches.  Not for exactness: small cold layers turn one rounding into 1e-5 of a
+  // centroid and more in either loop -- 2048 quadruples, k = 16, a spread of 350 tau, 24 seeds, C against float64: median 3.0e-6
+  // here and 1.2e-6 there, largest 1.5e-3 and 1.4e-3; at 240 tau 5.9e-7 and 6.9e-7, 4.9e-5 and 4.0e-5.)
   if (ctx->n_layers > 1 || ctx->in_groups) return 1;
   int grid = ctx->sms;
   const long long most = (ctx->m_total + MMA_LOOP_ROWS - 1) / MMA_LOOP_ROWS;
@@ -830,9 +832,10 @@ static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassP
       ctx->n_layers > ctx->sms)
     return 1;
   // Few weights and a cold softmax: the bins are nearly as many as the weights, and summarising them costs more than the
-  // iterations save.  (The weights' spread is not known here; it is of the order of 0.05.  30 iterations and the Jacobian-free
-  // backward, spread 0.03, one-launch loop over the weights against this one: m = 4096, k = 4: tau = 0.05 128 against 115 us,
-  // 0.01 103 against 119, 5e-4 104 against 146; m = 8192, k = 16: 5e-4 185 against 222, 2e-3 faster here.)
+  // iterations save.  What counts is tau against the weights' spread, which only the device knows: the bounds are absolute, for
+  // weights of the order of 0.05, and a layer in other units may take the slower of two right answers.  (30 iterations and the
+  // Jacobian-free backward, spread 0.03, one-launch loop over the weights against this one: m = 4096, k = 4: tau = 0.05 128 against
+  // 115 us, 0.01 103 against 119, 5e-4 104 against 146; m = 8192, k = 16: 5e-4 185 against 222, 2e-3 faster here.)
   const bool cold = (ctx->m_total <= 4096 && ctx->k <= 4 && ctx->tau < 0.03f) || (ctx->m_total <= 16384 && ctx->k <= 16 && ctx->tau < 1e-3f);
   if (ctx->n_layers == 1 && !ctx->in_groups && cold) return 1;
   for (int l = 0; l < ctx->n_layers; ++l)
@@ -1081,9 +1084,19 @@ int idkm_forward_batched(idkm_ctx* ctx, const float* W_cat, const int64_t* layer
     ++ctx->launches;
     mark(ctx, 1);
     rc = try_small_loop(ctx, wl, p, max_iter);
-    if (rc == 1) rc = try_mma_loop(ctx, wl, p, max_iter);
-    if (rc == 1) rc = launch_step_loop(ctx, wl, &p, max_iter);
+    ctx->route_forward = 1;
+    if (rc == 1) {
+      rc = try_mma_loop(ctx, wl, p, max_iter);
+      ctx->route_forward = 2;
+    }
+    if (rc == 1) {
+      rc = launch_step_loop(ctx, wl, &p, max_iter);
+      ctx->route_forward = 0;
+    }
+  } else {
+    ctx->route_forward = 3;
   }
+  ctx->route_adjoint = -1;
   nvtxRangePop();
   if (rc != IDKM_OK) return rc;
   mark(ctx, 2);
@@ -1151,13 +1164,18 @@ int idkm_backward(idkm_ctx* ctx, const float* dWq, idkm_mode mode, float adj_tol
   nvtxRangePop();
   if (rc != IDKM_OK) return rc;
   mark(ctx, 5);
+  ctx->route_adjoint = -1;
   if (solve) {
     nvtxRangePushA("idkm adjoint solve");
+    ctx->route_adjoint = scalar ? 5 : (jac_mma ? 4 : (explicit_jac ? (exact ? 3 : (jac_tile ? 2 : 1)) : 0));
     if (scalar) {
       rc = launch_scalar_pass(ctx, wl, p, SP_ADJOINT, dC_out);
     } else if (jac_mma) {
       rc = launch_jac_mma_adjoint(ctx, wl, p);
-      if (rc == 1) rc = launch_pass(ctx, ADJ, &p, adj_max_iter);
+      if (rc == 1) {
+        rc = launch_pass(ctx, ADJ, &p, adj_max_iter);
+        ctx->route_adjoint = 0;
+      }
     } else if (explicit_jac) {
       if (exact) p.max_iter = -1;                  // the epilogue solves (I - J^T) u = g instead of iterating
       rc = launch_pass(ctx, JACOBIAN, &p, 1);      // one pass forms J_C; the whole iteration runs on it in the epilogue
@@ -1593,6 +1611,14 @@ int idkm_count_busy_tickets(idkm_ctx* ctx, int* count_out) {
     }
   }
   *count_out = busy;
+  return IDKM_OK;
+}
+
+int idkm_last_route(const idkm_ctx* ctx, int* forward_out, int* adjoint_out) {
+  if (!ctx || !forward_out || !adjoint_out) return IDKM_ERR_NULL;
+  if (!ctx->have_forward) return IDKM_ERR_ORDER;
+  *forward_out = ctx->route_forward;
+  *adjoint_out = ctx->route_adjoint;
   return IDKM_OK;
 }
 

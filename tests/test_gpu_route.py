@@ -1,0 +1,37 @@
+"""What idkm_last_route says against the launches that a call makes (B200 only)."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m,d,k,layers,loop,adjoint,forward,backward", [
+    (20000, 1, 4, 1, 0, 0, "interval form", "interval sums"),
+    (20000, 1, 40, 3, 0, 1, "interval form", "fused passes"),
+    (20000, 1, 16, 1, 1, 2, "a launch per iteration", "exact solve on the explicit Jacobian"),
+    (20000, 2, 4, 2, 0, 0, "one-launch loop", "explicit Jacobian in registers"),
+    (20000, 4, 8, 1, 0, 0, "one-launch loop", "explicit Jacobian in tiles"),
+    (20000, 4, 16, 1, 0, 0, "one-launch loop of larger codebooks", "explicit Jacobian from the tensor cores"),
+    (20000, 4, 16, 4, 0, 0, "a launch per iteration", "explicit Jacobian from the tensor cores"),
+    (6000, 4, 256, 4, 0, 0, "a launch per iteration", "fused passes"),
+])
+def test_the_route_that_was_taken(m, d, k, layers, loop, adjoint, forward, backward):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(k)
+    W = torch.randn(m * layers, d, device="cuda", generator=g) * 0.03
+    offs = [m * l for l in range(layers + 1)]
+    C0 = torch.cat([W[a:a + k] for a in offs[:-1]]).contiguous()
+    ctx = B.Context()
+    ctx.set_forward_loop(loop)
+    ctx.set_adjoint_method(adjoint)
+    n0 = ctx.launches
+    ctx.forward(W, C0, 0.02, 0.0, 20, layer_offsets=offs)
+    n1 = ctx.launches
+    assert ctx.last_route() == {"forward": forward, "adjoint": "none"}
+    ctx.backward(torch.ones_like(W), B.IMPLICIT, 0.0, 40, 0.25)
+    n2 = ctx.launches
+    assert ctx.last_route() == {"forward": forward, "adjoint": backward}
+    assert (n1 - n0 >= 20) == (forward == "a launch per iteration")
+    assert (n2 - n1 >= 40) == (backward == "fused passes")
+    ctx.backward(torch.ones_like(W), B.JFB, 0.0, 0, 1.0)
+    assert ctx.last_route()["adjoint"] == "none"
