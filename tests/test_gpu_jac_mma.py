@@ -161,3 +161,29 @@ def test_the_largest_batches_keep_the_route(d, k, layers):
     if all(s == 0 for s in out[0][3]):
         assert_close(out[0][2], out[1][2], TOL_GRAD, "dC")
         assert_close(out[0][1], out[1][1], TOL_GRAD, "dW")
+
+
+@pytest.mark.parametrize("d,k", [(4, 64), (2, 128)])
+def test_a_layer_with_nothing_to_solve_ends_before_the_matrix(d, k):
+    """tau above the weights' spread: every centroid is in the mean, and the first step of the iteration changes nothing."""
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    W, C0, G, offs = data([30000, 20000], d, k, 0.02, 1)
+    W[30000:] *= 40.0                      # (the second layer does not collapse)
+    C0[k:] *= 40.0
+    W, C0, G = (torch.from_numpy(x).cuda() for x in (W, C0, G))
+    for layers in (1, 2):
+        n = offs[layers]
+        got = []
+        for method in (0, 1):
+            ctx = B.Context()
+            ctx.set_adjoint_method(method)
+            ctx.forward(W[:n], C0[:layers * k], 0.2, 0.0, 60, layer_offsets=offs[:layers + 1])
+            dW, dC = ctx.backward(G[:n], B.IMPLICIT, 1e-5, 200, 0.5)
+            got.append((dW.cpu().numpy(), dC.cpu().numpy(), [(i.status, i.adj_iters) for i in ctx.info()]))
+        assert got[0][2][0][1] == got[1][2][0][1] <= 1
+        if layers == 1:
+            assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+        else:
+            assert got[0][2][1][1] > 1 and abs(got[0][2][1][1] - got[1][2][1][1]) <= 1
+            assert_close(got[0][1], got[1][1], TOL_GRAD, "dC")
