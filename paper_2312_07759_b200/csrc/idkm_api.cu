@@ -711,6 +711,12 @@ static int try_mma_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassPara
   if (no_coop() || ctx->forward_loop != 0 || max_iter < 2 || (!ctx->squared && ctx->collapse_step != 0)) return 1;
   const MmaLoopEntry* e = mma_loop_entry(ctx->d, ctx->k, ctx->squared != 0);
   if (!e || !e->launch || ctx->k * ctx->d <= 32) return 1;
+  // (Large layers of the codebooks whose kernel keeps few loads in flight are faster by a launch per iteration: us an iteration, one
+  // launch and a launch each -- d = 2, k = 256: 12 M 1959 and 1965, 16 M 3147 and 2734, 32 M 6339 and 5452; k = 128: 12 M 967 and 1047,
+  // 16 M 1480 and 1459; d = 4, k = 32: 1 M 41 and 45, 4 M 137 and 132, 16 M 543 and 481; k = 64: 6 M 374 and 376, 16 M 1042 and 1013.
+  // The others, at 16 M: d = 2, k = 32 and 64 371 and 402, 738 and 784; d = 4, k = 16, 128 and 256 278 and 286, 1652 and 1934, 3283 and 3521.)
+  const long long mb = ctx->m_total * ctx->d / 250000;   // of weights
+  if (ctx->d == 2 ? (ctx->k > 64 && mb > 110) : (ctx->k > 16 && (ctx->k <= 32 ? mb > 48 : (ctx->k <= 64 && mb > 128)))) return 1;
   // (Single layers only: a batch keeps a launch per iteration.  A ResNet-18's, d = 4, k = 16: 64 us an iteration against 51 in a
   // version of this kernel for batches.  Not for exactness: small cold layers turn one rounding into 1e-5 of a
   // centroid and more in either loop -- 2048 quadruples, k = 16, a spread of 350 tau, 24 seeds, C against float64: median 3.0e-6

@@ -35,3 +35,20 @@ def test_the_route_that_was_taken(m, d, k, layers, loop, adjoint, forward, backw
     assert (n2 - n1 >= 40) == (backward == "fused passes")
     ctx.backward(torch.ones_like(W), B.JFB, 0.0, 0, 1.0)
     assert ctx.last_route()["adjoint"] == "none"
+
+
+@pytest.mark.parametrize("m,d,k,forward", [
+    (13_000_000, 2, 128, "one-launch loop of larger codebooks"), (14_000_000, 2, 128, "a launch per iteration"),
+    (3_000_000, 4, 32, "one-launch loop of larger codebooks"), (3_100_000, 4, 32, "a launch per iteration"),
+])
+def test_large_layers(m, d, k, forward):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(k)
+    W = torch.randn(m, d, device="cuda", generator=g) * 0.03
+    ctx = B.Context()
+    C = ctx.forward(W, W[:k].contiguous(), 0.01, 0.0, 3, want_Wq=False).C
+    assert ctx.last_route()["forward"] == forward
+    ctx.set_forward_loop(1)
+    ref = ctx.forward(W, W[:k].contiguous(), 0.01, 0.0, 3, want_Wq=False).C
+    assert float((C - ref).norm() / ref.norm()) < 1e-5
