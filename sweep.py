@@ -87,7 +87,9 @@ def run_point(ctx, B, torch, m, d, b, tau, cap):
         "dW_err_implicit": rel(dWi, dWr), "dW_err_jfb": rel(dWj, dWr),
         "dC_err_implicit": rel(dCi, dCr), "dC_err_jfb": rel(dCj, dCr),
     }
-    out["frac_of_roofline"] = out["step_roofline_ms"] / out["fwd_ms_per_iter"]
+    # (the interval form of scalar weights visits no pairs of a weight and a centroid, so the step's roofline says nothing there)
+    out["route"] = ctx.last_route()["forward"]
+    out["frac_of_roofline"] = None if out["route"] == "interval form" else out["step_roofline_ms"] / out["fwd_ms_per_iter"]
     return out
 
 
@@ -120,8 +122,9 @@ def main():
               "dW err implicit | dW err JFB |")
         print("|---|---|---|---|---|---|---|---|---|---|---|---|---|")
         for r in rows:
+            frac = "-" if r["frac_of_roofline"] is None else f"{r['frac_of_roofline']:.2f}"
             print(f"| {r['m']} | {r['d']} | {r['k']} | {r['tau']} | {r['fwd_iters']} | {r['fwd_residual']:.1e} | "
-                  f"{r['fwd_ms_per_iter']:.4f} | {r['step_roofline_ms']:.4f} | {r['frac_of_roofline']:.2f} | "
+                  f"{r['fwd_ms_per_iter']:.4f} | {r['step_roofline_ms']:.4f} | {frac} | "
                   f"{r['jfb_ms']:.3f} | {r['implicit_ms']:.3f} ({r['adj_iters']}) | {r['dW_err_implicit']:.1e} | "
                   f"{r['dW_err_jfb']:.1e} |")
 
