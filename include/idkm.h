@@ -327,10 +327,11 @@ int idkm_measure_pipe_rates(double* fp32_lane_ops_per_s, double* sfu_lane_ops_pe
  * inside the loop.  A layer leaves the loop at the iteration whose stop test passes; a batch leaves at the first
  * barrier at which every layer has.  Layers that collapse on the way step in the fp32 increment form (see
  * idkm_set_collapse_step).  Scalar weights (d = 1, Euclidean distance, either Wq_out given or k > 16) of any size and
- * number of layers up to the number of multiprocessors take the interval form instead: the weights are summarised once
- * in bins with moments, and an iteration works on the bins (or, for layers that bins do not suit -- tau far below the
- * weights' range, thousands of weights on one value -- weight by weight, in the same launch).  Single layers with d = 2 and k > 16, or d = 4 and k > 8,
- * of any size and either distance, have a one-launch loop of their own.  Everything else (larger layers of small
+ * number of layers up to the number of multiprocessors take the interval form instead (but for k <= 8 with max_iter <= 4, and
+ * few weights with a cold softmax): the weights are summarised once in bins with moments, and an iteration works on the bins
+ * (or, for layers that bins do not suit -- tau far below the weights' range, thousands of weights on one value -- weight by
+ * weight, in the same launch).  Single layers with d = 2 and k > 16, or d = 4 and k > 8, either distance, have a one-launch
+ * loop of their own (not the large layers of some of these codebooks, for which it is slower).  Everything else (larger layers of small
  * codebooks, other batches, max_iter < 2, the fp64 step for collapsing layers) takes one launch per iteration.  Every barrier wait is bounded
  * (about a second): if one runs out the kernel returns and the status of the layer (of every layer of a batch) is
  * IDKM_ERR_TIMEOUT.  1: always one launch per iteration

@@ -844,6 +844,10 @@ static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassP
   // 115 us, 0.01 103 against 119, 5e-4 104 against 146; m = 8192, k = 16: 5e-4 185 against 222, 2e-3 faster here.)
   const bool cold = (ctx->m_total <= 4096 && ctx->k <= 4 && ctx->tau < 0.03f) || (ctx->m_total <= 16384 && ctx->k <= 16 && ctx->tau < 1e-3f);
   if (ctx->n_layers == 1 && !ctx->in_groups && cold) return 1;
+  // Few iterations of a small codebook do not pay for the bins either.  (Forward and implicit backward of 20 steps, over the pairs
+  // and here, k = 4, 4 iterations: m = 36864 90 and 121 us, 1 M 129 and 143, 16 M 433 and 506; 6 iterations 100 and 124, 143 and 148, 502
+  // and 517; k = 16, 4 iterations, 1 M 227 and 166, 16 M 1611 and 576.)
+  if (max_iter <= 4 && ctx->k <= 8) return 1;
   for (int l = 0; l < ctx->n_layers; ++l)
     if (ctx->row_off[l + 1] - ctx->row_off[l] > 0x7fffffffLL) return 1;
   ScalarParams sp;

@@ -52,3 +52,17 @@ def test_large_layers(m, d, k, forward):
     ctx.set_forward_loop(1)
     ref = ctx.forward(W, W[:k].contiguous(), 0.01, 0.0, 3, want_Wq=False).C
     assert float((C - ref).norm() / ref.norm()) < 1e-5
+
+
+@pytest.mark.parametrize("k,iters,forward", [(4, 4, "one-launch loop"), (4, 5, "interval form"), (8, 4, "one-launch loop"), (9, 4, "interval form")])
+def test_few_iterations_do_without_bins(k, iters, forward):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(k)
+    W = torch.randn(30000, 1, device="cuda", generator=g) * 0.03
+    ctx = B.Context()
+    C = ctx.forward(W, W[:k].contiguous(), 0.01, 0.0, iters).C
+    assert ctx.last_route()["forward"] == forward
+    ctx.set_forward_loop(1)
+    ref = ctx.forward(W, W[:k].contiguous(), 0.01, 0.0, iters).C
+    assert float((C - ref).norm() / ref.norm()) < 1e-5

@@ -31,7 +31,7 @@ def test_sums_of_many_terms(m, k):
     C0 = torch.linspace(-0.06, 0.06, k, device="cuda").reshape(k, 1)
     G = 0.3 + 0.05 * torch.randn(m, 1, device="cuda", generator=g)
     ctx = B.Context()
-    C = ctx.forward(W, C0, 0.02, 0.0, 2).C
+    C = ctx.forward(W, C0, 0.02, 0.0, 5).C
     dC = ctx.backward(G, B.JFB, 0.0, 0, 1.0, want_dW=False)[1][:, 0].double()
     ref = reference(W, C, 0.02, G)
     err = float((dC - ref).norm() / ref.norm())
