@@ -12,10 +12,10 @@
 // integers, so results are reproducible although the grouping uses atomic counters.
 //
 // What bounds it.  Building: the grouping pass stores two bytes per weight to scattered places, 67 cycles a warp store
-// (110 us per 11.7 M weights on all SMs).  Iterating: the chain of one block a layer -- evaluate, sum, M-step, four meetings of
-// the block -- 2.6 us at k <= 4 to 6 us, whatever the number of weights.  Measured, loop with the summary against one that
-// visits the pairs: 21 layers of a ResNet-18, k = 4, 50 iterations 382 against 1473 us; k = 8, tau = 5e-4, 30 iterations 366
-// against 1268; 16 M weights, k = 16, 100 iterations 1.42 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 101
+// (110 us per 11.7 M weights on all SMs).  Iterating: the chain of one block a layer, 1.7 us at k <= 4 to 6 us, whatever the
+// number of weights (sc_iterate up to 16 centroids).  Measured, loop with the summary against one that
+// visits the pairs: 21 layers of a ResNet-18, k = 4, 50 iterations 352 against 1473 us; k = 8, tau = 5e-4, 30 iterations 380
+// against 1268; 16 M weights, k = 16, 100 iterations 1.26 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 68
 // against 112.
 //
 // Layers that bins do not suit -- tau below 1 / 5700 of the weights' range (1 / 2800 in layers beyond the eighth), which an outlier
@@ -174,11 +174,13 @@ struct ScLayer {
 };
 
 constexpr int SC_PARTS = 768;   // (centroid, slot) pairs: a slot per warp of an interval and two for its ends
+constexpr int SI_K = 16;        // up to this many centroids the iterations are sc_iterate's
+constexpr int SI_SLOTS = 52;    // (interval, slot) pairs there
 constexpr int SC_BELOW = 272;   // (centroid, warp) pairs of the scan of the centroids' fine bins
 struct ScShared {
   ScGrid g;
   ScLayer ly;              // (copy for the functions that are not inlined)
-  int ok, bad, flag, done, iters, dead, status;
+  int ok, bad, flag, steps, done, iters, dead, status;
   // what the evaluations without bins need (here, so that it does not live in registers in the others)
   unsigned int meet;       // barriers of the layer's blocks so far
   const float* W;          // the layer's weights, and this block's share
@@ -195,6 +197,7 @@ struct ScShared {
   double Ls[SC_PARTS][2];  // sums of lambda (and lambda x) over the interval right of a centroid, per slot
   double Ms[SC_PARTS][2];  // ... of mu over the interval left of it
   double Xs[SC_PARTS][2];  // ... of lambda mu over the interval right of it (last evaluation only)
+  alignas(16) double ev[SI_SLOTS][4];  // sc_iterate: per (interval, slot) sums of lambda, lambda x, mu, mu x
   double cnew[256], cold[256];   // the last M-step, for the stop test
   int dead_j[256];
   double qs[256];
@@ -1144,6 +1147,450 @@ __device__ __noinline__ bool sd_sums(ScShared& sh, const ScalarParams& sp, int l
   return true;
 }
 
+// ---- the iterations of up to SI_K centroids ----
+// What bounds an iteration is the latency of its chain, instruction by instruction.  So its parts overlap: the first warp takes
+// the M-step and publishes the centroids (meeting B1), then the even points and places (B2); a warp per centroid counts its
+// fine bin between the two and afterwards takes the ends of the two intervals the centroid borders; other warps have the
+// whole bins of an interval; at the third meeting (A) the first warp has all sums.  What a warp does is the same in every
+// iteration, and a centroid's fine bin (up to SI_HEAD of its places, and its record) stays in its warp's registers.  Nothing in
+// the loop may live in local memory: with the shared memory the block takes the L1 cache holds none of it, and every access
+// is a trip to L2; and a load whose value is used before the next one is issued is one more such trip.  Cycles an iteration,
+// before (counts, ends and M-step one after the other between meetings of the block) and now: 4096 weights, k = 4 5500 and 3300;
+// 36864, k = 8 6700 and 4600; 2.4 M, k = 4 8000 and 5900; 16 M, k = 16 24000 and 19800 (the fine bins hold thousands of weights).
+constexpr int SI_WORDS = 8, SI_HEAD = 64 * SI_WORDS;
+constexpr int SI_A = 2, SI_B1 = 3, SI_B2 = 4;   // hardware barriers
+__device__ __forceinline__ void si_arrive(int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(SC_T) : "memory"); }
+__device__ __forceinline__ void si_meet(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(SC_T) : "memory"); }
+// (interval, slot) pairs of an interval: warps that share its whole bins, then its left and its right end
+template <int LOG>
+__host__ __device__ constexpr int si_slots() { return LOG <= 2 ? 5 : (LOG == 3 ? 4 : 3); }
+
+struct SiBin {
+  int f;                      // fine bin, -1: none
+  unsigned int e0, e1;        // its elements
+  unsigned int w[SI_WORDS];   // 64 places each, two a lane; 0 (which no weight's place is) where there is none
+  double m[4];                // moments of the weights of earlier fine bins of the coarse bin
+};
+// (places start at a multiple of 8 elements of `grouped`)
+__device__ __forceinline__ long long si_base(const ScLayer& ly, const SiBin& bn) { return (ly.row0 + bn.e0) & ~7LL; }
+template <int N>
+__device__ __forceinline__ void si_words(const ScLayer& ly, long long base, int lo, int hi, SiBin& bn) {
+  const int e0 = 2 * (threadIdx.x & 31);
+  const unsigned int* g = reinterpret_cast<const unsigned int*>(ly.grouped + base) + (e0 >> 1);
+  const bool pairs = base + hi + 1 <= ly.total;   // (the last element of all may have no partner)
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int e = 64 * i + e0;
+    bn.w[i] = e + (pairs ? 0 : 1) < hi ? g[32 * i] : 0u;
+  }
+  if (!pairs && ((hi - 1) & 1) == 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (64 * i + e0 == hi - 1) bn.w[i] = (unsigned int)ly.grouped[base + hi - 1];
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int e = 64 * i + e0;
+    bn.w[i] &= (e >= lo && e < hi ? 0xffffu : 0u) | (e + 1 >= lo && e + 1 < hi ? 0xffff0000u : 0u);
+  }
+}
+__device__ __forceinline__ void si_bin_load(const ScLayer& ly, int f, SiBin& bn) {
+  const int lane = threadIdx.x & 31;
+  bn.f = f;
+  bn.e0 = ly.fstart[f];
+  bn.e1 = ly.fstart[f + 1];
+  const double2 r0 = reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4)[0], r1 = reinterpret_cast<const double2*>(ly.frec + (size_t)f * 4)[1];
+  const long long base = si_base(ly, bn);
+  const int lo = (int)(ly.row0 + bn.e0 - base), n = lo + (int)(bn.e1 - bn.e0), hi = n < SI_HEAD ? n : SI_HEAD;
+  // all loads first, then what is made of them
+  if (hi > 256) si_words<SI_WORDS>(ly, base, lo, hi, bn);
+  else if (hi > 64) si_words<4>(ly, base, lo, hi, bn);
+  else si_words<1>(ly, base, lo, hi, bn);
+  bn.m[0] = r0.x;
+  bn.m[1] = r0.y;
+  bn.m[2] = r1.x;
+  bn.m[3] = r1.y;
+}
+// Sums over n places p (from 1; 0: none) that lie below pv, those at it counting half, without a comparison: with S(x) the sum
+// of min(p, x), S(x) - S(x - 1) places are at x or beyond.  Two places per instruction.
+struct SiSum {
+  unsigned int a, b, c;   // S(pv), S(pv + 1), S(pv - 1)
+  int q2, q3, q4;
+};
+struct SiCut {
+  unsigned int a, b, c;   // pv, pv + 1, pv - 1 in both halves
+  int pv;
+};
+__device__ __forceinline__ SiCut si_cut(int pv) {
+  // beyond the ends of the scale: below everything the result is set to zero, above everything the three sums are equal
+  const unsigned int a = (unsigned int)(pv < 1 ? 1 : (pv > 65535 ? 65535 : pv)), b = a < 65535u ? a + 1u : a, c = pv > 65535 ? a : a - 1u;
+  SiCut t;
+  t.a = a * 0x10001u;
+  t.b = b * 0x10001u;
+  t.c = c * 0x10001u;
+  t.pv = pv;
+  return t;
+}
+// Powers of the place.  A fine bin is 1 / F of a coarse bin: from F = 8 on its third and fourth powers, from F = 64 on its second
+// change an interval's sums by less than 1e-8.
+__device__ __forceinline__ int si_powers(int F) { return F >= 64 ? 1 : (F >= 8 ? 2 : 4); }
+__device__ __forceinline__ void si_add(unsigned int x, const SiCut& t, int powers, SiSum& s) {
+  s.a = __dp2a_lo(__vminu2(x, t.a), 0x0101u, s.a);
+  s.b = __dp2a_lo(__vminu2(x, t.b), 0x0101u, s.b);
+  s.c = __dp2a_lo(__vminu2(x, t.c), 0x0101u, s.c);
+  if (powers > 1) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int u = (int)(i ? x >> 16 : x & 0xffffu), p = u > 0 ? u - 32768 : 0;
+      const int w = u < t.pv ? 2 : (u == t.pv ? 1 : 0);
+      if (powers == 2) {
+        s.q2 += w * ((p * p + 8192) >> 14);
+      } else {
+        int p2, p3, p4;
+        sc_powers(p, p2, p3, p4);
+        s.q2 += w * p2;
+        s.q3 += w * p3;
+        s.q4 += w * p4;
+      }
+    }
+  }
+}
+// Over the warp, n places in all (at most 2^15): twice the count and sums of powers.
+__device__ __forceinline__ void si_total(const SiSum& s, int n, const SiCut& t, int powers, double (&b)[5]) {
+  const unsigned int a = __reduce_add_sync(0xffffffffu, s.a), up = __reduce_add_sync(0xffffffffu, s.b - s.a), at = __reduce_add_sync(0xffffffffu, s.a - s.c);
+  const int lt2 = 2 * n - (int)(up + at), eq = (int)(at - up);   // up: beyond pv, at: at it or beyond
+  // twice the sum of the places below (the sum of all, those beyond counted as pv), those at pv half
+  const long long p2 = 2LL * a - (long long)(t.a & 0xffffu) * (2LL * at - eq);
+  const bool none = t.pv < 1;
+  b[0] += none ? 0.0 : (double)lt2;
+  b[1] += none ? 0.0 : (double)(p2 - 32768LL * lt2);
+  if (powers > 1) b[2] += (double)__reduce_add_sync(0xffffffffu, s.q2);
+  if (powers > 2) {
+    b[3] += (double)__reduce_add_sync(0xffffffffu, s.q3);
+    b[4] += (double)__reduce_add_sync(0xffffffffu, s.q4);
+  }
+}
+// What lies below a centroid in its coarse bin.
+struct SiBelow {
+  int c;
+  double n, m[4];
+};
+__device__ __forceinline__ void si_below(const ScShared& sh, const ScGrid& g, const ScLayer& ly, SiBin& bn, float v, SiBelow& o) {
+  const int lane = threadIdx.x & 31;
+  int place;
+  const int f = sc_fine_place(g, fminf(fmaxf(v, g.lo), g.hi), place);
+  // one beyond the ends of the scale where the centroid lies outside the weights' range
+  const int pv = v > g.hi ? 72768 : (v < g.lo ? -7232 : place + 32768);
+  if (bn.f != f) si_bin_load(ly, f, bn);
+  const int powers = si_powers(g.F);
+  const SiCut t = si_cut(pv);
+  SiSum s = {0u, 0u, 0u, 0, 0, 0};
+  const long long base = si_base(ly, bn), end = ly.row0 + bn.e1;
+  const int hi = end - base < SI_HEAD ? (int)(end - base) : SI_HEAD;
+#pragma unroll
+  for (int i = 0; i < SI_WORDS; ++i) {
+    if (i > 0 && 64 * i >= hi) break;
+    si_add(bn.w[i], t, powers, s);
+  }
+  double b[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  int n = hi - (int)(ly.row0 + bn.e0 - base);
+  // the weights that are not in registers, in stretches whose 32-bit sums cannot overflow
+  for (long long e = base + SI_HEAD; e < end;) {
+    uint4 q[4];
+    if (e + 1024 <= ly.total) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint4*>(ly.grouped + e + 256 * i + 8 * lane);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const long long x = e + 256 * i + 8 * lane;
+        q[i] = x < end ? sc_load8(ly.grouped, x, ly.total) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    if (e + 1024 > end) {
+      const int last = (int)(end - e) - 8 * lane;
+      auto cut = [&](unsigned int w, int h) { return (h < last ? w & 0xffffu : 0u) | (h + 1 < last ? w & 0xffff0000u : 0u); };
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        q[i] = make_uint4(cut(q[i].x, 256 * i), cut(q[i].y, 256 * i + 2), cut(q[i].z, 256 * i + 4), cut(q[i].w, 256 * i + 6));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      si_add(q[i].x, t, powers, s);
+      si_add(q[i].y, t, powers, s);
+      si_add(q[i].z, t, powers, s);
+      si_add(q[i].w, t, powers, s);
+    }
+    n += end - e < 1024 ? (int)(end - e) : 1024;
+    e += 1024;
+    if (n >= SC_CHUNK) {
+      si_total(s, n, t, powers, b);
+      s = SiSum{0u, 0u, 0u, 0, 0, 0};
+      n = 0;
+    }
+  }
+  si_total(s, n, t, powers, b);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) b[i] *= 0.5;
+  o.c = f >> g.fshift;
+  sc_shift(g, sc_fine_x0(g, f), b[0], b[1], b[2], b[3], b[4], o.m);
+  o.n = b[0] + ((double)bn.e0 - ly.rec.cn[o.c]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) o.m[i] += bn.m[i];
+}
+// Centroid j: the right end of interval j (even lanes) and the left end of interval j + 1 (odd lanes); where there is no such
+// interval, all weights beyond.
+template <int SLOTS>
+__device__ __forceinline__ void si_ends(ScShared& sh, const ScGrid& g, const ScLayer& ly, const SiBelow& o, int j) {
+  const int k = ly.k, lane = threadIdx.x & 31;
+  const bool left = lane & 1;
+  const int s = left ? j + 1 : j;
+  const bool inner = s > 0 && s < k;
+  const double v0 = (double)sh.v[0], ctr = sc_center(g, o.c), even = inner ? sh.even[s] : ctr;
+  const bool whole = left && inner && (sh.fb[inner ? s : j] >> g.fshift) != o.c;
+  const double nt = ly.rec.cn[g.nc], xt = ly.rec.cx[g.nc], xc = ly.rec.cx[o.c], nc = ly.rec.cn[o.c];
+  float r[5];   // the whole bin
+#pragma unroll
+  for (int i = 0; i < 5; ++i) r[i] = ly.rec.r[i * ly.rec.stride + o.c];
+  // everything below the centroid, or above it
+  double nn = o.n + nc, xx = fma(ctr, o.n, fma(g.hc, o.m[0], xc));
+  nn = left ? nt - nn : nn;
+  xx = left ? xt - xx : xx;
+  if (sh.n0 > 0) {   // weights that are exactly zero
+    const float v = left ? -sh.v[k - 1] : sh.v[0];
+    nn += (v > 0.f ? 1.0 : (v == 0.f ? 0.5 : 0.0)) * (double)sh.n0;
+  }
+  xx = fma(-v0, nn, xx);
+  // the piece below the right end; above the left end the whole bin (unless the right end lies in it) minus what is below
+  const ScCoef co = sc_coef((float)((ctr - even) * (double)ly.slope));
+  double n = o.n, m[4];
+  n = left ? (whole ? (double)r[0] : 0.0) - n : n;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) m[i] = left ? (whole ? (double)r[i + 1] : 0.0) - o.m[i] : o.m[i];
+  double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  sc_bin_sums<false, double>(co, g.eta, n, m[0], m[1], m[2], m[3], ctr - v0, g.hc, acc);
+  if (lane < 2) {
+    double2* d = reinterpret_cast<double2*>(sh.ev[s * SLOTS + (left ? SLOTS - 2 : SLOTS - 1)]);
+    d[0] = inner ? make_double2(acc[0], acc[1]) : make_double2(left ? nn : 0.0, left ? xx : 0.0);
+    d[1] = inner ? make_double2(acc[2], acc[3]) : make_double2(left ? 0.0 : nn, left ? 0.0 : xx);
+  }
+}
+// Interval s: the whole bins between its ends, dealt to the lanes of tw warps of which this is number `sub`.
+template <int SLOTS>
+__device__ __forceinline__ void si_bins(ScShared& sh, const ScGrid& g, const ScLayer& ly, int s, int sub, int tw) {
+  const int lane = threadIdx.x & 31;
+  const int cl = sh.fb[s - 1] >> g.fshift, cr = sh.fb[s] >> g.fshift;
+  const double even = sh.even[s], v0 = (double)sh.v[0];
+  double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (cr - cl >= 2) {   // (uniform)
+    // the zone where neither lambda nor mu vanishes: b0 .. b1 - 1
+    const double at = (even - g.ctr0) * g.inv_hc, zb = ly.zone * g.inv_hc;
+    int b0 = __double2int_rd(at - zb), b1 = __double2int_ru(at + zb) + 1;
+    b0 = b0 < cl + 1 ? cl + 1 : (b0 < cr ? b0 : cr);
+    b1 = b1 < cl + 1 ? cl + 1 : (b1 < cr ? b1 : cr);
+    const double slope = (double)ly.slope, z1 = g.hc * slope, z0 = (g.ctr0 - even) * slope, x0 = g.ctr0 - v0;
+    for (int b = b0 + sub * 32 + lane; b < b1; b += 32 * tw) {
+      const double bd = (double)b;
+      const float* r = ly.rec.r + b;
+      const int st = ly.rec.stride;
+      const ScCoef c = sc_coef((float)fma(bd, z1, z0));
+      sc_bin_sums<false, float>(c, g.eta, r[0], r[st], r[2 * st], r[3 * st], r[4 * st], fma(bd, g.hc, x0), g.hc, acc);
+    }
+    if (sub == 0 && lane < 2) {
+      // outside it: lambda = 1 left of it, mu = 1 right of it
+      const int lo = lane ? b1 : cl + 1, hi = lane ? cr : b0;
+      const double nn = ly.rec.cn[hi] - ly.rec.cn[lo], xx = fma(-v0, nn, ly.rec.cx[hi] - ly.rec.cx[lo]);
+      acc[0] += lane ? 0.0 : nn;
+      acc[1] += lane ? 0.0 : xx;
+      acc[2] += lane ? nn : 0.0;
+      acc[3] += lane ? xx : 0.0;
+    }
+  }
+  if (sub == 0 && lane == 0 && sh.n0 > 0) {
+    // the weights that are exactly zero (see sc_zeros)
+    const float vl = sh.v[s - 1], vr = sh.v[s];
+    const double n = (vl < 0.f && vr > 0.f ? 1.0 : ((vl == 0.f && vr > 0.f) || (vl < 0.f && vr == 0.f) ? 0.5 : 0.0)) * (double)sh.n0;
+    float lam, mu;
+    sc_lambda((float)(-even * (double)ly.slope), lam, mu);
+    acc[0] += n * (double)lam;
+    acc[1] -= v0 * (n * (double)lam);
+    acc[2] += n * (double)mu;
+    acc[3] -= v0 * (n * (double)mu);
+  }
+  __syncwarp();
+  // four sums over the warp: the first two levels also deal the sums out, so that lanes 0, 8, 16, 24 end with one each
+  const bool h4 = lane & 16, h3 = lane & 8;
+  double p = h4 ? acc[2] : acc[0], q = h4 ? acc[3] : acc[1];
+  p += __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[2], 16);
+  q += __shfl_xor_sync(0xffffffffu, h4 ? acc[1] : acc[3], 16);
+  double r = h3 ? q : p;
+  r += __shfl_xor_sync(0xffffffffu, h3 ? p : q, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  if ((lane & 7) == 0) sh.ev[s * SLOTS + sub][lane >> 3] = r;
+}
+// The last M-step, as the first warp's lanes hold it for the stop test.
+struct SiLast {
+  double cnew, cold, s;
+};
+// Algorithm 1's stop test (see sc_stop_test); result in all lanes: the loop is done.
+template <int LOG>
+__device__ __forceinline__ bool si_stop_test(ScShared& sh, const ScalarParams& sp, int layer, const SiLast& la, int test) {
+  const int j = threadIdx.x;
+  const bool own = j < sp.k;
+  const double d = own ? la.cnew - la.cold : 0.0, c = own ? la.cnew : 0.0;
+  double num = d * d, den = c * c;
+  const bool bad = __any_sync(0xffffffffu, own && !(la.s <= 1e300 && fabs(la.cnew) <= 1e300));
+  const int dead = __popc(__ballot_sync(0xffffffffu, own && !(la.s >= S_MIN)));
+#pragma unroll
+  for (int o = (1 << LOG) / 2; o > 0; o >>= 1) {
+    num += __shfl_xor_sync(0xffffffffu, num, o);
+    den += __shfl_xor_sync(0xffffffffu, den, o);
+  }
+  // (a reciprocal from an fp32 seed where that has the range)
+  const float res = sqrtf((float)(den > 1e-30 && den < 1e30 ? num * sc_rcp(den) : num / fmax(den, 1e-300)));
+  const bool stop = __shfl_sync(0xffffffffu, (int)(sp.tol > 0.f && res < sp.tol), 0);
+  if (j == 0) {
+    sh.iters = test;
+    sh.res = res;
+    sh.dead = dead;
+    if (test <= HIST_CAP) sp.p.hist_fwd[(size_t)layer * HIST_CAP + test - 1] = res;
+    if (bad) sh.status = ST_NONFINITE;
+    else if (stop) sh.status = ST_OK;
+    else if (sp.tol > 0.f && test >= sp.max_iter) sh.status = ST_MAXITER;
+    if (bad || stop) sh.done = test;
+  }
+  return bad || stop;
+}
+// Returns the number of M-steps.
+template <int LOG>
+__device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, int layer) {
+  constexpr int SLOTS = si_slots<LOG>();
+  static_assert(((1 << LOG) + 1) * SLOTS <= SI_SLOTS, "slots of the intervals");
+  const ScLayer& ly = sh.ly;
+  const ScGrid& g = sh.g;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = sp.k, max_iter = sp.max_iter;
+  for (int i = threadIdx.x; i < SI_SLOTS * 4; i += SC_T) (&sh.ev[0][0])[i] = 0.0;
+  if (threadIdx.x == 0) sh.flag = 0;
+  __syncthreads();
+  int it = 0;
+  if (warp == 0) {
+    const int j = lane, jc = j < k ? j : k - 1;
+    const bool own = j < k;
+    ScScan<LOG> scn;
+#pragma unroll
+    for (int l = 0; l < LOG; ++l) scn.cb[l] = scn.cf[l] = 0.0;
+    SiLast la = {0.0, 0.0, 1.0};
+    float cn = sh.v[jc];
+    for (;;) {
+      if (it == max_iter) break;
+      si_arrive(SI_B1);
+      double rP, rQ;
+      sc_tables_warp(sh, ly, cn, scn, rP, rQ);
+      si_arrive(SI_B2);
+      const bool done = it > 0 && si_stop_test<LOG>(sh, sp, layer, la, it);
+      si_meet(SI_A);
+      if (done) {
+        if (j == 0) sh.flag = 1;
+        if (it + 1 < max_iter) {   // (the others wait at the next evaluation's meetings)
+          si_arrive(SI_B1);
+          si_arrive(SI_B2);
+        }
+        break;
+      }
+      // ---- M-step (Algorithm 1, step 5) ----
+      const double v0 = (double)sh.v[0];
+      double x[2] = {0.0, 0.0}, y[2] = {0.0, 0.0};
+#pragma unroll
+      for (int q = 0; q < SLOTS; ++q) {
+        const double2 l = reinterpret_cast<const double2*>(sh.ev[(jc + 1) * SLOTS + q])[0], m = reinterpret_cast<const double2*>(sh.ev[jc * SLOTS + q])[1];
+        x[0] += l.x;
+        x[1] += l.y;
+        y[0] += m.x;
+        y[1] += m.y;
+      }
+      x[0] *= rP;   // (rP = rQ = 0 in lanes without a centroid)
+      x[1] *= rP;
+      y[0] *= rQ;
+      y[1] *= rQ;
+      sc_scan_both<2, LOG>(scn, x, y);
+      la.cold = (double)cn;
+      la.s = x[0] + y[0];
+      la.cnew = la.s >= S_MIN ? fma(x[1] + y[1], sc_rcp(la.s), v0) : la.cold;
+      cn = own ? (float)la.cnew : __int_as_float(0x7f800000);
+      // (the map keeps the order of the centroids up to rounding)
+      const float left = __shfl_up_sync(0xffffffffu, cn, 1);
+      if (__any_sync(0xffffffffu, own && j > 0 && !(left <= cn))) {
+        if (own) {
+          sh.vn[j] = cn;
+          sh.idn[j] = sh.id[j];
+        }
+        __syncwarp();
+        sc_sort(sh, k);
+      } else if (own) {
+        sh.v[j] = cn;
+      }
+      __syncwarp();
+      cn = sh.v[jc];
+      ++it;
+    }
+    if (j == 0) sh.steps = it;
+    if (own) {   // (for the stop test of the last M-step)
+      sh.cnew[j] = la.cnew;
+      sh.cold[j] = la.cold;
+      sh.dead_j[j] = (la.s >= S_MIN ? 0 : 1) + (!(la.s <= 1e300 && fabs(la.cnew) <= 1e300) ? 0x10000 : 0);
+    }
+  } else {
+    // centroid j by warp j + 1 (16 centroids: the last by the second warp, besides the first); intervals by the warps that are
+    // left, several each where there are enough, or by those of the first centroids besides
+    constexpr int OTHERS = SC_WARPS - 1;
+    int tw = 1, sub = 0, s = 0;   // this warp's interval, 0: none
+    const int t = warp - 1 - k, free_warps = OTHERS - k;
+    if (free_warps >= k - 1) {
+      if (k > 1) {
+        tw = free_warps / (k - 1);
+        tw = tw > SLOTS - 2 ? SLOTS - 2 : tw;
+        if (t >= 0 && t < (k - 1) * tw) {
+          s = t / tw + 1;
+          sub = t % tw;
+        }
+      }
+    } else {
+      const int u = t >= 0 ? t : (free_warps > 0 ? free_warps : 0) + warp - 1;
+      if (u < k - 1) s = u + 1;
+    }
+    const int j = warp - 1;
+    SiBin bn;
+    bn.f = -1;
+    bn.e0 = bn.e1 = 0u;
+#pragma unroll
+    for (int i = 0; i < SI_WORDS; ++i) bn.w[i] = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) bn.m[i] = 0.0;
+    SiBelow o;
+    while (it < max_iter) {
+      if (j < k) {
+        si_meet(SI_B1);
+        si_below(sh, g, ly, bn, sh.v[j], o);
+      } else {
+        si_arrive(SI_B1);
+      }
+      si_meet(SI_B2);
+      if (sh.flag) break;
+      if (j < k) si_ends<SLOTS>(sh, g, ly, o, j);
+      if (j + OTHERS < k) {
+        si_below(sh, g, ly, bn, sh.v[j + OTHERS], o);
+        si_ends<SLOTS>(sh, g, ly, o, j + OTHERS);
+      }
+      if (s > 0) si_bins<SLOTS>(sh, g, ly, s, sub, tw);
+      si_arrive(SI_A);
+      ++it;
+    }
+  }
+  __syncthreads();
+  return sh.steps;
+}
+
 constexpr int SI_T = 1024, SI_WARPS = SI_T / 32;
 // ---- first launch: layer states, working centroids, counters to zero, value range of the weights ----
 __global__ void __launch_bounds__(SI_T, 1) idkm_scalar_init(const __grid_constant__ ScalarParams sp) {
@@ -1350,7 +1797,8 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
       lin_scan<2, true>(ap, y, k, sh.tmp);
     }
   };
-  tables();
+  constexpr bool quick = !DIRECT && LOG > 0 && (1 << LOG) <= SI_K;   // the iterations are sc_iterate's
+  if constexpr (!quick) tables();
   ScBin keep;
   keep.f = -1;
   keep.groups = 0;
@@ -1360,7 +1808,12 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
   __syncthreads();
 
   int it = 0;
-  while (it < sp.max_iter) {
+  if constexpr (quick) {
+    it = sc_iterate<LOG>(sh, sp, layer);
+    tables();
+    __syncthreads();
+  }
+  while (!quick && it < sp.max_iter) {
     if constexpr (DIRECT) {
       if (!sd_sums(sh, sp, layer, false, it)) {
         if (leader) sc_give_up(sp, layer, ST_TIMEOUT);

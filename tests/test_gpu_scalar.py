@@ -85,6 +85,26 @@ def test_interval_form_against_the_oracle(kind, m, k, tau):
     check(W, C0, float(np.float32(tau)), 6, 5, alpha=0.5)
 
 
+# n nearly equal weights around a centroid: a fine bin of n weights (one load a lane and several, what stays in registers and what
+# does not), its start at any element of a layer with an odd start, the last weights of all; 1 to 16 centroids (two of them
+# with one warp), bins split into one, 8 and more than 64 (sums of four, two and one powers of the place)
+@pytest.mark.parametrize("n,k,m,tau,where", [
+    (1, 1, 5000, 0.01, "inside"), (57, 2, 20011, 0.01, "inside"), (63, 3, 20011, 5e-4, "inside"), (64, 4, 20011, 0.01, "last"),
+    (65, 5, 20011, 0.01, "inside"), (249, 8, 20011, 0.004, "last"), (257, 9, 20010, 0.01, "inside"), (505, 15, 20011, 0.01, "last"),
+    (512, 16, 20011, 0.01, "inside"), (513, 4, 20011, 5e-4, "last"), (521, 16, 1 << 20, 0.05, "inside"), (1537, 7, 20011, 0.01, "last"),
+    (2559, 16, 300001, 0.01, "inside"), (2571, 6, 300001, 0.02, "last"), (4000, 16, 1 << 20, 0.05, "last"), (4100, 4, 1 << 20, 0.05, "inside"),
+])
+def test_interval_form_with_a_crowded_bin(n, k, m, tau, where):
+    rng = np.random.default_rng(n + k)
+    at = 0.0201 if where == "inside" else 0.2
+    W = np.concatenate([rng.standard_normal(1001) * 0.03, rng.standard_normal(m) * 0.03, at + rng.uniform(-1e-6, 1e-6, n)])
+    W = W.astype(np.float32).reshape(-1, 1)
+    second = W[1001:, 0]
+    C0 = np.concatenate([rng.choice(np.unique(W[:1001]), size=k, replace=False), [np.float32(at)],
+                         rng.choice(np.unique(second[:m]), size=k - 1, replace=False)]).astype(np.float32).reshape(-1, 1)
+    check(W, C0, float(np.float32(tau)), 6, 5, alpha=0.5, offs=[0, 1001, W.shape[0]])
+
+
 def test_interval_form_on_ragged_batches():
     """Unaligned layer starts, layers of a few weights and of many blocks, one that collapses, in one call."""
     rng = np.random.default_rng(5)
