@@ -18,7 +18,9 @@ namespace idkm {
 
 constexpr int SC_T = 512;              // threads of a block of the loop kernel (128 registers each)
 constexpr int SC_WARPS = SC_T / 32;
-constexpr int SC_FINE_BIG = 32768;     // fine bins of a layer: the workspace holds this many for the largest layers ...
+constexpr int SC_FINE_BIG = 40960;     // fine bins of a layer: the workspace holds this many for the largest layers ...
+constexpr int SC_FINE_MOST = 32768;    // ... of which layers of less than SC_FINE_ROWS weights use this many at most,
+constexpr long long SC_FINE_ROWS = 8LL << 20;
 constexpr int SC_FINE_SMALL = 16384;   // ... and this many for the others
 constexpr int SC_BIG_LAYERS = 8;
 constexpr int SC_REC_SMEM = 3584;      // coarse bins whose records fit in shared memory (36 bytes each)

@@ -15,7 +15,7 @@
 // (110 us per 11.7 M weights on all SMs).  Iterating: the chain of one block a layer, 1.7 us at k <= 4 to 6 us, whatever the
 // number of weights (sc_iterate up to 16 centroids).  Measured, loop with the summary against one that
 // visits the pairs: 21 layers of a ResNet-18, k = 4, 50 iterations 352 against 1473 us; k = 8, tau = 5e-4, 30 iterations 380
-// against 1268; 16 M weights, k = 16, 100 iterations 1.26 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 68
+// against 1268; 16 M weights, k = 16, 100 iterations 1.09 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 68
 // against 112.
 //
 // Layers that bins do not suit -- tau below 1 / 5700 of the weights' range (1 / 2800 in layers beyond the eighth), which an outlier
@@ -63,6 +63,11 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   if (!(range > amax * 1e-6)) range = amax * 1e-6;
   const double hmin = amax * (1.0 / 2097152.0);   // indices stay below 2^21 in magnitude
   double hc = 0.17 * tau;
+  // (a layer of very many weights is given more fine bins, as its iterations look at all weights of the centroids' bins: 16 M
+  // weights, k = 16, 100 iterations, the whole call 1477 us with at most 32768 bins, 1306 with 40960; a layer of 2.4 M weights would
+  // go from 16640 to 33280 bins, whose prefix costs about what 50 iterations gain)
+  const int wide = m < SC_FINE_ROWS ? SC_FINE_MOST : cap;
+  if (cap > SC_FINE_MOST) cap = SC_FINE_MOST;
   if (hc < range / (double)(cap - 8)) hc = range / (double)(cap - 8);
   if (hc > range) hc = range;
   if (hc < hmin) hc = hmin;
@@ -71,7 +76,8 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   const long long nc0 = (long long)(range / hc) + 5;
   long long want = m / 64 < 512 ? 512 : m / 64;
   if (want < 16 * nc0) want = 16 * nc0 < m / 8 ? 16 * nc0 : (want < m / 8 ? m / 8 : want);
-  if (want > cap) want = cap;
+  const int most = cap < SC_FINE_MOST ? cap : wide;
+  if (want > most) want = most;
   int f = 0;
   while (f < 12 && hc / (double)(2 << f) >= hmin && (nc0 << (f + 1)) <= want) ++f;
   g.inv_hf = (float)((double)(1 << f) / hc);
@@ -1156,7 +1162,8 @@ __device__ __noinline__ bool sd_sums(ScShared& sh, const ScalarParams& sp, int l
 // the loop may live in local memory: with the shared memory the block takes the L1 cache holds none of it, and every access
 // is a trip to L2; and a load whose value is used before the next one is issued is one more such trip.  Cycles an iteration,
 // before (counts, ends and M-step one after the other between meetings of the block) and now: 4096 weights, k = 4 5500 and 3300;
-// 36864, k = 8 6700 and 4600; 2.4 M, k = 4 8000 and 5900; 16 M, k = 16 24000 and 19800 (the fine bins hold thousands of weights).
+// 36864, k = 8 6700 and 4600; 2.4 M, k = 4 8000 and 5900; 16 M, k = 16 24000 and 19800 (the fine bins hold thousands
+// of weights; with twice as many of them about 16000).
 constexpr int SI_WORDS = 8, SI_HEAD = 64 * SI_WORDS;
 constexpr int SI_A = 2, SI_B1 = 3, SI_B2 = 4;   // hardware barriers
 __device__ __forceinline__ void si_arrive(int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(SC_T) : "memory"); }

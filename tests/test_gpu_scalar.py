@@ -75,6 +75,7 @@ def check(W, C0, tau, iters, adj_iters, alpha=1.0, offs=None):
     ("normal", 50001, 256, 0.02), ("laplace", 65536, 16, 5e-4), ("normal", 8192, 8, 5e-5), ("laplace", 150000, 12, 2e-5),
     ("pruned", 120001, 4, 0.01), ("pruned", 30000, 7, 0.002), ("levels", 150001, 5, 0.004), ("offset", 40000, 4, 5e-4),
     ("outlier", 70000, 5, 0.003), ("outlier", 70000, 5, 2e-4), ("normal", 20000, 3, 10.0), ("normal", 1 << 20, 4, 0.002),
+    ("normal", 8 << 20, 16, 0.01), ("normal", (8 << 20) - 1, 16, 0.01),   # (either side of the rule for more fine bins)
 ])
 def test_interval_form_against_the_oracle(kind, m, k, tau):
     rng = np.random.default_rng(m + k)
