@@ -136,6 +136,11 @@ constexpr double SC_S2 = 16384.0 * SC_S1 * SC_S1;
 constexpr double SC_S3 = 536870912.0 * SC_S1 * SC_S1 * SC_S1;
 constexpr double SC_S4 = 17592186044416.0 * SC_S1 * SC_S1 * SC_S1 * SC_S1;
 constexpr int SC_CHUNK = 8192;   // elements whose 32-bit integer sums cannot overflow
+// Which powers of the place matter: a fine bin is 1 / F of a coarse bin, so the fourth and third power of a place inside it
+// change the interval's sums by less than 1e-8 from F = 64 on, and so does the square in the one bin that is split.  With
+// fewer fine bins all four do: 3000 of 4096 weights in a tenth of one coarse bin, F = 8, five iterations from 16 centroids within
+// the same tenth of it, centroids against float64: 2e-6 with all powers, 3e-5 without the third and the fourth.
+__device__ __forceinline__ bool sc_full(const ScGrid& g) { return g.F < 64; }
 
 // Moments about the coarse bin's centre, in units of the coarse width, of n weights of fine bin kf (0 .. F - 1) whose
 // integer sums of powers of the place are s1 .. s4.
@@ -384,10 +389,9 @@ __device__ __forceinline__ void sc_bin_load(const ScLayer& ly, int f, unsigned i
   }
 }
 // Sums over the bin's weights that lie below place pv, weights at pv itself counting half: twice the count and twice the
-// sums of the powers of the place.  Result in every lane.  Which powers matter: a fine bin is 1 / F of a coarse bin, so
-// the fourth and third power of a place inside it change the interval's sums by less than 1e-8 from F = 64 on, and so
-// does the square in the one bin that is split.  This part: the weights that are not in registers, eight places per
-// load, two loads in flight beyond the one being counted, in stretches whose 32-bit sums cannot overflow.
+// sums of the powers of the place.  Result in every lane.  `full`: see sc_full.  This part: the weights that are not in
+// registers, eight places per load, two loads in flight beyond the one being counted, in stretches whose 32-bit sums
+// cannot overflow.
 __device__ __noinline__ void sc_bin_below_rest(const ScLayer& ly, long long t0, long long t1, int pv, bool full, double* s) {
   const int lane = threadIdx.x & 31;
   for (long long tb = t0; tb < t1; tb += SC_CHUNK) {
@@ -820,7 +824,7 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
 // Both halves; the last warp first runs the stop test of the M-step before (`test` = its number, 0: none).
 template <bool EXTRA>
 __device__ __forceinline__ void sc_evaluate(ScShared& sh, const ScLayer& ly, ScBin& keep, const ScalarParams& sp, int layer, int test) {
-  const bool full = sh.g.F < 64;
+  const bool full = sc_full(sh.g);
   if (test > 0 && threadIdx.x >= SC_T - 32) sc_stop_test(sh, sp, layer, test);
   if (ly.k <= SC_WARPS) sc_scan_warps(sh, ly, keep, full);
   else sc_scan_quarters(sh, full);
@@ -1202,7 +1206,6 @@ __device__ __forceinline__ void si_words(const ScLayer& ly, long long base, int 
   }
 }
 __device__ __forceinline__ void si_bin_load(const ScLayer& ly, int f, SiBin& bn) {
-  const int lane = threadIdx.x & 31;
   bn.f = f;
   bn.e0 = ly.fstart[f];
   bn.e1 = ly.fstart[f + 1];
@@ -1219,14 +1222,15 @@ __device__ __forceinline__ void si_bin_load(const ScLayer& ly, int f, SiBin& bn)
   bn.m[3] = r1.y;
 }
 // Sums over n places p (from 1; 0: none) that lie below pv, those at it counting half, without a comparison: with S(x) the sum
-// of min(p, x), S(x) - S(x - 1) places are at x or beyond.  Two places per instruction.
+// of min(p, x), S(x) - S(x - 1) places are at x or beyond.  Two places per instruction.  Powers (`full`): of min(p, pv), those
+// beyond taken off again in si_total.
 struct SiSum {
   unsigned int a, b, c;   // S(pv), S(pv + 1), S(pv - 1)
   int q2, q3, q4;
 };
 struct SiCut {
   unsigned int a, b, c;   // pv, pv + 1, pv - 1 in both halves
-  int pv;
+  bool none;              // below the scale
 };
 __device__ __forceinline__ SiCut si_cut(int pv) {
   // beyond the ends of the scale: below everything the result is set to zero, above everything the three sums are equal
@@ -1235,46 +1239,42 @@ __device__ __forceinline__ SiCut si_cut(int pv) {
   t.a = a * 0x10001u;
   t.b = b * 0x10001u;
   t.c = c * 0x10001u;
-  t.pv = pv;
+  t.none = pv < 1;
   return t;
 }
-// Powers of the place.  A fine bin is 1 / F of a coarse bin: from F = 8 on its third and fourth powers, from F = 64 on its second
-// change an interval's sums by less than 1e-8.
-__device__ __forceinline__ int si_powers(int F) { return F >= 64 ? 1 : (F >= 8 ? 2 : 4); }
-__device__ __forceinline__ void si_add(unsigned int x, const SiCut& t, int powers, SiSum& s) {
-  s.a = __dp2a_lo(__vminu2(x, t.a), 0x0101u, s.a);
+__device__ __forceinline__ void si_add(unsigned int x, const SiCut& t, bool full, SiSum& s) {
+  const unsigned int y = __vminu2(x, t.a);
+  s.a = __dp2a_lo(y, 0x0101u, s.a);
   s.b = __dp2a_lo(__vminu2(x, t.b), 0x0101u, s.b);
   s.c = __dp2a_lo(__vminu2(x, t.c), 0x0101u, s.c);
-  if (powers > 1) {
+  if (full) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int u = (int)(i ? x >> 16 : x & 0xffffu), p = u > 0 ? u - 32768 : 0;
-      const int w = u < t.pv ? 2 : (u == t.pv ? 1 : 0);
-      if (powers == 2) {
-        s.q2 += w * ((p * p + 8192) >> 14);
-      } else {
-        int p2, p3, p4;
-        sc_powers(p, p2, p3, p4);
-        s.q2 += w * p2;
-        s.q3 += w * p3;
-        s.q4 += w * p4;
-      }
+      const int u = (int)(i ? y >> 16 : y & 0xffffu), p = u > 0 ? u - 32768 : 0;
+      int p2, p3, p4;
+      sc_powers(p, p2, p3, p4);
+      s.q2 += p2;
+      s.q3 += p3;
+      s.q4 += p4;
     }
   }
 }
-// Over the warp, n places in all (at most 2^15): twice the count and sums of powers.
-__device__ __forceinline__ void si_total(const SiSum& s, int n, const SiCut& t, int powers, double (&b)[5]) {
+// Over the warp, n places in all (fewer than SC_CHUNK + 1024): twice the count and sums of powers.
+__device__ __forceinline__ void si_total(const SiSum& s, int n, const SiCut& t, bool full, double (&b)[5]) {
   const unsigned int a = __reduce_add_sync(0xffffffffu, s.a), up = __reduce_add_sync(0xffffffffu, s.b - s.a), at = __reduce_add_sync(0xffffffffu, s.a - s.c);
-  const int lt2 = 2 * n - (int)(up + at), eq = (int)(at - up);   // up: beyond pv, at: at it or beyond
+  const int lt2 = 2 * n - (int)(up + at), over = (int)(at + up);   // up: beyond pv, at: at it or beyond
   // twice the sum of the places below (the sum of all, those beyond counted as pv), those at pv half
-  const long long p2 = 2LL * a - (long long)(t.a & 0xffffu) * (2LL * at - eq);
-  const bool none = t.pv < 1;
-  b[0] += none ? 0.0 : (double)lt2;
-  b[1] += none ? 0.0 : (double)(p2 - 32768LL * lt2);
-  if (powers > 1) b[2] += (double)__reduce_add_sync(0xffffffffu, s.q2);
-  if (powers > 2) {
-    b[3] += (double)__reduce_add_sync(0xffffffffu, s.q3);
-    b[4] += (double)__reduce_add_sync(0xffffffffu, s.q4);
+  const int pv = (int)(t.a & 0xffffu);
+  const long long p2 = 2LL * a - (long long)pv * over;
+  b[0] += t.none ? 0.0 : (double)lt2;
+  b[1] += t.none ? 0.0 : (double)(p2 - 32768LL * lt2);
+  if (full) {
+    int v2, v3, v4;
+    sc_powers(pv - 32768, v2, v3, v4);
+    const int q2 = __reduce_add_sync(0xffffffffu, s.q2), q3 = __reduce_add_sync(0xffffffffu, s.q3), q4 = __reduce_add_sync(0xffffffffu, s.q4);
+    b[2] += t.none ? 0.0 : (double)(2LL * q2 - (long long)v2 * over);
+    b[3] += t.none ? 0.0 : (double)(2LL * q3 - (long long)v3 * over);
+    b[4] += t.none ? 0.0 : (double)(2LL * q4 - (long long)v4 * over);
   }
 }
 // What lies below a centroid in its coarse bin.
@@ -1289,7 +1289,7 @@ __device__ __forceinline__ void si_below(const ScShared& sh, const ScGrid& g, co
   // one beyond the ends of the scale where the centroid lies outside the weights' range
   const int pv = v > g.hi ? 72768 : (v < g.lo ? -7232 : place + 32768);
   if (bn.f != f) si_bin_load(ly, f, bn);
-  const int powers = si_powers(g.F);
+  const bool full = sc_full(g);
   const SiCut t = si_cut(pv);
   SiSum s = {0u, 0u, 0u, 0, 0, 0};
   const long long base = si_base(ly, bn), end = ly.row0 + bn.e1;
@@ -1297,7 +1297,7 @@ __device__ __forceinline__ void si_below(const ScShared& sh, const ScGrid& g, co
 #pragma unroll
   for (int i = 0; i < SI_WORDS; ++i) {
     if (i > 0 && 64 * i >= hi) break;
-    si_add(bn.w[i], t, powers, s);
+    si_add(bn.w[i], t, full, s);
   }
   double b[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   int n = hi - (int)(ly.row0 + bn.e0 - base);
@@ -1323,20 +1323,20 @@ __device__ __forceinline__ void si_below(const ScShared& sh, const ScGrid& g, co
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      si_add(q[i].x, t, powers, s);
-      si_add(q[i].y, t, powers, s);
-      si_add(q[i].z, t, powers, s);
-      si_add(q[i].w, t, powers, s);
+      si_add(q[i].x, t, full, s);
+      si_add(q[i].y, t, full, s);
+      si_add(q[i].z, t, full, s);
+      si_add(q[i].w, t, full, s);
     }
     n += end - e < 1024 ? (int)(end - e) : 1024;
     e += 1024;
     if (n >= SC_CHUNK) {
-      si_total(s, n, t, powers, b);
+      si_total(s, n, t, full, b);
       s = SiSum{0u, 0u, 0u, 0, 0, 0};
       n = 0;
     }
   }
-  si_total(s, n, t, powers, b);
+  si_total(s, n, t, full, b);
 #pragma unroll
   for (int i = 0; i < 5; ++i) b[i] *= 0.5;
   o.c = f >> g.fshift;
@@ -2200,7 +2200,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
         const unsigned short* all = own ? grouped : sp.p.grouped;
         const long long row0 = own ? 0 : sp.row_off[layer], total = own ? m : sp.row_off[sp.n_layers];
         const int step = NB * SC_T / 8, ql = lane & 7;
-        const bool full = g.F < 64;   // (see sc_bin_below)
+        const bool full = sc_full(g);
         const unsigned int qmask = 0xffu << (lane & 24);
         int i = (b * SC_T + tid) >> 3;
         long long A0 = 0, A1 = 0;

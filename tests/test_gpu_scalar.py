@@ -106,6 +106,26 @@ def test_interval_form_with_a_crowded_bin(n, k, m, tau, where):
     check(W, C0, float(np.float32(tau)), 6, 5, alpha=0.5, offs=[0, 1001, W.shape[0]])
 
 
+# centroids within a fraction of a fine bin of each other, and most weights there with them: a coarse bin is split in 8, so that the
+# third and the fourth power of a weight's place in its fine bin count (without them 1.1e-5 to 3.3e-5, with them below 3e-6)
+@pytest.mark.parametrize("k,spread", [(4, 0.1), (4, 0.03), (16, 0.03), (16, 0.01)])
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_interval_form_with_close_centroids(k, spread, seed):
+    import torch
+    from oracle import idkm_ref as R
+    from paper_2312_07759_b200 import binding as B
+    tau = 0.05
+    rng = np.random.default_rng(1000 * seed + k)
+    near, far = rng.random(1500) * 0.02 * tau, rng.random(548) * 4.5 * tau
+    W = np.concatenate([near, -near, far, -far]).astype(np.float32).reshape(-1, 1)
+    C0 = ((2 * np.arange(k) + 1 - k) / k * spread * tau).astype(np.float32).reshape(-1, 1)
+    tau = float(np.float32(tau))
+    ctx = B.Context()
+    C = ctx.forward(torch.from_numpy(W).cuda(), torch.from_numpy(C0).cuda(), tau, 0.0, 5).C.cpu().numpy()
+    assert ctx.last_route()["forward"] == "interval form"
+    assert_close(C, R.forward(W.astype(np.float64), C0.astype(np.float64), tau, 0.0, 5)[0], TOL_C, "C")
+
+
 def test_interval_form_on_ragged_batches():
     """Unaligned layer starts, layers of a few weights and of many blocks, one that collapses, in one call."""
     rng = np.random.default_rng(5)
