@@ -202,10 +202,15 @@ static int jac_mma_min_iters(int d, int k) {
   return n < least ? least : n;
 }
 
-// Fine bins the workspace holds for n_layers layers of scalar weights: the largest layers get more.
-static int scalar_fine_total(int n_layers) {
+// Fine bins the workspace holds for a layer of scalar weights that `larger` layers come before in size.
+static int scalar_fine_bins(long long rows, int larger) {
+  return larger >= SC_BIG_LAYERS ? SC_FINE_SMALL : (rows < SC_FINE_ROWS ? SC_FINE_BIG : SC_FINE_MOST);
+}
+// ... for n_layers layers of m_total weights, however these are dealt to them.
+static int scalar_fine_total(int64_t m_total, int n_layers) {
   const int big = n_layers < SC_BIG_LAYERS ? n_layers : SC_BIG_LAYERS;
-  return big * SC_FINE_BIG + (n_layers - big) * SC_FINE_SMALL;
+  const int most = m_total / SC_FINE_ROWS < big ? (int)(m_total / SC_FINE_ROWS) : big;
+  return most * SC_FINE_MOST + (big - most) * SC_FINE_BIG + (n_layers - big) * SC_FINE_SMALL;
 }
 
 constexpr size_t NO_ROWSTAT = ~(size_t)0;
@@ -293,7 +298,7 @@ static bool make_layout(int64_t m_total, int d, int k, int n_layers, int sms, Wo
   w.sc_fine = 0;
   if (d == 1) {
     const int L = n_layers, K1 = k + 1;
-    const size_t nf = (size_t)scalar_fine_total(L);
+    const size_t nf = (size_t)scalar_fine_total(m_total, L);
     w.sc_fine = (int)nf;
     w.n_sc_grad_blocks = 2 * sms + L;
     w.n_sc_groups = w.n_sc_grad_blocks / RED_GROUP + 2 * L + 2;
@@ -804,7 +809,7 @@ static void scalar_params(const idkm_ctx* ctx, const WorkspaceLayout& wl, const 
         const long long r = ctx->row_off[o + 1] - ctx->row_off[o];
         larger += (r > rows || (r == rows && o < l));
       }
-    sp->fine_off[l + 1] = sp->fine_off[l] + (larger < SC_BIG_LAYERS ? SC_FINE_BIG : SC_FINE_SMALL);
+    sp->fine_off[l + 1] = sp->fine_off[l] + scalar_fine_bins(rows, larger);
   }
   for (int l = L + 1; l <= MAX_LAYERS; ++l) sp->fine_off[l] = sp->fine_off[L];
 }

@@ -63,11 +63,9 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   if (!(range > amax * 1e-6)) range = amax * 1e-6;
   const double hmin = amax * (1.0 / 2097152.0);   // indices stay below 2^21 in magnitude
   double hc = 0.17 * tau;
-  // (a layer of very many weights is given more fine bins, as its iterations look at all weights of the centroids' bins: 16 M
-  // weights, k = 16, 100 iterations, the whole call 1477 us with at most 32768 bins, 1306 with 40960; a layer of 2.4 M weights would
-  // go from 16640 to 33280 bins, whose prefix costs about what 50 iterations gain)
-  const int wide = m < SC_FINE_ROWS ? SC_FINE_MOST : cap;
-  if (cap > SC_FINE_MOST) cap = SC_FINE_MOST;
+  // (the widest coarse bins do not depend on the number of weights)
+  const int most = cap;
+  if (cap > SC_FINE_BIG) cap = SC_FINE_BIG;
   if (hc < range / (double)(cap - 8)) hc = range / (double)(cap - 8);
   if (hc > range) hc = range;
   if (hc < hmin) hc = hmin;
@@ -76,7 +74,6 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   const long long nc0 = (long long)(range / hc) + 5;
   long long want = m / 64 < 512 ? 512 : m / 64;
   if (want < 16 * nc0) want = 16 * nc0 < m / 8 ? 16 * nc0 : (want < m / 8 ? m / 8 : want);
-  const int most = cap < SC_FINE_MOST ? cap : wide;
   if (want > most) want = most;
   int f = 0;
   while (f < 12 && hc / (double)(2 << f) >= hmin && (nc0 << (f + 1)) <= want) ++f;
@@ -217,7 +214,7 @@ struct ScShared {
   double scan_x[SC_WARPS + 1];
 };
 constexpr int SC_SH_BYTES = (int)((sizeof(ScShared) + 255) / 256 * 256);
-constexpr int SC_BIN_BYTES = (SC_FINE_BIG * 4 > SC_REC_SMEM * SC_REC_BYTES + 16) ? SC_FINE_BIG * 4 : SC_REC_SMEM * SC_REC_BYTES + 16;
+constexpr int SC_BIN_BYTES = (SC_FINE_MOST * 4 > SC_REC_SMEM * SC_REC_BYTES + 16) ? SC_FINE_MOST * 4 : SC_REC_SMEM * SC_REC_BYTES + 16;
 // without bins (sd_pass): sums of every thread, of every warp, tables of the search
 constexpr int SD_COLS = SC_WARPS * 257 * 4 * 8, SD_WSUM = 8448, SD_BYTES = SD_COLS + SD_WSUM + (512 + 2 * 257) * 4;
 constexpr int SC_DYN = SC_SH_BYTES + (SC_BIN_BYTES > SD_BYTES ? SC_BIN_BYTES : SD_BYTES);
