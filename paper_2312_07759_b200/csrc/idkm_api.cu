@@ -202,17 +202,6 @@ static int jac_mma_min_iters(int d, int k) {
   return n < least ? least : n;
 }
 
-// Fine bins the workspace holds for a layer of scalar weights that `larger` layers come before in size.
-static int scalar_fine_bins(long long rows, int larger) {
-  return larger >= SC_BIG_LAYERS ? SC_FINE_SMALL : (rows < SC_FINE_ROWS ? SC_FINE_BIG : SC_FINE_MOST);
-}
-// ... for n_layers layers of m_total weights, however these are dealt to them.
-static int scalar_fine_total(int64_t m_total, int n_layers) {
-  const int big = n_layers < SC_BIG_LAYERS ? n_layers : SC_BIG_LAYERS;
-  const int most = m_total / SC_FINE_ROWS < big ? (int)(m_total / SC_FINE_ROWS) : big;
-  return most * SC_FINE_MOST + (big - most) * SC_FINE_BIG + (n_layers - big) * SC_FINE_SMALL;
-}
-
 constexpr size_t NO_ROWSTAT = ~(size_t)0;
 
 static int device_sm_count() {
@@ -800,7 +789,6 @@ static void scalar_params(const idkm_ctx* ctx, const WorkspaceLayout& wl, const 
   sp->wq_dtype = ctx->wq_dtype;
   const int L = ctx->n_layers;
   for (int l = 0; l <= MAX_LAYERS; ++l) sp->row_off[l] = ctx->row_off[l < L ? l : L];
-  // fine bins: the SC_BIG_LAYERS largest layers get the larger share
   for (int l = 0; l < L; ++l) {
     const long long rows = ctx->row_off[l + 1] - ctx->row_off[l];
     int larger = 0;
@@ -809,7 +797,7 @@ static void scalar_params(const idkm_ctx* ctx, const WorkspaceLayout& wl, const 
         const long long r = ctx->row_off[o + 1] - ctx->row_off[o];
         larger += (r > rows || (r == rows && o < l));
       }
-    sp->fine_off[l + 1] = sp->fine_off[l] + scalar_fine_bins(rows, larger);
+    sp->fine_off[l + 1] = sp->fine_off[l] + scalar_fine_bins(rows, larger, ctx->row_off[L]);
   }
   for (int l = L + 1; l <= MAX_LAYERS; ++l) sp->fine_off[l] = sp->fine_off[L];
 }

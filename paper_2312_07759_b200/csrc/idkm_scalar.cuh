@@ -13,17 +13,12 @@
 // coefficients a_j = exp(-(v_{j+1} - v_j)/tau) (Algorithm 1, step 5; Sections 4.1-4.3).
 #pragma once
 #include "idkm_kernels.cuh"
+#include "idkm_scalar_bins.h"
 
 namespace idkm {
 
 constexpr int SC_T = 512;              // threads of a block of the loop kernel (128 registers each)
 constexpr int SC_WARPS = SC_T / 32;
-// fine bins the workspace holds: for the largest layers of at least SC_FINE_ROWS weights (an iteration looks at all weights of the
-// centroids' bins: 16 M weights, k = 16, 100 iterations, the whole call 1477 us with at most 32768 bins, 1306 with 40960), for the
-// other ones of the SC_BIG_LAYERS largest, and for the rest
-constexpr int SC_FINE_MOST = 40960, SC_FINE_BIG = 32768, SC_FINE_SMALL = 16384;
-constexpr long long SC_FINE_ROWS = 8LL << 20;
-constexpr int SC_BIG_LAYERS = 8;
 constexpr int SC_REC_SMEM = 3584;      // coarse bins whose records fit in shared memory (36 bytes each)
 constexpr int SC_REC_BYTES = 36;
 constexpr int SC_SYNC_WORDS = 32;      // barrier words of one layer (one 128-byte line)

@@ -63,7 +63,7 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   if (!(range > amax * 1e-6)) range = amax * 1e-6;
   const double hmin = amax * (1.0 / 2097152.0);   // indices stay below 2^21 in magnitude
   double hc = 0.17 * tau;
-  // (the widest coarse bins do not depend on the number of weights)
+  // (how wide the coarse bins get does not depend on the number of weights)
   const int most = cap;
   if (cap > SC_FINE_BIG) cap = SC_FINE_BIG;
   if (hc < range / (double)(cap - 8)) hc = range / (double)(cap - 8);

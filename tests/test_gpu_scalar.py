@@ -75,7 +75,7 @@ def check(W, C0, tau, iters, adj_iters, alpha=1.0, offs=None):
     ("normal", 50001, 256, 0.02), ("laplace", 65536, 16, 5e-4), ("normal", 8192, 8, 5e-5), ("laplace", 150000, 12, 2e-5),
     ("pruned", 120001, 4, 0.01), ("pruned", 30000, 7, 0.002), ("levels", 150001, 5, 0.004), ("offset", 40000, 4, 5e-4),
     ("outlier", 70000, 5, 0.003), ("outlier", 70000, 5, 2e-4), ("normal", 20000, 3, 10.0), ("normal", 1 << 20, 4, 0.002),
-    ("normal", 8 << 20, 16, 0.01), ("normal", (8 << 20) - 1, 16, 0.01),   # (either side of the rule for more fine bins)
+    ("normal", 8 << 20, 16, 0.01), ("normal", (8 << 20) - 1, 16, 0.01),
 ])
 def test_interval_form_against_the_oracle(kind, m, k, tau):
     rng = np.random.default_rng(m + k)
@@ -84,6 +84,33 @@ def test_interval_form_against_the_oracle(kind, m, k, tau):
     u = np.unique(W)
     C0 = rng.choice(u, size=min(k, u.size), replace=False).reshape(-1, 1).astype(np.float32)
     check(W, C0, float(np.float32(tau)), 6, 5, alpha=0.5)
+
+
+def bins(W, tau, cap):
+    """Fine bins of a layer that may have `cap` of them: coarse bins 0.17 tau wide, each split in a power of two."""
+    m, span, floor = W.size, float(W.max()) - float(W.min()), min(cap, 32768) - 8
+    width = max(0.17 * tau, span / floor)
+    coarse = int(span / width) + 5
+    want = max(m // 64, 512)
+    if want < 16 * coarse:
+        want = 16 * coarse if 16 * coarse < m // 8 else max(want, m // 8)
+    f = 1
+    while coarse * f * 2 <= min(want, cap):
+        f *= 2
+    return coarse * f
+
+
+# either side of the rule for more than 32768 fine bins, at a tau where they make a difference: the layer's size, its share of the
+# call, the size of the call (one layer that may have them, besides others that may not)
+@pytest.mark.parametrize("sizes", [(10 << 20,), ((10 << 20) - 1,), ((10 << 20) + 3, 4099, 1001), ((10 << 20) + 3, (10 << 20) + 4)])
+def test_interval_form_with_the_most_bins(sizes):
+    rng = np.random.default_rng(len(sizes))
+    offs = [0] + [int(x) for x in np.cumsum(sizes)]
+    W = (rng.standard_normal((offs[-1], 1)) * 0.03).astype(np.float32)
+    tau = float(np.float32((float(W[:sizes[0]].max()) - float(W[:sizes[0]].min())) / 140.5 / 0.17))
+    assert bins(W[:sizes[0]], tau, 32768) <= 20000 and 32768 < bins(W[:sizes[0]], tau, 40960) <= 40960
+    C0 = np.concatenate([rng.choice(np.unique(W[a:b]), size=8, replace=False) for a, b in zip(offs, offs[1:])]).reshape(-1, 1)
+    check(W, C0, tau, 6, 3, alpha=0.5, offs=offs)
 
 
 # n nearly equal weights around a centroid: a fine bin of n weights (one load a lane and several, what stays in registers and what

@@ -38,13 +38,12 @@ def test_host_only_calls_work_without_a_device():
 
 
 def test_scalar_layers_reserve_the_bins_they_can_use():
-    """A fine bin takes 76 bytes; only a layer of 8 M weights can use more than 32768 of them, and enough room for the largest
-    call is enough for every smaller one."""
+    """A fine bin takes 76 bytes; only one layer of 10 M weights or more can use more than 32768 of them, and enough room for the
+    largest call is enough for every smaller one."""
     from paper_2312_07759_b200 import binding as B
-    rows = 8 << 20
+    rows = 10 << 20
     size = lambda m, layers=1: B.workspace_bytes(m, 1, 4, layers)
-    assert size(rows - 1) == size(4096) and size(rows) - size(rows - 1) == 8192 * 76
-    assert size(3 * rows - 1, 64) - size(4096, 64) == 2 * 8192 * 76
+    assert size(rows - 1) == size(4096) and size(rows) - size(rows - 1) == 8192 * 76 == size(9 * rows, 64) - size(4096, 64)
     for layers in (1, 3, 64):
         sizes = [size(m, layers) for m in (4096, rows - 1, rows, 2 * rows, 4 * rows, 5 * rows, 8 * rows, 9 * rows, 64 * rows)]
         assert sizes == sorted(sizes)
