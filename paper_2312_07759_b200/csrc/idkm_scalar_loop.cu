@@ -1159,8 +1159,8 @@ __device__ __noinline__ bool sd_sums(ScShared& sh, const ScalarParams& sp, int l
 // the M-step and publishes the centroids (meeting B1), then the even points and places (B2); a warp per centroid counts its
 // fine bin between the two and afterwards takes the ends of the two intervals the centroid borders; other warps have the
 // whole bins of an interval; at the third meeting (A) the first warp has all sums.  What a warp does is the same in every
-// iteration, and a centroid's fine bin (up to SI_HEAD of its places, and its record) stays in its warp's registers.  Nothing in
-// the loop may live in local memory: with the shared memory the block takes the L1 cache holds none of it, and every access
+// iteration, and a centroid's fine bin (up to SI_HEAD of its places, and its record) stays in its warp's registers, unless the
+// warp has two centroids (16 of them).  Nothing in the loop may live in local memory: with the shared memory the block takes the L1 cache holds none of it, and every access
 // is a trip to L2; and a load whose value is used before the next one is issued is one more such trip.  Cycles an iteration,
 // before (counts, ends and M-step one after the other between meetings of the block) and now: 4096 weights, k = 4 5500 and 3300;
 // 36864, k = 8 6700 and 4600; 2.4 M, k = 4 8000 and 5900; 16 M, k = 16 24000 and 19800 (the fine bins hold thousands
@@ -1343,9 +1343,9 @@ __device__ __forceinline__ void si_below(const ScShared& sh, const ScGrid& g, co
   for (int i = 0; i < 4; ++i) o.m[i] += bn.m[i];
 }
 // Centroid j: the right end of interval j (even lanes) and the left end of interval j + 1 (odd lanes); where there is no such
-// interval, all weights beyond.
+// interval, all weights beyond.  `pairs` of lanes have a centroid each.
 template <int SLOTS>
-__device__ __forceinline__ void si_ends(ScShared& sh, const ScGrid& g, const ScLayer& ly, const SiBelow& o, int j) {
+__device__ __forceinline__ void si_ends(ScShared& sh, const ScGrid& g, const ScLayer& ly, const SiBelow& o, int j, int pairs) {
   const int k = ly.k, lane = threadIdx.x & 31;
   const bool left = lane & 1;
   const int s = left ? j + 1 : j;
@@ -1373,7 +1373,7 @@ __device__ __forceinline__ void si_ends(ScShared& sh, const ScGrid& g, const ScL
   for (int i = 0; i < 4; ++i) m[i] = left ? (whole ? (double)r[i + 1] : 0.0) - o.m[i] : o.m[i];
   double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   sc_bin_sums<false, double>(co, g.eta, n, m[0], m[1], m[2], m[3], ctr - v0, g.hc, acc);
-  if (lane < 2) {
+  if (lane < 2 * pairs) {
     double2* d = reinterpret_cast<double2*>(sh.ev[s * SLOTS + (left ? SLOTS - 2 : SLOTS - 1)]);
     d[0] = inner ? make_double2(acc[0], acc[1]) : make_double2(left ? nn : 0.0, left ? xx : 0.0);
     d[1] = inner ? make_double2(acc[2], acc[3]) : make_double2(left ? 0.0 : nn, left ? 0.0 : xx);
@@ -1493,6 +1493,10 @@ __device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, 
       sc_tables_warp(sh, ly, cn, scn, rP, rQ);
       si_arrive(SI_B2);
       const bool done = it > 0 && si_stop_test<LOG>(sh, sp, layer, la, it);
+      if (LOG == 4 && k == SC_WARPS && !done) {
+        __syncwarp();
+        si_bins<SLOTS>(sh, g, ly, 1, 0, 1);
+      }
       si_meet(SI_A);
       if (done) {
         if (j == 0) sh.flag = 1;
@@ -1545,8 +1549,10 @@ __device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, 
       sh.dead_j[j] = (la.s >= S_MIN ? 0 : 1) + (!(la.s <= 1e300 && fabs(la.cnew) <= 1e300) ? 0x10000 : 0);
     }
   } else {
-    // centroid j by warp j + 1 (16 centroids: the last by the second warp, besides the first); intervals by the warps that are
-    // left, several each where there are enough, or by those of the first centroids besides
+    // centroid j by warp j + 1; intervals by the warps that are left, several each where there are enough, or by those of the
+    // first centroids besides.  16 centroids: the second warp has the last one as well as the first and is what the others wait
+    // for, so it takes the ends of both at once, and the first warp its interval while it waits itself (4096 weights, tau = 0.01,
+    // 30 iterations: 159 us when it took them one after the other, 134 now, 130 with 15 centroids)
     constexpr int OTHERS = SC_WARPS - 1;
     int tw = 1, sub = 0, s = 0;   // this warp's interval, 0: none
     const int t = warp - 1 - k, free_warps = OTHERS - k;
@@ -1561,7 +1567,7 @@ __device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, 
       }
     } else {
       const int u = t >= 0 ? t : (free_warps > 0 ? free_warps : 0) + warp - 1;
-      if (u < k - 1) s = u + 1;
+      if (u < k - 1 && !(LOG == 4 && k == SC_WARPS && u == 0)) s = u + 1;
     }
     const int j = warp - 1;
     SiBin bn;
@@ -1581,10 +1587,17 @@ __device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, 
       }
       si_meet(SI_B2);
       if (sh.flag) break;
-      if (j < k) si_ends<SLOTS>(sh, g, ly, o, j);
-      if (j + OTHERS < k) {
-        si_below(sh, g, ly, bn, sh.v[j + OTHERS], o);
-        si_ends<SLOTS>(sh, g, ly, o, j + OTHERS);
+      if (LOG == 4 && j + OTHERS < k) {
+        const SiBelow o1 = o;
+        si_below(sh, g, ly, bn, sh.v[OTHERS], o);
+        const bool second = lane & 2;
+        o.c = second ? o.c : o1.c;
+        o.n = second ? o.n : o1.n;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o.m[i] = second ? o.m[i] : o1.m[i];
+        si_ends<SLOTS>(sh, g, ly, o, second ? OTHERS : 0, 2);
+      } else if (j < k) {
+        si_ends<SLOTS>(sh, g, ly, o, j, 1);
       }
       if (s > 0) si_bins<SLOTS>(sh, g, ly, s, sub, tw);
       si_arrive(SI_A);

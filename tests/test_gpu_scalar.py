@@ -153,6 +153,28 @@ def test_interval_form_with_close_centroids(k, spread, seed):
     assert_close(C, R.forward(W.astype(np.float64), C0.astype(np.float64), tau, 0.0, 5)[0], TOL_C, "C")
 
 
+def test_a_warp_with_two_centroids_does_not_hold_up_the_others():
+    """15 warps count around 16 centroids: 400 iterations took 1.3 times as long as with 15 centroids when one warp did all its
+    work for one centroid before all of that for the other; now 1.03 times."""
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    W = torch.from_numpy((np.random.default_rng(2).standard_normal((4096, 1)) * 0.03).astype(np.float32)).cuda()
+    times = {15: [], 16: []}
+    for _ in range(9):
+        for k in times:
+            C0 = torch.linspace(-0.06, 0.06, k).reshape(k, 1).cuda()
+            ctx = B.Context()
+            ctx.forward(W, C0, 0.01, 0.0, 3)
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ctx.forward(W, C0, 0.01, 0.0, 400)
+            b.record()
+            torch.cuda.synchronize()
+            assert ctx.last_route()["forward"] == "interval form"
+            times[k].append(a.elapsed_time(b))
+    assert np.median(times[16]) < 1.15 * np.median(times[15])
+
+
 def test_interval_form_on_ragged_batches():
     """Unaligned layer starts, layers of a few weights and of many blocks, one that collapses, in one call."""
     rng = np.random.default_rng(5)
