@@ -1393,13 +1393,23 @@ __device__ __forceinline__ void si_bins(ScShared& sh, const ScGrid& g, const ScL
     b0 = b0 < cl + 1 ? cl + 1 : (b0 < cr ? b0 : cr);
     b1 = b1 < cl + 1 ? cl + 1 : (b1 < cr ? b1 : cr);
     const double slope = (double)ly.slope, z1 = g.hc * slope, z0 = (g.ctr0 - even) * slope, x0 = g.ctr0 - v0;
-    for (int b = b0 + sub * 32 + lane; b < b1; b += 32 * tw) {
+    const float* r = ly.rec.r;
+    const int st = ly.rec.stride, step = 32 * tw;
+    auto add = [&](int b) {
       const double bd = (double)b;
-      const float* r = ly.rec.r + b;
-      const int st = ly.rec.stride;
       const ScCoef c = sc_coef((float)fma(bd, z1, z0));
-      sc_bin_sums<false, float>(c, g.eta, r[0], r[st], r[2 * st], r[3 * st], r[4 * st], fma(bd, g.hc, x0), g.hc, acc);
-    }
+      sc_bin_sums<false, float>(c, g.eta, r[b], r[st + b], r[2 * st + b], r[3 * st + b], r[4 * st + b], fma(bd, g.hc, x0), g.hc, acc);
+    };
+    int b = b0 + sub * 32 + lane;
+    // where a lane has more than four (a cold softmax: the zone holds up to 390) two at a time, as one is a chain of some hundred
+    // cycles: 21 layers of a ResNet-18, tau = 5e-4, k = 7, 30 iterations 515 us one by one, 494 so.  (9 to 16 centroids gain 3 %
+    // there and lose 1 % where an interval has few bins.)
+    if (SLOTS > 3 && b1 - b0 > 4 * step)
+      for (; b + step < b1; b += 2 * step) {
+        add(b);
+        add(b + step);
+      }
+    for (; b < b1; b += step) add(b);
     if (sub == 0 && lane < 2) {
       // outside it: lambda = 1 left of it, mu = 1 right of it
       const int lo = lane ? b1 : cl + 1, hi = lane ? cr : b0;
@@ -1557,13 +1567,17 @@ __device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, 
     int tw = 1, sub = 0, s = 0;   // this warp's interval, 0: none
     const int t = warp - 1 - k, free_warps = OTHERS - k;
     if (free_warps >= k - 1) {
-      if (k > 1) {
-        tw = free_warps / (k - 1);
-        tw = tw > SLOTS - 2 ? SLOTS - 2 : tw;
-        if (t >= 0 && t < (k - 1) * tw) {
-          s = t / tw + 1;
-          sub = t % tw;
+      // (warps that do not go round: to the outer intervals, which hold the most bins)
+      int first = 0;
+      for (int i = 0; i < k - 1; ++i) {
+        int n = free_warps / (k - 1) + (i < free_warps % (k - 1) ? 1 : 0);
+        n = n > SLOTS - 2 ? SLOTS - 2 : n;
+        if (t >= first && t < first + n) {
+          s = (i & 1) ? k - 1 - (i >> 1) : 1 + (i >> 1);
+          sub = t - first;
+          tw = n;
         }
+        first += n;
       }
     } else {
       const int u = t >= 0 ? t : (free_warps > 0 ? free_warps : 0) + warp - 1;

@@ -153,6 +153,16 @@ def test_interval_form_with_close_centroids(k, spread, seed):
     assert_close(C, R.forward(W.astype(np.float64), C0.astype(np.float64), tau, 0.0, 5)[0], TOL_C, "C")
 
 
+# a softmax so cold that an interval holds up to 390 bins which count: 1 to 3 warps for each, some intervals with a warp more than
+# others, bins two at a time and one by one
+@pytest.mark.parametrize("k", [2, 3, 4, 5, 6, 7, 8, 9, 13, 15, 16])
+def test_interval_form_with_many_bins_in_an_interval(k):
+    rng = np.random.default_rng(k)
+    W = (rng.standard_normal((120001, 1)) * 0.06).astype(np.float32)
+    C0 = np.linspace(-0.15, 0.16, k).astype(np.float32).reshape(k, 1) if k < 9 else rng.choice(W[:, 0], k, replace=False).reshape(k, 1)
+    check(W, C0, float(np.float32(3e-4)), 6, 5, alpha=0.5)
+
+
 def test_a_warp_with_two_centroids_does_not_hold_up_the_others():
     """15 warps count around 16 centroids: 400 iterations took 1.3 times as long as with 15 centroids when one warp did all its
     work for one centroid before all of that for the other; now 1.03 times."""
