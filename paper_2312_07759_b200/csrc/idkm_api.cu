@@ -832,14 +832,18 @@ static int try_scalar_loop(idkm_ctx* ctx, const WorkspaceLayout& wl, const PassP
     return 1;
   // Few weights and a cold softmax: the bins are nearly as many as the weights, and summarising them costs more than the
   // iterations save.  What counts is tau against the weights' spread, which only the device knows: the bounds are absolute, for
-  // weights of the order of 0.05, and a layer in other units may take the slower of two right answers.  (30 iterations and the
-  // Jacobian-free backward, spread 0.03, one-launch loop over the weights against this one: m = 4096, k = 4: tau = 0.05 128 against
-  // 115 us, 0.01 103 against 119, 5e-4 104 against 146; m = 8192, k = 16: 5e-4 185 against 222, 2e-3 faster here.)
-  const bool cold = (ctx->m_total <= 4096 && ctx->k <= 4 && ctx->tau < 0.03f) || (ctx->m_total <= 16384 && ctx->k <= 16 && ctx->tau < 1e-3f);
-  if (ctx->n_layers == 1 && !ctx->in_groups && cold) return 1;
+  // weights of the order of 0.05, and a layer in other units may take the slower of two right answers.  (us, 30 iterations and the
+  // Jacobian-free backward, spread 0.03, one-launch loop over the weights against this one.  m = 2048, k = 4: tau = 1e-3 89 and 103,
+  // 0.01 89 and 87; k = 8: 5e-4 123 and 149, 1e-3 123 and 124.  m = 4096, k = 4: 1e-3 103 and 107, 5e-3 103 and 89; k = 8: 5e-4 150
+  // and 155, 7e-4 150 and 140.  m = 8192, k = 4: 3e-4 150 and 156, 5e-4 150 and 134; k = 12: 3e-4 185 and 216, 5e-4 185 and 175;
+  // k = 16: 5e-4 185 and 193, 7e-4 185 and 177.  5 iterations, m = 8192, k = 8: 5e-4 73 and 89, 1e-3 73 and 75.)
+  float below = ctx->m_total > 2048 && max_iter >= 20 ? (ctx->m_total > 4096 && ctx->k <= 12 ? 5e-4f : 7e-4f) : 1e-3f;
+  if (ctx->k <= 4 && ctx->m_total <= 4096) below = ctx->m_total <= 2048 ? 0.03f : 2.5e-3f;
+  if (ctx->n_layers == 1 && !ctx->in_groups && ctx->m_total <= 16384 && ctx->k <= 16 && ctx->tau < below) return 1;
   // Few iterations of a small codebook do not pay for the bins either.  (Forward and implicit backward of 20 steps, over the pairs
-  // and here, k = 4, 4 iterations: m = 36864 90 and 121 us, 1 M 129 and 143, 16 M 433 and 506; 6 iterations 100 and 124, 143 and 148, 502
-  // and 517; k = 16, 4 iterations, 1 M 227 and 166, 16 M 1611 and 576.)
+  // and here, k = 4, 4 iterations: m = 36864 71 and 93 us, 1 M 107 and 117, 16 M 407 and 489; 6 iterations 80 and 97, 123 and 121, 475
+  // and 497; k = 8, 4 iterations: 93 and 97, 132 and 125, but 16 M 814 and 509: from 4 M weights on 5 to 8 centroids would gain here.
+  // k = 16, 4 iterations, 1 M 204 and 132, 16 M 1587 and 547.)
   if (max_iter <= 4 && ctx->k <= 8) return 1;
   for (int l = 0; l < ctx->n_layers; ++l)
     if (ctx->row_off[l + 1] - ctx->row_off[l] > 0x7fffffffLL) return 1;

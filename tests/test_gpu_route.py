@@ -66,3 +66,26 @@ def test_few_iterations_do_without_bins(k, iters, forward):
     ctx.set_forward_loop(1)
     ref = ctx.forward(W, W[:k].contiguous(), 0.01, 0.0, iters).C
     assert float((C - ref).norm() / ref.norm()) < 1e-5
+
+
+# either side of the lines between the loop over few cold weights and the interval form: rows, centroids, iterations, tau
+@pytest.mark.parametrize("m,k,iters,tau,forward", [
+    (2048, 4, 30, 0.029, "one-launch loop"), (2048, 4, 30, 0.031, "interval form"), (2049, 4, 30, 0.0024, "one-launch loop"),
+    (2049, 4, 5, 0.0026, "interval form"), (4096, 4, 30, 0.0024, "one-launch loop"), (4096, 2, 30, 0.0026, "interval form"),
+    (2048, 5, 30, 9.9e-4, "one-launch loop"), (2048, 16, 30, 1.1e-3, "interval form"), (2049, 5, 30, 6.9e-4, "one-launch loop"),
+    (4096, 16, 20, 7.1e-4, "interval form"), (4096, 16, 19, 7.1e-4, "one-launch loop"), (4097, 4, 20, 5e-4, "interval form"),
+    (4097, 12, 20, 4.9e-4, "one-launch loop"), (16384, 12, 19, 9.9e-4, "one-launch loop"), (16384, 13, 20, 6.9e-4, "one-launch loop"),
+    (16384, 16, 20, 7.1e-4, "interval form"), (16385, 3, 20, 1e-4, "interval form"), (16384, 17, 20, 1e-4, "interval form"),
+])
+def test_few_cold_weights(m, k, iters, tau, forward):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(m + k)
+    W = torch.randn(m, 1, device="cuda", generator=g) * 0.03
+    C0 = torch.sort(W[:, 0])[0][((torch.arange(k, device="cuda") + 0.5) * m / k).long()].reshape(k, 1).contiguous()
+    ctx = B.Context()
+    C = ctx.forward(W, C0, tau, 0.0, iters).C
+    assert ctx.last_route()["forward"] == forward
+    ctx.set_forward_loop(1)
+    ref = ctx.forward(W, C0, tau, 0.0, iters).C
+    assert float((C - ref).norm() / ref.norm()) < 1e-5
