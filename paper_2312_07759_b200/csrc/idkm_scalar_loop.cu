@@ -353,19 +353,16 @@ __device__ __forceinline__ uint4 sc_load8(const unsigned short* grouped, long lo
   return make_uint4(x[0], x[1], x[2], x[3]);
 }
 
-// A fine bin as a warp sees it: up to SC_HEAD of its weights in registers (kept from one iteration to the next while the
-// centroid stays in the bin), the rest read again every time.
+// A fine bin as a warp of the last evaluation sees it: up to SC_HEAD of its weights in registers.
 constexpr int SC_HEAD = 248;
 struct ScBin {
-  int f;                  // fine bin, -1: none
   int groups;             // of 32 weights in pe
   int pe[8];              // places (40001: no weight)
   long long t0, t1;       // the rest, as elements of `grouped` (t0 is a multiple of 8)
 };
 // (n warps share a bin: this one takes share `sub`, boundaries at multiples of 8)
-__device__ __forceinline__ void sc_bin_load(const ScLayer& ly, int f, unsigned int e0, unsigned int e1, int sub, int n, ScBin& bn) {
+__device__ __forceinline__ void sc_bin_load(const ScLayer& ly, unsigned int e0, unsigned int e1, int sub, int n, ScBin& bn) {
   const int lane = threadIdx.x & 31;
-  bn.f = f;
   long long A0 = ly.row0 + e0, A1 = ly.row0 + e1;
   if (n > 1) {
     const long long len = A1 - A0, b = A0, e = A1;
@@ -552,16 +549,17 @@ __device__ __noinline__ void sc_stop_test(ScShared& sh, const ScalarParams& sp, 
   }
   }
 
-// First half of an evaluation: the weights of every centroid's fine bin below it.  Up to 16 centroids: a warp (or two) each;
-// `keep` is the bin this warp had in the evaluation before, in registers.  More: eight lanes each, eight places per load.
-__device__ __forceinline__ void sc_scan_warps(ScShared& sh, const ScLayer& ly, ScBin& keep, bool full) {
+// First half of an evaluation: the weights of every centroid's fine bin below it.  Up to 16 centroids (the last evaluation only:
+// the others are sc_iterate's): a warp (or two) each.  More: eight lanes each, eight places per load.
+__device__ __forceinline__ void sc_scan_warps(ScShared& sh, const ScLayer& ly, bool full) {
   const int lane = threadIdx.x & 31, t = threadIdx.x >> 5;
   if (t >= ly.k << ly.wl) return;
   const int j = t >> ly.wl, sub = t & ((1 << ly.wl) - 1);
   const int f = sh.fb[j];
-  if (keep.f != f) sc_bin_load(ly, f, ly.fstart[f], ly.fstart[f + 1], sub, 1 << ly.wl, keep);
+  ScBin bn;
+  sc_bin_load(ly, ly.fstart[f], ly.fstart[f + 1], sub, 1 << ly.wl, bn);
   double s[5];
-  sc_bin_below(sh.ly, keep, sh.pv[j], full, s);
+  sc_bin_below(sh.ly, bn, sh.pv[j], full, s);
   if (lane == 0) {
 #pragma unroll
     for (int i = 0; i < 5; ++i) sh.bs[t][i] = s[i];
@@ -820,10 +818,10 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
 
 // Both halves; the last warp first runs the stop test of the M-step before (`test` = its number, 0: none).
 template <bool EXTRA>
-__device__ __forceinline__ void sc_evaluate(ScShared& sh, const ScLayer& ly, ScBin& keep, const ScalarParams& sp, int layer, int test) {
+__device__ __forceinline__ void sc_evaluate(ScShared& sh, const ScLayer& ly, const ScalarParams& sp, int layer, int test) {
   const bool full = sc_full(sh.g);
   if (test > 0 && threadIdx.x >= SC_T - 32) sc_stop_test(sh, sp, layer, test);
-  if (ly.k <= SC_WARPS) sc_scan_warps(sh, ly, keep, full);
+  if (EXTRA && ly.k <= SC_WARPS) sc_scan_warps(sh, ly, full);
   else sc_scan_quarters(sh, full);
   __syncthreads();
   sc_sum_intervals<EXTRA>(sh, ly, full);
@@ -1622,11 +1620,11 @@ __device__ __forceinline__ int sc_iterate(ScShared& sh, const ScalarParams& sp, 
   return sh.steps;
 }
 
-constexpr int SI_T = 1024, SI_WARPS = SI_T / 32;
+constexpr int SC_INIT_T = 1024, SC_INIT_WARPS = SC_INIT_T / 32;
 // ---- first launch: layer states, working centroids, counters to zero, value range of the weights ----
-__global__ void __launch_bounds__(SI_T, 1) idkm_scalar_init(const __grid_constant__ ScalarParams sp) {
-  __shared__ float red_lo[SI_WARPS], red_hi[SI_WARPS];
-  __shared__ unsigned int red_z[SI_WARPS];
+__global__ void __launch_bounds__(SC_INIT_T, 1) idkm_scalar_init(const __grid_constant__ ScalarParams sp) {
+  __shared__ float red_lo[SC_INIT_WARPS], red_hi[SC_INIT_WARPS];
+  __shared__ unsigned int red_z[SC_INIT_WARPS];
   grid_dependency_sync();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = sp.k;
   const int layer = sc_layer_of_block(sp, (int)blockIdx.x);
@@ -1644,12 +1642,12 @@ __global__ void __launch_bounds__(SI_T, 1) idkm_scalar_init(const __grid_constan
       sp.p.st[layer] = s;
     }
   }
-  for (int i = (int)blockIdx.x * SI_T + tid; i < sp.n_group_rows; i += (int)gridDim.x * SI_T) sp.p.gtick[i] = 0u;
+  for (int i = (int)blockIdx.x * SC_INIT_T + tid; i < sp.n_group_rows; i += (int)gridDim.x * SC_INIT_T) sp.p.gtick[i] = 0u;
   for (int h = 0; h < 2; ++h)
-    for (int i = (int)blockIdx.x * SI_T + tid; i < sp.p.n_pair_ticks[h]; i += (int)gridDim.x * SI_T) sp.p.pair_ticks[h][i] = 0u;
+    for (int i = (int)blockIdx.x * SC_INIT_T + tid; i < sp.p.n_pair_ticks[h]; i += (int)gridDim.x * SC_INIT_T) sp.p.pair_ticks[h][i] = 0u;
   const int cap = sp.fine_off[layer + 1] - sp.fine_off[layer];
   if (NB > 1)
-    for (int i = b * SI_T + tid; i < cap; i += NB * SI_T) sp.p.gcount[sp.fine_off[layer] + i] = 0u;
+    for (int i = b * SC_INIT_T + tid; i < cap; i += NB * SC_INIT_T) sp.p.gcount[sp.fine_off[layer] + i] = 0u;
   const long long r0 = m * b / NB, r1 = m * (b + 1) / NB;
   float lo = __int_as_float(0x7f800000), hi = -lo;
   int bad = 0;
@@ -1662,14 +1660,14 @@ __global__ void __launch_bounds__(SI_T, 1) idkm_scalar_init(const __grid_constan
     hi = z ? hi : fmaxf(hi, w);
   };
   long long r = r0 + tid;
-  for (; r + 7 * SI_T < r1; r += 8 * SI_T) {
+  for (; r + 7 * SC_INIT_T < r1; r += 8 * SC_INIT_T) {
     float w[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = __ldg(Wl + r + i * SI_T);
+    for (int i = 0; i < 8; ++i) w[i] = __ldg(Wl + r + i * SC_INIT_T);
 #pragma unroll
     for (int i = 0; i < 8; ++i) take(w[i]);
   }
-  for (; r < r1; r += SI_T) take(__ldg(Wl + r));
+  for (; r < r1; r += SC_INIT_T) take(__ldg(Wl + r));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -1830,12 +1828,6 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
   };
   constexpr bool quick = !DIRECT && LOG > 0 && (1 << LOG) <= SI_K;   // the iterations are sc_iterate's
   if constexpr (!quick) tables();
-  ScBin keep;
-  keep.f = -1;
-  keep.groups = 0;
-  keep.t0 = keep.t1 = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) keep.pe[i] = 40001;
   __syncthreads();
 
   int it = 0;
@@ -1851,7 +1843,7 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
         return;
       }
     } else {
-      sc_evaluate<false>(sh, ly, keep, sp, layer, it);
+      sc_evaluate<false>(sh, ly, sp, layer, it);
       __syncthreads();
     }
     if (sh.done) break;
@@ -1918,7 +1910,7 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
     }
     if (!leader) return;
   } else {
-    sc_evaluate<true>(sh, ly, keep, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
+    sc_evaluate<true>(sh, ly, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
   }
   __syncthreads();
   if (tid < kw * 32) {
@@ -2400,7 +2392,7 @@ __global__ void __launch_bounds__(SC_T, 1) idkm_scalar_loop(const __grid_constan
 }
 
 cudaError_t launch_scalar_init(const ScalarParams& sp, int grid, cudaStream_t stream) {
-  idkm_scalar_init<<<grid, SI_T, 0, stream>>>(sp);
+  idkm_scalar_init<<<grid, SC_INIT_T, 0, stream>>>(sp);
   return cudaGetLastError();
 }
 
