@@ -115,12 +115,14 @@ def test_interval_form_with_the_most_bins(sizes):
 
 # n nearly equal weights around a centroid: a fine bin of n weights (one load a lane and several, what stays in registers and what
 # does not), its start at any element of a layer with an odd start, the last weights of all; 1 to 16 centroids (two of them
-# with one warp), bins split into one, 8 and more than 64 (sums of four, two and one powers of the place)
+# with one warp), bins split into one, 8 and more than 64 (sums of four and of one power of the place)
 @pytest.mark.parametrize("n,k,m,tau,where", [
     (1, 1, 5000, 0.01, "inside"), (57, 2, 20011, 0.01, "inside"), (63, 3, 20011, 5e-4, "inside"), (64, 4, 20011, 0.01, "last"),
     (65, 5, 20011, 0.01, "inside"), (249, 8, 20011, 0.004, "last"), (257, 9, 20010, 0.01, "inside"), (505, 15, 20011, 0.01, "last"),
     (512, 16, 20011, 0.01, "inside"), (513, 4, 20011, 5e-4, "last"), (521, 16, 1 << 20, 0.05, "inside"), (1537, 7, 20011, 0.01, "last"),
     (2559, 16, 300001, 0.01, "inside"), (2571, 6, 300001, 0.02, "last"), (4000, 16, 1 << 20, 0.05, "last"), (4100, 4, 1 << 20, 0.05, "inside"),
+    (9300, 5, 5 << 20, 0.05, "inside"), (19000, 16, 5 << 20, 0.05, "last"), (12000, 2, 5 << 20, 0.01, "inside"),
+    (11000, 6, 5 << 20, 0.002, "inside"),   # (sums taken up in between)
 ])
 def test_interval_form_with_a_crowded_bin(n, k, m, tau, where):
     rng = np.random.default_rng(n + k)
@@ -183,6 +185,42 @@ def test_a_warp_with_two_centroids_does_not_hold_up_the_others():
             assert ctx.last_route()["forward"] == "interval form"
             times[k].append(a.elapsed_time(b))
     assert np.median(times[16]) < 1.15 * np.median(times[15])
+
+
+# where the stop falls decides which of the block's meetings the first warp still goes to: after the first step, on the last
+# iteration but one and on the last, with room left, and never; codebooks with and without warps of their own for the intervals.
+# (at most 4 iterations of up to 8 centroids take another loop, one centroid stands still after one step)
+@pytest.mark.parametrize("k,stop,caps", [
+    (1, 2, (5, 6, 40)), (4, 4, (5, 6, 40)), (4, 5, (5, 6, 7)), (8, 1, (5,)), (8, 7, (7, 8, 9, 40)), (9, 1, (2, 3, 9)), (15, 2, (2, 3, 4)),
+    (16, 1, (2, 3, 40)), (16, 2, (2, 3, 4)), (16, 9, (9, 10, 11, 40)),
+])
+@pytest.mark.parametrize("m", [20011, 400003])
+def test_interval_form_stops_where_it_should(k, stop, caps, m):
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    W = torch.from_numpy((np.random.default_rng(m + k).standard_normal((m, 1)) * 0.03).astype(np.float32)).cuda()
+    C0 = torch.linspace(-0.05, 0.06, k).reshape(k, 1).cuda()
+
+    def call(tol, cap):
+        ctx = B.Context()
+        fr = ctx.forward(W, C0, 0.01, tol, cap)
+        torch.cuda.synchronize()
+        assert ctx.last_route()["forward"] == "interval form"
+        return ctx.info()[0], ctx.history(0), fr.C.cpu().numpy(), fr.Wq.cpu().numpy()
+
+    res = call(0.0, 40)[1]
+    assert all(res[stop - 1] < r for r in res[:stop - 1])
+    tol = float(np.float32(res[stop - 1] * (1 + 1e-4) + 1e-30))
+    assert all(tol < r for r in res[:stop - 1])
+    for cap in caps:
+        info, hist, C, Wq = call(tol, cap)
+        assert (info.status, info.fwd_iters) == (B.OK, stop) and np.array_equal(hist, res[:stop])
+        if not (k <= 8 and stop <= 4):
+            _, _, Cs, Wqs = call(0.0, stop) if stop > 1 else (None, None, C, Wq)
+            assert np.array_equal(C, Cs) and np.array_equal(Wq, Wqs)
+    if k > 1:
+        info, hist, _, _ = call(float(np.float32(min(res) * 0.5)), max(caps))
+        assert (info.status, info.fwd_iters) == (B.MAXITER, max(caps)) and np.array_equal(hist, res[:max(caps)])
 
 
 def test_interval_form_on_ragged_batches():
