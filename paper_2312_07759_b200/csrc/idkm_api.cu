@@ -797,7 +797,7 @@ static void scalar_params(const idkm_ctx* ctx, const WorkspaceLayout& wl, const 
         const long long r = ctx->row_off[o + 1] - ctx->row_off[o];
         larger += (r > rows || (r == rows && o < l));
       }
-    sp->fine_off[l + 1] = sp->fine_off[l] + scalar_fine_bins(rows, larger, ctx->row_off[L]);
+    sp->fine_off[l + 1] = sp->fine_off[l] + scalar_fine_bins(rows, larger, ctx->in_groups ? ctx->batch_m : ctx->row_off[L]);
   }
   for (int l = L + 1; l <= MAX_LAYERS; ++l) sp->fine_off[l] = sp->fine_off[L];
 }

@@ -84,3 +84,25 @@ def test_a_group_takes_the_routes_of_the_whole_call(d, k, rows, tau):
     groups = n[0] / n[1]
     assert groups == int(groups) and 2 <= groups <= 4
     assert [i.status for i in out[0][4]] == [i.status for i in out[1][4]]
+
+
+def test_a_group_uses_the_bins_of_the_whole_call():
+    """Two large layers of scalar weights, neither of which has most of the call: a group of one of them must not take the finer
+    bins of a call of its own (the centroids would differ in their last bits)."""
+    import torch
+    from paper_2312_07759_b200 import binding as B
+    rng = np.random.default_rng(4)
+    rows = [(10 << 20) + 5, (10 << 20) + 3]
+    offs = [0, rows[0], sum(rows)]
+    W = rng.standard_normal((offs[-1], 1), dtype=np.float32) * np.float32(0.03)
+    G = np.full_like(W, 0.01)
+    C0 = np.concatenate([np.linspace(-0.08, 0.07, 12, dtype=np.float32)] * 2).reshape(-1, 1)
+    tau = (float(W.max()) - float(W.min())) / 140.5 / 0.17
+    ctx = B.Context()
+    n0 = ctx.launches
+    C = ctx.quantize_host(W, C0, G, tau, 0.0, 20, B.JFB, 0.0, 0, 1.0, layer_offsets=offs)[0]
+    assert ctx.launches - n0 >= 8           # (two groups)
+    ref = B.Context().forward(torch.from_numpy(W).cuda(), torch.from_numpy(C0).cuda(), tau, 0.0, 20, layer_offsets=offs).C
+    assert np.array_equal(C, ref.cpu().numpy())
+    alone = [B.Context().forward(torch.from_numpy(W[a:b]).cuda(), torch.from_numpy(C0[:12]).cuda(), tau, 0.0, 20).C for a, b in zip(offs, offs[1:])]
+    assert not np.array_equal(C, torch.cat(alone).cpu().numpy())
