@@ -12,10 +12,11 @@
 // integers, so results are reproducible although the grouping uses atomic counters.
 //
 // What bounds it.  Building: the grouping pass stores two bytes per weight to scattered places, 67 cycles a warp store
-// (110 us per 11.7 M weights on all SMs).  Iterating: the chain of one block a layer, 1.7 us at k <= 4 to 6 us, whatever the
-// number of weights (sc_iterate up to 16 centroids).  Measured, loop with the summary against one that
-// visits the pairs: 21 layers of a ResNet-18, k = 4, 50 iterations 352 against 1473 us; k = 8, tau = 5e-4, 30 iterations 380
-// against 1268; 16 M weights, k = 16, 100 iterations 1.09 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 68
+// (110 us per 11.7 M weights on all SMs).  Iterating: the chain of one block a layer, and where the centroids' fine bins hold
+// thousands of weights, counting these: up to 16 centroids (sc_iterate) 1.5 us for 4096 weights, k = 4, to 6.0 for 16 M, k = 16;
+// more 4.0 (36864, k = 17) to 25 and 92 (16 M, k = 32 and 256).  Measured, loop with the summary against one that
+// visits the pairs: 21 layers of a ResNet-18, k = 4, 50 iterations 312 against 1473 us; k = 8, tau = 5e-4, 30 iterations 359
+// against 1268; 16 M weights, k = 16, 100 iterations 0.87 against 10.4 ms; 4096 weights, k = 4, tau = 0.05, 30 iterations 71
 // against 112.
 //
 // Layers that bins do not suit -- tau below 1 / 5700 of the weights' range (1 / 2800 in layers beyond the eighth), which an outlier
@@ -69,7 +70,7 @@ __device__ ScGrid sc_make_grid(float lo, float hi, double tau, long long m, int 
   if (hc < range / (double)(cap - 8)) hc = range / (double)(cap - 8);
   if (hc > range) hc = range;
   if (hc < hmin) hc = hmin;
-  // fine bins: about 64 weights each; 16 to a coarse bin (see sc_bin_below) while they hold 8 weights; as many as the
+  // fine bins: about 64 weights each; 16 to a coarse bin (see sc_full) while they hold 8 weights; as many as the
   // workspace holds
   const long long nc0 = (long long)(range / hc) + 5;
   long long want = m / 64 < 512 ? 512 : m / 64;
@@ -135,8 +136,8 @@ constexpr double SC_S4 = 17592186044416.0 * SC_S1 * SC_S1 * SC_S1 * SC_S1;
 constexpr int SC_CHUNK = 8192;   // elements whose 32-bit integer sums cannot overflow
 // Which powers of the place matter: a fine bin is 1 / F of a coarse bin, so the fourth and third power of a place inside it
 // change the interval's sums by less than 1e-8 from F = 64 on, and so does the square in the one bin that is split.  With
-// fewer fine bins all four do: 3000 of 4096 weights in a tenth of one coarse bin, F = 8, five iterations from 16 centroids within
-// the same tenth of it, centroids against float64: 2e-6 with all powers, 3e-5 without the third and the fourth.
+// fewer fine bins all four do: 3000 of 4096 weights in a quarter of one coarse bin, F = 8, five iterations from 16 centroids in a
+// third of it, centroids against float64: 2e-6 with all powers, 3e-5 without the third and the fourth.
 __device__ __forceinline__ bool sc_full(const ScGrid& g) { return g.F < 64; }
 
 // Moments about the coarse bin's centre, in units of the coarse width, of n weights of fine bin kf (0 .. F - 1) whose
@@ -1159,10 +1160,12 @@ __device__ __noinline__ bool sd_sums(ScShared& sh, const ScalarParams& sp, int l
 // whole bins of an interval; at the third meeting (A) the first warp has all sums.  What a warp does is the same in every
 // iteration, and a centroid's fine bin (up to SI_HEAD of its places, and its record) stays in its warp's registers, unless the
 // warp has two centroids (16 of them).  Nothing in the loop may live in local memory: with the shared memory the block takes the L1 cache holds none of it, and every access
-// is a trip to L2; and a load whose value is used before the next one is issued is one more such trip.  Cycles an iteration,
-// before (counts, ends and M-step one after the other between meetings of the block) and now: 4096 weights, k = 4 5500 and 3300;
-// 36864, k = 8 6700 and 4600; 2.4 M, k = 4 8000 and 5900; 16 M, k = 16 24000 and 19800 (the fine bins hold thousands
-// of weights; with twice as many of them about 16000).
+// is a trip to L2; and a load whose value is used before the next one is issued is one more such trip.  Cycles an iteration, in
+// brackets the loop in which the whole block goes through counts, ends and M-step one after the other: 4096 weights, k = 4 3000
+// (5500); 36864, k = 8 3800 (6700), k = 15 and 16 5400 and 5600; 2.4 M, k = 4 3600 (8000), k = 8 at tau = 5e-4 6900; 16 M, k = 4
+// 6400, k = 16 11800 (24000 with half as many fine bins): there the centroids' bins hold 2000 weights and more.  Under ncu 36864
+// weights, k = 16: issue slots 36 % busy, a warp waits at the meetings for 2.5 cycles of every instruction issued, for fixed
+// latencies 2.1, for shared memory 1.5; no access to local memory.
 constexpr int SI_WORDS = 8, SI_HEAD = 64 * SI_WORDS;
 constexpr int SI_A = 2, SI_B1 = 3, SI_B2 = 4;   // hardware barriers
 __device__ __forceinline__ void si_arrive(int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(SC_T) : "memory"); }
