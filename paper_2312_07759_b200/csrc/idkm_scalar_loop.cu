@@ -818,11 +818,11 @@ __device__ __forceinline__ void sc_sum_intervals(ScShared& sh, const ScLayer& ly
 }
 
 // Both halves; the last warp first runs the stop test of the M-step before (`test` = its number, 0: none).
-template <bool EXTRA>
+template <bool EXTRA, bool WARPS>
 __device__ __forceinline__ void sc_evaluate(ScShared& sh, const ScLayer& ly, const ScalarParams& sp, int layer, int test) {
   const bool full = sc_full(sh.g);
   if (test > 0 && threadIdx.x >= SC_T - 32) sc_stop_test(sh, sp, layer, test);
-  if (EXTRA && ly.k <= SC_WARPS) sc_scan_warps(sh, ly, full);
+  if constexpr (WARPS) sc_scan_warps(sh, ly, full);
   else sc_scan_quarters(sh, full);
   __syncthreads();
   sc_sum_intervals<EXTRA>(sh, ly, full);
@@ -1846,7 +1846,7 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
         return;
       }
     } else {
-      sc_evaluate<false>(sh, ly, sp, layer, it);
+      sc_evaluate<false, quick>(sh, ly, sp, layer, it);
       __syncthreads();
     }
     if (sh.done) break;
@@ -1913,7 +1913,7 @@ __device__ __forceinline__ void sc_rest(ScShared& sh, const ScalarParams& sp, in
     }
     if (!leader) return;
   } else {
-    sc_evaluate<true>(sh, ly, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
+    sc_evaluate<true, quick>(sh, ly, sp, layer, (it == sp.max_iter && !sh.done) ? it : 0);
   }
   __syncthreads();
   if (tid < kw * 32) {
